@@ -75,7 +75,7 @@ WsLayout ws_layout(const Geom& g) {
   const size_t esz = g.f32 ? 4 : 2;
   size_t off = 0;
   l.y_off = off;      off = align_up(off + tiles * g.Nloc * g.d * sizeof(__nv_bfloat16), 256);
-  l.sq_off = off;     off = align_up(off + tiles * g.Nloc * g.Nloc * sizeof(int16_t), 256);
+  l.sq_off = off;     off = align_up(off + tiles * g.Nloc * sq_pitch(g.Nloc) * sizeof(uint16_t), 256);
   l.logits_off = off; off = align_up(off + (size_t)gm.B * gm.P * gm.Dloc * gm.Nloc * sizeof(float), 256);
   l.wts_off = off;    off = align_up(off + (weights_tc_supported(gm) ? weights_tc_scratch_bytes(gm) : 0), 256);
   l.gidx_off = off;   off = align_up(off + (g.global_merge ? (size_t)g.B * g.D * sizeof(int32_t) : 0), 256);
@@ -106,10 +106,10 @@ static cudaError_t do_select(const Geom& g, const void* x, int32_t* idx, char* w
                              cudaStream_t s) {
   const WsLayout l = ws_layout(g);
   __nv_bfloat16* y = (__nv_bfloat16*)(ws + l.y_off);
-  int16_t* sq = (int16_t*)(ws + l.sq_off);
+  uint16_t* sq = (uint16_t*)(ws + l.sq_off);
   cudaError_t e = launch_quantise(g, x, y, s);
   if (e != cudaSuccess) return e;
-  e = gram_tc_supported(g) ? launch_gram_tc(g, y, sq, dev_status, s) : launch_gram_ffma(g, y, sq, s);
+  e = launch_gram_tc(g, y, sq, dev_status, s);
   if (e != cudaSuccess) return e;
   return launch_greedy(g, sq, idx, s);
 }

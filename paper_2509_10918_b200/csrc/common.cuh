@@ -16,6 +16,10 @@ namespace toma {
 // Fixed-point cosine similarity constants (see toma_select in toma.h).
 constexpr double kCosScaleTimesOne = 0.99 * 4096.0;  // token length 0.99 in units of 2^-12
 constexpr int kDiagQ = 4014;                          // rint(0.99^2 * 4096)
+// The similarity matrix in the workspace: entry S + kSqBias (unsigned, below 2^13: |S| <= 4014), rows of sq_pitch()
+// entries (16-byte aligned), 0 behind the tile's tokens.
+constexpr int kSqBias = 4096;
+__host__ __device__ constexpr int sq_pitch(int nloc) { return (nloc + 7) & ~7; }
 constexpr int kMaxNloc = 1024;
 constexpr int kMaxDim = 4096;
 
@@ -71,10 +75,8 @@ cudaError_t raise_dynamic_smem(Kernel kernel, int bytes, std::atomic<unsigned lo
 
 // ---- launchers (each returns cudaGetLastError() of its launches) ----
 cudaError_t launch_quantise(const Geom& g, const void* x, __nv_bfloat16* y, cudaStream_t s);
-cudaError_t launch_gram_ffma(const Geom& g, const __nv_bfloat16* y, int16_t* sq, cudaStream_t s);
-bool gram_tc_supported(const Geom& g);
-cudaError_t launch_gram_tc(const Geom& g, const __nv_bfloat16* y, int16_t* sq, uint32_t* dev_status, cudaStream_t s);
-cudaError_t launch_greedy(const Geom& g, const int16_t* sq, int32_t* idx, cudaStream_t s);
+cudaError_t launch_gram_tc(const Geom& g, const __nv_bfloat16* y, uint16_t* sq, uint32_t* dev_status, cudaStream_t s);
+cudaError_t launch_greedy(const Geom& g, const uint16_t* sq, int32_t* idx, cudaStream_t s);
 // `wu`: where the un-normalised shares A^T go in the weight buffer's layout, or nullptr.
 cudaError_t launch_weights_simt(const Geom& g, const void* x, const int32_t* idx, void* w, void* wu, float* logits,
                                 cudaStream_t s);

@@ -2,8 +2,9 @@
 // greedy selection consumes).  Input is the quantised token directions y (bf16, tile-major
 // [tile][N_loc][d]); every y is k * 2^-12 with an integer k of at most 8 significant bits and
 // |y| < 1, so every partial sum of y_i . y_j is a multiple of 2^-24 below 1 and the fp32
-// accumulation in tensor memory is exact whatever the order.  Output S_q[i][j] =
-// rint(<y_i, y_j> * 4096) as int16, diagonal forced to 4014.
+// accumulation in tensor memory is exact whatever the order.  Output S_q[i][j] + 4096 with S_q[i][j] =
+// rint(<y_i, y_j> * 4096), diagonal forced to 4014 (see sq_pitch() for the layout).  Any N_loc: rows and columns past
+// the tile are zero-filled by TMA and stored as 0 up to the row pitch.
 // grid (tile, 128-row block, column block of <= 256); warp 0 TMA, warp 1 MMA, warps 2..5 epilogue.
 #include "common.cuh"
 #include "tc.cuh"
@@ -25,7 +26,7 @@ struct GramBars {
 
 __global__ void __launch_bounds__(192, 1)
 gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
-               int16_t* __restrict__ sq, int Nloc, int d, int n_cols, uint32_t* dev_status) {
+               uint16_t* __restrict__ sq, int Nloc, int d, int n_cols, uint32_t* dev_status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int a_bytes = 128 * 128, b_bytes = n_cols * 128;
@@ -90,7 +91,8 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
     if (mbar_wait(&bar->done, 0, dev_status, abort_flag)) {
       tc_fence_after();
-      int16_t* row = sq + ((size_t)tile * Nloc + (i < Nloc ? i : 0)) * Nloc + n0;
+      const int pitch = sq_pitch(Nloc);
+      uint16_t* row = sq + ((size_t)tile * Nloc + (i < Nloc ? i : 0)) * pitch + n0;
       for (int j0 = 0; j0 < n_cols; j0 += 32) {
         uint32_t r[32];
         tmem_ld32(taddr + j0, r);
@@ -98,16 +100,18 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         if (i < Nloc) {
 #pragma unroll
           for (int e = 0; e < 32; e += 8) {
-            if (j0 + e >= n_cols) break;
+            if (j0 + e >= n_cols || n0 + j0 + e >= pitch) break;
             uint32_t pk[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
               const int ja = n0 + j0 + e + 2 * u;
-              int lo = __float2int_rn(__uint_as_float(r[e + 2 * u]) * 4096.f);
-              int hi = __float2int_rn(__uint_as_float(r[e + 2 * u + 1]) * 4096.f);
-              if (ja == i) lo = kDiagQ;
-              if (ja + 1 == i) hi = kDiagQ;
-              pk[u] = ((uint32_t)hi << 16) | ((uint32_t)lo & 0xFFFFu);
+              int lo = __float2int_rn(__uint_as_float(r[e + 2 * u]) * 4096.f) + kSqBias;
+              int hi = __float2int_rn(__uint_as_float(r[e + 2 * u + 1]) * 4096.f) + kSqBias;
+              if (ja == i) lo = kDiagQ + kSqBias;
+              if (ja + 1 == i) hi = kDiagQ + kSqBias;
+              if (ja >= Nloc) lo = 0;
+              if (ja + 1 >= Nloc) hi = 0;
+              pk[u] = ((uint32_t)hi << 16) | (uint32_t)lo;
             }
             *reinterpret_cast<uint4*>(row + j0 + e) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
           }
@@ -125,14 +129,8 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 
 }  // namespace
 
-bool gram_tc_supported(const Geom& g) {
-  if (g.Nloc % 16 != 0) return false;
-  if (g.Nloc > 256 && g.Nloc % 256 != 0) return false;
-  return true;
-}
-
-cudaError_t launch_gram_tc(const Geom& g, const __nv_bfloat16* y, int16_t* sq, uint32_t* dev_status, cudaStream_t s) {
-  const int n_cols = g.Nloc > 256 ? 256 : g.Nloc;
+cudaError_t launch_gram_tc(const Geom& g, const __nv_bfloat16* y, uint16_t* sq, uint32_t* dev_status, cudaStream_t s) {
+  const int n_cols = g.Nloc > 256 ? 256 : (g.Nloc + 15) & ~15;  // MMA N: a multiple of 16
   CUtensorMap ta, tb;
   const uint64_t dims[3] = {(uint64_t)g.d, (uint64_t)g.Nloc, (uint64_t)g.B * g.P};
   const uint64_t strides[2] = {(uint64_t)g.d * 2, (uint64_t)g.Nloc * g.d * 2};
@@ -143,7 +141,7 @@ cudaError_t launch_gram_tc(const Geom& g, const __nv_bfloat16* y, int16_t* sq, u
   const int smem = 1024 + kStages * (128 * 128 + n_cols * 128) + 256;
   static std::atomic<unsigned long long> smem_raised{0};
   if (cudaError_t e = raise_dynamic_smem(gram_tc_kernel, 200 * 1024, smem_raised); e != cudaSuccess) return e;
-  dim3 grid(g.B * g.P, (g.Nloc + 127) / 128, g.Nloc / n_cols);
+  dim3 grid(g.B * g.P, (g.Nloc + 127) / 128, (g.Nloc + n_cols - 1) / n_cols);
   const cudaError_t le = launch_dependent(gram_tc_kernel, grid, dim3(192), (size_t)smem, s, ta, tb, sq, g.Nloc, g.d, n_cols, dev_status);
   count_launch();
   return le != cudaSuccess ? le : cudaGetLastError();

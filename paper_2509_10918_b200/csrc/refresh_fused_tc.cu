@@ -5,8 +5,7 @@
 //      Gram products on the tensor cores: S = y y^T (exact in fp32: every partial sum is a multiple of 2^-24
 //      below 1) and G = x x^T, both 64 x 64 in tensor memory;
 //   2. rounds S to the fixed-point S_q in shared memory and runs the greedy rounds on it in ONE warp (two
-//      candidates and two cached maxima per lane: no barrier, no list; a round is a warp reduction, two row
-//      reads, two ballots and a walk over the few columns whose maximum improved);
+//      candidates and two cached maxima per lane, no block barrier; several picks per round: greedy.cuh);
 //   3. takes the logits of Sec. 4.2.1 out of G - the logit of source k and destination i is G[idx_i][k] scaled,
 //      so no second contraction and no gathered copy of the destinations is needed -, softmax over the
 //      destinations per source, row sums per destination in a fixed order, and writes A~^T as hi and lo planes.
@@ -14,9 +13,8 @@
 // longer over it than the kernel takes as a whole).
 // Warp 0, 1: thread = token = tensor-memory lane (warp 0 runs the greedy rounds); warp 2: TMA producer;
 // warp 3: MMA issuer.
-#include <climits>
-
 #include "common.cuh"
+#include "greedy.cuh"
 #include "tc.cuh"
 
 namespace toma {
@@ -51,67 +49,40 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
-// Greedy rounds of Algorithm 2 on a 64 x 64 S_q in shared memory, by one warp.  Lane l owns candidates l and
-// l + 32 (their gains) and the cached maxima m[l], m[l + 32].  Exact integer gains, ties to the lowest index,
-// selected tokens excluded: the same picks as greedy_kernel.
-__device__ __forceinline__ void greedy_one_warp(const int16_t* S, int Dloc, int lane, int* sel, int32_t* out) {
-  const int j0 = lane, j1 = lane + 32;
-  int sum0 = 0, sum1 = 0;
-  for (int i = 0; i < kTok; ++i) {
-    sum0 += S[i * kTok + j0];
-    sum1 += S[i * kTok + j1];
+// Algorithm 2 on a 64 x 64 S_q (biased, two tokens to a word) in shared memory, by one warp; the rounds are
+// greedy.cuh's.  Lane l owns tokens 2 l and 2 l + 1.
+__device__ __forceinline__ void greedy_one_warp(const uint32_t* S, int Dloc, int lane, greedy::Shared<kTok>& sh, int* sel, int32_t* out) {
+  constexpr int kPitchW = kTok / 2;
+  uint32_t sum0 = 0, sum1 = 0;
+#pragma unroll
+  for (int j0 = 0; j0 < kTok; j0 += 8) {
+    uint32_t t = 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) t += S[(j0 + u) * kPitchW + lane];  // eight entries below 2^13 per half: no carry
+    sum0 += t & 0xFFFFu;
+    sum1 += t >> 16;
   }
-  // first pick: argmax of the column sums (they may be negative), lowest index on ties
-  int g = sum0 >= sum1 ? sum0 : sum1, gi = sum0 >= sum1 ? j0 : j1;
-  const int gmax = __reduce_max_sync(0xffffffffu, g);
-  int pick = __reduce_min_sync(0xffffffffu, g == gmax ? gi : INT_MAX);
-  bool sel0 = pick == j0, sel1 = pick == j1;
-  if (lane == 0) {
-    sel[0] = pick;
-    out[0] = pick;
+  // first pick: the largest column sum, lowest index on ties
+  const uint32_t first_key = __reduce_max_sync(0xffffffffu, max(greedy::make_key(sum0, 2 * lane), greedy::make_key(sum1, 2 * lane + 1)));
+  const int first = greedy::key_index(first_key);
+  const uint16_t* mrow = reinterpret_cast<const uint16_t*>(S + first * kPitchW);
+  uint32_t g0 = 0, g1 = 0, ms = 0;
+#pragma unroll
+  for (int j0 = 0; j0 < kTok; j0 += 8) {
+    uint32_t t = 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const uint32_t mj = mrow[j0 + u];
+      ms += mj;
+      t += greedy::max_u16x2(S[(j0 + u) * kPitchW + lane], mj * 0x10001u);
+    }
+    g0 += t & 0xFFFFu;
+    g1 += t >> 16;
   }
-  int m0 = S[pick * kTok + j0], m1 = S[pick * kTok + j1];
-  int g0 = 0, g1 = 0;
-  {
-    const int16_t* mrow = S + pick * kTok;
-    for (int i = 0; i < kTok; ++i) {
-      const int mi = mrow[i];
-      g0 += max((int)S[i * kTok + j0] - mi, 0);
-      g1 += max((int)S[i * kTok + j1] - mi, 0);
-    }
-  }
-  for (int r = 1; r < Dloc; ++r) {
-    // gain (< 2^23) and 255 - index in one positive key: the largest key is the largest gain, lowest index
-    const int k0 = sel0 ? -1 : (g0 << 8) | (255 - j0), k1 = sel1 ? -1 : (g1 << 8) | (255 - j1);
-    pick = 255 - (__reduce_max_sync(0xffffffffu, max(k0, k1)) & 255);
-    sel0 = sel0 || pick == j0;
-    sel1 = sel1 || pick == j1;
-    if (lane == 0) {
-      sel[r] = pick;
-      out[r] = pick;
-    }
-    const int s0 = S[pick * kTok + j0], s1 = S[pick * kTok + j1];
-    unsigned b0 = __ballot_sync(0xffffffffu, s0 > m0), b1 = __ballot_sync(0xffffffffu, s1 > m1);
-    // columns whose cached maximum improves: g_j += relu(S[i][j] - new) - relu(S[i][j] - old)
-    while (b0) {
-      const int l = __ffs(b0) - 1;
-      b0 &= b0 - 1;
-      const int old = __shfl_sync(0xffffffffu, m0, l), nw = __shfl_sync(0xffffffffu, s0, l);
-      const int v0 = S[l * kTok + j0], v1 = S[l * kTok + j1];
-      g0 += max(v0 - nw, 0) - max(v0 - old, 0);
-      g1 += max(v1 - nw, 0) - max(v1 - old, 0);
-    }
-    while (b1) {
-      const int l = __ffs(b1) - 1;
-      b1 &= b1 - 1;
-      const int old = __shfl_sync(0xffffffffu, m1, l), nw = __shfl_sync(0xffffffffu, s1, l);
-      const int v0 = S[(l + 32) * kTok + j0], v1 = S[(l + 32) * kTok + j1];
-      g0 += max(v0 - nw, 0) - max(v0 - old, 0);
-      g1 += max(v1 - nw, 0) - max(v1 - old, 0);
-    }
-    m0 = max(m0, s0);
-    m1 = max(m1, s1);
-  }
+  if (lane == 0) sel[0] = first;
+  greedy::rounds<true, false, kTok>(S, kPitchW, kTok, Dloc, 1, lane, first, g0 - ms, g1 - ms, sh, sel);
+  __syncwarp();
+  for (int r = lane; r < Dloc; r += 32) out[r] = sel[r];
 }
 
 __device__ __forceinline__ void rows_sync() { asm volatile("bar.sync 1, 64;" ::: "memory"); }  // warps 0 and 1
@@ -124,12 +95,13 @@ refresh_small_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_cons
   // ring, then one slab of padding: an MMA reads 128 operand rows, of which only the first 64 exist; the other 64
   // are whatever follows the slab (their accumulator rows are never read)
   uint8_t* ring = smem;
-  int16_t* S = reinterpret_cast<int16_t*>(ring + kRing * kStageBytes + kSlab);  // [64][64]
+  uint16_t* S = reinterpret_cast<uint16_t*>(ring + kRing * kStageBytes + kSlab);  // [64][64]
   float* G = reinterpret_cast<float*>(S + kTok * kTok);                         // [64][kPitch]
   float* A = G + kTok * kPitch;                                                 // shares [D_loc][kPitch]
   float* zinv = A + kTok * kPitch;                                              // [64]
   int* sel = reinterpret_cast<int*>(zinv + kTok);                               // [64]
-  RBars* bar = reinterpret_cast<RBars*>(sel + kTok);
+  greedy::Shared<kTok>* lists = reinterpret_cast<greedy::Shared<kTok>*>(sel + kTok);
+  RBars* bar = reinterpret_cast<RBars*>(lists + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tile_b = blockIdx.x, b = tile_b / p.P, tile = tile_b - b * p.P;
@@ -199,7 +171,7 @@ refresh_small_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_cons
         tmem_wait_ld();
 #pragma unroll
         for (int e = 0; e < 32; ++e)
-          S[(c0 + e) * kTok + r] = (c0 + e == r) ? (int16_t)kDiagQ : (int16_t)__float2int_rn(__uint_as_float(v[e]) * 4096.f);
+          S[(c0 + e) * kTok + r] = (uint16_t)((c0 + e == r ? kDiagQ : __float2int_rn(__uint_as_float(v[e]) * 4096.f)) + kSqBias);
       }
 #pragma unroll
       for (int c0 = 0; c0 < kTok; c0 += 32) {
@@ -215,7 +187,7 @@ refresh_small_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_cons
     rows_sync();
     if (bar->go) {
       // ---- Algorithm 2
-      if (warp == 0) greedy_one_warp(S, p.Dloc, lane, sel, p.idx + (size_t)tile_b * p.Dloc);
+      if (warp == 0) greedy_one_warp(reinterpret_cast<const uint32_t*>(S), p.Dloc, lane, *lists, sel, p.idx + (size_t)tile_b * p.Dloc);
       rows_sync();
       // ---- Sec. 4.2.1: thread = source token k; logit of destination i is G[idx_i][k] / (tau sqrt(d))
       const int Dl = p.Dloc;
@@ -257,7 +229,7 @@ refresh_small_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_cons
   }
 }
 
-constexpr int kRefreshSmem = 1024 + kRing * kStageBytes + kSlab + kTok * kTok * 2 + 2 * kTok * kPitch * 4 + 2 * kTok * 4 + 256;
+constexpr int kRefreshSmem = 1024 + kRing * kStageBytes + kSlab + kTok * kTok * 2 + 2 * kTok * kPitch * 4 + 2 * kTok * 4 + (int)sizeof(greedy::Shared<kTok>) + 256;
 static_assert(sizeof(RBars) <= 256, "barrier block outgrew its reservation");
 
 }  // namespace

@@ -83,10 +83,20 @@ extern "C" toma_status toma_select_static(const toma_desc* desc, const void* x, 
   void* base = nullptr;
   if (scratch_for_current_device(&base) != cudaSuccess) return TOMA_ERR_CUDA;
   __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(base);
-  int16_t* sq = reinterpret_cast<int16_t*>(static_cast<unsigned char*>(base) + y_bytes);
+  uint16_t* sq = reinterpret_cast<uint16_t*>(static_cast<unsigned char*>(base) + y_bytes);
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = launch_quantise(g, x, y, s);
-  if (e == cudaSuccess) e = gram_tc_supported(g) ? launch_gram_tc(g, y, sq, dev_status, s) : launch_gram_ffma(g, y, sq, s);
-  if (e == cudaSuccess) e = launch_greedy(g, sq, idx, s);
+  // The matrices' rows are padded to 16 bytes: as many tiles at a time as the rest of the array holds that way
+  // (all of them, except where unpadded matrices would just fit).
+  const size_t per_tile = (size_t)g.Nloc * sq_pitch(g.Nloc) * sizeof(uint16_t);
+  const size_t fit = ((size_t)TOMA_STATIC_SCRATCH_BYTES - y_bytes) / per_tile;
+  if (fit == 0) return TOMA_ERR_SCRATCH_LIMIT;
+  for (size_t t0 = 0; t0 < tiles && e == cudaSuccess; t0 += fit) {
+    Geom part = g;  // these two launches see the tiles as one flat sequence
+    part.B = 1;
+    part.P = (int)(tiles - t0 < fit ? tiles - t0 : fit);
+    e = launch_gram_tc(part, y + t0 * g.Nloc * g.d, sq, dev_status, s);
+    if (e == cudaSuccess) e = launch_greedy(part, sq, idx + t0 * g.Dloc, s);
+  }
   return e == cudaSuccess ? TOMA_OK : TOMA_ERR_CUDA;
 }

@@ -1083,3 +1083,18 @@ def test_results_are_deterministic(toma):
     wa, wb = a.weights(), b.weights()
     assert np.array_equal(wa, wb)
     assert np.array_equal(a.merge(), b.merge())
+
+
+@pytest.mark.parametrize("th,tw,ratio", [(1, 1, 0.0), (3, 5, 0.2), (7, 9, 0.5), (5, 13, 0.0), (8, 16, 0.25), (3, 43, 0.5), (15, 17, 0.5), (1, 256, 0.5),
+                                         (1, 257, 0.9), (16, 21, 0.0), (1, 337, 0.5), (18, 19, 0.5), (31, 33, 0.25)])
+def test_selection_at_the_edges_of_its_kernels(toma, th, tw, ratio):
+    """Tiles around the limits of the greedy kernel's forms (64 tokens per warp, one warp; 336 in shared memory; 16 warps) and
+    with ragged rows: every pick equals the oracle's, down to the last one (ratio 0 ranks all tokens, zero gains included)."""
+    cfg = gen.config("cfg2", batch=2, grid_h=th, grid_w=2 * tw, tile_h=th, tile_w=tw, dim=64, n_heads=1, merge_ratio=ratio, noise_sigma=0.4)
+    x_host = gen.features(cfg)
+    idx = Run(toma, cfg, x_host).select()
+    for b in range(cfg.batch):
+        for p in range(cfg.n_tiles):
+            want, margin = O.select_tile(tile_tokens(cfg, x_host, b, p), od(cfg))
+            assert margin > O.FRAGILE_MARGIN
+            assert np.array_equal(idx[b, p], want)
