@@ -94,6 +94,11 @@ cudaError_t launch_merge_tc(const Geom& g, const void* w, const void* x, void* x
                             uint32_t* dev_status, cudaStream_t s);
 cudaError_t launch_unmerge_tc(const Geom& g, const void* w, const void* y, void* out, uint32_t* dev_status,
                               cudaStream_t s);
+// The same for regions of any shape (rows of at most 128 tokens).
+bool ragged_tc_supported(const Geom& g);
+cudaError_t launch_merge_ragged(const Geom& g, const void* w, const void* x, void* xm, void* zero, size_t zero_bytes, uint32_t* dev_status,
+                                cudaStream_t s);
+cudaError_t launch_unmerge_ragged(const Geom& g, const void* w, const void* y, void* out, uint32_t* dev_status, cudaStream_t s);
 cudaError_t launch_copy_extra(const Geom& g, const void* src, void* dst, bool merging, cudaStream_t s);
 // Scratch of the tensor-core attention (tickets and partial results of split work units).
 size_t attention_tc_workspace_bytes(int B, int L, int heads, int dh);

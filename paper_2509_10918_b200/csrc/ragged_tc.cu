@@ -1,0 +1,367 @@
+// Merge X_m = A~ X (Sec. 4.2.1) and unmerge A~^T X' (Sec. 4.2.2) on the sm_100a tensor cores for regions of any
+// shape: N_loc no multiple of 64, D_loc no multiple of 16 - what divides an image whose sides are no powers of
+// two.  (Regions that are whole 64-token boxes take linear_tc.cu.)
+//
+// Two things stand in the way of feeding such regions through TMA alone, and decide the design:
+//   * A region's tokens are rows of tile_w tokens.  A TMA box takes r whole tile rows, r tile_w <= 64 (or 128) tokens
+//     of consecutive slots; the last box of a region is a map of its own with the rows that are left, so that no
+//     token of a neighbouring region is ever read.  The contraction is padded to 16 with zero weights.
+//   * The weight planes [N_loc][D_loc] have rows of 2 D_loc bytes, which are neither 16-byte aligned nor a legal
+//     TMA stride.  They are gathered instead: eight warps read the aligned 16-byte packets that cover eight weights,
+//     shift them into place and write the 128-byte-swizzled operand tile; the same warps are the epilogue later.
+// The weights are the A operand of both (destinations on M for the merge, MN-major; tokens on M for the unmerge,
+// K-major), the tokens / attended rows the MN-major B operand with 128 or 256 channels: a weight block is then
+// gathered once per 128 or 256 channels, and every thread of the epilogue holds one output row.
+// Per CTA: warp 0 TMA, warp 1 MMA, warps 2..9 gather and epilogue.
+#include "common.cuh"
+#include "tc.cuh"
+
+namespace toma {
+
+using namespace tc;
+
+namespace {
+
+constexpr int kWorkers = 256;       // threads of the gather / epilogue warps
+constexpr int kMaxStages = 4;
+
+struct RgBars {
+  uint64_t full[kMaxStages], empty[kMaxStages], done;
+  uint32_t tmem_base;
+  int abort_flag;
+};
+
+struct RgParams {
+  int P, tiles_x, th, tw, Nloc, Dloc, d;
+  int rows;        // tile rows of a full box
+  int nch;         // channels per CTA (a multiple of 64, at most 256)
+  int stages;
+  int kc;          // contraction rows of a stage (64 or 128; unmerge: 64)
+  const __nv_bfloat16* w;
+  const uint8_t* w_end;
+  uint32_t* zero;  // merge only: words cleared on the side (the attention kernel's tickets)
+  int zero_words;
+};
+
+// Eight consecutive weights starting `off` elements into a plane, the first `n` of them real and the rest 0.
+__device__ __forceinline__ void funnel8(const uint4& lo, const uint4& hi, uint32_t sh, int n, uint32_t (&v)[4]) {
+  uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+  if (sh & 8u) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) w[i] = w[i + 2];
+  }
+  if (sh & 4u) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) w[i] = w[i + 1];
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    v[i] = (sh & 2u) ? __funnelshift_r(w[i], w[i + 1], 16) : w[i];
+    if (2 * i >= n) v[i] = 0u;
+    else if (2 * i + 1 >= n) v[i] &= 0xFFFFu;
+  }
+}
+
+// One weight block into its swizzled operand tile(s): kRows rows starting at plane row `row0` (rows >= n_rows become
+// 0), kChunks groups of eight columns starting at `col0` (columns >= D_loc become 0), both planes.  Slab s holds
+// columns 64 s .. 64 s + 63; `slab_bytes` apart, planes `plane_bytes` apart.
+template <int kChunks>
+__device__ __forceinline__ void gather_block(const RgParams& p, const uint8_t* plane0, int t, int rows_total, int row0, int n_rows, int col0,
+                                             uint8_t* dst, int slab_bytes, int plane_bytes) {
+  constexpr int kRowStep = kWorkers / kChunks;
+  const int ch = t % kChunks, r0 = t / kChunks;
+  const int n = min(8, p.Dloc - (col0 + ch * 8));
+  if (n <= 0) return;  // zero since the start
+  uint8_t* out = dst + (ch >> 3) * slab_bytes;
+  const size_t plane_stride = (size_t)p.Nloc * p.Dloc * 2;
+  const bool aligned = ((p.Dloc & 7) == 0);  // then every packet starts on 16 bytes
+  for (int rb = r0; rb < rows_total; rb += 4 * kRowStep) {
+    uint4 lo[2][4], hi[2][4];
+    uint32_t sh[2][4];
+#pragma unroll
+    for (int pl = 0; pl < 2; ++pl)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int row = rb + u * kRowStep;
+        lo[pl][u] = hi[pl][u] = make_uint4(0u, 0u, 0u, 0u);
+        sh[pl][u] = 0u;
+        if (row < n_rows) {
+          const uint8_t* a = plane0 + pl * plane_stride + ((size_t)(row0 + row) * p.Dloc + col0 + ch * 8) * 2;
+          const uint32_t s = (uint32_t)(reinterpret_cast<uintptr_t>(a) & 15);
+          const uint4* q = reinterpret_cast<const uint4*>(a - s);
+          sh[pl][u] = s;
+          if (aligned) {
+            lo[pl][u] = __ldg(q);
+          } else if (reinterpret_cast<const uint8_t*>(q + 2) <= p.w_end) {
+            lo[pl][u] = __ldg(q);
+            if (s + 2 * n > 16) hi[pl][u] = __ldg(q + 1);
+          } else {  // the last packets of the buffer: nothing behind its end is read
+            __align__(16) __nv_bfloat16 e[8];
+            for (int i = 0; i < 8; ++i) e[i] = i < n ? reinterpret_cast<const __nv_bfloat16*>(a)[i] : __float2bfloat16_rn(0.f);
+            lo[pl][u] = *reinterpret_cast<const uint4*>(e);
+            sh[pl][u] = 0u;
+          }
+        }
+      }
+#pragma unroll
+    for (int pl = 0; pl < 2; ++pl)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int row = rb + u * kRowStep;
+        if (row < rows_total) {
+          uint32_t v[4];
+          funnel8(lo[pl][u], hi[pl][u], sh[pl][u], n, v);
+          *reinterpret_cast<uint4*>(out + pl * plane_bytes + sw128_offset(row, ch & 7)) = make_uint4(v[0], v[1], v[2], v[3]);
+        }
+      }
+  }
+}
+
+// Epilogue: this warp's 32 accumulator rows (tensor-memory lanes 32 (warp & 3) ..), columns [c_lo, c_hi), as bf16 into
+// the staged slabs [128 rows][64 channels], the layout of the output map's box.
+__device__ __forceinline__ void stage_rows(uint8_t* so, uint32_t taddr, int row, int c_lo, int c_hi) {
+  for (int c = c_lo; c < c_hi; c += 32) {
+    uint32_t r[32];
+    tmem_ld32(taddr + c, r);
+    tmem_wait_ld();
+    uint8_t* slab = so + (c >> 6) * (128 * 128);
+#pragma unroll
+    for (int e = 0; e < 32; e += 8) {
+      __align__(16) __nv_bfloat162 q[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) q[u] = __floats2bfloat162_rn(__uint_as_float(r[e + 2 * u]), __uint_as_float(r[e + 2 * u + 1]));
+      *reinterpret_cast<uint4*>(slab + sw128_offset(row, ((c & 63) + e) >> 3)) = *reinterpret_cast<const uint4*>(q);
+    }
+  }
+}
+
+// kMerge: M = destinations, contraction over the region's tokens, box by box.  Otherwise M = one box of tokens,
+// contraction over the destinations, 64 at a time.
+//   grid: (channel block, M block, region)
+//   tm_b / tm_b_tail: the B operand (merge: tokens, a full box and the region's last box; unmerge: attended rows, once)
+//   tm_o / tm_o_tail: the output (merge: merged rows, once; unmerge: tokens, a full box and the region's last box)
+template <bool kMerge>
+__global__ void __launch_bounds__(64 + kWorkers, 1)
+ragged_kernel(const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ CUtensorMap tm_b_tail,
+              const __grid_constant__ CUtensorMap tm_o, const __grid_constant__ CUtensorMap tm_o_tail, const RgParams p, uint32_t* dev_status) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int batch = blockIdx.z, mb = blockIdx.y, c0 = blockIdx.x * p.nch;
+  const int b = batch / p.P, tile = batch - b * p.P;
+  const int ty = tile / p.tiles_x, tx = tile - ty * p.tiles_x;
+  const int n_ch = min(p.nch, p.d - c0), slabs = (n_ch + 63) / 64, n_mma = slabs * 64;
+  const int n_boxes = (p.th + p.rows - 1) / p.rows, tail_rows = p.th - (n_boxes - 1) * p.rows;
+  // A: merge [2 planes][2 slabs of 64 destinations][kc tokens][128 B]; unmerge [2 planes][128 tokens][64 destinations]
+  const int a_slab = kMerge ? p.kc * 128 : 128 * 128, a_plane = kMerge ? 2 * a_slab : a_slab;
+  const int b_slab = p.kc * 128;
+  const int stage_bytes = 2 * a_plane + (p.nch / 64) * b_slab;
+  RgBars* bar = reinterpret_cast<RgBars*>(smem + p.stages * stage_bytes);
+  const int nk = kMerge ? n_boxes : (p.Dloc + 63) / 64;
+  const uint32_t ncols = p.nch > 128 ? 256u : p.nch > 64 ? 128u : 64u;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(&bar->full[s], 1 + kWorkers / 32);
+      mbar_init(&bar->empty[s], 1);
+    }
+    mbar_init(&bar->done, 1);
+    bar->abort_flag = 0;
+    mbar_fence_init();
+    prefetch_tmap(&tm_b);
+    prefetch_tmap(&tm_b_tail);
+    prefetch_tmap(&tm_o);
+    prefetch_tmap(&tm_o_tail);
+  }
+  // what no load ever writes has to be a finite number: padding rows of the B operand, padding columns of A
+  for (int e = threadIdx.x; e < p.stages * stage_bytes / 16; e += blockDim.x) reinterpret_cast<uint4*>(smem)[e] = make_uint4(0u, 0u, 0u, 0u);
+  fence_proxy_async();
+  dependency_wait();
+  if (threadIdx.x == 0) release_dependents();
+  if (warp == 1) tmem_alloc(&bar->tmem_base, ncols);
+  if (kMerge && p.zero_words > 0) {
+    const int cta = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    const int n_thr = gridDim.x * gridDim.y * gridDim.z * blockDim.x;
+    for (int i = cta * blockDim.x + threadIdx.x; i < p.zero_words; i += n_thr) p.zero[i] = 0u;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = bar->tmem_base;
+  volatile int* abort_flag = &bar->abort_flag;
+
+  if (warp == 0) {
+    if (elect_one()) {
+      for (int k = 0; k < nk; ++k) {
+        const int s = k % p.stages;
+        if (k >= p.stages && !mbar_wait(&bar->empty[s], ((k / p.stages) - 1) & 1, dev_status, abort_flag)) break;
+        uint8_t* sb = smem + s * stage_bytes + 2 * a_plane;
+        if (kMerge) {
+          const bool tail = k == n_boxes - 1;
+          mbar_expect_tx(&bar->full[s], slabs * (tail ? tail_rows : p.rows) * p.tw * 128);
+          for (int c = 0; c < slabs; ++c)
+            tma_load_4d(sb + c * b_slab, tail ? &tm_b_tail : &tm_b, &bar->full[s], c0 + c * 64, tx * p.tw, ty * p.th + k * p.rows, b);
+        } else {
+          mbar_expect_tx(&bar->full[s], slabs * b_slab);
+          for (int c = 0; c < slabs; ++c) tma_load_4d(sb + c * b_slab, &tm_b, &bar->full[s], c0 + c * 64, k * 64, tile, b);
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (elect_one()) {
+      const uint32_t idesc = idesc_f16(kFmtBF16, kFmtBF16, kMerge, true, 128, n_mma);
+      bool ok = true;
+      for (int k = 0; k < nk; ++k) {
+        const int s = k % p.stages;
+        if (!mbar_wait(&bar->full[s], (k / p.stages) & 1, dev_status, abort_flag)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t aa = smem_u32(smem + s * stage_bytes), ba = aa + 2 * a_plane;
+        const int len = kMerge ? (k == n_boxes - 1 ? tail_rows : p.rows) * p.tw : min(64, p.Dloc - k * 64);
+        const int ksteps = (len + 15) / 16;
+        for (int kk = 0; kk < ksteps; ++kk) {
+          const uint64_t bd = smem_desc_sw128(ba + kk * 2048, b_slab, 1024);
+#pragma unroll
+          for (int pl = 0; pl < 2; ++pl) {
+            const uint64_t ad = kMerge ? smem_desc_sw128(aa + pl * a_plane + kk * 2048, a_slab, 1024)
+                                       : smem_desc_sw128(aa + pl * a_plane + kk * 32, 16, 1024);
+            mma_ss(tmem, ad, bd, idesc, k > 0 || kk > 0 || pl > 0);
+          }
+        }
+        mma_commit(&bar->empty[s]);
+      }
+      if (ok) mma_commit(&bar->done);
+    }
+  } else {
+    const int t = threadIdx.x - 64;
+    const uint8_t* plane0 = reinterpret_cast<const uint8_t*>(p.w) + (size_t)batch * 2 * p.Nloc * p.Dloc * 2;
+    const int box_tok = p.rows * p.tw;
+    bool ok = true;
+    for (int k = 0; k < nk; ++k) {
+      const int s = k % p.stages;
+      // one answer per warp
+      if (k >= p.stages) ok = __all_sync(0xffffffffu, mbar_wait(&bar->empty[s], ((k / p.stages) - 1) & 1, dev_status, abort_flag));
+      if (!ok) break;
+      uint8_t* sa = smem + s * stage_bytes;
+      if (kMerge) {
+        const int len = (k == n_boxes - 1 ? tail_rows : p.rows) * p.tw;
+        gather_block<16>(p, plane0, t, (box_tok + 15) & ~15, k * box_tok, len, mb * 128, sa, a_slab, a_plane);
+      } else {
+        const int len = (mb == n_boxes - 1 ? tail_rows : p.rows) * p.tw;
+        gather_block<8>(p, plane0, t, len, mb * box_tok, len, k * 64, sa, a_slab, a_plane);
+        if (k == nk - 1 && k >= p.stages) {  // columns past D_loc still hold an earlier block's weights
+          const int first = (p.Dloc - k * 64 + 7) / 8, last = ((p.Dloc - k * 64 + 15) / 16) * 2;
+          for (int e = t; e < (last - first) * 256; e += kWorkers) {
+            const int ch = first + e / 256, pl = (e >> 7) & 1, row = e & 127;
+            *reinterpret_cast<uint4*>(sa + pl * a_plane + sw128_offset(row, ch)) = make_uint4(0u, 0u, 0u, 0u);
+          }
+        }
+      }
+      fence_proxy_async();  // the MMA reads what these threads wrote
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar->full[s]);
+    }
+    if (ok && __all_sync(0xffffffffu, mbar_wait(&bar->done, 0, dev_status, abort_flag))) {
+      tc_fence_after();
+      // every load has been consumed: the stages are the output's staging area
+      const int quarter = warp & 3, half = (warp - 2) >> 2, row = quarter * 32 + lane;
+      const int mid = ((n_mma / 2) + 31) & ~31;
+      stage_rows(smem, tmem + ((uint32_t)(quarter * 32) << 16), row, half ? mid : 0, half ? n_mma : mid);
+      fence_proxy_async();  // the staged rows are read by the TMA engine
+      asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory");
+      if (t == 0) {
+        for (int c = 0; c < slabs; ++c) {
+          const void* src = smem + c * (128 * 128);
+          if (kMerge) tma_store_4d(&tm_o, src, c0 + c * 64, mb * 128, tile, b);  // rows past the region's D_loc are clipped
+          else tma_store_4d(mb == n_boxes - 1 ? &tm_o_tail : &tm_o, src, c0 + c * 64, tx * p.tw, ty * p.th + mb * p.rows, b);
+        }
+        tma_store_commit();
+        tma_store_wait_read();  // shared memory must outlive the engine's reads
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, ncols);
+  }
+}
+
+bool token_map(const Geom& g, const void* x, int rows, CUtensorMap* tm) {
+  const uint64_t dims[4] = {(uint64_t)g.d, (uint64_t)g.W, (uint64_t)g.H, (uint64_t)g.B};
+  const uint64_t strides[3] = {(uint64_t)g.d * 2, (uint64_t)g.W * g.d * 2, (uint64_t)g.tokens_all() * g.d * 2};
+  const uint32_t box[4] = {64, (uint32_t)g.tw, (uint32_t)rows, 1};
+  return encode_tmap_16bit(tm, x, 4, dims, strides, box);
+}
+
+// merged / attended rows as (channel, destination, region, batch): a box never reaches into the next region's rows
+bool merged_map(const Geom& g, const void* m, int rows, CUtensorMap* tm) {
+  const uint64_t dims[4] = {(uint64_t)g.d, (uint64_t)g.Dloc, (uint64_t)g.P, (uint64_t)g.B};
+  const uint64_t strides[3] = {(uint64_t)g.d * 2, (uint64_t)g.Dloc * g.d * 2, (uint64_t)g.Lm * g.d * 2};
+  const uint32_t box[4] = {64, (uint32_t)rows, 1, 1};
+  return encode_tmap_16bit(tm, m, 4, dims, strides, box);
+}
+
+template <bool kMerge>
+cudaError_t launch_ragged(const Geom& g, const void* w, const void* in, void* out, void* zero, size_t zero_bytes, uint32_t* dev_status,
+                          cudaStream_t s) {
+  RgParams p;
+  p.P = g.P; p.tiles_x = g.tiles_x; p.th = g.th; p.tw = g.tw; p.Nloc = g.Nloc; p.Dloc = g.Dloc; p.d = g.d;
+  // merge: boxes of at most 64 tokens keep a stage small (rows wider than that: 128); unmerge: a box is the M block
+  p.kc = kMerge && g.tw > 64 ? 128 : 64;
+  const int box_max = kMerge ? p.kc : 128;
+  p.rows = box_max / g.tw < g.th ? box_max / g.tw : g.th;
+  const int n_boxes = (g.th + p.rows - 1) / p.rows, tail = g.th - (n_boxes - 1) * p.rows;
+  const int m_blocks = kMerge ? (g.Dloc + 127) / 128 : n_boxes;
+  // 256 channels per CTA halve how often the weights are gathered; 128 where that would leave SMs without a CTA
+  const long long wide = (long long)g.B * g.P * m_blocks * ((g.d + 255) / 256);
+  p.nch = g.d > 128 && wide >= sm_count() ? 256 : 128;
+  if (g.d <= 64) p.nch = 64;
+  p.w = (const __nv_bfloat16*)w;
+  p.w_end = (const uint8_t*)w + (size_t)g.B * g.P * g.Nloc * g.Dloc * 4;
+  p.zero = (uint32_t*)zero;
+  p.zero_words = (int)(zero_bytes / 4);
+  CUtensorMap tb, tbt, to, tot;
+  bool ok;
+  if (kMerge) ok = token_map(g, in, p.rows, &tb) && token_map(g, in, tail, &tbt) && merged_map(g, out, 128, &to);
+  else ok = merged_map(g, in, 64, &tb) && token_map(g, out, p.rows, &to) && token_map(g, out, tail, &tot);
+  if (!ok) return cudaErrorInvalidValue;
+  if (kMerge) tot = to;
+  else tbt = tb;
+  const int a_plane = kMerge ? 2 * p.kc * 128 : 128 * 128;
+  const int stage_bytes = 2 * a_plane + (p.nch / 64) * p.kc * 128;
+  const int nk = kMerge ? n_boxes : (g.Dloc + 63) / 64;
+  // two stages of the narrow form leave room for a second CTA on the SM; the wide form runs alone
+  p.stages = p.nch > 128 || p.kc > 64 ? (220 * 1024) / stage_bytes : 2;
+  p.stages = p.stages > 3 ? 3 : p.stages;
+  if (p.stages > nk) p.stages = nk;
+  int ring = p.stages * stage_bytes;
+  const int staging = (p.nch / 64) * 128 * 128;
+  if (ring < staging) {  // a single stage: as many as the staged output needs
+    p.stages = (staging + stage_bytes - 1) / stage_bytes;
+    ring = p.stages * stage_bytes;
+  }
+  const int smem = 1024 + ring + 256;
+  static std::atomic<unsigned long long> raised{0};
+  if (cudaError_t e = raise_dynamic_smem(ragged_kernel<kMerge>, 227 * 1024, raised); e != cudaSuccess) return e;
+  const dim3 grid((unsigned)((g.d + p.nch - 1) / p.nch), (unsigned)m_blocks, (unsigned)(g.B * g.P));
+  const cudaError_t e = launch_dependent(ragged_kernel<kMerge>, grid, dim3(64 + kWorkers), (size_t)smem, s, tb, tbt, to, tot, p, dev_status);
+  count_launch();
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace
+
+// bf16 regions whose rows fit a TMA box of 128 tokens (grid z holds 65535 regions).
+bool ragged_tc_supported(const Geom& g) { return !g.f32 && g.tw <= 128 && (long long)g.B * g.P <= 65535; }
+
+cudaError_t launch_merge_ragged(const Geom& g, const void* w, const void* x, void* xm, void* zero, size_t zero_bytes, uint32_t* dev_status,
+                                cudaStream_t s) {
+  return launch_ragged<true>(g, w, x, xm, zero, zero_bytes, dev_status, s);
+}
+
+cudaError_t launch_unmerge_ragged(const Geom& g, const void* w, const void* y, void* out, uint32_t* dev_status, cudaStream_t s) {
+  return launch_ragged<false>(g, w, y, out, nullptr, 0, dev_status, s);
+}
+
+}  // namespace toma

@@ -1098,3 +1098,40 @@ def test_selection_at_the_edges_of_its_kernels(toma, th, tw, ratio):
             want, margin = O.select_tile(tile_tokens(cfg, x_host, b, p), od(cfg))
             assert margin > O.FRAGILE_MARGIN
             assert np.array_equal(idx[b, p], want)
+
+
+RAGGED = [  # tile_h, tile_w, ratio, dim, heads: boxes of whole tile rows with a tail, D_loc of every alignment, rows over 64 tokens
+    (18, 14, 0.5, 640, 10), (19, 13, 0.5, 128, 2), (9, 7, 0.4, 64, 1), (5, 27, 0.3, 72, 1), (3, 65, 0.5, 128, 2), (2, 100, 0.25, 320, 5),
+    (1, 128, 0.5, 64, 1), (24, 25, 0.75, 192, 3), (17, 3, 0.9, 328, 1), (16, 16, 0.41, 640, 10), (28, 28, 0.2, 64, 1), (1, 1, 0.0, 64, 1),
+]
+
+
+@pytest.mark.parametrize("th,tw,ratio,dim,heads", RAGGED)
+@pytest.mark.parametrize("unmerge", ["transpose", "shares"])
+def test_regions_of_any_shape_parity(toma, th, tw, ratio, dim, heads, unmerge):
+    """Weights, merge and unmerge of regions that are no whole 64-token boxes, bf16, against the oracle; text tokens behind them."""
+    cfg = gen.config("cfg2", batch=2, grid_h=2 * th, grid_w=3 * tw, tile_h=th, tile_w=tw, dim=dim, n_heads=heads, head_dim=dim // heads,
+                     merge_ratio=ratio, n_extra=3)
+    x_host = gen.features(cfg)
+    run = Run(toma, cfg, x_host, unmerge_mode=unmerge)
+    idx = run.select()
+    dense = run.weights()
+    merged = run.merge()
+    y_dev = (run.xm.float() * 0.25).to(run.xm.dtype)  # as in test_edge_shapes: keeps the outputs below 8
+    unmerged = run.unmerge(y_dev)
+    y_host = to_host64(y_dev)
+    d_loc = gd(toma, cfg)
+    ids = O.tile_token_ids(cfg.grid_h, cfg.grid_w, cfg.tile_h, cfg.tile_w)
+    for b in range(cfg.batch):
+        for p in range(cfg.n_tiles):
+            xt = tile_tokens(cfg, x_host, b, p)
+            want_idx, _ = O.select_tile(xt, od(cfg))
+            assert np.array_equal(idx[b, p], want_idx)
+            w = O.merge_weights(xt, want_idx, cfg.tau)
+            assert np.abs(dense[b, p] - w).max() <= 6e-4
+            sl = slice(p * d_loc, (p + 1) * d_loc)
+            assert_close(merged[b, sl], O.merge(w, xt), "bf16", "merge")
+            u = w if unmerge == "transpose" else O.softmax_shares(xt, want_idx, cfg.tau)
+            assert_close(unmerged[b, ids[p]], O.unmerge(u, y_host[b, sl]), "bf16", "unmerge")
+        assert np.array_equal(merged[b, cfg.n_tiles * d_loc:], x_host[b, cfg.n_tokens:].astype(np.float64))
+        assert np.array_equal(unmerged[b, cfg.n_tokens:], y_host[b, cfg.n_tiles * d_loc:])
