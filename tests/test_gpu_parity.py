@@ -1103,6 +1103,7 @@ def test_selection_at_the_edges_of_its_kernels(toma, th, tw, ratio):
 RAGGED = [  # tile_h, tile_w, ratio, dim, heads: boxes of whole tile rows with a tail, D_loc of every alignment, rows over 64 tokens
     (18, 14, 0.5, 640, 10), (19, 13, 0.5, 128, 2), (9, 7, 0.4, 64, 1), (5, 27, 0.3, 72, 1), (3, 65, 0.5, 128, 2), (2, 100, 0.25, 320, 5),
     (1, 128, 0.5, 64, 1), (24, 25, 0.75, 192, 3), (17, 3, 0.9, 328, 1), (16, 16, 0.41, 640, 10), (28, 28, 0.2, 64, 1), (1, 1, 0.0, 64, 1),
+    (11, 67, 0.5, 128, 2), (31, 33, 0.61, 64, 1), (24, 32, 0.51, 64, 1),  # 11 and 11 source blocks; 6 of them, 376 destinations
 ]
 
 
@@ -1135,3 +1136,26 @@ def test_regions_of_any_shape_parity(toma, th, tw, ratio, dim, heads, unmerge):
             assert_close(unmerged[b, ids[p]], O.unmerge(u, y_host[b, sl]), "bf16", "unmerge")
         assert np.array_equal(merged[b, cfg.n_tiles * d_loc:], x_host[b, cfg.n_tokens:].astype(np.float64))
         assert np.array_equal(unmerged[b, cfg.n_tokens:], y_host[b, cfg.n_tiles * d_loc:])
+
+
+@pytest.mark.parametrize("gh,gw,th,tw,ratio", [(18, 28, 9, 14, 0.5), (30, 42, 10, 21, 0.5), (15, 26, 15, 13, 0.43)])
+def test_global_merge_of_ragged_images_parity(toma, gh, gw, th, tw, ratio):
+    """The image as one region of any shape: the same kernels with up to 630 destinations, which is past the 512 of a block."""
+    cfg = gen.config("cfg2", batch=2, grid_h=gh, grid_w=gw, tile_h=th, tile_w=tw, dim=128, n_heads=2, merge_ratio=ratio)
+    x_host = gen.features(cfg)
+    run = Run(toma, cfg, x_host, global_merge=True)
+    idx = run.select()
+    d = cfg.n_tiles * gd(toma, cfg)
+    run.t.toma_merge_weights(run.desc, run.x, run.idx, run.w, run.ws, run.status)
+    dense_dev = torch.empty((cfg.batch, 1, d, cfg.n_tokens), dtype=torch.float32, device="cuda")
+    run.t.toma_weights_export(run.desc, run.w, dense_dev)
+    run.ok()
+    merged = run.merge()
+    y_dev = (run.xm.float() * 0.25).to(run.xm.dtype)
+    unmerged = run.unmerge(y_dev)
+    for b in range(cfg.batch):
+        gdest = O.global_destinations(idx[b], O.tile_token_ids(cfg.grid_h, cfg.grid_w, cfg.tile_h, cfg.tile_w))
+        w = O.merge_weights(x_host[b], gdest, cfg.tau)
+        assert np.abs(dense_dev[b, 0].double().cpu().numpy() - w).max() <= 6e-4
+        assert_close(merged[b], O.merge(w, x_host[b]), "bf16", "merge")
+        assert_close(unmerged[b], O.unmerge(w, to_host64(y_dev)[b]), "bf16", "unmerge")
