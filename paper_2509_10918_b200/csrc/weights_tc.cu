@@ -260,7 +260,7 @@ weights_logits_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
 //   by then) and copied out, one plane after the other.
 // ------------------------------------------------------------------------------------------------
 template <int kMB, bool kCluster = false>
-__global__ void __launch_bounds__(64 + 128 * kMB, 1)
+__global__ void __launch_bounds__(64 + 256 * kMB, 1)
 weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_x_tail,
                      const __grid_constant__ CUtensorMap tm_d,
                      __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ wu, const WParams p, uint32_t* dev_status) {
@@ -275,7 +275,8 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   WBars* bar = reinterpret_cast<WBars*>(smem + p.stages * stage_bytes);
   float* zw = reinterpret_cast<float*>(bar + 1);  // [4 kMB warps][D_loc] partial row sums
   float* zinv = zw + 4 * kMB * Dl;                // [D_loc] reciprocal row sums of the tile
-  float* zpart = zinv + Dl;                       // [m_blocks][D_loc] cluster form: every block's row sums
+  float* red = zinv + Dl;                         // [2 halves][128 kMB] maxima, then denominators, of a token's two threads
+  float* zpart = red + 256 * kMB;                 // [m_blocks][D_loc] cluster form: every block's row sums
   static_assert(!kCluster || kMB == 1, "the cluster form has one source block per CTA");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int batch = kCluster ? blockIdx.x / p.m_blocks : blockIdx.x;
@@ -293,7 +294,7 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
       mbar_init(&bar->empty[s], 1);
     }
     mbar_init(&bar->done, 1);
-    if (kCluster && p.m_blocks > 1) mbar_init(&bar->z_in, (uint32_t)(128 * (p.m_blocks - 1)));  // every epilogue thread of the peers arrives once
+    if (kCluster && p.m_blocks > 1) mbar_init(&bar->z_in, (uint32_t)(256 * (p.m_blocks - 1)));  // every epilogue thread of the peers arrives once
     bar->abort_flag = 0;
     mbar_fence_init();
     prefetch_tmap(&tm_x);
@@ -347,86 +348,108 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
       if (ok) mma_commit(&bar->done);
     }
   } else {
-    const int mb = (warp - 2) >> 2, quarter = warp & 3;
-    const int k_loc = quarter * 32 + lane;  // source row inside its block = tensor-memory lane
+    // Two threads per source token (tensor-memory lane), one for each half of the destinations: the passes over the
+    // row are bound by exponentials, tensor-memory reads and shuffles of one thread, and a CTA has the SM to itself.
+    const int mb = (warp - 2) >> 3, half = ((warp - 2) >> 2) & 1, quarter = warp & 3;
+    const int k_loc = quarter * 32 + lane;  // source row inside its block
     const int m_valid = tail && mb == kMB - 1 ? p.tail_tok : p.m_tok;
     const bool valid = k_loc < m_valid;
+    const int mid = ((Dl + 1) / 2 + 31) & ~31;
+    const int lo_col = half ? mid : 0, hi_col = half ? Dl : min(mid, Dl);  // this thread's destinations
     const uint32_t taddr = tmem + mb * ncols_mb + ((uint32_t)(quarter * 32) << 16);
     float* zrow = zw + (mb * 4 + quarter) * Dl;
-    float neg_m = 0.f, inv = 0.f;
-    const bool ok = mbar_wait(&bar->done, 0, dev_status, abort_flag);
-    if (ok) {
-      tc_fence_after();
+    float* mine = red + half * (128 * kMB) + mb * 128 + k_loc;
+    const float* other = red + (half ^ 1) * (128 * kMB) + mb * 128 + k_loc;
+    const int pair_bar = 2 + mb * 4 + quarter;
+    auto pair_sync = [&] { asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory"); };
+    float inv = 0.f;
+    // one answer per warp, then one per pair of warps (they meet at barriers): NaN says that a wait ran out
+    bool ok = __all_sync(0xffffffffu, mbar_wait(&bar->done, 0, dev_status, abort_flag));
+    if (ok) tc_fence_after();
+    {
       // pass 1: maximum logit over the destinations
       float mx = -INFINITY;
-      for (int i0 = 0; i0 < Dl; i0 += 32) {
-        uint32_t r[32];
-        tmem_ld32(taddr + i0, r);
-        tmem_wait_ld();
+      if (ok)
+        for (int i0 = lo_col; i0 < hi_col; i0 += 32) {
+          uint32_t r[32];
+          tmem_ld32(taddr + i0, r);
+          tmem_wait_ld();
 #pragma unroll
-        for (int e = 0; e < 32; ++e)
-          if (i0 + e < Dl) mx = fmaxf(mx, __uint_as_float(r[e]));
-      }
-      neg_m = -mx * p.scale_log2;
-      // pass 2: denominator of the token's softmax
+          for (int e = 0; e < 32; ++e)
+            if (i0 + e < hi_col) mx = fmaxf(mx, __uint_as_float(r[e]));
+        }
+      *mine = ok ? mx : __int_as_float(0x7fffffff);
+      pair_sync();
+      ok = ok && !(*other != *other);
+      mx = fmaxf(mx, *other);
+      const float neg_m = -mx * p.scale_log2;
+      pair_sync();
+      // pass 2: the exponentials, left in place of the logits, and the denominator of the token's softmax
       float sum = 0.f;
-      for (int i0 = 0; i0 < Dl; i0 += 32) {
-        uint32_t r[32];
-        tmem_ld32(taddr + i0, r);
-        tmem_wait_ld();
+      if (ok)
+        for (int i0 = lo_col; i0 < hi_col; i0 += 32) {
+          uint32_t r[32];
+          tmem_ld32(taddr + i0, r);
+          tmem_wait_ld();
 #pragma unroll
-        for (int e = 0; e < 32; ++e)
-          if (i0 + e < Dl) sum += fast_exp2(fmaf(__uint_as_float(r[e]), p.scale_log2, neg_m));
-      }
+          for (int e = 0; e < 32; ++e) {
+            const float v = fast_exp2(fmaf(__uint_as_float(r[e]), p.scale_log2, neg_m));
+            if (i0 + e < hi_col) sum += v;
+            r[e] = __float_as_uint(v);
+          }
+          tmem_st32(taddr + i0, r);
+        }
+      tmem_wait_st();
+      *mine = sum;
+      pair_sync();
+      sum = half ? *other + sum : sum + *other;
       inv = valid ? 1.f / sum : 0.f;
       // pass 3: the shares' sums over this warp's 32 source tokens, per destination
-      for (int i0 = 0; i0 < Dl; i0 += 32) {
-        uint32_t r[32];
-        tmem_ld32(taddr + i0, r);
-        tmem_wait_ld();
-        float a[32];
+      if (ok)
+        for (int i0 = lo_col; i0 < hi_col; i0 += 32) {
+          uint32_t r[32];
+          tmem_ld32(taddr + i0, r);
+          tmem_wait_ld();
+          float a[32];
 #pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          const float v = fast_exp2(fmaf(__uint_as_float(r[e]), p.scale_log2, neg_m)) * inv;
-          a[e] = (valid && i0 + e < Dl) ? v : 0.f;
-        }
-        // transpose-reduce: afterwards lane c holds the sum over the warp's 32 rows of column i0 + c
+          for (int e = 0; e < 32; ++e) a[e] = (valid && i0 + e < hi_col) ? __uint_as_float(r[e]) * inv : 0.f;
+          // transpose-reduce: afterwards lane c holds the sum over the warp's 32 rows of column i0 + c
 #pragma unroll
-        for (int off = 16, n = 32; off >= 1; off >>= 1, n >>= 1) {
-          const bool upper = (lane & off) != 0;
+          for (int off = 16, n = 32; off >= 1; off >>= 1, n >>= 1) {
+            const bool upper = (lane & off) != 0;
 #pragma unroll
-          for (int c = 0; c < n / 2; ++c) {
-            const float send = upper ? a[c] : a[c + n / 2];
-            const float keep = upper ? a[c + n / 2] : a[c];
-            a[c] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+            for (int c = 0; c < n / 2; ++c) {
+              const float send = upper ? a[c] : a[c + n / 2];
+              const float keep = upper ? a[c + n / 2] : a[c];
+              a[c] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+            }
           }
+          if (i0 + lane < hi_col) zrow[i0 + lane] = a[0];
         }
-        if (i0 + lane < Dl) zrow[i0 + lane] = a[0];
-      }
     }
     // the tile's row sums: warps of a block pairwise, then the blocks in order (a fixed order: the
     // result does not depend on scheduling); a row sum that underflowed to 0 gives a zero row
-    asm volatile("bar.sync 1, %0;" ::"n"(128 * kMB) : "memory");
+    asm volatile("bar.sync 1, %0;" ::"n"(256 * kMB) : "memory");
     if (kCluster) {
       // this block's sums go to every peer, the peers' arrive here; all add the blocks' sums in rank order
-      for (int i = threadIdx.x - 64; i < Dl; i += 128) {
+      for (int i = threadIdx.x - 64; i < Dl; i += 256) {
         const float* q = zw + i;
         zpart[rank * Dl + i] = (q[0] + q[Dl]) + (q[2 * Dl] + q[3 * Dl]);
       }
       for (int q = 0; q < p.m_blocks; ++q) {
         if (q == rank) continue;
         const uint32_t dst = peer_addr(smem_u32(zpart + rank * Dl), (uint32_t)q);
-        for (int i = threadIdx.x - 64; i < Dl; i += 128) st_peer_f32(dst + 4u * (uint32_t)i, zpart[rank * Dl + i]);
+        for (int i = threadIdx.x - 64; i < Dl; i += 256) st_peer_f32(dst + 4u * (uint32_t)i, zpart[rank * Dl + i]);
         mbar_arrive_peer(peer_addr(smem_u32(&bar->z_in), (uint32_t)q));
       }
       const bool got = p.m_blocks == 1 || mbar_wait_cluster(&bar->z_in, 0, dev_status, abort_flag);
-      for (int i = threadIdx.x - 64; i < Dl; i += 128) {
+      for (int i = threadIdx.x - 64; i < Dl; i += 256) {
         float z = 0.f;
         for (int q = 0; q < p.m_blocks; ++q) z += zpart[q * Dl + i];
         zinv[i] = got && z > 0.f ? 1.f / z : 0.f;
       }
     } else {
-      for (int i = threadIdx.x - 64; i < Dl; i += 128 * kMB) {
+      for (int i = threadIdx.x - 64; i < Dl; i += 256 * kMB) {
         float z = 0.f;
 #pragma unroll
         for (int m = 0; m < kMB; ++m) {
@@ -436,33 +459,35 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         zinv[i] = z > 0.f ? 1.f / z : 0.f;
       }
     }
-    asm volatile("bar.sync 1, %0;" ::"n"(128 * kMB) : "memory");
-    if (ok && valid && Dl % 8 == 0) {
+    asm volatile("bar.sync 1, %0;" ::"n"(256 * kMB) : "memory");
+    if (ok && Dl % 8 == 0) {
       // pass 4: A~_ik = A_ik / Z_i, written as row k of A~^T [N_loc][D_loc], hi plane then lo plane
       const size_t plane = (size_t)p.Nloc * Dl;
-      const size_t row = (size_t)((mb + rank) * p.m_tok + k_loc) * Dl;
+      const size_t row = (size_t)((mb + rank) * p.m_tok + (valid ? k_loc : 0)) * Dl;
       __nv_bfloat16* t_hi = w + (size_t)batch * 2 * plane + row;
       __nv_bfloat16* u_hi = wu ? wu + (size_t)batch * 2 * plane + row : nullptr;
-      for (int i0 = 0; i0 < Dl; i0 += 32) {
+      for (int i0 = lo_col; i0 < hi_col; i0 += 32) {
         uint32_t r[32];
         tmem_ld32(taddr + i0, r);
         tmem_wait_ld();
 #pragma unroll
         for (int e0 = 0; e0 < 32; e0 += 8) {
-          if (i0 + e0 >= Dl) break;  // D_loc is a multiple of 8
+          if (i0 + e0 >= hi_col) break;  // D_loc is a multiple of 8
           __align__(16) __nv_bfloat16 hi[8], lo[8], uh[8], ul[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
-            const float a = fast_exp2(fmaf(__uint_as_float(r[e0 + e]), p.scale_log2, neg_m)) * inv;
+            const float a = __uint_as_float(r[e0 + e]) * inv;
             const float v = a * zinv[i0 + e0 + e];
             hi[e] = __float2bfloat16_rn(v);
             lo[e] = __float2bfloat16_rn(v - __bfloat162float(hi[e]));
             uh[e] = __float2bfloat16_rn(a);
             ul[e] = __float2bfloat16_rn(a - __bfloat162float(uh[e]));
           }
-          *reinterpret_cast<uint4*>(t_hi + i0 + e0) = *reinterpret_cast<const uint4*>(hi);
-          *reinterpret_cast<uint4*>(t_hi + plane + i0 + e0) = *reinterpret_cast<const uint4*>(lo);
-          if (u_hi) {
+          if (valid) {
+            *reinterpret_cast<uint4*>(t_hi + i0 + e0) = *reinterpret_cast<const uint4*>(hi);
+            *reinterpret_cast<uint4*>(t_hi + plane + i0 + e0) = *reinterpret_cast<const uint4*>(lo);
+          }
+          if (valid && u_hi) {
             *reinterpret_cast<uint4*>(u_hi + i0 + e0) = *reinterpret_cast<const uint4*>(uh);
             *reinterpret_cast<uint4*>(u_hi + plane + i0 + e0) = *reinterpret_cast<const uint4*>(ul);
           }
@@ -470,7 +495,7 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
       }
     }
     if (ok && Dl % 8 != 0) {
-      // the same for rows that are not 16-byte aligned: this warp's rows of a plane are one contiguous range, staged
+      // the same for rows that are not 16-byte aligned: a pair's 32 rows of a plane are one contiguous range, staged
       // with the range's own misalignment so that its middle is copied in aligned packets
       const size_t plane = (size_t)p.Nloc * Dl;
       const int n_rows = max(0, min(32, m_valid - quarter * 32));
@@ -478,26 +503,26 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
       for (int pl = 0; pl < (wu ? 4 : 2); ++pl) {
         __nv_bfloat16* g = (pl < 2 ? w : wu) + ((size_t)batch * 2 + (pl & 1)) * plane + (size_t)((mb + rank) * p.m_tok + quarter * 32) * Dl;
         const int mis = (int)(reinterpret_cast<uintptr_t>(g) & 15);
-        __nv_bfloat16* mine = reinterpret_cast<__nv_bfloat16*>(stage + mis) + lane * Dl;
-        for (int i0 = 0; i0 < Dl; i0 += 32) {
+        __nv_bfloat16* row = reinterpret_cast<__nv_bfloat16*>(stage + mis) + lane * Dl;
+        for (int i0 = lo_col; i0 < hi_col; i0 += 32) {
           uint32_t r[32];
           tmem_ld32(taddr + i0, r);
           tmem_wait_ld();
           if (valid) {
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
-              if (i0 + e >= Dl) break;
-              const float a = fast_exp2(fmaf(__uint_as_float(r[e]), p.scale_log2, neg_m)) * inv;
+              if (i0 + e >= hi_col) break;
+              const float a = __uint_as_float(r[e]) * inv;
               const float v = pl < 2 ? a * zinv[i0 + e] : a;
               const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-              mine[i0 + e] = (pl & 1) ? __float2bfloat16_rn(v - __bfloat162float(hi)) : hi;
+              row[i0 + e] = (pl & 1) ? __float2bfloat16_rn(v - __bfloat162float(hi)) : hi;
             }
           }
         }
-        __syncwarp();
+        pair_sync();
         uint8_t* gb = reinterpret_cast<uint8_t*>(g) - mis;
         const int end = mis + n_rows * Dl * 2;  // bytes [mis, end) of the staged packets
-        for (int o = lane * 16; o < end; o += 512) {
+        for (int o = (half * 32 + lane) * 16; o < end; o += 1024) {
           if (o >= mis && o + 16 <= end) {
             *reinterpret_cast<uint4*>(gb + o) = *reinterpret_cast<const uint4*>(stage + o);
           } else {
@@ -505,7 +530,7 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
               *reinterpret_cast<__nv_bfloat16*>(gb + q) = *reinterpret_cast<const __nv_bfloat16*>(stage + q);
           }
         }
-        __syncwarp();
+        pair_sync();
       }
     }
   }
@@ -759,16 +784,16 @@ cudaError_t launch_weights_tc(const Geom& g, const void* x, const int32_t* idx, 
     if (p.stages > nk) p.stages = nk;
     if (g.Dloc % 8 != 0)  // the ring doubles as the staging area of the plane rows
       while (p.stages * stage_bytes < 4 * ((32 * g.Dloc * 2 + 47) & ~15)) ++p.stages;
-    const int smem = 1024 + p.stages * stage_bytes + (int)sizeof(WBars) + (4 * mb + 1 + (cluster ? mblocks : 0)) * g.Dloc * 4 + 64;
+    const int smem = 1024 + p.stages * stage_bytes + (int)sizeof(WBars) + ((4 * mb + 1 + (cluster ? mblocks : 0)) * g.Dloc + 256 * mb) * 4 + 64;
     if (fused) {
       static std::atomic<unsigned long long> raised2{0};
       if (cudaError_t e = raise_dynamic_smem(weights_fused_kernel<2>, 227 * 1024, raised2); e != cudaSuccess) return e;
-      le = launch_dependent(weights_fused_kernel<2>, dim3((unsigned)tiles), dim3(320), (size_t)smem, s, tx, txt, td,
+      le = launch_dependent(weights_fused_kernel<2>, dim3((unsigned)tiles), dim3(64 + 512), (size_t)smem, s, tx, txt, td,
                             (__nv_bfloat16*)w, (__nv_bfloat16*)wu, p, dev_status);
     } else {
       static std::atomic<unsigned long long> raised1{0};
       if (cudaError_t e = raise_dynamic_smem(weights_fused_kernel<1, true>, 227 * 1024, raised1); e != cudaSuccess) return e;
-      le = launch_dependent_cluster(weights_fused_kernel<1, true>, dim3((unsigned)(mblocks * tiles)), dim3(192), (size_t)smem, mblocks, s, tx, txt,
+      le = launch_dependent_cluster(weights_fused_kernel<1, true>, dim3((unsigned)(mblocks * tiles)), dim3(64 + 256), (size_t)smem, mblocks, s, tx, txt,
                                     td, (__nv_bfloat16*)w, (__nv_bfloat16*)wu, p, dev_status);
     }
     count_launch();
