@@ -76,7 +76,7 @@ WsLayout ws_layout(const Geom& g) {
   size_t off = 0;
   l.y_off = off;      off = align_up(off + tiles * g.Nloc * g.d * sizeof(__nv_bfloat16), 256);
   l.sq_off = off;     off = align_up(off + tiles * g.Nloc * sq_pitch(g.Nloc) * sizeof(uint16_t), 256);
-  l.logits_off = off; off = align_up(off + (size_t)gm.B * gm.P * ((gm.Dloc + 3) & ~3) * gm.Nloc * sizeof(float), 256);
+  l.logits_off = off; off = align_up(off + (size_t)gm.B * gm.P * gm.Dloc * gm.Nloc * sizeof(float), 256);
   l.wts_off = off;    off = align_up(off + (weights_tc_supported(gm) ? weights_tc_scratch_bytes(gm) : 0), 256);
   l.gidx_off = off;   off = align_up(off + (g.global_merge ? (size_t)g.B * g.D * sizeof(int32_t) : 0), 256);
   l.xm_off = off;     off = align_up(off + (size_t)g.B * g.Lm * g.d * esz, 256);

@@ -9,11 +9,8 @@
 //      block, the partial row sums sum_k A_ik.
 //   3. weights_normalise_kernel: A~_ik = A_ik / sum_k' A_ik' with the partial sums added in a
 //      fixed order, stored as A~^T [N_loc][D_loc] split into a hi and a lo bf16 plane.
-// Regions of at most 512 destinations and 8 source blocks take weights_fused_kernel instead of 2 and 3: one
-// CTA per source block, the blocks of a region a thread-block cluster (or one CTA for both blocks of a region where
-// there are many), the row normalisation applied in the epilogue of the logits contraction.
-// A source block is as many whole rows of a region as 128 tokens hold - any region shape whose rows are at most 128
-// tokens; its last block has a TMA map of its own, so that no token of a neighbouring region is read.
+// Tiles of at most 256 tokens and 256 destinations take weights_fused_kernel instead of 2 and 3: one
+// CTA per tile, the row normalisation applied in the epilogue of the logits contraction.
 #include "common.cuh"
 #include "tc.cuh"
 
@@ -34,11 +31,7 @@ struct WBars {
 
 struct WParams {
   int P, tiles_x, th, tw, W, Nloc, Dloc, d, n_all;
-  int rows;     // region rows per source block
-  int m_tok;    // source tokens per block: rows * tw, at most 128
-  int m_blocks; // source blocks of a region; the last one has tail_tok tokens
-  int tail_tok;
-  int pitch;    // row pitch of the shares in memory: D_loc rounded up to 4
+  int m_tok;    // source tokens per CTA (128, or N_loc when the tile is smaller)
   int stages;
   float scale_log2;  // log2(e) / (tau * sqrt(d))
   int d_block;  // destinations per CTA: D_loc itself, or 512 when D_loc is larger (blockIdx.z picks the block)
@@ -68,8 +61,7 @@ __device__ __forceinline__ float fast_exp2(float x) {
 }
 
 __global__ void __launch_bounds__(192, 1)
-weights_logits_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_x_tail,
-                      const __grid_constant__ CUtensorMap tm_d,
+weights_logits_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_d,
                       float* __restrict__ shares, float* __restrict__ zpart, const WParams p, uint32_t* dev_status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -88,11 +80,10 @@ weights_logits_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
   const int batch = blockIdx.x, mblk = blockIdx.y, k_base = mblk * p.m_tok;
   const int b = batch / p.P, tile = batch - b * p.P;
   const int ty = tile / p.tiles_x, tx = tile - ty * p.tiles_x;
-  const bool tail = mblk == p.m_blocks - 1;
-  const int m_valid = tail ? p.tail_tok : p.m_tok;  // source tokens of this block
+  const int rows_per_box = p.m_tok / p.tw;
   const int nk = (p.d + kKC - 1) / kKC;
   const uint32_t ncols = n_mma > 256 ? 512u : n_mma > 128 ? 256u : n_mma > 64 ? 128u : n_mma > 32 ? 64u : 32u;
-  const int box_bytes_a = m_valid * 128;
+  const int box_bytes_a = p.m_tok * 128;
   const int box_d0 = Dl > 256 ? 256 : Dl, box_d1 = Dl - box_d0;
 
   if (threadIdx.x == 0) {
@@ -103,7 +94,7 @@ weights_logits_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     mbar_init(&bar->done, 1);
     bar->abort_flag = 0;
     mbar_fence_init();
-    prefetch_tmap(tail ? &tm_x_tail : &tm_x);
+    prefetch_tmap(&tm_x);
     prefetch_tmap(&tm_d);
   }
   dependency_wait();  // before tensor memory is held and before any global access
@@ -122,7 +113,7 @@ weights_logits_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         if (k >= p.stages && !mbar_wait(&bar->empty[s], ((k / p.stages) - 1) & 1, dev_status, abort_flag)) break;
         uint8_t* sa = smem + s * stage_bytes;
         mbar_expect_tx(&bar->full[s], box_bytes_a + b_load_bytes);
-        tma_load_4d(sa, tail ? &tm_x_tail : &tm_x, &bar->full[s], k * kKC, tx * p.tw, ty * p.th + mblk * p.rows, b);
+        tma_load_4d(sa, &tm_x, &bar->full[s], k * kKC, tx * p.tw, ty * p.th + mblk * rows_per_box, b);
         tma_load_3d(sa + a_bytes, &tm_d, &bar->full[s], k * kKC, d_base, batch);
         if (box_d1 > 0) tma_load_3d(sa + a_bytes + 256 * 128, &tm_d, &bar->full[s], k * kKC, d_base + 256, batch);
       }
@@ -150,21 +141,18 @@ weights_logits_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
   } else {
     const int quarter = warp & 3;
     const int k_loc = quarter * 32 + lane;              // source row inside this CTA
-    const bool valid = k_loc < m_valid;
+    const bool valid = k_loc < p.m_tok;
     const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
     float* zrow = zw + quarter * Dl;
     if (mbar_wait(&bar->done, 0, dev_status, abort_flag)) {
       tc_fence_after();
       if (p.raw) {  // scaled logits only: the row's other destination blocks are in other CTAs
-        float* dst = shares + ((size_t)batch * p.Nloc + k_base + (valid ? k_loc : 0)) * p.pitch + d_base;
+        float* dst = shares + ((size_t)batch * p.Nloc + k_base + (valid ? k_loc : 0)) * p.Dloc + d_base;
         for (int i0 = 0; i0 < Dl; i0 += 32) {
           uint32_t r[32];
           tmem_ld32(taddr + i0, r);
           tmem_wait_ld();
           if (valid) {
-#pragma unroll
-            for (int e = 0; e < 32; ++e)
-              if (i0 + e >= Dl) r[e] = 0xFF800000u;  // -inf: the padding of the last row packet
 #pragma unroll
             for (int e = 0; e < 32; e += 4)
               if (i0 + e < Dl)
@@ -197,7 +185,7 @@ weights_logits_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
       }
       const float inv = valid ? 1.f / sum : 0.f;
       // pass 3: shares, their store, and the per-warp column sums
-      float* dst = shares + ((size_t)batch * p.Nloc + k_base + (valid ? k_loc : 0)) * p.pitch;
+      float* dst = shares + ((size_t)batch * p.Nloc + k_base + (valid ? k_loc : 0)) * p.Dloc;
       for (int i0 = 0; i0 < p.Dloc; i0 += 32) {
         uint32_t r[32];
         tmem_ld32(taddr + i0, r);
@@ -249,43 +237,37 @@ weights_logits_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
 // up across the tile through shared memory, and the row normalisation 1/Z_i applied as the
 // accumulators are read a last time: A~^T leaves the kernel as its hi and lo bf16 planes, and the
 // fp32 shares never exist in memory.
-//   kMB: source blocks per CTA (1 or 2).  Warp 0 TMA, warp 1 MMA, then four epilogue warps
+//   kMB: 128-source blocks per tile (1 or 2).  Warp 0 TMA, warp 1 MMA, then four epilogue warps
 //   per source block (thread = source token = tensor-memory lane).
-//   kCluster (with kMB = 1): the source blocks of a region are the CTAs of a cluster (up to 8), which send each other
-//   their parts of the row sums (a store into every peer's shared memory per destination, counted on a barrier of
-//   the peer's) and add the blocks' sums in rank order.  64 regions of 1024 tokens with 512 destinations took 144 us
-//   for the logits and 98 us for normalising them through fp32 shares in memory.
-//   D_loc % 8 != 0: rows of the planes are not aligned, and a thread per row would write two bytes to 32 lines at a
-//   time; a warp's 32 rows, which are one contiguous range of a plane, are staged in shared memory (the ring is free
-//   by then) and copied out, one plane after the other.
+//   kPair (with kMB = 1): a tile of two source blocks is shared by the two CTAs of a cluster, one block each,
+//   which send each other their halves of the row sums (a store into the peer's shared memory per
+//   destination, counted on a barrier of the peer's) - for launches of few tiles, where one CTA per tile would
+//   leave most SMs idle and each CTA bound by what one SM takes in.
 // ------------------------------------------------------------------------------------------------
-template <int kMB, bool kCluster = false>
-__global__ void __launch_bounds__(64 + 256 * kMB, 1)
-weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_x_tail,
-                     const __grid_constant__ CUtensorMap tm_d,
+template <int kMB, bool kPair = false>
+__global__ void __launch_bounds__(64 + 128 * kMB, 1)
+weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_d,
                      __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ wu, const WParams p, uint32_t* dev_status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int Dl = p.Dloc;
   const int n_mma = (Dl + 15) & ~15;  // MMA N: destinations padded to 16
-  const int n0 = n_mma > 256 ? 256 : n_mma, n1 = n_mma - n0;  // an MMA takes at most 256 columns (n1 > 0 only with kMB = 1)
   const int a_bytes = 128 * 128;      // one source block of a stage (only m_tok rows are loaded)
   const int b_bytes = ((((Dl + 7) & ~7) * 128 + 1023) / 1024) * 1024;
   const int stage_bytes = kMB * a_bytes + b_bytes;
   WBars* bar = reinterpret_cast<WBars*>(smem + p.stages * stage_bytes);
   float* zw = reinterpret_cast<float*>(bar + 1);  // [4 kMB warps][D_loc] partial row sums
   float* zinv = zw + 4 * kMB * Dl;                // [D_loc] reciprocal row sums of the tile
-  float* red = zinv + Dl;                         // [2 halves][128 kMB] maxima, then denominators, of a token's two threads
-  float* zpart = red + 256 * kMB;                 // [m_blocks][D_loc] cluster form: every block's row sums
-  static_assert(!kCluster || kMB == 1, "the cluster form has one source block per CTA");
+  float* zpeer = zinv + Dl;                       // [D_loc] paired form: the peer block's row sums
+  static_assert(!kPair || kMB == 1, "the paired form has one source block per CTA");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int batch = kCluster ? blockIdx.x / p.m_blocks : blockIdx.x;
-  const int rank = kCluster ? (int)blockIdx.x - batch * p.m_blocks : 0;  // in the cluster = the region's source block of this CTA
+  const int batch = kPair ? blockIdx.x >> 1 : blockIdx.x;
+  const int half = kPair ? (int)(blockIdx.x & 1) : 0;  // = rank in the cluster: the tile's source block of this CTA
   const int b = batch / p.P, tile = batch - b * p.P;
   const int ty = tile / p.tiles_x, tx = tile - ty * p.tiles_x;
-  const bool tail = rank + kMB == p.m_blocks;  // this CTA has the region's last block (of kMB, the last)
+  const int rows_per_box = p.m_tok / p.tw;
   const int nk = (p.d + kKC - 1) / kKC;
-  const uint32_t ncols_mb = n_mma > 256 ? 512u : n_mma > 128 ? 256u : n_mma > 64 ? 128u : n_mma > 32 ? 64u : 32u;
+  const uint32_t ncols_mb = n_mma > 128 ? 256u : n_mma > 64 ? 128u : n_mma > 32 ? 64u : 32u;
   const uint32_t ncols = kMB * ncols_mb;  // a power of two again (kMB is 1 or 2)
 
   if (threadIdx.x == 0) {
@@ -294,11 +276,10 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
       mbar_init(&bar->empty[s], 1);
     }
     mbar_init(&bar->done, 1);
-    if (kCluster && p.m_blocks > 1) mbar_init(&bar->z_in, (uint32_t)(256 * (p.m_blocks - 1)));  // every epilogue thread of the peers arrives once
+    mbar_init(&bar->z_in, 128);  // every epilogue thread of the peer arrives once
     bar->abort_flag = 0;
     mbar_fence_init();
     prefetch_tmap(&tm_x);
-    prefetch_tmap(&tm_x_tail);
     prefetch_tmap(&tm_d);
   }
   dependency_wait();  // before tensor memory is held and before any global access
@@ -307,7 +288,7 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (kCluster) cluster_sync();  // the peers' barriers are initialised before anything is sent to it
+  if (kPair) cluster_sync();  // the peer's barrier is initialised before anything is sent to it
   const uint32_t tmem = bar->tmem_base;
   volatile int* abort_flag = &bar->abort_flag;
 
@@ -317,18 +298,15 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         const int s = k % p.stages;
         if (k >= p.stages && !mbar_wait(&bar->empty[s], ((k / p.stages) - 1) & 1, dev_status, abort_flag)) break;
         uint8_t* sa = smem + s * stage_bytes;
-        mbar_expect_tx(&bar->full[s], ((kMB - 1) * p.m_tok + (tail ? p.tail_tok : p.m_tok)) * 128 + (Dl > 256 ? 512 : Dl) * 128);
+        mbar_expect_tx(&bar->full[s], kMB * p.m_tok * 128 + Dl * 128);
         for (int mb = 0; mb < kMB; ++mb)
-          tma_load_4d(sa + mb * a_bytes, tail && mb == kMB - 1 ? &tm_x_tail : &tm_x, &bar->full[s], k * kKC, tx * p.tw,
-                      ty * p.th + (mb + rank) * p.rows, b);
+          tma_load_4d(sa + mb * a_bytes, &tm_x, &bar->full[s], k * kKC, tx * p.tw, ty * p.th + (mb + half) * rows_per_box, b);
         tma_load_3d(sa + kMB * a_bytes, &tm_d, &bar->full[s], k * kKC, 0, batch);
-        if (kMB == 1 && Dl > 256) tma_load_3d(sa + kMB * a_bytes + 256 * 128, &tm_d, &bar->full[s], k * kKC, 256, batch);
       }
     }
   } else if (warp == 1) {
     if (elect_one()) {
-      const uint32_t idesc = idesc_f16(kFmtBF16, kFmtBF16, false, false, 128, n0);
-      const uint32_t idesc1 = idesc_f16(kFmtBF16, kFmtBF16, false, false, 128, n1 > 0 ? n1 : 16);
+      const uint32_t idesc = idesc_f16(kFmtBF16, kFmtBF16, false, false, 128, n_mma);
       bool ok = true;
       for (int k = 0; k < nk; ++k) {
         const int s = k % p.stages;
@@ -338,118 +316,91 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
 #pragma unroll
         for (int mb = 0; mb < kMB; ++mb)
 #pragma unroll
-          for (int kk = 0; kk < kKC / 16; ++kk) {
-            const uint64_t ad = smem_desc_sw128(aa + mb * a_bytes + kk * 32, 16, 1024);
-            mma_ss(tmem + mb * ncols_mb, ad, smem_desc_sw128(ba + kk * 32, 16, 1024), idesc, k > 0 || kk > 0);
-            if (kMB == 1 && n1 > 0) mma_ss(tmem + 256, ad, smem_desc_sw128(ba + 256 * 128 + kk * 32, 16, 1024), idesc1, k > 0 || kk > 0);
-          }
+          for (int kk = 0; kk < kKC / 16; ++kk)
+            mma_ss(tmem + mb * ncols_mb, smem_desc_sw128(aa + mb * a_bytes + kk * 32, 16, 1024),
+                   smem_desc_sw128(ba + kk * 32, 16, 1024), idesc, k > 0 || kk > 0);
         mma_commit(&bar->empty[s]);
       }
       if (ok) mma_commit(&bar->done);
     }
   } else {
-    // Two threads per source token (tensor-memory lane), one for each half of the destinations: the passes over the
-    // row are bound by exponentials, tensor-memory reads and shuffles of one thread, and a CTA has the SM to itself.
-    const int mb = (warp - 2) >> 3, half = ((warp - 2) >> 2) & 1, quarter = warp & 3;
-    const int k_loc = quarter * 32 + lane;  // source row inside its block
-    const int m_valid = tail && mb == kMB - 1 ? p.tail_tok : p.m_tok;
-    const bool valid = k_loc < m_valid;
-    const int mid = ((Dl + 1) / 2 + 31) & ~31;
-    const int lo_col = half ? mid : 0, hi_col = half ? Dl : min(mid, Dl);  // this thread's destinations
+    const int mb = (warp - 2) >> 2, quarter = warp & 3;
+    const int k_loc = quarter * 32 + lane;  // source row inside its block = tensor-memory lane
+    const bool valid = k_loc < p.m_tok;
     const uint32_t taddr = tmem + mb * ncols_mb + ((uint32_t)(quarter * 32) << 16);
     float* zrow = zw + (mb * 4 + quarter) * Dl;
-    float* mine = red + half * (128 * kMB) + mb * 128 + k_loc;
-    const float* other = red + (half ^ 1) * (128 * kMB) + mb * 128 + k_loc;
-    const int pair_bar = 2 + mb * 4 + quarter;
-    auto pair_sync = [&] { asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory"); };
-    float inv = 0.f;
-    // one answer per warp, then one per pair of warps (they meet at barriers): NaN says that a wait ran out
-    bool ok = __all_sync(0xffffffffu, mbar_wait(&bar->done, 0, dev_status, abort_flag));
-    if (ok) tc_fence_after();
-    {
+    float neg_m = 0.f, inv = 0.f;
+    const bool ok = mbar_wait(&bar->done, 0, dev_status, abort_flag);
+    if (ok) {
+      tc_fence_after();
       // pass 1: maximum logit over the destinations
       float mx = -INFINITY;
-      if (ok)
-        for (int i0 = lo_col; i0 < hi_col; i0 += 32) {
-          uint32_t r[32];
-          tmem_ld32(taddr + i0, r);
-          tmem_wait_ld();
+      for (int i0 = 0; i0 < Dl; i0 += 32) {
+        uint32_t r[32];
+        tmem_ld32(taddr + i0, r);
+        tmem_wait_ld();
 #pragma unroll
-          for (int e = 0; e < 32; ++e)
-            if (i0 + e < hi_col) mx = fmaxf(mx, __uint_as_float(r[e]));
-        }
-      *mine = ok ? mx : __int_as_float(0x7fffffff);
-      pair_sync();
-      ok = ok && !(*other != *other);
-      mx = fmaxf(mx, *other);
-      const float neg_m = -mx * p.scale_log2;
-      pair_sync();
-      // pass 2: the exponentials, left in place of the logits, and the denominator of the token's softmax
+        for (int e = 0; e < 32; ++e)
+          if (i0 + e < Dl) mx = fmaxf(mx, __uint_as_float(r[e]));
+      }
+      neg_m = -mx * p.scale_log2;
+      // pass 2: denominator of the token's softmax
       float sum = 0.f;
-      if (ok)
-        for (int i0 = lo_col; i0 < hi_col; i0 += 32) {
-          uint32_t r[32];
-          tmem_ld32(taddr + i0, r);
-          tmem_wait_ld();
+      for (int i0 = 0; i0 < Dl; i0 += 32) {
+        uint32_t r[32];
+        tmem_ld32(taddr + i0, r);
+        tmem_wait_ld();
 #pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            const float v = fast_exp2(fmaf(__uint_as_float(r[e]), p.scale_log2, neg_m));
-            if (i0 + e < hi_col) sum += v;
-            r[e] = __float_as_uint(v);
-          }
-          tmem_st32(taddr + i0, r);
-        }
-      tmem_wait_st();
-      *mine = sum;
-      pair_sync();
-      sum = half ? *other + sum : sum + *other;
+        for (int e = 0; e < 32; ++e)
+          if (i0 + e < Dl) sum += fast_exp2(fmaf(__uint_as_float(r[e]), p.scale_log2, neg_m));
+      }
       inv = valid ? 1.f / sum : 0.f;
       // pass 3: the shares' sums over this warp's 32 source tokens, per destination
-      if (ok)
-        for (int i0 = lo_col; i0 < hi_col; i0 += 32) {
-          uint32_t r[32];
-          tmem_ld32(taddr + i0, r);
-          tmem_wait_ld();
-          float a[32];
+      for (int i0 = 0; i0 < Dl; i0 += 32) {
+        uint32_t r[32];
+        tmem_ld32(taddr + i0, r);
+        tmem_wait_ld();
+        float a[32];
 #pragma unroll
-          for (int e = 0; e < 32; ++e) a[e] = (valid && i0 + e < hi_col) ? __uint_as_float(r[e]) * inv : 0.f;
-          // transpose-reduce: afterwards lane c holds the sum over the warp's 32 rows of column i0 + c
-#pragma unroll
-          for (int off = 16, n = 32; off >= 1; off >>= 1, n >>= 1) {
-            const bool upper = (lane & off) != 0;
-#pragma unroll
-            for (int c = 0; c < n / 2; ++c) {
-              const float send = upper ? a[c] : a[c + n / 2];
-              const float keep = upper ? a[c + n / 2] : a[c];
-              a[c] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-            }
-          }
-          if (i0 + lane < hi_col) zrow[i0 + lane] = a[0];
+        for (int e = 0; e < 32; ++e) {
+          const float v = fast_exp2(fmaf(__uint_as_float(r[e]), p.scale_log2, neg_m)) * inv;
+          a[e] = (valid && i0 + e < Dl) ? v : 0.f;
         }
+        // transpose-reduce: afterwards lane c holds the sum over the warp's 32 rows of column i0 + c
+#pragma unroll
+        for (int off = 16, n = 32; off >= 1; off >>= 1, n >>= 1) {
+          const bool upper = (lane & off) != 0;
+#pragma unroll
+          for (int c = 0; c < n / 2; ++c) {
+            const float send = upper ? a[c] : a[c + n / 2];
+            const float keep = upper ? a[c + n / 2] : a[c];
+            a[c] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+          }
+        }
+        if (i0 + lane < Dl) zrow[i0 + lane] = a[0];
+      }
     }
     // the tile's row sums: warps of a block pairwise, then the blocks in order (a fixed order: the
     // result does not depend on scheduling); a row sum that underflowed to 0 gives a zero row
-    asm volatile("bar.sync 1, %0;" ::"n"(256 * kMB) : "memory");
-    if (kCluster) {
-      // this block's sums go to every peer, the peers' arrive here; all add the blocks' sums in rank order
-      for (int i = threadIdx.x - 64; i < Dl; i += 256) {
+    asm volatile("bar.sync 1, %0;" ::"n"(128 * kMB) : "memory");
+    if (kPair) {
+      // this block's sums go to the peer, the peer's arrive here; both add block 0 + block 1 in that order
+      const uint32_t peer = (uint32_t)(half ^ 1);
+      const uint32_t peer_z = peer_addr(smem_u32(zpeer), peer);
+      for (int i = threadIdx.x - 64; i < Dl; i += 128) {
         const float* q = zw + i;
-        zpart[rank * Dl + i] = (q[0] + q[Dl]) + (q[2 * Dl] + q[3 * Dl]);
+        const float z = (q[0] + q[Dl]) + (q[2 * Dl] + q[3 * Dl]);
+        zinv[i] = z;  // own half, for now
+        st_peer_f32(peer_z + 4u * (uint32_t)i, z);
       }
-      for (int q = 0; q < p.m_blocks; ++q) {
-        if (q == rank) continue;
-        const uint32_t dst = peer_addr(smem_u32(zpart + rank * Dl), (uint32_t)q);
-        for (int i = threadIdx.x - 64; i < Dl; i += 256) st_peer_f32(dst + 4u * (uint32_t)i, zpart[rank * Dl + i]);
-        mbar_arrive_peer(peer_addr(smem_u32(&bar->z_in), (uint32_t)q));
-      }
-      const bool got = p.m_blocks == 1 || mbar_wait_cluster(&bar->z_in, 0, dev_status, abort_flag);
-      for (int i = threadIdx.x - 64; i < Dl; i += 256) {
-        float z = 0.f;
-        for (int q = 0; q < p.m_blocks; ++q) z += zpart[q * Dl + i];
-        zinv[i] = got && z > 0.f ? 1.f / z : 0.f;
+      mbar_arrive_peer(peer_addr(smem_u32(&bar->z_in), peer));
+      const bool got = mbar_wait_cluster(&bar->z_in, 0, dev_status, abort_flag);
+      for (int i = threadIdx.x - 64; i < Dl; i += 128) {
+        const float z = !got ? 0.f : half == 0 ? zinv[i] + zpeer[i] : zpeer[i] + zinv[i];
+        zinv[i] = z > 0.f ? 1.f / z : 0.f;
       }
     } else {
-      for (int i = threadIdx.x - 64; i < Dl; i += 256 * kMB) {
+      for (int i = threadIdx.x - 64; i < Dl; i += 128 * kMB) {
         float z = 0.f;
 #pragma unroll
         for (int m = 0; m < kMB; ++m) {
@@ -459,78 +410,37 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         zinv[i] = z > 0.f ? 1.f / z : 0.f;
       }
     }
-    asm volatile("bar.sync 1, %0;" ::"n"(256 * kMB) : "memory");
-    if (ok && Dl % 8 == 0) {
+    asm volatile("bar.sync 1, %0;" ::"n"(128 * kMB) : "memory");
+    if (ok && valid) {
       // pass 4: A~_ik = A_ik / Z_i, written as row k of A~^T [N_loc][D_loc], hi plane then lo plane
       const size_t plane = (size_t)p.Nloc * Dl;
-      const size_t row = (size_t)((mb + rank) * p.m_tok + (valid ? k_loc : 0)) * Dl;
+      const size_t row = (size_t)((mb + half) * p.m_tok + k_loc) * Dl;
       __nv_bfloat16* t_hi = w + (size_t)batch * 2 * plane + row;
       __nv_bfloat16* u_hi = wu ? wu + (size_t)batch * 2 * plane + row : nullptr;
-      for (int i0 = lo_col; i0 < hi_col; i0 += 32) {
+      for (int i0 = 0; i0 < Dl; i0 += 32) {
         uint32_t r[32];
         tmem_ld32(taddr + i0, r);
         tmem_wait_ld();
 #pragma unroll
         for (int e0 = 0; e0 < 32; e0 += 8) {
-          if (i0 + e0 >= hi_col) break;  // D_loc is a multiple of 8
+          if (i0 + e0 >= Dl) break;  // D_loc is a multiple of 8
           __align__(16) __nv_bfloat16 hi[8], lo[8], uh[8], ul[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
-            const float a = __uint_as_float(r[e0 + e]) * inv;
+            const float a = fast_exp2(fmaf(__uint_as_float(r[e0 + e]), p.scale_log2, neg_m)) * inv;
             const float v = a * zinv[i0 + e0 + e];
             hi[e] = __float2bfloat16_rn(v);
             lo[e] = __float2bfloat16_rn(v - __bfloat162float(hi[e]));
             uh[e] = __float2bfloat16_rn(a);
             ul[e] = __float2bfloat16_rn(a - __bfloat162float(uh[e]));
           }
-          if (valid) {
-            *reinterpret_cast<uint4*>(t_hi + i0 + e0) = *reinterpret_cast<const uint4*>(hi);
-            *reinterpret_cast<uint4*>(t_hi + plane + i0 + e0) = *reinterpret_cast<const uint4*>(lo);
-          }
-          if (valid && u_hi) {
+          *reinterpret_cast<uint4*>(t_hi + i0 + e0) = *reinterpret_cast<const uint4*>(hi);
+          *reinterpret_cast<uint4*>(t_hi + plane + i0 + e0) = *reinterpret_cast<const uint4*>(lo);
+          if (u_hi) {
             *reinterpret_cast<uint4*>(u_hi + i0 + e0) = *reinterpret_cast<const uint4*>(uh);
             *reinterpret_cast<uint4*>(u_hi + plane + i0 + e0) = *reinterpret_cast<const uint4*>(ul);
           }
         }
-      }
-    }
-    if (ok && Dl % 8 != 0) {
-      // the same for rows that are not 16-byte aligned: a pair's 32 rows of a plane are one contiguous range, staged
-      // with the range's own misalignment so that its middle is copied in aligned packets
-      const size_t plane = (size_t)p.Nloc * Dl;
-      const int n_rows = max(0, min(32, m_valid - quarter * 32));
-      uint8_t* stage = smem + (mb * 4 + quarter) * ((32 * Dl * 2 + 47) & ~15);
-      for (int pl = 0; pl < (wu ? 4 : 2); ++pl) {
-        __nv_bfloat16* g = (pl < 2 ? w : wu) + ((size_t)batch * 2 + (pl & 1)) * plane + (size_t)((mb + rank) * p.m_tok + quarter * 32) * Dl;
-        const int mis = (int)(reinterpret_cast<uintptr_t>(g) & 15);
-        __nv_bfloat16* row = reinterpret_cast<__nv_bfloat16*>(stage + mis) + lane * Dl;
-        for (int i0 = lo_col; i0 < hi_col; i0 += 32) {
-          uint32_t r[32];
-          tmem_ld32(taddr + i0, r);
-          tmem_wait_ld();
-          if (valid) {
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-              if (i0 + e >= hi_col) break;
-              const float a = __uint_as_float(r[e]) * inv;
-              const float v = pl < 2 ? a * zinv[i0 + e] : a;
-              const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-              row[i0 + e] = (pl & 1) ? __float2bfloat16_rn(v - __bfloat162float(hi)) : hi;
-            }
-          }
-        }
-        pair_sync();
-        uint8_t* gb = reinterpret_cast<uint8_t*>(g) - mis;
-        const int end = mis + n_rows * Dl * 2;  // bytes [mis, end) of the staged packets
-        for (int o = (half * 32 + lane) * 16; o < end; o += 1024) {
-          if (o >= mis && o + 16 <= end) {
-            *reinterpret_cast<uint4*>(gb + o) = *reinterpret_cast<const uint4*>(stage + o);
-          } else {
-            for (int q = max(o, mis); q < min(o + 16, end); q += 2)
-              *reinterpret_cast<__nv_bfloat16*>(gb + q) = *reinterpret_cast<const __nv_bfloat16*>(stage + q);
-          }
-        }
-        pair_sync();
       }
     }
   }
@@ -540,7 +450,7 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     tc_fence_after();
     tmem_dealloc(tmem, ncols);
   }
-  if (kCluster) cluster_sync();  // no CTA's shared memory goes away while a peer could still write to it
+  if (kPair) cluster_sync();  // neither CTA's shared memory goes away while the other could still write to it
 }
 
 __global__ void __launch_bounds__(256)
@@ -587,48 +497,13 @@ weights_normalise_kernel(const float* __restrict__ shares, const float* __restri
   }
 }
 
-// The same for D_loc % 4 != 0, whose plane rows are not aligned: a warp per row, consecutive lanes on consecutive weights.
-__global__ void __launch_bounds__(256)
-weights_normalise_ragged_kernel(const float* __restrict__ shares, const float* __restrict__ zpart, __nv_bfloat16* __restrict__ w,
-                                __nv_bfloat16* __restrict__ wu, int Nloc, int Dloc, int pitch, int mblocks) {
-  extern __shared__ float zs[];
-  dependency_wait();  // launched with programmatic stream serialisation
-  if (threadIdx.x == 0) release_dependents();
-  const size_t batch = blockIdx.y;
-  for (int i = threadIdx.x; i < Dloc; i += blockDim.x) {
-    float z = 0.f;
-    for (int mb = 0; mb < mblocks; ++mb) z += zpart[(batch * mblocks + mb) * Dloc + i];
-    zs[i] = z > 0.f ? 1.f / z : 0.f;  // a row sum that underflowed to 0 gives a zero row
-  }
-  __syncthreads();
-  const size_t plane = (size_t)Nloc * Dloc;
-  const int lane = threadIdx.x & 31;
-  for (int row = blockIdx.x * 8 + (threadIdx.x >> 5); row < Nloc; row += gridDim.x * 8) {
-    const float* src = shares + (batch * Nloc + row) * pitch;
-    __nv_bfloat16* t = w + batch * 2 * plane + (size_t)row * Dloc;
-    __nv_bfloat16* u = wu ? wu + batch * 2 * plane + (size_t)row * Dloc : nullptr;
-#pragma unroll 4
-    for (int i = lane; i < Dloc; i += 32) {
-      const float a = src[i], v = a * zs[i];
-      const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-      t[i] = hi;
-      t[plane + i] = __float2bfloat16_rn(v - __bfloat162float(hi));
-      if (u) {
-        const __nv_bfloat16 uh = __float2bfloat16_rn(a);
-        u[i] = uh;
-        u[plane + i] = __float2bfloat16_rn(a - __bfloat162float(uh));
-      }
-    }
-  }
-}
-
 // Softmax over the destination axis for rows of scaled logits (log2 domain) that span several
 // destination blocks: shares[row][i] <- 2^(v_i - max) / sum.  One warp per source row, 32 rows per
 // CTA; the CTA then leaves, per destination, the sum of its 32 rows of shares in zblk (rows added in
 // row order, so the result does not depend on scheduling).
 constexpr int kSoftmaxRows = 32;
 __global__ void __launch_bounds__(256)
-softmax_rows_kernel(float* __restrict__ shares, float* __restrict__ zblk, int Nloc, int Dloc, int pitch) {
+softmax_rows_kernel(float* __restrict__ shares, float* __restrict__ zblk, int Nloc, int Dloc) {
   dependency_wait();
   if (threadIdx.x == 0) release_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -637,23 +512,23 @@ softmax_rows_kernel(float* __restrict__ shares, float* __restrict__ zblk, int Nl
   for (int rr = 0; rr < kSoftmaxRows / 8; ++rr) {
     const int row = row0 + warp * (kSoftmaxRows / 8) + rr;
     if (row >= Nloc) break;
-    float4* v = reinterpret_cast<float4*>(shares + (batch * Nloc + row) * pitch);  // padding: -inf, share 0
+    float4* v = reinterpret_cast<float4*>(shares + (batch * Nloc + row) * Dloc);
     float mx = -INFINITY;
-    for (int q = lane; q < pitch / 4; q += 32) {
+    for (int q = lane; q < Dloc / 4; q += 32) {
       const float4 a = v[q];
       mx = fmaxf(fmaxf(mx, fmaxf(a.x, a.y)), fmaxf(a.z, a.w));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     float sum = 0.f;
-    for (int q = lane; q < pitch / 4; q += 32) {
+    for (int q = lane; q < Dloc / 4; q += 32) {
       const float4 a = v[q];
       sum += (fast_exp2(a.x - mx) + fast_exp2(a.y - mx)) + (fast_exp2(a.z - mx) + fast_exp2(a.w - mx));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     const float inv = 1.f / sum;
-    for (int q = lane; q < pitch / 4; q += 32) {
+    for (int q = lane; q < Dloc / 4; q += 32) {
       float4 a = v[q];
       a.x = fast_exp2(a.x - mx) * inv;
       a.y = fast_exp2(a.y - mx) * inv;
@@ -664,11 +539,11 @@ softmax_rows_kernel(float* __restrict__ shares, float* __restrict__ zblk, int Nl
   }
   __syncthreads();  // the CTA's rows are final (and visible to the whole CTA)
   const int rows = min(kSoftmaxRows, Nloc - row0);
-  const float* base = shares + (batch * Nloc + row0) * pitch;
+  const float* base = shares + (batch * Nloc + row0) * Dloc;
   float* out = zblk + (batch * gridDim.x + blockIdx.x) * Dloc;
   for (int i = threadIdx.x; i < Dloc; i += blockDim.x) {
     float acc = 0.f;
-    for (int r = 0; r < rows; ++r) acc += base[(size_t)r * pitch + i];
+    for (int r = 0; r < rows; ++r) acc += base[(size_t)r * Dloc + i];
     out[i] = acc;
   }
 }
@@ -707,29 +582,23 @@ __global__ void __launch_bounds__(256) z_reduce_kernel(const float* __restrict__
 
 }  // namespace
 
-namespace {
-// Source blocks of a region: as many whole region rows as 128 tokens hold.
-struct Blocks {
-  int rows, m_tok, n, tail_rows;
-};
-Blocks source_blocks(const Geom& g) {
-  Blocks b;
-  b.rows = 128 / g.tw < g.th ? 128 / g.tw : g.th;
-  b.m_tok = b.rows * g.tw;
-  b.n = (g.th + b.rows - 1) / b.rows;
-  b.tail_rows = g.th - (b.n - 1) * b.rows;
-  return b;
+bool weights_tc_supported(const Geom& g) {
+  if (g.f32) return false;
+  const int m_tok = g.Nloc < 128 ? g.Nloc : 128;
+  if (g.Nloc % m_tok != 0 || m_tok % 8 != 0) return false;
+  if (g.tw > m_tok || m_tok % g.tw != 0 || g.th % (m_tok / g.tw) != 0 || g.tw > 256 || m_tok / g.tw > 256) return false;
+  if (g.Dloc % 4 != 0) return false;
+  if (g.Dloc > 512 && g.Nloc % kSoftmaxRows != 0) return false;  // blocked form: softmax in a second kernel
+  return true;
 }
-}  // namespace
-
-bool weights_tc_supported(const Geom& g) { return !g.f32 && g.tw <= 128; }
 
 size_t weights_tc_scratch_bytes(const Geom& g) {  // gathered destinations + partial row sums
   const size_t tiles = (size_t)g.B * g.P;
+  const int m_tok = g.Nloc < 128 ? g.Nloc : 128;
   const size_t dest = tiles * g.Dloc * g.d * 2 + 256;
   if (g.Dloc > 512)  // blocked form: per-row-block sums, then their total
-    return dest + tiles * ((size_t)(g.Nloc + kSoftmaxRows - 1) / kSoftmaxRows) * g.Dloc * 4 + 256 + tiles * g.Dloc * 4 + 256;
-  return dest + tiles * source_blocks(g).n * g.Dloc * 4 + 256;
+    return dest + tiles * ((size_t)g.Nloc / kSoftmaxRows) * g.Dloc * 4 + 256 + tiles * g.Dloc * 4 + 256;
+  return dest + tiles * (g.Nloc / m_tok) * g.Dloc * 4 + 256;
 }
 
 cudaError_t launch_weights_tc(const Geom& g, const void* x, const int32_t* idx, void* w, void* wu, float* shares,
@@ -738,17 +607,12 @@ cudaError_t launch_weights_tc(const Geom& g, const void* x, const int32_t* idx, 
   WParams p;
   p.P = g.P; p.tiles_x = g.tiles_x; p.th = g.th; p.tw = g.tw; p.W = g.W; p.Nloc = g.Nloc; p.Dloc = g.Dloc; p.d = g.d;
   p.n_all = (int)g.tokens_all();
-  const Blocks blk = source_blocks(g);
-  p.rows = blk.rows;
-  p.m_tok = blk.m_tok;
-  p.m_blocks = blk.n;
-  p.tail_tok = blk.tail_rows * g.tw;
-  p.pitch = (g.Dloc + 3) & ~3;
+  p.m_tok = g.Nloc < 128 ? g.Nloc : 128;
   p.scale_log2 = g.logit_scale * 1.4426950408889634f;
   const bool blocked = g.Dloc > 512;  // more destinations than one CTA's tensor memory holds
   p.d_block = blocked ? 512 : g.Dloc;
   p.raw = blocked ? 1 : 0;
-  const int mblocks = blk.n;
+  const int mblocks = g.Nloc / p.m_tok;
   __nv_bfloat16* dg = (__nv_bfloat16*)scratch;
   float* zpart = (float*)((char*)scratch + ((tiles * g.Dloc * g.d * 2 + 255) / 256) * 256);
 
@@ -759,42 +623,53 @@ cudaError_t launch_weights_tc(const Geom& g, const void* x, const int32_t* idx, 
   count_launch();
   if (le != cudaSuccess) return le;
 
-  CUtensorMap tx, txt, td;
-  // Up to 512 destinations and 8 source blocks: one kernel, no fp32 shares in memory.  A region's blocks are a cluster;
-  // two blocks go into one CTA instead where there are enough regions to occupy the SMs anyway (a CTA takes in its
-  // operands at a few tens of bytes per clock whatever else it does: 77 against 91 us on 256 regions, 30 against
-  // 26 us on 32 regions).
-  const bool fused = g.Dloc <= 256 && g.Dloc % 8 == 0 && mblocks == 2 && (int)tiles >= sm_count() / 2;
-  const bool cluster = !fused && g.Dloc <= 512 && mblocks <= 8;
+  CUtensorMap tx, td;
+  // One CTA per tile, no fp32 shares in memory.  With two source blocks per tile the fused form halves the
+  // CTA count, and a CTA takes in its operands at a few tens of bytes per clock whatever else it does: it
+  // wins once there are enough tiles to occupy the SMs anyway (measured: 77 against 91 us on 256 tiles, 30
+  // against 26 us on 32 tiles); with one source block per tile it only saves the second kernel.
+  const bool fused = g.Dloc <= 256 && g.Dloc % 8 == 0 && (mblocks == 1 || (mblocks == 2 && (int)tiles >= sm_count() / 2));
+  // few tiles of two source blocks: the fused form with the tile shared by a cluster of two CTAs (one block each)
+  const bool paired = !fused && g.Dloc <= 256 && g.Dloc % 8 == 0 && mblocks == 2;
   const uint64_t xdims[4] = {(uint64_t)g.d, (uint64_t)g.W, (uint64_t)g.H, (uint64_t)g.B};
   const uint64_t xstr[3] = {(uint64_t)g.d * 2, (uint64_t)g.W * g.d * 2, (uint64_t)g.tokens_all() * g.d * 2};
-  const uint32_t xbox[4] = {64, (uint32_t)g.tw, (uint32_t)blk.rows, 1}, xbox_tail[4] = {64, (uint32_t)g.tw, (uint32_t)blk.tail_rows, 1};
+  const uint32_t xbox[4] = {64, (uint32_t)g.tw, (uint32_t)(p.m_tok / g.tw), 1};
   const uint64_t ddims[3] = {(uint64_t)g.d, (uint64_t)g.Dloc, (uint64_t)tiles};
   const uint64_t dstr[2] = {(uint64_t)g.d * 2, (uint64_t)g.Dloc * g.d * 2};
   const uint32_t dbox[3] = {64, (uint32_t)(g.Dloc > 256 ? 256 : g.Dloc), 1};
-  if (!encode_tmap_16bit(&tx, x, 4, xdims, xstr, xbox) || !encode_tmap_16bit(&txt, x, 4, xdims, xstr, xbox_tail) || !encode_tmap_16bit(&td, dg, 3, ddims, dstr, dbox))
+  if (!encode_tmap_16bit(&tx, x, 4, xdims, xstr, xbox) || !encode_tmap_16bit(&td, dg, 3, ddims, dstr, dbox))
     return cudaErrorInvalidValue;
   const int b_rows = g.Dloc > 256 ? 512 : ((g.Dloc + 7) & ~7);
   const int nk = (g.d + kKC - 1) / kKC;
-  if (fused || cluster) {
-    const int mb = fused ? 2 : 1;  // source blocks per CTA
-    const int stage_bytes = mb * 128 * 128 + ((b_rows * 128 + 1023) / 1024) * 1024;
-    p.stages = (176 * 1024) / stage_bytes;
+  if (paired) {
+    const int stage_bytes = 128 * 128 + ((b_rows * 128 + 1023) / 1024) * 1024;
+    p.stages = (200 * 1024) / stage_bytes;
     p.stages = p.stages > 4 ? 4 : p.stages;
     if (p.stages > nk) p.stages = nk;
-    if (g.Dloc % 8 != 0)  // the ring doubles as the staging area of the plane rows
-      while (p.stages * stage_bytes < 4 * ((32 * g.Dloc * 2 + 47) & ~15)) ++p.stages;
-    const int smem = 1024 + p.stages * stage_bytes + (int)sizeof(WBars) + ((4 * mb + 1 + (cluster ? mblocks : 0)) * g.Dloc + 256 * mb) * 4 + 64;
-    if (fused) {
+    const int smem = 1024 + p.stages * stage_bytes + (int)sizeof(WBars) + (4 + 2) * g.Dloc * 4 + 64;
+    static std::atomic<unsigned long long> raised_p{0};
+    if (cudaError_t e = raise_dynamic_smem(weights_fused_kernel<1, true>, 227 * 1024, raised_p); e != cudaSuccess) return e;
+    le = launch_dependent_cluster(weights_fused_kernel<1, true>, dim3((unsigned)(2 * tiles)), dim3(192), (size_t)smem, 2, s, tx, td,
+                                  (__nv_bfloat16*)w, (__nv_bfloat16*)wu, p, dev_status);
+    count_launch();
+    return le != cudaSuccess ? le : cudaGetLastError();
+  }
+  if (fused) {
+    const int stage_bytes = mblocks * 128 * 128 + ((b_rows * 128 + 1023) / 1024) * 1024;
+    p.stages = (200 * 1024) / stage_bytes;
+    p.stages = p.stages > 4 ? 4 : p.stages;
+    if (p.stages > nk) p.stages = nk;
+    const int smem = 1024 + p.stages * stage_bytes + (int)sizeof(WBars) + (4 * mblocks + 2) * g.Dloc * 4 + 64;
+    if (mblocks == 2) {
       static std::atomic<unsigned long long> raised2{0};
       if (cudaError_t e = raise_dynamic_smem(weights_fused_kernel<2>, 227 * 1024, raised2); e != cudaSuccess) return e;
-      le = launch_dependent(weights_fused_kernel<2>, dim3((unsigned)tiles), dim3(64 + 512), (size_t)smem, s, tx, txt, td,
+      le = launch_dependent(weights_fused_kernel<2>, dim3((unsigned)tiles), dim3(320), (size_t)smem, s, tx, td,
                             (__nv_bfloat16*)w, (__nv_bfloat16*)wu, p, dev_status);
     } else {
       static std::atomic<unsigned long long> raised1{0};
-      if (cudaError_t e = raise_dynamic_smem(weights_fused_kernel<1, true>, 227 * 1024, raised1); e != cudaSuccess) return e;
-      le = launch_dependent_cluster(weights_fused_kernel<1, true>, dim3((unsigned)(mblocks * tiles)), dim3(64 + 256), (size_t)smem, mblocks, s, tx, txt,
-                                    td, (__nv_bfloat16*)w, (__nv_bfloat16*)wu, p, dev_status);
+      if (cudaError_t e = raise_dynamic_smem(weights_fused_kernel<1>, 227 * 1024, raised1); e != cudaSuccess) return e;
+      le = launch_dependent(weights_fused_kernel<1>, dim3((unsigned)tiles), dim3(192), (size_t)smem, s, tx, td,
+                            (__nv_bfloat16*)w, (__nv_bfloat16*)wu, p, dev_status);
     }
     count_launch();
     return le != cudaSuccess ? le : cudaGetLastError();
@@ -806,17 +681,17 @@ cudaError_t launch_weights_tc(const Geom& g, const void* x, const int32_t* idx, 
   static std::atomic<unsigned long long> smem_raised{0};
   if (cudaError_t e = raise_dynamic_smem(weights_logits_kernel, 200 * 1024, smem_raised); e != cudaSuccess) return e;
   dim3 grid((unsigned)tiles, mblocks, (g.Dloc + p.d_block - 1) / p.d_block);
-  le = launch_dependent(weights_logits_kernel, grid, dim3(192), (size_t)smem, s, tx, txt, td, shares, zpart, p, dev_status);
+  le = launch_dependent(weights_logits_kernel, grid, dim3(192), (size_t)smem, s, tx, td, shares, zpart, p, dev_status);
   count_launch();
   if (le != cudaSuccess) return le;
   const float* zsrc = zpart;
   int zblocks = mblocks;
   if (blocked) {  // softmax over the full rows, then the destinations' row sums in two deterministic steps
-    const int nrb = (g.Nloc + kSoftmaxRows - 1) / kSoftmaxRows;
+    const int nrb = g.Nloc / kSoftmaxRows;
     float* zblk = zpart;
     float* z = (float*)((char*)zblk + ((tiles * nrb * g.Dloc * 4 + 255) / 256) * 256);
     le = launch_dependent(softmax_rows_kernel, dim3((unsigned)nrb, (unsigned)tiles), dim3(256), 0, s, shares,
-                          zblk, g.Nloc, g.Dloc, p.pitch);
+                          zblk, g.Nloc, g.Dloc);
     count_launch();
     if (le != cudaSuccess) return le;
     le = launch_dependent(z_reduce_kernel, dim3((unsigned)((g.Dloc + 31) / 32), (unsigned)tiles), dim3(256), 0, s,
@@ -825,17 +700,6 @@ cudaError_t launch_weights_tc(const Geom& g, const void* x, const int32_t* idx, 
     if (le != cudaSuccess) return le;
     zsrc = z;
     zblocks = 1;
-  }
-  if (g.Dloc % 4 != 0) {
-    static std::atomic<unsigned long long> raised_r{0};
-    if (g.Dloc * 4 > 48 * 1024)
-      if (cudaError_t e = raise_dynamic_smem(weights_normalise_ragged_kernel, 200 * 1024, raised_r); e != cudaSuccess) return e;
-    int blocks = (g.Nloc + 31) / 32;  // four rows per warp
-    blocks = blocks > 1024 ? 1024 : blocks;
-    le = launch_dependent(weights_normalise_ragged_kernel, dim3((unsigned)blocks, (unsigned)tiles), dim3(256), (size_t)g.Dloc * 4, s,
-                          (const float*)shares, zsrc, (__nv_bfloat16*)w, (__nv_bfloat16*)wu, g.Nloc, g.Dloc, p.pitch, zblocks);
-    count_launch();
-    return le != cudaSuccess ? le : cudaGetLastError();
   }
   const int quads = g.Nloc * g.Dloc / 4;
   int nblocks = (quads + 1023) / 1024;  // four quads per thread
