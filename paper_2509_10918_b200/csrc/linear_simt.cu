@@ -3,51 +3,238 @@
 // (Sec. 4.2.2).  They serve the fp32 mode (whose 1e-4 tolerance rules out
 // reduced-precision tensor-core inputs) and every shape the tensor-core kernels do not
 // cover.
+#include <math.h>
+
 #include "common.cuh"
 
 namespace toma {
 
-// C[m][n] = sum_k A(m,k) B(k,n) for one batch entry (blockIdx.z); 64x64x16 tiles,
-// 256 threads, 4x4 outputs per thread.  `Op` supplies the element accessors.
-template <class Op, typename AccT>
-__global__ void __launch_bounds__(256) simt_gemm_kernel(Op op) {
-  __shared__ float As[16][65];
-  __shared__ float Bs[16][65];
-  const int batch = blockIdx.z;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  AccT acc[4][4] = {};
-  for (int k0 = 0; k0 < op.K; k0 += 16) {
-    for (int e = threadIdx.x; e < 64 * 16; e += 256) {
-      int r, c;
-      if (Op::a_k_contig) { r = e >> 4; c = e & 15; } else { r = e & 63; c = e >> 6; }
-      As[c][r] = (m0 + r < op.M && k0 + c < op.K) ? op.a(batch, m0 + r, k0 + c) : 0.f;
-      if (Op::b_k_contig) { r = e >> 4; c = e & 15; } else { r = e & 63; c = e >> 6; }
-      Bs[c][r] = (n0 + r < op.N && k0 + c < op.K) ? op.b(batch, k0 + c, n0 + r) : 0.f;
+// Four consecutive elements as floats; `vec`: the address is aligned for one load of all four.
+__device__ __forceinline__ float4 load4(const float* p, int n, bool vec) {
+  if (vec && n >= 4) return *reinterpret_cast<const float4*>(p);
+  return make_float4(n > 0 ? p[0] : 0.f, n > 1 ? p[1] : 0.f, n > 2 ? p[2] : 0.f, n > 3 ? p[3] : 0.f);
+}
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p, int n, bool vec) {
+  if (vec && n >= 4) {
+    const uint2 q = *reinterpret_cast<const uint2*>(p);
+    return make_float4(__uint_as_float(q.x << 16), __uint_as_float(q.x & 0xFFFF0000u), __uint_as_float(q.y << 16),
+                       __uint_as_float(q.y & 0xFFFF0000u));
+  }
+  return make_float4(n > 0 ? to_f32(p[0]) : 0.f, n > 1 ? to_f32(p[1]) : 0.f, n > 2 ? to_f32(p[2]) : 0.f, n > 3 ? to_f32(p[3]) : 0.f);
+}
+
+// Two columns of a row of sums: two floats in a 64-bit register, so that one packed fma (one issue slot) serves both,
+// or two doubles.
+struct Sum2f {
+  unsigned long long v;
+  __device__ __forceinline__ void fma(unsigned long long a2, unsigned long long b2) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(v) : "l"(a2), "l"(b2)); }
+  __device__ __forceinline__ void get(float* o) const { asm("mov.b64 {%0, %1}, %2;" : "=f"(o[0]), "=f"(o[1]) : "l"(v)); }
+};
+struct Sum2d {
+  double x, y;
+  __device__ __forceinline__ void fma(unsigned long long a2, unsigned long long b2) {
+    float a, b0, b1;
+    asm("{\n\t.reg .f32 t;\n\tmov.b64 {%0, t}, %1;\n\t}" : "=f"(a) : "l"(a2));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(b0), "=f"(b1) : "l"(b2));
+    x = ::fma((double)a, (double)b0, x);
+    y = ::fma((double)a, (double)b1, y);
+  }
+  __device__ __forceinline__ void get(double* o) const { o[0] = x; o[1] = y; }
+  __device__ __forceinline__ void add(double a, double b) { x += a, y += b; }
+};
+
+template <typename AccT> struct SumOf { typedef Sum2f Pair; };
+template <> struct SumOf<double> { typedef Sum2d Pair; };
+
+// C[m][n] = sum_k A(m,k) B(k,n) for one batch entry (blockIdx.z), every sum one chain of fused multiply-adds in
+// ascending k (the result does not depend on the tile form).  Tile BM x BN, TM x TN outputs per thread, 16
+// contraction steps per stage: the next stage's operands are on their way into registers (16-byte loads along the
+// operand's contiguous axis) while the current one is multiplied out of shared memory, two stages deep.  Both
+// operands lie there as [k][row], rows swizzled by 8 ((k / 4) % 4), which keeps groups of eight together for the
+// 16-byte reads and the transposing stores free of bank conflicts.
+// KG > 1 (double sums only, where the order of addition does not show): that many thread groups share a tile, each with
+// a part of every stage's k, and add up through shared memory at the end: for products too small to fill the SMs.
+// `Op`: a_ptr / b_ptr give the contiguous line of an operand (a row m or n if k runs along it, else a row k).
+constexpr int kBK = 16;
+template <int kRows>
+__device__ __forceinline__ constexpr int swz(int k4) { return 8 * (k4 & 3 & (kRows / 8 - 1)); }
+
+template <class Op, typename AccT, int BM, int BN, int TM, int TN, int KG>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, KG > 1 || BM == 128 ? 2 : 4) simt_gemm_kernel(const Op op) {
+  using Acc = typename SumOf<AccT>::Pair;
+  constexpr int kGroup = (BM / TM) * (BN / TN), kThreads = kGroup * KG;
+  constexpr int kPackA = BM * kBK / 4, kPackB = BN * kBK / 4;  // 4-element packets of a stage
+  constexpr int kVecA = (kPackA + kThreads - 1) / kThreads, kVecB = (kPackB + kThreads - 1) / kThreads;
+  __shared__ __align__(16) float As[2][kBK][BM];
+  __shared__ __align__(16) float Bs[2][kBK][BN];
+  const int batch = blockIdx.z, m0 = blockIdx.y * BM, n0 = blockIdx.x * BN, tid = threadIdx.x;
+  const int in_group = tid % kGroup, kg = tid / kGroup;
+  const int tn = in_group % (BN / TN) * 4, tm = in_group / (BN / TN) * TM;  // columns tn .. + 3, and with TN = 8 BN / 2 further on
+  // packet e of an operand: k along the line: line e / 4, k 4 (e % 4); else: k e / (rows / 4), rows 4 (e % (rows / 4))
+  float4 ra[kVecA], rb[kVecB];
+  typename Op::APtr pa[kVecA];  // lines of an operand with k along them stay the same for the whole sum
+  typename Op::BPtr pb[kVecB];
+  bool ha[kVecA], hb[kVecB];    // ... and are there
+  if (Op::a_k_contig) {
+#pragma unroll
+    for (int v = 0; v < kVecA; ++v) {
+      const int r = m0 + (tid + v * kThreads) / 4;
+      ha[v] = r < op.M && tid + v * kThreads < kPackA;
+      pa[v] = op.a_ptr(batch, ha[v] ? r : 0);
     }
-    __syncthreads();
+  }
+  if (Op::b_k_contig) {
 #pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      float a[4], b[4];
+    for (int v = 0; v < kVecB; ++v) {
+      const int r = n0 + (tid + v * kThreads) / 4;
+      hb[v] = r < op.N && tid + v * kThreads < kPackB;
+      pb[v] = op.b_ptr(batch, hb[v] ? r : 0);
+    }
+  }
+  auto fetch = [&](int k0) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        a[u] = As[c][ty * 4 + u];
-        b[u] = Bs[c][tx * 4 + u];
+    for (int v = 0; v < kVecA; ++v) {
+      const int e = tid + v * kThreads;
+      if (Op::a_k_contig) {
+        const int k = k0 + 4 * (e & 3);
+        ra[v] = ha[v] ? load4(pa[v] + k, op.K - k, op.a_vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+      } else {
+        const int k = k0 + e / (BM / 4), r = m0 + 4 * (e % (BM / 4));
+        ra[v] = e < kPackA && k < op.K && r < op.M ? load4(op.a_ptr(batch, k) + r, op.M - r, op.a_vec) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
+    }
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+    for (int v = 0; v < kVecB; ++v) {
+      const int e = tid + v * kThreads;
+      if (Op::b_k_contig) {
+        const int k = k0 + 4 * (e & 3);
+        rb[v] = hb[v] ? load4(pb[v] + k, op.K - k, op.b_vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+      } else {
+        const int k = k0 + e / (BN / 4), r = n0 + 4 * (e % (BN / 4));
+        rb[v] = e < kPackB && k < op.K && r < op.N ? load4(op.b_ptr(batch, k) + r, op.N - r, op.b_vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+  };
+  auto put = [&](int st) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] += (AccT)a[u] * (AccT)b[v];
+    for (int v = 0; v < kVecA; ++v) {
+      const int e = tid + v * kThreads;
+      if (kPackA % kThreads && e >= kPackA) continue;
+      if (Op::a_k_contig) {
+        const int r = e / 4, k = 4 * (e & 3), c = r ^ swz<BM>(e & 3);
+        As[st][k][c] = ra[v].x;
+        As[st][k + 1][c] = ra[v].y;
+        As[st][k + 2][c] = ra[v].z;
+        As[st][k + 3][c] = ra[v].w;
+      } else {
+        const int k = e / (BM / 4), r = 4 * (e % (BM / 4));
+        *reinterpret_cast<float4*>(&As[st][k][r ^ swz<BM>(k >> 2)]) = ra[v];
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < kVecB; ++v) {
+      const int e = tid + v * kThreads;
+      if (kPackB % kThreads && e >= kPackB) continue;
+      if (Op::b_k_contig) {
+        const int r = e / 4, k = 4 * (e & 3), c = r ^ swz<BN>(e & 3);
+        Bs[st][k][c] = rb[v].x; Bs[st][k + 1][c] = rb[v].y; Bs[st][k + 2][c] = rb[v].z; Bs[st][k + 3][c] = rb[v].w;
+      } else {
+        const int k = e / (BN / 4), r = 4 * (e % (BN / 4));
+        *reinterpret_cast<float4*>(&Bs[st][k][r ^ swz<BN>(k >> 2)]) = rb[v];
+      }
+    }
+  };
+  Acc acc[TM][TN / 2] = {};
+  fetch(0);
+  put(0);
+  __syncthreads();
+  int st = 0;
+  for (int k0 = 0; k0 < op.K; k0 += kBK, st ^= 1) {
+    const bool more = k0 + kBK < op.K;
+    if (more) fetch(k0 + kBK);
+#pragma unroll
+    for (int kk = 0; kk < kBK / KG; ++kk) {
+      const int k = KG == 1 ? kk : kg * (kBK / KG) + kk;
+      float4 a[TM / 4];
+      ulonglong2 b[TN / 4];
+#pragma unroll
+      for (int u = 0; u < TM / 4; ++u) a[u] = *reinterpret_cast<const float4*>(&As[st][k][(tm + 4 * u) ^ swz<BM>(k >> 2)]);
+#pragma unroll
+      for (int u = 0; u < TN / 4; ++u) b[u] = *reinterpret_cast<const ulonglong2*>(&Bs[st][k][(tn + u * (BN / 2)) ^ swz<BN>(k >> 2)]);
+#pragma unroll
+      for (int u = 0; u < TM / 4; ++u) {
+        const float av[4] = {a[u].x, a[u].y, a[u].z, a[u].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          unsigned long long a2;
+          asm("mov.b64 %0, {%1, %1};" : "=l"(a2) : "f"(av[e]));
+#pragma unroll
+          for (int q = 0; q < TN / 4; ++q) {
+            acc[4 * u + e][2 * q].fma(a2, b[q].x);
+            acc[4 * u + e][2 * q + 1].fma(a2, b[q].y);
+          }
+        }
+      }
+    }
+    if (more) {
+      put(st ^ 1);  // last read before the previous barrier
+      __syncthreads();
+    }
+  }
+  if constexpr (KG > 1) {  // groups 1 .. KG - 1 hand their sums to group 0
+    __shared__ AccT part[KG - 1][TM * TN][kGroup];
+    if (kg > 0) {
+#pragma unroll
+      for (int u = 0; u < TM; ++u)
+#pragma unroll
+        for (int q = 0; q < TN / 2; ++q) {
+          AccT v[2];
+          acc[u][q].get(v);
+          part[kg - 1][u * TN + 2 * q][in_group] = v[0];
+          part[kg - 1][u * TN + 2 * q + 1][in_group] = v[1];
+        }
     }
     __syncthreads();
+    if (kg > 0) return;
+#pragma unroll
+    for (int u = 0; u < TM; ++u)
+#pragma unroll
+      for (int q = 0; q < TN / 2; ++q)
+#pragma unroll
+        for (int g = 0; g < KG - 1; ++g) acc[u][q].add(part[g][u * TN + 2 * q][in_group], part[g][u * TN + 2 * q + 1][in_group]);
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
+  for (int u = 0; u < TM; ++u) {
+    const int m = m0 + tm + u;
+    if (m >= op.M) break;
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int m = m0 + ty * 4 + u, n = n0 + tx * 4 + v;
-      if (m < op.M && n < op.N) op.store(batch, m, n, acc[u][v]);
+    for (int q = 0; q < TN / 4; ++q) {
+      const int n = n0 + tn + q * (BN / 2);
+      AccT v[4];
+      acc[u][2 * q].get(v);
+      acc[u][2 * q + 1].get(v + 2);
+      if (n < op.N) op.store4(batch, m, n, op.N - n, v);
     }
+  }
+}
+
+// Four consecutive outputs of a row, `n` of them real.
+template <typename T>
+__device__ __forceinline__ void put4(T* p, int n, bool vec, const float (&v)[4]) {
+  if (vec && n >= 4) {
+    if constexpr (sizeof(T) == 4) {
+      *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+      __align__(8) __nv_bfloat16 h[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) from_f32(h[e], v[e]);
+      *reinterpret_cast<uint2*>(p) = *reinterpret_cast<const uint2*>(h);
+    }
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (e < n) from_f32(p[e], v[e]);
+  }
 }
 
 struct TileMap {
@@ -86,23 +273,45 @@ static TileMap make_map(const Geom& g) {
   return TileMap{g.P, g.tiles_x, g.th, g.tw, g.W, g.Nloc, g.Dloc, g.d, (int)g.tokens_all(), g.Lm};
 }
 
+// Stored weights A~^T as an operand: the fp32 plane, or the sum of the two bf16 planes.
+struct SplitW {
+  const __nv_bfloat16* hi;
+  size_t plane;
+  __device__ __forceinline__ SplitW operator+(int e) const { return SplitW{hi + e, plane}; }
+};
+__device__ __forceinline__ float4 load4(const SplitW& p, int n, bool) {
+  float v[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) v[e] = e < n ? to_f32(p.hi[e]) + to_f32(p.hi[p.plane + e]) : 0.f;
+  return make_float4(v[0], v[1], v[2], v[3]);
+}
+
+__device__ __forceinline__ const float* w_line(const float* w, int batch, size_t off, size_t plane) { return w + batch * plane + off; }
+__device__ __forceinline__ SplitW w_line(const __nv_bfloat16* w, int batch, size_t off, size_t plane) {
+  return SplitW{w + batch * 2 * plane + off, plane};
+}
+template <typename WT> struct WLine { typedef const float* Ptr; };
+template <> struct WLine<__nv_bfloat16> { typedef SplitW Ptr; };
+
 // logits[batch][i][k] = <X[idx_i], X_k> * scale
 template <typename T>
 struct LogitsOp {
   static constexpr bool a_k_contig = true, b_k_contig = true;
+  typedef const T* APtr;
+  typedef const T* BPtr;
   int M, N, K;
+  bool a_vec, b_vec;
   TileMap tm;
   const T* x;
   const int32_t* idx;
   float* logits;
   float scale;
-  __device__ __forceinline__ float a(int batch, int i, int c) const {
-    return to_f32(x[tm.x_row(batch, idx[(size_t)batch * tm.Dloc + i]) * tm.d + c]);
-  }
-  __device__ __forceinline__ float b(int batch, int c, int k) const { return to_f32(x[tm.x_row(batch, k) * tm.d + c]); }
+  __device__ __forceinline__ const T* a_ptr(int batch, int i) const { return x + tm.x_row(batch, idx[(size_t)batch * tm.Dloc + i]) * tm.d; }
+  __device__ __forceinline__ const T* b_ptr(int batch, int k) const { return x + tm.x_row(batch, k) * tm.d; }
   template <typename AccT>
-  __device__ __forceinline__ void store(int batch, int i, int k, AccT v) const {
-    logits[((size_t)batch * tm.Dloc + i) * tm.Nloc + k] = (float)(v * (AccT)scale);
+  __device__ __forceinline__ void store4(int batch, int i, int k, int n, const AccT* v) const {
+    const float f[4] = {(float)(v[0] * (AccT)scale), (float)(v[1] * (AccT)scale), (float)(v[2] * (AccT)scale), (float)(v[3] * (AccT)scale)};
+    put4(logits + ((size_t)batch * tm.Dloc + i) * tm.Nloc + k, n, tm.Nloc % 4 == 0, f);
   }
 };
 
@@ -110,17 +319,19 @@ struct LogitsOp {
 template <typename T, typename WT>
 struct MergeOp {
   static constexpr bool a_k_contig = false, b_k_contig = false;
+  typedef typename WLine<WT>::Ptr APtr;
+  typedef const T* BPtr;
   int M, N, K;
+  bool a_vec, b_vec;
   TileMap tm;
   const WT* w;
   const T* x;
   T* xm;
-  __device__ __forceinline__ float a(int batch, int i, int k) const {
-    return w_load(w, batch, (size_t)k * tm.Dloc + i, (size_t)tm.Nloc * tm.Dloc);
-  }
-  __device__ __forceinline__ float b(int batch, int k, int c) const { return to_f32(x[tm.x_row(batch, k) * tm.d + c]); }
-  __device__ __forceinline__ void store(int batch, int i, int c, float v) const {
-    from_f32(xm[tm.m_row(batch, i) * tm.d + c], v);
+  __device__ __forceinline__ APtr a_ptr(int batch, int k) const { return w_line(w, batch, (size_t)k * tm.Dloc, (size_t)tm.Nloc * tm.Dloc); }
+  __device__ __forceinline__ const T* b_ptr(int batch, int k) const { return x + tm.x_row(batch, k) * tm.d; }
+  __device__ __forceinline__ void store4(int batch, int i, int c, int n, const float* v) const {
+    const float f[4] = {v[0], v[1], v[2], v[3]};
+    put4(xm + tm.m_row(batch, i) * tm.d + c, n, true, f);
   }
 };
 
@@ -128,84 +339,192 @@ struct MergeOp {
 template <typename T, typename WT>
 struct UnmergeOp {
   static constexpr bool a_k_contig = true, b_k_contig = false;
+  typedef typename WLine<WT>::Ptr APtr;
+  typedef const T* BPtr;
   int M, N, K;
+  bool a_vec, b_vec;
   TileMap tm;
   const WT* w;
   const T* y;
   T* out;
-  __device__ __forceinline__ float a(int batch, int k, int i) const {
-    return w_load(w, batch, (size_t)k * tm.Dloc + i, (size_t)tm.Nloc * tm.Dloc);
-  }
-  __device__ __forceinline__ float b(int batch, int i, int c) const { return to_f32(y[tm.m_row(batch, i) * tm.d + c]); }
-  __device__ __forceinline__ void store(int batch, int k, int c, float v) const {
-    from_f32(out[tm.x_row(batch, k) * tm.d + c], v);
+  __device__ __forceinline__ APtr a_ptr(int batch, int k) const { return w_line(w, batch, (size_t)k * tm.Dloc, (size_t)tm.Nloc * tm.Dloc); }
+  __device__ __forceinline__ const T* b_ptr(int batch, int i) const { return y + tm.m_row(batch, i) * tm.d; }
+  __device__ __forceinline__ void store4(int batch, int k, int c, int n, const float* v) const {
+    const float f[4] = {v[0], v[1], v[2], v[3]};
+    put4(out + tm.x_row(batch, k) * tm.d + c, n, true, f);
   }
 };
 
-template <class Op, typename AccT>
-static void run_gemm(const Op& op, int batches, cudaStream_t s) {
-  dim3 grid((op.N + 63) / 64, (op.M + 63) / 64, batches);
-  simt_gemm_kernel<Op, AccT><<<grid, 256, 0, s>>>(op);
+template <class Op, typename AccT, int BM, int BN, int TM, int TN, int KG = 1>
+static void run_tile(const Op& op, int batches, cudaStream_t s) {
+  const dim3 grid((op.N + BN - 1) / BN, (op.M + BM - 1) / BM, batches);
+  simt_gemm_kernel<Op, AccT, BM, BN, TM, TN, KG><<<grid, (BM / TM) * (BN / TN) * KG, 0, s>>>(op);
   count_launch();
 }
 
-// Softmax over the destination axis for every source token (a token's shares sum to 1).
-// One thread per (tile, source k); logits[batch][i][k] is overwritten with A_ik.
-__global__ void __launch_bounds__(128) softmax_dest_kernel(float* __restrict__ logits, int Nloc, int Dloc) {
+// Tile form: the least work on the fullest SM, padding included.  A larger tile reads its operands less often per
+// multiply-add (rel: its measured rate per SM against the 128 x 128 form once eight warps or more are resident); with
+// fewer warps an SM cannot hide its latencies and runs in proportion slower.
+struct TileForm {
+  int bm, bn, warps;
+  double rel;
+};
+static int pick_form(const TileForm* f, int n, int M, int N, int batches) {
+  int best = 0;
+  double best_cost = 0.0;
+  for (int i = 0; i < n; ++i) {
+    const double ctas = (double)((M + f[i].bm - 1) / f[i].bm) * ((N + f[i].bn - 1) / f[i].bn) * batches;
+    const double per_sm = ceil(ctas / sm_count()), warps = per_sm * f[i].warps;
+    const double cost = per_sm * f[i].bm * f[i].bn / f[i].rel * (warps < 8 ? 8 / warps : 1.0);
+    if (i == 0 || cost < best_cost) best = i, best_cost = cost;
+  }
+  return best;
+}
+
+template <class Op, typename AccT>
+static void run_gemm(const Op& op, int batches, cudaStream_t s) {
+  if constexpr (sizeof(AccT) == 8) {
+    static constexpr TileForm forms[] = {{64, 64, 8, 1.0}, {32, 32, 8, 0.8}, {16, 32, 4, 0.7}};
+    switch (pick_form(forms, 3, op.M, op.N, batches)) {
+      case 0: run_tile<Op, AccT, 64, 64, 4, 4>(op, batches, s); break;
+      case 1: run_tile<Op, AccT, 32, 32, 4, 4, 4>(op, batches, s); break;
+      default: run_tile<Op, AccT, 16, 32, 4, 4, 4>(op, batches, s);
+    }
+  } else {
+    static constexpr TileForm forms[] = {{128, 128, 8, 1.0}, {64, 64, 4, 0.85}, {32, 64, 4, 0.6}};
+    switch (pick_form(forms, 3, op.M, op.N, batches)) {
+      case 0: run_tile<Op, AccT, 128, 128, 8, 8>(op, batches, s); break;
+      case 1: run_tile<Op, AccT, 64, 64, 4, 8>(op, batches, s); break;
+      default: run_tile<Op, AccT, 32, 64, 4, 4>(op, batches, s);
+    }
+  }
+}
+
+// Softmax over the destination axis for every source token (a token's shares sum to 1); logits[batch][i][k] is
+// overwritten with A_ik.  A CTA takes 32 source tokens: maxima and exponentials by all its threads (eight rows of 128
+// bytes at a time), the denominator of a token by one thread in destination order, out of shared memory.
+constexpr int kSoftTok = 32, kSoftThreads = 512;
+__global__ void __launch_bounds__(kSoftThreads) softmax_dest_kernel(float* __restrict__ logits, int Nloc, int Dloc) {
+  extern __shared__ float e_smem[];  // [D_loc][32] exponentials
+  __shared__ float red[kSoftThreads / 32][kSoftTok];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = blockIdx.x * kSoftTok + lane;
+  constexpr int kWarps = kSoftThreads / 32;
+  const bool live = k < Nloc;
+  float* L = logits + (size_t)blockIdx.y * Dloc * Nloc + (live ? k : 0);
+  float mx = -INFINITY;
+#pragma unroll 8
+  for (int i = warp; i < Dloc; i += kWarps) {
+    const float v = L[(size_t)i * Nloc];
+    e_smem[i * kSoftTok + lane] = v;
+    mx = fmaxf(mx, v);
+  }
+  red[warp][lane] = mx;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) mx = fmaxf(mx, red[w][lane]);
+#pragma unroll 4
+  for (int i = warp; i < Dloc; i += kWarps) e_smem[i * kSoftTok + lane] = expf(e_smem[i * kSoftTok + lane] - mx);
+  __syncthreads();
+  if (warp == 0) {
+    float sum = 0.f;
+#pragma unroll 16
+    for (int i = 0; i < Dloc; ++i) sum += e_smem[i * kSoftTok + lane];
+    red[0][lane] = 1.f / sum;
+  }
+  __syncthreads();
+  const float inv = red[0][lane];
+  if (live) {
+#pragma unroll 4
+    for (int i = warp; i < Dloc; i += kWarps) L[(size_t)i * Nloc] = e_smem[i * kSoftTok + lane] * inv;
+  }
+}
+// The same without shared memory for more destinations than it holds (global merge): one thread per source token.
+__global__ void __launch_bounds__(128) softmax_dest_long_kernel(float* __restrict__ logits, int Nloc, int Dloc) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= Nloc) return;
   float* L = logits + (size_t)blockIdx.y * Dloc * Nloc + k;
   float mx = -INFINITY;
+#pragma unroll 8
   for (int i = 0; i < Dloc; ++i) mx = fmaxf(mx, L[(size_t)i * Nloc]);
   float sum = 0.f;
+#pragma unroll 8
   for (int i = 0; i < Dloc; ++i) {
     const float e = expf(L[(size_t)i * Nloc] - mx);
     L[(size_t)i * Nloc] = e;
     sum += e;
   }
   const float inv = 1.f / sum;
+#pragma unroll 8
   for (int i = 0; i < Dloc; ++i) L[(size_t)i * Nloc] *= inv;
 }
 
-// Row normalisation: one warp per (tile, destination i); writes A~^T[k][i] = A_ik / sum_k' A_ik'
-// and, when wu is given, the shares themselves, A^T[k][i] = A_ik, in the same layout.
+// Row normalisation of 32 destinations of a region: A~^T[k][i] = A_ik / sum_k' A_ik' and, when wu is given, the shares
+// themselves, A^T[k][i] = A_ik, in the same layout.  A row's sum is a warp's (32 strided partial sums, then a tree); the
+// planes are written through a 32 x 32 transpose in shared memory, so that consecutive lanes write consecutive weights.
 template <typename WT>
 __global__ void __launch_bounds__(256) rownorm_kernel(const float* __restrict__ A, WT* __restrict__ w, WT* __restrict__ wu,
-                                                      int Nloc, int Dloc, int rows_total) {
-  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (row >= rows_total) return;
-  const int batch = row / Dloc, i = row - batch * Dloc;
-  const float* a = A + (size_t)row * Nloc;
-  float z = 0.f;
-  for (int k = lane; k < Nloc; k += 32) z += a[k];
+                                                      int Nloc, int Dloc) {
+  __shared__ float inv[32];
+  __shared__ float tr[8][32][33];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int batch = blockIdx.y, i0 = blockIdx.x * 32;
+  const int ni = min(32, Dloc - i0);
+  const float* a = A + ((size_t)batch * Dloc + i0) * Nloc;
+  for (int r = warp; r < ni; r += 8) {
+    float z = 0.f;
+#pragma unroll 8
+    for (int k = lane; k < Nloc; k += 32) z += a[(size_t)r * Nloc + k];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-  const float inv = z > 0.f ? 1.f / z : 0.f;
+    for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+    if (lane == 0) inv[r] = z > 0.f ? 1.f / z : 0.f;
+  }
+  __syncthreads();
   const size_t plane = (size_t)Nloc * Dloc;
-  for (int k = lane; k < Nloc; k += 32) w_store(w, batch, (size_t)k * Dloc + i, plane, a[k] * inv);
-  if (wu)
-    for (int k = lane; k < Nloc; k += 32) w_store(wu, batch, (size_t)k * Dloc + i, plane, a[k]);
+  for (int k0 = (blockIdx.z * 8 + warp) * 32; k0 < Nloc; k0 += gridDim.z * 256) {
+    const int nk = min(32, Nloc - k0);
+#pragma unroll 16
+    for (int r = 0; r < 32; ++r) tr[warp][lane][r] = r < ni && lane < nk ? a[(size_t)r * Nloc + k0 + lane] : 0.f;
+    __syncwarp();
+    if (lane < ni) {
+      const float f = inv[lane];
+#pragma unroll 4
+      for (int k = 0; k < nk; ++k) {
+        const float v = tr[warp][k][lane];
+        const size_t off = (size_t)(k0 + k) * Dloc + i0 + lane;
+        w_store(w, batch, off, plane, v * f);
+        if (wu) w_store(wu, batch, off, plane, v);
+      }
+    }
+    __syncwarp();
+  }
 }
 
 cudaError_t launch_weights_simt(const Geom& g, const void* x, const int32_t* idx, void* w, void* wu, float* logits,
                                 cudaStream_t s) {
   const int batches = g.B * g.P;
-  if (g.f32) {
-    LogitsOp<float> op{g.Dloc, g.Nloc, g.d, make_map(g), (const float*)x, idx, logits, g.logit_scale};
+  if (g.f32) {  // fp32 mode sums the logits in double: a logit of some hundreds has to be right to its last fp32 bit
+    LogitsOp<float> op{g.Dloc, g.Nloc, g.d, true, true, make_map(g), (const float*)x, idx, logits, g.logit_scale};
     run_gemm<LogitsOp<float>, double>(op, batches, s);
   } else {
-    LogitsOp<__nv_bfloat16> op{g.Dloc, g.Nloc, g.d, make_map(g), (const __nv_bfloat16*)x, idx, logits, g.logit_scale};
+    LogitsOp<__nv_bfloat16> op{g.Dloc, g.Nloc, g.d, true, true, make_map(g), (const __nv_bfloat16*)x, idx, logits, g.logit_scale};
     run_gemm<LogitsOp<__nv_bfloat16>, float>(op, batches, s);
   }
-  softmax_dest_kernel<<<dim3((g.Nloc + 127) / 128, batches), 128, 0, s>>>(logits, g.Nloc, g.Dloc);
+  const size_t smem = (size_t)g.Dloc * kSoftTok * 4;
+  if (smem <= 200 * 1024) {
+    static std::atomic<unsigned long long> raised{0};
+    if (cudaError_t e = raise_dynamic_smem(softmax_dest_kernel, 200 * 1024, raised); e != cudaSuccess) return e;
+    softmax_dest_kernel<<<dim3((g.Nloc + kSoftTok - 1) / kSoftTok, batches), kSoftThreads, smem, s>>>(logits, g.Nloc, g.Dloc);
+  } else {
+    softmax_dest_long_kernel<<<dim3((g.Nloc + 127) / 128, batches), 128, 0, s>>>(logits, g.Nloc, g.Dloc);
+  }
   count_launch();
-  const int rows = batches * g.Dloc;
-  const int blocks = (rows * 32 + 255) / 256;
-  if (g.f32)
-    rownorm_kernel<float><<<blocks, 256, 0, s>>>(logits, (float*)w, (float*)wu, g.Nloc, g.Dloc, rows);
-  else
-    rownorm_kernel<__nv_bfloat16><<<blocks, 256, 0, s>>>(logits, (__nv_bfloat16*)w, (__nv_bfloat16*)wu, g.Nloc, g.Dloc, rows);
+  // a CTA per 32 destinations, their source tokens split further where that leaves SMs idle (each part sums the rows anew)
+  const int blocks = (g.Dloc + 31) / 32;
+  int parts = 1;
+  while (parts < 8 && (long long)blocks * batches * parts < sm_count() && parts * 256 < g.Nloc) parts *= 2;
+  const dim3 grid(blocks, batches, parts);
+  if (g.f32) rownorm_kernel<float><<<grid, 256, 0, s>>>(logits, (float*)w, (float*)wu, g.Nloc, g.Dloc);
+  else rownorm_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(logits, (__nv_bfloat16*)w, (__nv_bfloat16*)wu, g.Nloc, g.Dloc);
   count_launch();
   return cudaGetLastError();
 }
@@ -243,11 +562,11 @@ cudaError_t launch_copy_extra(const Geom& g, const void* src, void* dst, bool me
 cudaError_t launch_merge_simt(const Geom& g, const void* w, const void* x, void* xm, cudaStream_t s) {
   const int batches = g.B * g.P;
   if (g.f32) {
-    MergeOp<float, float> op{g.Dloc, g.d, g.Nloc, make_map(g), (const float*)w, (const float*)x, (float*)xm};
+    MergeOp<float, float> op{g.Dloc, g.d, g.Nloc, g.Dloc % 4 == 0, true, make_map(g), (const float*)w, (const float*)x, (float*)xm};
     run_gemm<MergeOp<float, float>, float>(op, batches, s);
     copy_extra<float>(g, (const float*)x, (float*)xm, true, s);
   } else {
-    MergeOp<__nv_bfloat16, __nv_bfloat16> op{g.Dloc, g.d, g.Nloc, make_map(g), (const __nv_bfloat16*)w, (const __nv_bfloat16*)x,
+    MergeOp<__nv_bfloat16, __nv_bfloat16> op{g.Dloc, g.d, g.Nloc, false, true, make_map(g), (const __nv_bfloat16*)w, (const __nv_bfloat16*)x,
                                       (__nv_bfloat16*)xm};
     run_gemm<MergeOp<__nv_bfloat16, __nv_bfloat16>, float>(op, batches, s);
     copy_extra<__nv_bfloat16>(g, (const __nv_bfloat16*)x, (__nv_bfloat16*)xm, true, s);
@@ -258,11 +577,11 @@ cudaError_t launch_merge_simt(const Geom& g, const void* w, const void* x, void*
 cudaError_t launch_unmerge_simt(const Geom& g, const void* w, const void* y, void* out, cudaStream_t s) {
   const int batches = g.B * g.P;
   if (g.f32) {
-    UnmergeOp<float, float> op{g.Nloc, g.d, g.Dloc, make_map(g), (const float*)w, (const float*)y, (float*)out};
+    UnmergeOp<float, float> op{g.Nloc, g.d, g.Dloc, g.Dloc % 4 == 0, true, make_map(g), (const float*)w, (const float*)y, (float*)out};
     run_gemm<UnmergeOp<float, float>, float>(op, batches, s);
     copy_extra<float>(g, (const float*)y, (float*)out, false, s);
   } else {
-    UnmergeOp<__nv_bfloat16, __nv_bfloat16> op{g.Nloc, g.d, g.Dloc, make_map(g), (const __nv_bfloat16*)w, (const __nv_bfloat16*)y,
+    UnmergeOp<__nv_bfloat16, __nv_bfloat16> op{g.Nloc, g.d, g.Dloc, false, true, make_map(g), (const __nv_bfloat16*)w, (const __nv_bfloat16*)y,
                                         (__nv_bfloat16*)out};
     run_gemm<UnmergeOp<__nv_bfloat16, __nv_bfloat16>, float>(op, batches, s);
     copy_extra<__nv_bfloat16>(g, (const __nv_bfloat16*)y, (__nv_bfloat16*)out, false, s);
@@ -274,26 +593,30 @@ cudaError_t launch_unmerge_simt(const Geom& g, const void* w, const void* y, voi
 template <typename T>
 struct LinearOp {
   static constexpr bool a_k_contig = true, b_k_contig = false;
+  typedef const T* APtr;
+  typedef const T* BPtr;
   int M, N, K;
+  bool a_vec, b_vec;
   const T* a_;
   const T* w_;
   T* c_;
   int act;
-  __device__ __forceinline__ float a(int, int m, int k) const { return to_f32(a_[(size_t)m * K + k]); }
-  __device__ __forceinline__ float b(int, int k, int n) const { return to_f32(w_[(size_t)k * N + n]); }
-  template <typename AccT>
-  __device__ __forceinline__ void store(int, int m, int n, AccT v) const {
-    const float f = (float)v;
-    from_f32(c_[(size_t)m * N + n], act == kActGelu ? gelu(f) : f);
+  __device__ __forceinline__ const T* a_ptr(int, int m) const { return a_ + (size_t)m * K; }
+  __device__ __forceinline__ const T* b_ptr(int, int k) const { return w_ + (size_t)k * N; }
+  __device__ __forceinline__ void store4(int, int m, int n, int left, const float* v) const {
+    float f[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) f[e] = act == kActGelu ? gelu(v[e]) : v[e];
+    put4(c_ + (size_t)m * N + n, left, N % 4 == 0, f);
   }
 };
 
 cudaError_t launch_linear_simt(int M, int N, int K, bool f32, const void* a, const void* w, void* c, int act, cudaStream_t s) {
   if (f32) {
-    LinearOp<float> op{M, N, K, (const float*)a, (const float*)w, (float*)c, act};
+    LinearOp<float> op{M, N, K, K % 4 == 0, N % 4 == 0, (const float*)a, (const float*)w, (float*)c, act};
     run_gemm<LinearOp<float>, float>(op, 1, s);
   } else {
-    LinearOp<__nv_bfloat16> op{M, N, K, (const __nv_bfloat16*)a, (const __nv_bfloat16*)w, (__nv_bfloat16*)c, act};
+    LinearOp<__nv_bfloat16> op{M, N, K, K % 4 == 0, N % 4 == 0, (const __nv_bfloat16*)a, (const __nv_bfloat16*)w, (__nv_bfloat16*)c, act};
     run_gemm<LinearOp<__nv_bfloat16>, float>(op, 1, s);
   }
   return cudaGetLastError();
