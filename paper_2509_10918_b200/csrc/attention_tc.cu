@@ -37,6 +37,8 @@
 // registers for both the maximum and the exponentials.
 // Keys past the sequence end are zero-filled by TMA and masked out; query rows past the end are
 // computed on zeros and not written.
+#include <mutex>
+
 #include "attention_core.cuh"
 #include "common.cuh"
 #include "tc.cuh"
@@ -855,15 +857,13 @@ int cut_spans(int T, int nblk, long long C, int gmax, int* bounds) {
 // otherwise spans cut at single key tiles: evenly where a span holds two units or more (the pieces' costs are
 // small beside it), else so that the longest span, pieces' costs included, is as short as possible (the
 // smallest budget C for which a left-to-right cut needs no more spans than there are CTAs).
-Spans plan_spans(int units, int nblk) {
+Spans make_spans(int units, int nblk, int gmax, int forced) {
   Spans sp = {};
   sp.nblk = nblk;
   sp.T = units * nblk;
-  const int gmax = max_ctas();
   const int whole_tiles = ((units + gmax - 1) / gmax) * nblk;  // longest CTA with whole units
   const int even_tiles = (sp.T + gmax - 1) / gmax;             // longest CTA with an even cut
   int mode = whole_tiles <= even_tiles + kSplitCostTiles ? 0 : 1;
-  const int forced = g_tune_attention_split.load(std::memory_order_relaxed);  // test-only override
   if (forced == 0 || forced == 1) mode = forced;
   sp.split = mode;
   const int quantum = mode == 0 ? nblk : 1;
@@ -880,7 +880,13 @@ Spans plan_spans(int units, int nblk) {
     }
   } else if (mode == 1) {
     // spans of less than two units: the pieces' costs decide
-    long long lo = 2 + kPieceCostPartial, hi = 2LL * sp.T + (long long)kPieceCostPartial * (units + 2);
+    // (no budget below an even share of the tiles will do; the search climbs from there before it bisects)
+    long long lo = 2LL * sp.T / gmax > 2 + kPieceCostPartial ? 2LL * sp.T / gmax : 2 + kPieceCostPartial, step = 4, hi = lo;
+    while (!cut_spans(sp.T, nblk, hi, gmax, sp.bounds)) {
+      lo = hi + 1;
+      hi += step;
+      step *= 2;
+    }
     while (lo < hi) {  // cut_spans succeeds for every budget from some value on
       const long long mid = (lo + hi) / 2;
       if (cut_spans(sp.T, nblk, mid, gmax, sp.bounds)) hi = mid;
@@ -896,6 +902,37 @@ Spans plan_spans(int units, int nblk) {
     }
   }
   return sp;
+}
+
+// The plan of a launch, kept from call to call: it depends on these four numbers alone, and working it out costs the
+// host 15 to 40 us - as much as the kernel of a small call takes.  Bounded: the least recently used of 32 plans goes.
+void plan_spans(int units, int nblk, Spans* out) {
+  struct Entry {
+    int units = 0, nblk = 0, gmax = 0, forced = 0;
+    unsigned long long used = 0;
+    Spans sp;
+  };
+  static std::mutex mu;
+  static Entry cache[32];
+  static unsigned long long clock = 0;
+  const int gmax = max_ctas(), forced = g_tune_attention_split.load(std::memory_order_relaxed);  // test-only override
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    for (Entry& e : cache)
+      if (e.used && e.units == units && e.nblk == nblk && e.gmax == gmax && e.forced == forced) {
+        e.used = ++clock;
+        *out = e.sp;
+        return;
+      }
+  }
+  *out = make_spans(units, nblk, gmax, forced);
+  std::lock_guard<std::mutex> lock(mu);
+  Entry* oldest = cache;
+  for (Entry& e : cache)
+    if (e.used < oldest->used) oldest = &e;
+  oldest->units = units, oldest->nblk = nblk, oldest->gmax = gmax, oldest->forced = forced;
+  oldest->used = ++clock;
+  oldest->sp = *out;
 }
 
 template <int DH>
@@ -917,7 +954,8 @@ cudaError_t launch(int B, int L, int heads, const void* q, const void* k, const 
   const long long units = (long long)B * heads * ((L + kUM - 1) / kUM);
   const int nblk = (L + kBN - 1) / kBN;
   if (units * nblk > 0x7fffffffLL) return cudaErrorInvalidValue;  // iteration indices are 32-bit
-  const Spans sp = plan_spans((int)units, nblk);
+  Spans sp;
+  plan_spans((int)units, nblk, &sp);
   const size_t tb = ticket_bytes(B, L, heads);
   if (sp.split && !tickets_clean) {  // units are split: their tickets start at zero
     e = cudaMemsetAsync(ws, 0, tb, s);
@@ -944,7 +982,8 @@ int attention_tc_plan(int B, int L, int heads, int info[4], int* bounds, int* ow
   const long long units = (long long)B * heads * ((L + kUM - 1) / kUM);
   const int nblk = (L + kBN - 1) / kBN;
   if (units * nblk > 0x7fffffffLL) return 0;
-  const Spans sp = plan_spans((int)units, nblk);
+  Spans sp;
+  plan_spans((int)units, nblk, &sp);
   info[0] = sp.G;
   info[1] = sp.split;
   info[2] = (int)units;
