@@ -6,6 +6,9 @@
 #include "common.cuh"
 #include "tc.cuh"
 
+#ifndef TOMA_POLY
+#define TOMA_POLY(e) (((e) & 6) == 6)
+#endif
 namespace toma {
 namespace attn {
 
@@ -43,6 +46,11 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
 __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
 // 2^x for x <= ~9 on the FMA pipe, two at a time: round to nearest integer with the 1.5*2^23 trick, degree-3
@@ -184,6 +192,36 @@ __device__ __forceinline__ bool softmax_tile(uint32_t sb, uint32_t ob, float sca
   tmem_st16(sb + 16, pk);
   tmem_wait_st();
   return true;
+}
+
+// ------------------------------------------------------------------ softmax against a reference with headroom
+// P = 2^(S c - m) of 32 columns as packed bf16 for a reference m that lies 2^kHeadroom above the scores seen when it was
+// set.  Everything is floating point, so the common factor costs no precision; what it buys is that the reference need
+// not follow the row maximum: no maximum is taken before the exponentials.  Instead `big` collects bit 14 of every
+// result, which is set exactly when P >= 2 (or is no number): then, and only then, the scores have outgrown the headroom
+// and the caller moves the reference.  sum2: fp32 sums of the even and the odd columns.
+// One pair of columns in four takes the polynomial of ex2_poly2 on the FMA pipe, the others MUFU.
+constexpr float kHeadroom = 32.f;
+
+__device__ __forceinline__ void chunk_exp_ref(const uint32_t (&r)[32], uint32_t (&pk)[16], float scale, float neg_m, uint64_t& sum2, uint32_t& big) {
+  const uint64_t c2 = pack2(scale, scale), m2 = pack2(neg_m, neg_m);
+#pragma unroll
+  for (int e = 0; e < 32; e += 2) {
+    const uint64_t x2 = fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), c2, m2);
+    float p0, p1;
+    if (TOMA_POLY(e)) {
+      ex2_poly2(x2, p0, p1);
+    } else {
+      float x0, x1;
+      unpack2(x2, x0, x1);
+      p0 = ex2_mufu(x0);
+      p1 = ex2_mufu(x1);
+    }
+    sum2 = add2(sum2, pack2(p0, p1));
+    pk[e >> 1] = pack_bf16_rn(p0, p1);
+  }
+#pragma unroll
+  for (int e = 0; e < 16; e += 2) big |= pk[e] | pk[e + 1];
 }
 
 // 32 accumulator columns of one row, scaled and rounded to bf16: 64 contiguous bytes.

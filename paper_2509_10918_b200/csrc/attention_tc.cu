@@ -43,6 +43,9 @@
 #include "common.cuh"
 #include "tc.cuh"
 
+#ifndef TOMA_ISS
+#define TOMA_ISS (DH == 128 ? 2 : 1)
+#endif
 namespace toma {
 
 using namespace tc;
@@ -51,11 +54,12 @@ using namespace attn;
 namespace {
 
 constexpr int kUM = 2 * kBM;  // queries per work unit
-constexpr int kThreads = 384;
+constexpr int kSoftWarps = 16;
+constexpr int kThreads = (kSoftWarps + 4) * 32;
 
 template <int DH>
 struct AttCfg {
-  static constexpr int kStages = 4;                        // K/V ring depth (S runs two tiles ahead of P V)
+  static constexpr int kStages = DH == 64 ? 8 : 4;         // K/V ring depth (S runs two tiles ahead of P V)
   static constexpr int kQBufs = DH == 64 ? 2 : 1;          // Q buffers: the next unit's Q lands under this unit's tail
   static constexpr int kChunks = DH / 64;                  // 64-column (128-byte) slabs per row
   static constexpr int kQSlab = kBM * 128;                 // 128 query rows x 128 B
@@ -63,28 +67,29 @@ struct AttCfg {
   static constexpr int kQBytes = 2 * kQTile;               // both query tiles of a unit
   static constexpr int kKvSlab = kBN * 128;                // 64 key rows x 128 B
   static constexpr int kKvBytes = kChunks * kKvSlab;       // one K or V tile
-  static constexpr bool kSumMma = DH == 64;                // row sums on the tensor pipe, truncated P
-  static constexpr int kOnesBytes = kSumMma ? kBN * 128 : 0;  // [64 keys][64] bf16 ones: the N chunk after V in the PV operand
-  static constexpr int kOutBytes = 8 * 32 * 128;           // per softmax warp: 32 output rows of one 64-channel slab, staged for a TMA store
+  static constexpr int kOutBytes = kSoftWarps * 32 * 64;   // per softmax warp: 32 output rows of 32 channels, staged for a TMA store
   static constexpr int kBarBytes = 512;
-  static constexpr int kSmemBytes = 1024 + kQBufs * kQBytes + 2 * kStages * kKvBytes + kOnesBytes + kOutBytes + kBarBytes;
+  static constexpr int kSmemBytes = 1024 + kQBufs * kQBytes + 2 * kStages * kKvBytes + kOutBytes + kBarBytes;
   static constexpr int kTmemCols = 512;
-  // Threads that issue MMAs.  With two, each query tile has its own (on different schedulers): neither waits behind
-  // the other tile's barrier.  Timed: 2-3.5 % faster at head_dim 128, 0-1.4 % slower at head_dim 64.
-  static constexpr int kIssuers = DH == 128 ? 2 : 1;
-  // S buffer (q, b) at column (2 q + b) * 64; O_q (and, behind it, the row sums) from column 256
-  static constexpr int kColS = 0, kColO = 256, kOStride = DH == 64 ? 96 : 128;
+  static constexpr int kIssuers = TOMA_ISS;  // threads that issue MMAs
+  // Tensor memory: a pipeline (query tile q, parity h) has 64 columns of S (P takes the first 32) and, at head_dim 64, an
+  // accumulator of its own; at head_dim 128 the two pipelines of a query tile share one.
+  static constexpr bool kOwnO = DH == 64;
+  __device__ static constexpr uint32_t s_col(int q, int h) { return kOwnO ? (q * 2 + h) * 128 : q * 256 + h * 64; }
+  __device__ static constexpr uint32_t o_col(int q, int h) { return kOwnO ? (q * 2 + h) * 128 + 64 : q * 256 + 128; }
 };
 
 struct Barriers {
-  uint64_t q_full[2], q_empty[2];     // per piece: Q landed / every S MMA of the piece has read Q
-  uint64_t k_full[4], kv_empty[4];    // per tile: K and V landed / every MMA that reads them is done
-  uint64_t s_full[2][2], p_full[2][2];  // per tile and query tile: S ready for the softmax / P ready for the PV MMAs
-  uint64_t o_done[2], o_free[2];      // per piece and query tile: accumulator complete / epilogue has read it
-  uint64_t pub_ready, pub_done;       // first partial piece: written by the softmax warps / published, tickets drawn
-  uint32_t first_ticket[8];           // per softmax warp: ticket its first (partial) piece drew
-  uint32_t others_done;               // set by the publisher when the span's last unit has all its other pieces in scratch
-  uint32_t poll_stop[2];              // set by each softmax group when the answer is no longer needed
+  uint64_t q_full[2], q_empty[2];       // per piece: Q landed / every S MMA of the piece has read Q
+  uint64_t k_full[8], kv_empty[8];      // per tile: K and V landed / every MMA that reads them is done
+  uint64_t s_full[2][2], p_full[2][2];  // per tile and pipeline: S ready for the softmax / P ready for the PV MMAs
+  uint64_t pv_done[2][2];               // the tile's PV MMAs are complete
+  uint64_t o_free[2];                   // per piece and query tile: the epilogue has read the accumulators
+  uint64_t pub_ready, pub_done;         // first partial piece: written by the softmax warps / published, tickets drawn
+  uint32_t first_ticket[kSoftWarps];    // per softmax warp: ticket its first (partial) piece drew
+  uint32_t move[8];                     // shared accumulator: a warp of this row group wants the reference moved
+  uint32_t others_done;                 // set by the publisher when the span's last unit has all its other pieces in scratch
+  uint32_t poll_stop[2];                // set by each softmax group when the answer is no longer needed
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -176,13 +181,14 @@ __device__ __forceinline__ const float* slot_of(const float* pieces, const Spans
   return pieces + (size_t)(2 * g + (u > first_unit ? 1 : 0)) * piece_floats<DH>();
 }
 
-// Adds up the pieces of one query row of unit u, left by CTAs g_first..g_last:
+// Adds up the pieces of one query row of unit u (channels [ch, ch + DH / 2) of the head), left by CTAs g_first..g_last:
 //   O = sum_i 2^(m_i - M) O_i / sum_i 2^(m_i - M) l_i,  M = max_i m_i  (m in the log2 domain).
 // Contributors are taken two at a time so that their loads are in flight together, and summed in
-// ascending CTA order with one fused multiply-add each, starting from zero: finish_piece's direct
-// path follows the same order, so the result does not depend on which path a launch takes.  Loads bypass L1: the pieces were written by other SMs during this launch.
+// ascending CTA order with one fused multiply-add each, starting from zero: finish_partial's direct
+// path follows the same order, so the result does not depend on which path a launch takes.  Loads bypass L1: the pieces
+// were written by other SMs during this launch.
 template <int DH>
-__device__ __noinline__ void combine_rows(const float* pieces, const Spans& sp, int u, int g_first, int g_last, int row,
+__device__ __noinline__ void combine_rows(const float* pieces, const Spans& sp, int u, int g_first, int g_last, int row, int ch,
                                           __nv_bfloat16* dst) {
   constexpr size_t kM = (size_t)kUM * DH, kL = (size_t)kUM * DH + kUM;
   float M = -INFINITY;
@@ -192,11 +198,11 @@ __device__ __noinline__ void combine_rows(const float* pieces, const Spans& sp, 
     M = max3(M, __ldcg(sa + kM + row), __ldcg(sb + kM + row));
   }
 #pragma unroll 1
-  for (int half = 0; half < DH / 64; ++half) {  // 64 accumulator columns at a time
+  for (int c0 = ch; c0 < ch + DH / 2; c0 += 16) {  // 16 accumulator columns at a time
     float denom = 0.f;
-    float acc[64];
+    float acc[16];
 #pragma unroll
-    for (int e = 0; e < 64; ++e) acc[e] = 0.f;
+    for (int e = 0; e < 16; ++e) acc[e] = 0.f;
     for (int g = g_first; g <= g_last; g += 2) {
       const float* sa = slot_of<DH>(pieces, sp, g, u);
       const float* sb = g < g_last ? slot_of<DH>(pieces, sp, g + 1, u) : sa;
@@ -204,33 +210,28 @@ __device__ __noinline__ void combine_rows(const float* pieces, const Spans& sp, 
       const float mb = __ldcg(sb + kM + row), lb = __ldcg(sb + kL + row);
       const float wa = ex2_mufu(ma - M), wb = g < g_last ? ex2_mufu(mb - M) : 0.f;
       denom = fmaf(wb, lb, fmaf(wa, la, denom));
+      float4 va[4], vb[4];
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        float4 va[8], vb[8];
+      for (int q = 0; q < 4; ++q) {
+        va[q] = __ldcg(reinterpret_cast<const float4*>(sa) + (size_t)(c0 / 4 + q) * kUM + row);
+        vb[q] = __ldcg(reinterpret_cast<const float4*>(sb) + (size_t)(c0 / 4 + q) * kUM + row);
+      }
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          va[q] = __ldcg(reinterpret_cast<const float4*>(sa) + (size_t)(half * 16 + c * 8 + q) * kUM + row);
-          vb[q] = __ldcg(reinterpret_cast<const float4*>(sb) + (size_t)(half * 16 + c * 8 + q) * kUM + row);
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          float* a4 = &acc[c * 32 + 4 * q];
-          a4[0] = fmaf(wb, vb[q].x, fmaf(wa, va[q].x, a4[0]));
-          a4[1] = fmaf(wb, vb[q].y, fmaf(wa, va[q].y, a4[1]));
-          a4[2] = fmaf(wb, vb[q].z, fmaf(wa, va[q].z, a4[2]));
-          a4[3] = fmaf(wb, vb[q].w, fmaf(wa, va[q].w, a4[3]));
-        }
+      for (int q = 0; q < 4; ++q) {
+        float* a4 = &acc[4 * q];
+        a4[0] = fmaf(wb, vb[q].x, fmaf(wa, va[q].x, a4[0]));
+        a4[1] = fmaf(wb, vb[q].y, fmaf(wa, va[q].y, a4[1]));
+        a4[2] = fmaf(wb, vb[q].z, fmaf(wa, va[q].z, a4[2]));
+        a4[3] = fmaf(wb, vb[q].w, fmaf(wa, va[q].w, a4[3]));
       }
     }
     if (!dst) continue;
     const float inv = 1.f / denom;
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      uint32_t r[32];
-#pragma unroll
-      for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(acc[c * 32 + e]);
-      store_row32(dst + half * 64 + c * 32, r, inv);
-    }
+    for (int e = 0; e < 16; e += 8)
+      *reinterpret_cast<uint4*>(dst + c0 + e) =
+          make_uint4(pack_bf16_rn(acc[e] * inv, acc[e + 1] * inv), pack_bf16_rn(acc[e + 2] * inv, acc[e + 3] * inv),
+                     pack_bf16_rn(acc[e + 4] * inv, acc[e + 5] * inv), pack_bf16_rn(acc[e + 6] * inv, acc[e + 7] * inv));
   }
 }
 
@@ -259,42 +260,91 @@ __device__ __forceinline__ uint32_t take_ticket(uint32_t* ticket, int lane) {
   return __shfl_sync(0xffffffffu, t, 0);
 }
 
-// The per-thread view of a softmax thread: its query tile, its row in the unit, its accumulator.
+// The per-thread view of a softmax thread.  Two threads share a query row, both on its tensor-memory lane: each has every
+// second key tile (its pipeline, `half`) and, at the end of a piece, half of the head's channels.
 struct Row {
-  int q;        // query tile (softmax warp group) 0 or 1
-  int warp;     // softmax warp 0..7 = ticket column
+  int q;        // query tile 0 or 1
+  int half;
+  int warp;     // softmax warp 0..15 = ticket column
   int lane;
   int row;      // query row inside the unit, 0..255
-  uint32_t ob;  // tensor-memory address of this row's accumulator
+  uint32_t tm;  // this row's tensor-memory lane
 };
+// Both warps of a row group meet at a barrier of their own.
+__device__ __forceinline__ int pair_of(const Row& t) { return t.q * 4 + (t.warp & 3); }
+__device__ __forceinline__ void pair_sync(const Row& t) {
+  __syncwarp();
+  asm volatile("bar.sync %0, 64;" ::"r"(1 + pair_of(t)) : "memory");
+}
 // Where a softmax warp stages its output rows, and the map they are stored through: kept out of Row (the softmax
 // loop holds a Row in registers) and derived where a piece ends.
 struct OutStage {
-  uint8_t* stage;           // this warp's 4 KB of the output staging area (it lies right below the barriers)
-  const CUtensorMap* tm_o;  // output as (channel, token, batch), box = 64 channels x 32 tokens
+  uint8_t* stage;           // this warp's 2 KB of the output staging area (it lies right below the barriers)
+  const CUtensorMap* tm_o;  // output as (channel, token, batch), box = 32 channels x 32 tokens
 };
 template <int DH>
-__device__ __forceinline__ OutStage out_stage(const void* bar, int warp, const CUtensorMap* tm_o) {
-  return OutStage{const_cast<uint8_t*>(reinterpret_cast<const uint8_t*>(bar)) - AttCfg<DH>::kOutBytes + warp * 4096, tm_o};
+__device__ __forceinline__ uint8_t* stage_of(const void* bar, int warp) {
+  return const_cast<uint8_t*>(reinterpret_cast<const uint8_t*>(bar)) - AttCfg<DH>::kOutBytes + warp * 2048;
 }
-
-// Output rows leave through shared memory: a thread puts 32 channels of its row (scaled, bf16) into its warp's
-// staged slab (64 channels x 32 rows, 128-byte swizzled = the output map's box), and when a slab is complete the
-// warp stores it with one TMA store - whole lines instead of 16-byte stores to 32 different rows per warp
-// instruction.  Rows past the end of the sequence are clipped by the store.
-__device__ __forceinline__ void stage_half(const OutStage& os, int lane, int half, const uint32_t (&r)[32], float inv) {
+// Two words of this thread's for the other thread of the row, through the (then idle) staging areas.
+template <int DH>
+__device__ __forceinline__ uint2 exchange(const Row& t, const void* bar, uint32_t a, uint32_t b) {
+  volatile uint32_t* mine = reinterpret_cast<volatile uint32_t*>(stage_of<DH>(bar, t.warp)) + t.lane;
+  const volatile uint32_t* other = reinterpret_cast<volatile uint32_t*>(stage_of<DH>(bar, t.warp ^ 4)) + t.lane;
+  mine[0] = a;
+  mine[32] = b;
+  pair_sync(t);
+  const uint2 o = make_uint2(other[0], other[32]);
+  pair_sync(t);  // read: the areas may be written again
+  return o;
+}
+// A row at the end of a piece: reference and row sum of both pipelines together, and what their accumulators count in it
+// (own accumulators only; 0: nothing, not even if it is no number).
+struct Joint {
+  float m, l, w0, w1;
+};
+template <int DH>
+__device__ __forceinline__ Joint join_halves(const Row& t, const void* bar, float m, float l) {
+  const uint2 o = exchange<DH>(t, bar, __float_as_uint(m), __float_as_uint(l));
+  const float mo = __uint_as_float(o.x), lo = __uint_as_float(o.y);
+  Joint r;
+  r.m = fmaxf(m, mo);
+  const float own = ex2_mufu(m - r.m), oth = ex2_mufu(mo - r.m);  // a pipeline without a tile: 2^-inf = 0
+  r.w0 = t.half ? oth : own;
+  r.w1 = t.half ? own : oth;
+  r.l = t.half ? fmaf(r.w1, l, r.w0 * lo) : fmaf(r.w1, lo, r.w0 * l);
+  return r;
+}
+// 16 accumulator columns of the row, both pipelines' together.
+template <int DH>
+__device__ __forceinline__ void read_o16(const Row& t, const Joint& jn, int c, uint32_t (&r)[16]) {
+  using C = AttCfg<DH>;
+  tmem_ld16(t.tm + C::o_col(t.q, 0) + c, r);
+  if constexpr (C::kOwnO) {
+    uint32_t r1[16];
+    tmem_ld16(t.tm + C::o_col(t.q, 1) + c, r1);
+    tmem_wait_ld();
 #pragma unroll
-  for (int e = 0; e < 32; e += 8) {
-    uint4 v;
-    v.x = pack_bf16_rn(__uint_as_float(r[e]) * inv, __uint_as_float(r[e + 1]) * inv);
-    v.y = pack_bf16_rn(__uint_as_float(r[e + 2]) * inv, __uint_as_float(r[e + 3]) * inv);
-    v.z = pack_bf16_rn(__uint_as_float(r[e + 4]) * inv, __uint_as_float(r[e + 5]) * inv);
-    v.w = pack_bf16_rn(__uint_as_float(r[e + 6]) * inv, __uint_as_float(r[e + 7]) * inv);
-    *reinterpret_cast<uint4*>(os.stage + sw128_offset(lane, half * 4 + (e >> 3))) = v;
+    for (int e = 0; e < 16; ++e) {
+      const float a = jn.w0 != 0.f ? jn.w0 * __uint_as_float(r[e]) : 0.f;
+      r[e] = __float_as_uint(jn.w1 != 0.f ? fmaf(jn.w1, __uint_as_float(r1[e]), a) : a);
+    }
+  } else {
+    tmem_wait_ld();
   }
 }
-// The same for 16 channels (quarter 0..3 of the slab's 64).
-__device__ __forceinline__ void stage_quarter(const OutStage& os, int lane, int quarter, const uint32_t (&r)[16], float inv) {
+// The last products of both pipelines, in a piece of `cnt` tiles whose last is number `last_n` of the span.
+__device__ __forceinline__ bool wait_o(const Row& t, Barriers* bar, int last_n, int cnt, uint32_t* dev_status) {
+  bool ok = mbar_wait(&bar->pv_done[t.q][last_n & 1], (last_n >> 1) & 1, dev_status, &bar->abort_flag);
+  if (cnt > 1) ok = ok && mbar_wait(&bar->pv_done[t.q][(last_n - 1) & 1], ((last_n - 1) >> 1) & 1, dev_status, &bar->abort_flag);
+  return __all_sync(0xffffffffu, ok);
+}
+
+// Output rows leave through shared memory: a thread puts 16 channels of its row (scaled, bf16) into its warp's staged
+// slab (32 channels x 32 rows, 64-byte swizzled = the output map's box), and when the slab is complete the
+// warp stores it with one TMA store - whole sectors instead of 16-byte stores to 32 different rows per warp
+// instruction.  Rows past the end of the sequence are clipped by the store.
+__device__ __forceinline__ void stage16(const OutStage& os, int lane, int part, const uint32_t (&r)[16], float inv) {
 #pragma unroll
   for (int e = 0; e < 16; e += 8) {
     uint4 v;
@@ -302,7 +352,7 @@ __device__ __forceinline__ void stage_quarter(const OutStage& os, int lane, int 
     v.y = pack_bf16_rn(__uint_as_float(r[e + 2]) * inv, __uint_as_float(r[e + 3]) * inv);
     v.z = pack_bf16_rn(__uint_as_float(r[e + 4]) * inv, __uint_as_float(r[e + 5]) * inv);
     v.w = pack_bf16_rn(__uint_as_float(r[e + 6]) * inv, __uint_as_float(r[e + 7]) * inv);
-    *reinterpret_cast<uint4*>(os.stage + sw128_offset(lane, quarter * 2 + (e >> 3))) = v;
+    *reinterpret_cast<uint4*>(os.stage + lane * 64 + (((part * 2 + (e >> 3)) ^ ((lane >> 1) & 3)) << 4)) = v;
   }
 }
 // Whole warp.  (ch0, row0, b): first channel of the slab, first token of the warp's 32 rows, batch item.
@@ -327,35 +377,32 @@ __device__ __forceinline__ void warp_rows_of(int u, const Row& t, int L, int hea
 }
 
 // End of a piece that covers all keys of its unit (the only kind when units are kept whole), run by
-// the softmax warps: wait for the accumulator, normalise, write the rows out.  Returns false when
+// the softmax warps: wait for the accumulators, normalise, write the rows out.  Returns false when
 // the wait ran out.
 template <int DH>
-__device__ __forceinline__ bool finish_whole(const Row& t, Barriers* bar, int unit, int pc, float l, const CUtensorMap* tm_o, int L,
-                                             int heads, uint32_t* dev_status) {
-  using C = AttCfg<DH>;
-  if (!mbar_wait(&bar->o_done[t.q], pc & 1, dev_status, &bar->abort_flag)) return false;
+__device__ __noinline__ bool finish_whole(Row t, Barriers* bar, Piece p, int last_n, Joint jn, const CUtensorMap* tm_o, int L, int heads,
+                                          uint32_t* dev_status) {
+  if (!wait_o(t, bar, last_n, p.cnt, dev_status)) return false;
   tc_fence_after();
-  if (C::kSumMma) {
-    uint32_t rs[16];
-    tmem_ld16(t.ob + DH, rs);
-    tmem_wait_ld();
-    l = __uint_as_float(rs[0]);
-  }
   int b, ch0, row0;
-  warp_rows_of<DH>(unit, t, L, heads, b, ch0, row0);
-  const OutStage os = out_stage<DH>(bar, t.warp, tm_o);
-  const float inv = 1.f / l;
-#pragma unroll
-  for (int c = 0; c < DH / 32; ++c) {
-    uint32_t r[32];
-    tmem_ld32(t.ob + c * 32, r);
-    tmem_wait_ld();
-    stage_half(os, t.lane, c & 1, r, inv);
-    if (c & 1) flush_slab(os, t.lane, ch0 + (c >> 1) * 64, row0, b, L);
+  warp_rows_of<DH>(p.u, t, L, heads, b, ch0, row0);
+  const OutStage os{stage_of<DH>(bar, t.warp), tm_o};
+  const float inv = 1.f / jn.l;
+  const int c0 = t.half * (DH / 2);
+#pragma unroll 1
+  for (int c = c0; c < c0 + DH / 2; c += 32) {
+    uint32_t r[16];
+    read_o16<DH>(t, jn, c, r);
+    stage16(os, t.lane, 0, r, inv);
+    read_o16<DH>(t, jn, c + 16, r);
+    stage16(os, t.lane, 1, r, inv);
+    if (c + 32 >= c0 + DH / 2) {
+      tc_fence_before();
+      __syncwarp();
+      if (t.lane == 0) mbar_arrive(&bar->o_free[t.q]);  // the next piece's first PV product may overwrite the accumulator
+    }
+    flush_slab(os, t.lane, ch0 + c, row0, b, L);
   }
-  tc_fence_before();
-  __syncwarp();
-  if (t.lane == 0) mbar_arrive(&bar->o_free[t.q]);  // the next piece's first PV product may overwrite the accumulator
   return true;
 }
 
@@ -364,34 +411,29 @@ __device__ __forceinline__ bool finish_whole(const Row& t, Barriers* bar, int un
 //     published (it ran at the start of its own span, so it normally has), is added to that
 //     contributor's piece straight from tensor memory and written out: nothing of it goes through
 //     scratch, and the other piece is fetched while the last MMAs drain;
-//   - any other piece is left in scratch with its reference maximum and row sum and a (unit, warp)
+//   - any other piece is left in scratch with its reference and row sum and a (unit, warp)
 //     ticket is drawn; the warp that draws a unit's last ticket adds its pieces up.  A last piece
 //     does that here; a first piece, with more of the span to come, hands the fence and the
 //     tickets' round trips to the publisher thread and looks at the outcome in settle_first_piece.
 // Every decision that ends in a warp-wide operation is taken once per warp (lane 0 reads, the warp
-// gets the value by shuffle), so a warp always goes one way as a whole.
+// gets the value by shuffle), so a warp always goes one way as a whole.  Both warps of a row write the row's reference
+// and sum (the same values), so that each one's ticket covers what it needs.
 // Out of line (it runs at most twice per CTA and is register-hungry).  Returns false when the wait
 // ran out.
 template <int DH>
-__device__ __noinline__ bool finish_partial(Row t, Barriers* bar, Piece p, int pc, bool last_of_span, float m_used, float l,
+__device__ __noinline__ bool finish_partial(Row t, Barriers* bar, Piece p, int pc, int last_n, bool last_of_span, Joint jn,
                                             __nv_bfloat16* o, const CUtensorMap* tm_o, int L, int heads, const Spans& sp,
                                             uint32_t* tickets, float* pieces, uint32_t* dev_status) {
-  using C = AttCfg<DH>;
   constexpr size_t kM = (size_t)kUM * DH, kL = (size_t)kUM * DH + kUM;
-  const int row = t.row, lane = t.lane;
-  uint32_t* ticket = tickets + (size_t)p.u * 8 + t.warp;
+  const int row = t.row, lane = t.lane, c0 = t.half * (DH / 2);
+  uint32_t* ticket = tickets + (size_t)p.u * kSoftWarps + t.warp;
   // a partial piece lies in the unit the span starts in or in the one it ends in
   const int which = p.u == sp.bound(blockIdx.x) / sp.nblk ? 0 : 1;
   const int g_first = sp.unit_lo[which][blockIdx.x], g_last = sp.unit_hi[which][blockIdx.x];
   bool own_first = false;  // this CTA is the lower of the two contributors
-  // The direct path comes in two forms.  The wide one holds 64 columns of the other piece in registers (the
-  // function then spills); the lean one takes 16 columns at a time with the next 16 on their way.  Timed as a
-  // whole, the kernel is 3-4 % faster with the lean form at head_dim 128 and 5-7 % slower at head_dim 64, where
-  // the register allocation of the tile loop changes with this function's needs: each keeps the form that wins.
-  constexpr bool kLean = DH == 128;
-  const float* other = nullptr;
+  const float4* other = nullptr;
   float m_o = 0.f, l_o = 0.f;
-  float4 vo[kLean ? 4 : 16];
+  float4 vo[4];  // 16 columns of the other piece, the next 16 on their way
   // the publisher warp watches the tickets of the span's last unit; its answer carries the
   // acquire that orders the loads below after the other contributor's writes
   uint32_t others = 0;
@@ -401,117 +443,72 @@ __device__ __noinline__ bool finish_partial(Row t, Barriers* bar, Piece p, int p
     others = __shfl_sync(0xffffffffu, others, 0);
   }
   const bool direct = others == 1u;
-  if (last_of_span && (row & (kBM - 1)) == 0) *(volatile uint32_t*)&bar->poll_stop[t.q] = 1u;
+  if (last_of_span && (row & (kBM - 1)) == 0 && t.half == 0) *(volatile uint32_t*)&bar->poll_stop[t.q] = 1u;
   if (direct) {
     own_first = (int)blockIdx.x == g_first;
-    other = slot_of<DH>(pieces, sp, own_first ? g_last : g_first, p.u);
-    m_o = __ldcg(other + kM + row);
-    l_o = __ldcg(other + kL + row);
+    const float* slot = slot_of<DH>(pieces, sp, own_first ? g_last : g_first, p.u);
+    m_o = __ldcg(slot + kM + row);
+    l_o = __ldcg(slot + kL + row);
+    other = reinterpret_cast<const float4*>(slot) + row;
 #pragma unroll
-    for (int q = 0; q < (kLean ? 4 : 16); ++q) vo[q] = __ldcg(reinterpret_cast<const float4*>(other) + (size_t)q * kUM + row);
+    for (int q = 0; q < 4; ++q) vo[q] = __ldcg(other + (size_t)(c0 / 4 + q) * kUM);
   }
-  if (!mbar_wait(&bar->o_done[t.q], pc & 1, dev_status, &bar->abort_flag)) return false;
+  if (!wait_o(t, bar, last_n, p.cnt, dev_status)) return false;
   tc_fence_after();
-  if (C::kSumMma) {
-    uint32_t rs[16];
-    tmem_ld16(t.ob + DH, rs);
-    tmem_wait_ld();
-    l = __uint_as_float(rs[0]);
-  }
-  __nv_bfloat16* dst = out_row<DH>(o, p.u, row, L, heads);
   int b_item, ch0, row0;
   warp_rows_of<DH>(p.u, t, L, heads, b_item, ch0, row0);
-  const OutStage os = out_stage<DH>(bar, t.warp, tm_o);
   float* slot = pieces + (size_t)(2 * blockIdx.x + (pc > 0 ? 1 : 0)) * piece_floats<DH>();
-  float w_own = 1.f, w_o = 0.f, inv = 1.f;
   if (direct) {
-    const float M = fmaxf(m_used, m_o);
-    w_own = ex2_mufu(m_used - M);
-    w_o = ex2_mufu(m_o - M);
-    inv = 1.f / (own_first ? fmaf(w_o, l_o, w_own * l) : fmaf(w_own, l, w_o * l_o));
-  }
-  // rows of the piece into its scratch slot (32 columns at a time)
-  auto to_scratch = [&](int c, const uint32_t (&r)[32]) {
+    const OutStage os{stage_of<DH>(bar, t.warp), tm_o};
+    const float M = fmaxf(jn.m, m_o);
+    const float w_own = ex2_mufu(jn.m - M), w_o = ex2_mufu(m_o - M);
+    const float inv = 1.f / (own_first ? fmaf(w_o, l_o, w_own * jn.l) : fmaf(w_own, jn.l, w_o * l_o));
+#pragma unroll 1
+    for (int c = c0; c < c0 + DH / 2; c += 16) {
+      float4 vc[4];
 #pragma unroll
-    for (int e = 0; e < 32; e += 4)
-      reinterpret_cast<float4*>(slot)[(size_t)(c * 8 + (e >> 2)) * kUM + row] =
-          make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]), __uint_as_float(r[e + 2]), __uint_as_float(r[e + 3]));
-  };
-  if constexpr (kLean) {
-    if (direct) {
+      for (int q = 0; q < 4; ++q) vc[q] = vo[q];
+      if (c + 16 < c0 + DH / 2) {
 #pragma unroll
-      for (int c = 0; c < DH / 16; ++c) {
-        float4 vc[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) vc[q] = vo[q];
-        if (c + 1 < DH / 16) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) vo[q] = __ldcg(reinterpret_cast<const float4*>(other) + (size_t)((c + 1) * 4 + q) * kUM + row);
-        }
-        uint32_t r[16];
-        tmem_ld16(t.ob + c * 16, r);
-        tmem_wait_ld();
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float vv[4] = {vc[q].x, vc[q].y, vc[q].z, vc[q].w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float own = __uint_as_float(r[4 * q + e]);
-            r[4 * q + e] = __float_as_uint(own_first ? fmaf(w_o, vv[e], w_own * own) : fmaf(w_own, own, w_o * vv[e]));
-          }
-        }
-        stage_quarter(os, t.lane, c & 3, r, inv);
-        if ((c & 3) == 3) flush_slab(os, t.lane, ch0 + (c >> 2) * 64, row0, b_item, L);
+        for (int q = 0; q < 4; ++q) vo[q] = __ldcg(other + (size_t)((c + 16) / 4 + q) * kUM);
       }
-    } else {
+      uint32_t r[16];
+      read_o16<DH>(t, jn, c, r);
 #pragma unroll
-      for (int c = 0; c < DH / 32; ++c) {
-        uint32_t r[32];
-        tmem_ld32(t.ob + c * 32, r);
-        tmem_wait_ld();
-        to_scratch(c, r);
+      for (int q = 0; q < 4; ++q) {
+        const float vv[4] = {vc[q].x, vc[q].y, vc[q].z, vc[q].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float own = __uint_as_float(r[4 * q + e]);
+          r[4 * q + e] = __float_as_uint(own_first ? fmaf(w_o, vv[e], w_own * own) : fmaf(w_own, own, w_o * vv[e]));
+        }
       }
+      stage16(os, lane, (c >> 4) & 1, r, inv);
+      if ((c >> 4) & 1) flush_slab(os, lane, ch0 + c - 16, row0, b_item, L);
     }
   } else {
+#pragma unroll 1
+    for (int c = c0; c < c0 + DH / 2; c += 16) {
+      uint32_t r[16];
+      read_o16<DH>(t, jn, c, r);
 #pragma unroll
-    for (int c = 0; c < DH / 32; ++c) {
-      uint32_t r[32];
-      tmem_ld32(t.ob + c * 32, r);
-      tmem_wait_ld();
-      if (direct) {
-        if (c > 0 && (c & 1) == 0) {  // next 64 columns of the other piece
-#pragma unroll
-          for (int q = 0; q < 16; ++q) vo[q] = __ldcg(reinterpret_cast<const float4*>(other) + (size_t)(c * 8 + q) * kUM + row);
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const float4 v = vo[(c & 1) * 8 + q];
-          const float vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float own = __uint_as_float(r[4 * q + e]);
-            r[4 * q + e] = __float_as_uint(own_first ? fmaf(w_o, vv[e], w_own * own) : fmaf(w_own, own, w_o * vv[e]));
-          }
-        }
-        stage_half(os, t.lane, c & 1, r, inv);
-        if (c & 1) flush_slab(os, t.lane, ch0 + (c >> 1) * 64, row0, b_item, L);
-      } else {
-        to_scratch(c, r);
-      }
+      for (int e = 0; e < 16; e += 4)
+        reinterpret_cast<float4*>(slot)[(size_t)((c + e) / 4) * kUM + row] =
+            make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]), __uint_as_float(r[e + 2]), __uint_as_float(r[e + 3]));
     }
   }
   tc_fence_before();
   __syncwarp();
   if (lane == 0) mbar_arrive(&bar->o_free[t.q]);  // the next piece's first PV product may overwrite the accumulator
   if (direct) return true;
-  slot[kM + row] = m_used;
-  slot[kL + row] = l;
+  slot[kM + row] = jn.m;
+  slot[kL + row] = jn.l;
   if (!last_of_span) {  // the publisher thread fences, draws the tickets and leaves them for settle_first_piece
     __syncwarp();
     if (lane == 0) mbar_arrive(&bar->pub_ready);
   } else if (take_ticket(ticket, lane) == (uint32_t)(g_last - g_first)) {
     __threadfence();
-    combine_rows<DH>(pieces, sp, p.u, g_first, g_last, row, dst);
+    combine_rows<DH>(pieces, sp, p.u, g_first, g_last, row, c0, out_row<DH>(o, p.u, row, L, heads));
   }
   return true;
 }
@@ -529,16 +526,113 @@ __device__ __noinline__ void settle_first_piece(Barriers* bar, int it_begin, int
   if (!mbar_wait(&bar->pub_done, 0, dev_status, &bar->abort_flag)) return;
   if (bar->first_ticket[t.warp] != (uint32_t)(g_last - g_first)) return;
   __threadfence();
-  combine_rows<DH>(pieces, sp, u, g_first, g_last, t.row, out_row<DH>(o, u, t.row, L, heads));
+  combine_rows<DH>(pieces, sp, u, g_first, g_last, t.row, t.half * (DH / 2), out_row<DH>(o, u, t.row, L, heads));
 }
 
-// The ragged last key tile of a sequence: out of line, so that the hot loop holds one copy of the
-// softmax code.
+// Largest score (log2 domain) of this row in a tile, the first `valid` of its columns counting.
+__device__ __noinline__ float tile_max(uint32_t s_addr, int valid, float scale_log2) {
+  float mx = -INFINITY;
+#pragma unroll 1
+  for (int c = 0; c < valid; c += 16) {
+    uint32_t r[16];
+    tmem_ld16(s_addr + c, r);
+    tmem_wait_ld();
+#pragma unroll
+    for (int e = 0; e < 16; ++e) mx = c + e < valid ? fmaxf(mx, __uint_as_float(r[e])) : mx;
+  }
+  return mx * scale_log2;
+}
+// The reference for a row whose scores have reached `mx`.
+__device__ __forceinline__ float reference(float mx, float m_used) { return mx > m_used + 1.f ? ceilf(mx) + kHeadroom : m_used; }
+// Columns [c0, c1) of this row's accumulator times `factor` (a power of two: exact).
+__device__ __forceinline__ void scale_o(uint32_t o_addr, int c0, int c1, float factor) {
+#pragma unroll 1
+  for (int c = c0; c < c1; c += 16) {
+    uint32_t r[16];
+    tmem_ld16(o_addr + c, r);
+    tmem_wait_ld();
+#pragma unroll
+    for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * factor);
+    tmem_st16(o_addr + c, r);
+  }
+  tmem_wait_st();
+}
+
+// Own accumulators (head_dim 64): some row of this warp has scores that outgrew its reference.  Such rows get a new one,
+// kHeadroom above the tile's largest score, and the pipeline's accumulator is multiplied by the power of two between the
+// two (references are whole numbers).  Out of line, it hardly ever runs.  Returns the new reference.
 template <int DH>
-__device__ __noinline__ bool softmax_tile_ragged(uint32_t sb, uint32_t ob, float scale_log2, int valid, int j, float& m_used,
-                                                 float& l, uint64_t* pv_done, uint32_t pv_parity, uint32_t* dev_status,
-                                                 volatile int* abort_flag) {
-  return softmax_tile<DH, AttCfg<DH>::kSumMma, true>(sb, ob, scale_log2, valid, j, m_used, l, pv_done, pv_parity, dev_status, abort_flag);
+__device__ __noinline__ float move_reference(Row t, Barriers* bar, uint32_t s_addr, int valid, float scale_log2, float m_used, bool have_o, int n,
+                                             uint32_t* dev_status) {
+  const float m_new = reference(tile_max(s_addr, valid, scale_log2), m_used);
+  // every product issued so far must have landed
+  if (have_o && __all_sync(0xffffffffu, mbar_wait(&bar->pv_done[t.q][t.half], ((n >> 1) - 1) & 1, dev_status, &bar->abort_flag))) {
+    tc_fence_after();
+    scale_o(t.tm + AttCfg<DH>::o_col(t.q, t.half), 0, DH, ex2_mufu(m_used - m_new));
+  }
+  return m_new;
+}
+
+// Shared accumulator (head_dim 128): the two warps of a row group have one reference per row, and moving it takes both.
+// Each brings the number of its next tile whose P it has not stored (`next`; kNoTile at the end of the piece), whether
+// that tile's S lies ready (`have_s`; the warp that asks has it), and whether it asks.  Tiles below the smaller `next`
+// have been multiplied or will be without further ado; the only other P there can be is that of tile min + 1, stored by
+// the other warp and waiting behind it: it is rescaled where it lies.  Returns the new reference, and whether anybody
+// asked (two warps at the end of their piece just meet here).
+constexpr int kNoTile = 1 << 30;
+struct Meeting {
+  float m;
+  bool asked;
+};
+template <int DH>
+__device__ __noinline__ Meeting meet(Row t, Barriers* bar, uint32_t s_addr, int valid, float scale_log2, float m_used, bool ask, bool have_s, int next,
+                                     int first_n, int last_n, uint32_t* dev_status) {
+  using C = AttCfg<DH>;
+  const float mx = have_s ? tile_max(s_addr, valid, scale_log2) : -INFINITY;
+  const uint2 o = exchange<DH>(t, bar, __float_as_uint(mx), (uint32_t)next * 2u + (ask ? 1u : 0u));
+  if (!ask && !(o.y & 1u)) return Meeting{m_used, false};
+  const int other_next = (int)(o.y >> 1), low = min(next, other_next);
+  const float m_new = reference(fmaxf(mx, __uint_as_float(o.x)), m_used);
+  const float factor = ex2_mufu(m_used - m_new);
+  if (low > first_n && low != kNoTile) {  // products of the piece's tiles below `low`: in order, so the last one tells
+    const bool ok = mbar_wait(&bar->pv_done[t.q][(low - 1) & 1], ((low - 1) >> 1) & 1, dev_status, &bar->abort_flag);
+    if (__all_sync(0xffffffffu, ok)) {
+      tc_fence_after();
+      scale_o(t.tm + C::o_col(t.q, 0), t.half * (DH / 2), (t.half + 1) * (DH / 2), factor);
+    }
+  }
+  if ((low & 1) != t.half && next > low + 1 && low < last_n) {  // this warp has stored P of tile low + 1
+#pragma unroll 1
+    for (int c = 0; c < 32; c += 16) {
+      uint32_t r[16];
+      tmem_ld16(s_addr + c, r);
+      tmem_wait_ld();
+#pragma unroll
+      for (int e = 0; e < 16; ++e)
+        r[e] = pack_bf16_rn(__uint_as_float(r[e] << 16) * factor, __uint_as_float(r[e] & 0xFFFF0000u) * factor);
+      tmem_st16(s_addr + c, r);
+    }
+    tmem_wait_st();
+  }
+  tc_fence_before();
+  if (t.lane == 0) *(volatile uint32_t*)&bar->move[pair_of(t)] = 0u;
+  pair_sync(t);
+  tc_fence_after();
+  return Meeting{m_new, true};
+}
+
+// Waits for a tile's S, or for the row group's other warp to want the reference moved.  One answer per warp.
+enum class Wait { kReady, kMove, kAborted };
+__device__ __forceinline__ Wait wait_s_or_move(uint64_t* bar, uint32_t parity, const volatile uint32_t* move, uint32_t* dev_status,
+                                               volatile int* abort_flag) {
+  for (uint32_t it = 0; it < kSpinLimit; ++it) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return Wait::kReady;
+    if (__any_sync(0xffffffffu, *move != 0u)) return Wait::kMove;
+    if ((it & 1023u) == 1023u && __any_sync(0xffffffffu, *abort_flag)) return Wait::kAborted;
+  }
+  *abort_flag = 1;
+  if (dev_status) atomicOr(dev_status, kStatusTimeout);
+  return Wait::kAborted;
 }
 
 template <int DH>
@@ -554,8 +648,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   uint8_t* sQ = smem;
   uint8_t* sK = sQ + C::kQBufs * C::kQBytes;
   uint8_t* sV = sK + C::kStages * C::kKvBytes;
-  uint8_t* sOnes = sV + C::kStages * C::kKvBytes;
-  uint8_t* sOut = sOnes + C::kOnesBytes;
+  uint8_t* sOut = sV + C::kStages * C::kKvBytes;
   Barriers* bar = reinterpret_cast<Barriers*>(sOut + C::kOutBytes);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -564,32 +657,29 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   const int it_begin = sp.bound(blockIdx.x), it_end = sp.bound(blockIdx.x + 1);
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(&bar->q_full[s], 1);
-      mbar_init(&bar->q_empty[s], C::kIssuers);
-      mbar_init(&bar->o_done[s], 1);
-      mbar_init(&bar->o_free[s], 4);  // one arrival per softmax warp of the group
-      for (int b = 0; b < 2; ++b) {
-        mbar_init(&bar->s_full[s][b], 1);
-        mbar_init(&bar->p_full[s][b], 4);
+    for (int q = 0; q < 2; ++q) {
+      mbar_init(&bar->q_full[q], 1);
+      mbar_init(&bar->q_empty[q], C::kIssuers);
+      for (int h = 0; h < 2; ++h) {
+        mbar_init(&bar->s_full[q][h], 1);
+        mbar_init(&bar->p_full[q][h], 4);  // one arrival per softmax warp of the pipeline
+        mbar_init(&bar->pv_done[q][h], 1);
       }
-      bar->poll_stop[s] = 0;
+      mbar_init(&bar->o_free[q], 8);
+      bar->poll_stop[q] = 0;
     }
     for (int s = 0; s < C::kStages; ++s) {
       mbar_init(&bar->k_full[s], 1);
       mbar_init(&bar->kv_empty[s], C::kIssuers);
     }
-    mbar_init(&bar->pub_ready, 8);
+    for (int g = 0; g < 8; ++g) bar->move[g] = 0;
+    mbar_init(&bar->pub_ready, kSoftWarps);
     mbar_init(&bar->pub_done, 1);
     bar->others_done = 0;
     bar->abort_flag = 0;
     mbar_fence_init();
   }
-  if (C::kSumMma) {  // bf16 1.0 everywhere: the layout's swizzle is irrelevant for a constant tile
-    for (int e = threadIdx.x; e < C::kOnesBytes / 4; e += blockDim.x) reinterpret_cast<uint32_t*>(sOnes)[e] = 0x3F803F80u;
-    fence_proxy_async();
-  }
-  if (threadIdx.x == 256) {  // descriptor fetches overlap the previous kernel's tail
+  if (threadIdx.x == kSoftWarps * 32) {  // descriptor fetches overlap the previous kernel's tail
     prefetch_tmap(&tm_q);
     prefetch_tmap(&tm_k);
     prefetch_tmap(&tm_v);
@@ -597,82 +687,76 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   }
   dependency_wait();
   if (threadIdx.x == 0) release_dependents();
-  if (warp == 9) tmem_alloc(&bar->tmem_base, C::kTmemCols);
+  if (warp == 17) tmem_alloc(&bar->tmem_base, C::kTmemCols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bar->tmem_base;
   volatile int* abort_flag = &bar->abort_flag;
 
-  if (warp == 8) {
+  if (warp == 16) {
     // ------------------------------------------------------------------ TMA producer
     if (elect_one()) {
       Cursor c;
-      for (c.init(it_begin, it_end, nblk); c.valid(); c.next()) {
+      int u = 0, key0 = 0, b = 0, ch0 = 0;
+      for (c.init(it_begin, it_end, nblk); c.valid(); c.next(), key0 += kBN) {
         if (c.j == 0) {
-          const int u = c.it / nblk;
-          const int bh = u / nq, q0 = (u - bh * nq) * kUM, b = bh / heads, h = bh - b * heads;
-          const int qb = c.pc % C::kQBufs;
+          u = c.it / nblk, key0 = (c.it - u * nblk) * kBN;
+          const int bh = u / nq, q0 = (u - bh * nq) * kUM, qb = c.pc % C::kQBufs;
+          b = bh / heads, ch0 = (bh - b * heads) * DH;
           // a Q buffer is free once the S MMAs of the piece that used it have read it
           if (c.pc >= C::kQBufs && !mbar_wait(&bar->q_empty[qb], ((c.pc / C::kQBufs) - 1) & 1, dev_status, abort_flag)) break;
           mbar_expect_tx(&bar->q_full[qb], C::kQBytes);
           for (int t = 0; t < 2; ++t)
             for (int ch = 0; ch < C::kChunks; ++ch)
-              tma_load_3d(sQ + qb * C::kQBytes + t * C::kQTile + ch * C::kQSlab, &tm_q, &bar->q_full[qb], h * DH + ch * 64,
-                          q0 + t * kBM, b);
+              tma_load_3d(sQ + qb * C::kQBytes + t * C::kQTile + ch * C::kQSlab, &tm_q, &bar->q_full[qb], ch0 + ch * 64, q0 + t * kBM, b);
         }
-        const int u = c.it / nblk, k0 = c.it - u * nblk;
-        const int bh = u / nq, b = bh / heads, h = bh - b * heads;
         const int s = c.n % C::kStages;
         if (c.n >= C::kStages && !mbar_wait(&bar->kv_empty[s], ((c.n / C::kStages) - 1) & 1, dev_status, abort_flag)) break;
-        const int key0 = (k0 + c.j) * kBN;
         mbar_expect_tx(&bar->k_full[s], 2 * C::kKvBytes);  // K and V of a tile arrive under one barrier
         for (int ch = 0; ch < C::kChunks; ++ch)
-          tma_load_3d(sK + s * C::kKvBytes + ch * C::kKvSlab, &tm_k, &bar->k_full[s], h * DH + ch * 64, key0, b);
+          tma_load_3d(sK + s * C::kKvBytes + ch * C::kKvSlab, &tm_k, &bar->k_full[s], ch0 + ch * 64, key0, b);
         for (int ch = 0; ch < C::kChunks; ++ch)
-          tma_load_3d(sV + s * C::kKvBytes + ch * C::kKvSlab, &tm_v, &bar->k_full[s], h * DH + ch * 64, key0, b);
+          tma_load_3d(sV + s * C::kKvBytes + ch * C::kKvSlab, &tm_v, &bar->k_full[s], ch0 + ch * 64, key0, b);
       }
     }
-  } else if (warp == 9 || (warp == 11 && C::kIssuers == 2)) {
+  } else if (warp == 17 || (warp == 19 && C::kIssuers == 2)) {
     // ------------------------------------------------------------------ MMA issuer(s)
     // A thread's MMAs execute in the order it issues them: the S product of tile n+2 goes into the buffer whose
     // P the PV product of tile n, issued just before by the same thread, still reads.  The two query tiles'
     // products are independent of each other: one thread issues both, or each tile has its own thread
     // (query tiles [q_lo, q_hi) here); the barriers that both tiles' products free count one arrival per thread.
-    const int q_lo = C::kIssuers == 2 && warp == 11 ? 1 : 0, q_hi = C::kIssuers == 2 && warp == 9 ? 1 : 2;
+    const int q_lo = C::kIssuers == 2 && warp == 19 ? 1 : 0, q_hi = C::kIssuers == 2 && warp == 17 ? 1 : 2;
     if (elect_one()) {
       constexpr uint32_t idesc_s = idesc_f16(kFmtBF16, kFmtBF16, false, false, kBM, kBN);
-      // With row sums on the tensor pipe the B operand is [V | ones]: N = DH + 16, the 16 extra
-      // columns come from a constant slab of ones placed one "leading byte offset" after V's slab,
-      // so one MMA per 16 keys updates O and the row sums (which sit right behind O in tensor memory).
-      constexpr uint32_t idesc_o = idesc_f16(kFmtBF16, kFmtBF16, false, true, kBM, C::kSumMma ? DH + 16 : DH);
+      constexpr uint32_t idesc_o = idesc_f16(kFmtBF16, kFmtBF16, false, true, kBM, DH);
       // Descriptors are built once and advanced by adding a constant to the 14-bit start-address
       // field (no carry: all tiles live below 256 KB).
       const uint64_t q_desc0 = smem_desc_sw128(smem_u32(sQ), 16, 1024);
       const uint64_t k_desc0 = smem_desc_sw128(smem_u32(sK), 16, 1024);
-      const uint32_t v_addr0 = smem_u32(sV), ones_addr = smem_u32(sOnes);
+      const uint64_t v_desc0 = smem_desc_sw128(smem_u32(sV), C::kKvSlab, 1024);
       Cursor cs, cp;  // the S products run two tiles ahead of the PV products
       cs.init(it_begin, it_end, nblk);
       cp.init(it_begin, it_end, nblk);
-      bool ok = true;
       // Q of the piece and K of the tile that `cs` points at have landed
       auto s_inputs = [&]() -> bool {
         if (cs.j == 0 && !mbar_wait(&bar->q_full[cs.pc % C::kQBufs], (cs.pc / C::kQBufs) & 1, dev_status, abort_flag)) return false;
         return mbar_wait(&bar->k_full[cs.n % C::kStages], (cs.n / C::kStages) & 1, dev_status, abort_flag);
       };
       auto issue_s = [&](int q) {
-        const int s = cs.n % C::kStages, b = cs.n & 1, qb = cs.pc % C::kQBufs;
+        const int s = cs.n % C::kStages, h = cs.n & 1, qb = cs.pc % C::kQBufs;
         const uint64_t qd = q_desc0 + (uint64_t)((qb * C::kQBytes + q * C::kQTile) >> 4);
         const uint64_t kd = k_desc0 + (uint64_t)((s * C::kKvBytes) >> 4);
-        const uint32_t t_s = tmem + C::kColS + (2 * q + b) * kBN;
+        const uint32_t t_s = tmem + C::s_col(q, h);
 #pragma unroll
         for (int kk = 0; kk < DH / 16; ++kk) {
           const uint64_t qoff = (uint64_t)(((kk >> 2) * C::kQSlab + (kk & 3) * 32) >> 4);
           const uint64_t koff = (uint64_t)(((kk >> 2) * C::kKvSlab + (kk & 3) * 32) >> 4);
           mma_ss(t_s, qd + qoff, kd + koff, idesc_s, kk > 0);
         }
-        mma_commit(&bar->s_full[q][b]);
+        mma_commit(&bar->s_full[q][h]);
       };
+      bool ok = true;
       for (int pre = 0; pre < 2 && ok && cs.valid(); ++pre) {
         ok = s_inputs();
         if (!ok) break;
@@ -682,26 +766,23 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         cs.next();
       }
       while (ok && cp.valid()) {
-        const int s = cp.n % C::kStages, b = cp.n & 1;
+        const int s = cp.n % C::kStages, h = cp.n & 1;
         const bool more = cs.valid();
-        const uint32_t va = v_addr0 + s * C::kKvBytes;
-        const uint64_t vd = smem_desc_sw128(va, C::kSumMma ? ones_addr - va : (uint32_t)C::kKvSlab, 1024);
+        const uint64_t vd = v_desc0 + (uint64_t)((s * C::kKvBytes) >> 4);
+        const bool fresh = cp.j == 0 || (C::kOwnO && cp.j == 1);  // the accumulator's first product of the piece
 #pragma unroll
         for (int q = q_lo; q < q_hi; ++q) {
           // P ready implies that the K/V tile has landed
-          if (!mbar_wait(&bar->p_full[q][b], (cp.n >> 1) & 1, dev_status, abort_flag)) { ok = false; break; }
+          if (!mbar_wait(&bar->p_full[q][h], (cp.n >> 1) & 1, dev_status, abort_flag)) { ok = false; break; }
           // the first product of a piece overwrites the accumulator the previous epilogue reads
-          if (cp.j == 0 && cp.pc > 0 && !mbar_wait(&bar->o_free[q], (cp.pc - 1) & 1, dev_status, abort_flag)) { ok = false; break; }
+          if (fresh && cp.pc > 0 && !mbar_wait(&bar->o_free[q], (cp.pc - 1) & 1, dev_status, abort_flag)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t t_o = tmem + C::kColO + q * C::kOStride;
-          const uint32_t t_p = tmem + C::kColS + (2 * q + b) * kBN;
+          const uint32_t t_o = tmem + C::o_col(q, h), t_p = tmem + C::s_col(q, h);
 #pragma unroll
           for (int kk = 0; kk < kBN / 16; ++kk)  // 16 keys per MMA: 8 packed columns of P, 16 rows of V
-            mma_ts(t_o, t_p + kk * 8, vd + (uint64_t)((kk * 2048) >> 4), idesc_o, cp.j > 0 || kk > 0);
-          // One phase per piece: the next piece's products wait for o_free, which the epilogue gives
-          // only after it has seen this phase, so a waiter is never two phases behind.
-          if (cp.last_of_piece()) mma_commit(&bar->o_done[q]);
-          if (q == q_hi - 1) mma_commit(&bar->kv_empty[s]);  // frees the K/V slot; also "PV of this tile has landed" for a rescale
+            mma_ts(t_o, t_p + kk * 8, vd + (uint64_t)((kk * 2048) >> 4), idesc_o, !fresh || kk > 0);
+          mma_commit(&bar->pv_done[q][h]);
+          if (q == q_hi - 1) mma_commit(&bar->kv_empty[s]);
           if (more) {
             if (q == q_lo) {
               ok = s_inputs();
@@ -719,35 +800,35 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         cp.next();
       }
     }
-  } else if (warp == 10) {
+  } else if (warp == 18) {
     // ------------------------------------------------------------------ publisher
     if (lane == 0) {
       // When the span's first piece is partial and more pieces follow, make that piece
-      // visible to the other CTAs and draw its eight tickets here, off the softmax warps' path.
+      // visible to the other CTAs and draw its tickets here, off the softmax warps' path.
       const int u = it_begin / nblk;
       const bool early = (it_begin > u * nblk || it_end < (u + 1) * nblk) && it_end > (u + 1) * nblk;
       if (early && mbar_wait(&bar->pub_ready, 0, dev_status, abort_flag)) {
         __threadfence();
-        uint32_t t[8];
+        uint32_t t[kSoftWarps];
 #pragma unroll
-        for (int w = 0; w < 8; ++w) t[w] = atomicAdd(&tickets[(size_t)u * 8 + w], 1u);
+        for (int w = 0; w < kSoftWarps; ++w) t[w] = atomicAdd(&tickets[(size_t)u * kSoftWarps + w], 1u);
 #pragma unroll
-        for (int w = 0; w < 8; ++w) bar->first_ticket[w] = t[w];
+        for (int w = 0; w < kSoftWarps; ++w) bar->first_ticket[w] = t[w];
         mbar_arrive(&bar->pub_done);
       }
       // When the span ends inside a unit that one other CTA shares, that CTA ran its part at the
-      // start of its span and has normally published it long since.  Watch its eight tickets (acquire)
+      // start of its span and has normally published it long since.  Watch its tickets (acquire)
       // and leave the answer in shared memory for the softmax warps: they add the two pieces up
       // straight from tensor memory if the answer is there when their last piece ends, and go
       // through scratch and tickets otherwise.  Polling keeps the ticket out of their registers.
       const int ul = (it_end - 1) / nblk;
       if (it_end < (ul + 1) * nblk && sp.unit_hi[1][blockIdx.x] == sp.unit_lo[1][blockIdx.x] + 1) {
-        const uint32_t* tk = tickets + (size_t)ul * 8;
+        const uint32_t* tk = tickets + (size_t)ul * kSoftWarps;
         for (uint32_t spin = 0; spin < kSpinLimit; ++spin) {
           if ((*(volatile uint32_t*)&bar->poll_stop[0] && *(volatile uint32_t*)&bar->poll_stop[1]) || *abort_flag) break;
           bool all = true;
 #pragma unroll
-          for (int w = 0; w < 8; ++w) all = all && ld_acquire_gpu(tk + w) == 1u;
+          for (int w = 0; w < kSoftWarps; ++w) all = all && ld_acquire_gpu(tk + w) == 1u;
           if (all) {
             st_release_cta(&bar->others_done, 1u);
             break;
@@ -756,43 +837,115 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         }
       }
     }
-  } else if (warp < 8) {
-    // ------------------------------------------------------------------ softmax / correction / epilogue
+  } else if (warp < kSoftWarps) {
+    // ------------------------------------------------------------------ softmax / epilogue
     Row t;
-    t.q = warp >> 2, t.warp = warp, t.lane = lane;
-    t.row = warp * 32 + lane;  // query row inside the unit; (warp & 3) * 32 + lane is its tensor-memory lane
-    const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-    t.ob = tmem + lane_addr + C::kColO + t.q * C::kOStride;
+    t.q = warp >> 3, t.half = (warp >> 2) & 1, t.warp = warp, t.lane = lane;
+    t.row = t.q * kBM + (warp & 3) * 32 + lane;  // query row inside the unit; (warp & 3) * 32 + lane is its tensor-memory lane
+    t.tm = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t s_addr = t.tm + C::s_col(t.q, t.half);
+    uint64_t* s_bar = &bar->s_full[t.q][t.half];
+    volatile uint32_t* move = &bar->move[pair_of(t)];
+    // A warp whose wait ran out goes on without waiting: the two warps of a row meet at barriers, and neither may
+    // stay away (the results are void, and the status word says so).
     bool ok = true;
-    int n = 0, pc = 0;
-    for (int it = it_begin; ok && it < it_end; ++pc) {
+    int pc = 0;
+    for (int it = it_begin; it < it_end; ++pc) {
       const Piece p = piece_at(it, it_end, nblk);
+      // number of the piece's first tile: the tiles of this pipeline are those of its parity
+      const int n0 = it - it_begin, last_n = n0 + p.cnt - 1;
       it += p.cnt;
-      float m_used = -INFINITY, l = 0.f;
-      for (int j = 0; j < p.cnt; ++j, ++n) {
-        const int b = n & 1;
-        const uint32_t sb = tmem + lane_addr + C::kColS + (2 * t.q + b) * kBN;
-        if (!mbar_wait(&bar->s_full[t.q][b], (n >> 1) & 1, dev_status, abort_flag)) { ok = false; break; }
-        tc_fence_after();
-        const int valid = L - (p.k0 + j) * kBN;  // keys of this tile inside the sequence (>= 64: all)
-        uint64_t* pvb = &bar->kv_empty[(n + C::kStages - 1) % C::kStages];  // barrier the previous tile's PV commits to
-        const uint32_t pvp = (uint32_t)(((n - 1) / C::kStages) & 1);
-        if (valid >= kBN) ok = softmax_tile<DH, C::kSumMma, false>(sb, t.ob, scale_log2, kBN, j, m_used, l, pvb, pvp, dev_status, abort_flag);
-        else ok = softmax_tile_ragged<DH>(sb, t.ob, scale_log2, valid, j, m_used, l, pvb, pvp, dev_status, abort_flag);
-        if (!ok) break;
+      float m_used = -INFINITY;
+      uint64_t l2 = 0;
+      if constexpr (!C::kOwnO) {  // one reference for both pipelines: out of the piece's first tile
+        float mx = -INFINITY;
+        if ((n0 & 1) == t.half) {
+          ok = ok && __all_sync(0xffffffffu, mbar_wait(s_bar, (n0 >> 1) & 1, dev_status, abort_flag));
+          tc_fence_after();
+          mx = tile_max(s_addr, min(32, L - p.k0 * kBN), scale_log2);
+        }
+        m_used = ceilf(fmaxf(mx, __uint_as_float(exchange<DH>(t, bar, __float_as_uint(mx), 0u).x))) + kHeadroom;
+      }
+      auto moved_to = [&](float m_new) {
+        const float f = ex2_mufu(m_used - m_new);
+        l2 = mul2(l2, pack2(f, f));
+        m_used = m_new;
+      };
+      bool first = true;
+      for (int j = (n0 ^ t.half) & 1; j < p.cnt; j += 2) {
+        const int n = n0 + j, valid = min(kBN, L - (p.k0 + j) * kBN);  // keys of this tile inside the sequence
+        if constexpr (C::kOwnO) {
+          ok = ok && mbar_wait(s_bar, (n >> 1) & 1, dev_status, abort_flag);
+          __syncwarp();
+          tc_fence_after();
+          if (first) m_used = ceilf(tile_max(s_addr, min(valid, 32), scale_log2)) + kHeadroom;
+        } else {
+          while (ok) {
+            const Wait w = wait_s_or_move(s_bar, (n >> 1) & 1, move, dev_status, abort_flag);
+            if (w == Wait::kReady) break;
+            if (w == Wait::kAborted) ok = false;
+            else moved_to(meet<DH>(t, bar, s_addr, valid, scale_log2, m_used, false, false, n, n0, last_n, dev_status).m);
+          }
+          tc_fence_after();
+        }
+        uint32_t pk[32];
+        uint64_t sum2;
+        bool asked = false;  // a second time would not help (scores that are no numbers)
+#pragma unroll 1
+        for (;;) {
+          uint32_t big = 0;
+          sum2 = 0;
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            uint32_t r[32];
+            tmem_ld32(s_addr + c * 32, r);
+            tmem_wait_ld(r);
+            if (valid < (c + 1) * 32) {  // keys that are not there
+#pragma unroll
+              for (int e = 0; e < 32; ++e)
+                if (c * 32 + e >= valid) r[e] = 0xFF800000u;  // -inf
+            }
+            chunk_exp_ref(r, *reinterpret_cast<uint32_t(*)[16]>(&pk[c * 16]), scale_log2, -m_used, sum2, big);
+          }
+          const bool grown = __any_sync(0xffffffffu, (big & 0x40004000u) != 0u) && !asked;
+          if constexpr (C::kOwnO) {
+            if (!grown) break;
+            moved_to(move_reference<DH>(t, bar, s_addr, valid, scale_log2, m_used, !first, n, dev_status));
+          } else {
+            if (!grown && __all_sync(0xffffffffu, *move == 0u)) break;
+            if (grown && lane == 0) *move = 1u;
+            moved_to(meet<DH>(t, bar, s_addr, valid, scale_log2, m_used, grown, true, n, n0, last_n, dev_status).m);
+          }
+          asked = asked || grown;
+        }
+        first = false;
+        l2 = add2(l2, sum2);
+        tmem_st32(s_addr, pk);
+        tmem_wait_st();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&bar->p_full[t.q][b]);
+        if (lane == 0) mbar_arrive(&bar->p_full[t.q][t.half]);
       }
-      if (!ok) break;
-      if (p.cnt == nblk) ok = finish_whole<DH>(t, bar, p.u, pc, l, &tm_o, L, heads, dev_status);
-      else ok = finish_partial<DH>(t, bar, p, pc, it >= it_end, m_used, l, o, &tm_o, L, heads, sp, tickets, pieces, dev_status);
+      if constexpr (!C::kOwnO) {  // the other warp may still want to move the reference
+        for (;;) {
+          const Meeting mt = meet<DH>(t, bar, s_addr, 0, scale_log2, m_used, false, false, kNoTile, n0, last_n, dev_status);
+          if (!mt.asked) break;
+          moved_to(mt.m);
+        }
+      }
+      float l, l_odd;
+      unpack2(l2, l, l_odd);
+      const Joint jn = join_halves<DH>(t, bar, m_used, l + l_odd);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) continue;
+      if (p.cnt == nblk) ok = finish_whole<DH>(t, bar, p, last_n, jn, &tm_o, L, heads, dev_status);
+      else ok = finish_partial<DH>(t, bar, p, pc, last_n, it >= it_end, jn, o, &tm_o, L, heads, sp, tickets, pieces, dev_status);
     }
-    if (ok) settle_first_piece<DH>(bar, it_begin, it_end, t, o, L, heads, sp, pieces, dev_status);
+    if (__all_sync(0xffffffffu, ok)) settle_first_piece<DH>(bar, it_begin, it_end, t, o, L, heads, sp, pieces, dev_status);
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 9) {
+  if (warp == 17) {
     tc_fence_after();
     tmem_dealloc(tmem, C::kTmemCols);
   }
@@ -800,7 +953,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 
 size_t ticket_bytes(int B, int L, int heads) {
   const size_t units = (size_t)B * heads * ((L + kUM - 1) / kUM);
-  return (units * 8 * sizeof(uint32_t) + 255) & ~(size_t)255;
+  return (units * kSoftWarps * sizeof(uint32_t) + 255) & ~(size_t)255;
 }
 
 int max_ctas() {
@@ -944,7 +1097,7 @@ cudaError_t launch(int B, int L, int heads, const void* q, const void* k, const 
   const uint64_t strides[2] = {(uint64_t)heads * DH * 2, (uint64_t)L * heads * DH * 2};
   const uint32_t box_q[3] = {64, kBM, 1};
   const uint32_t box_kv[3] = {64, kBN, 1};
-  const uint32_t box_o[3] = {64, 32, 1};  // a softmax warp's 32 rows of one 64-channel slab
+  const uint32_t box_o[3] = {32, 32, 1};  // a softmax warp's 32 rows of 32 channels
   if (!encode_tmap_16bit(&tq, q, 3, dims, strides, box_q) || !encode_tmap_16bit(&tk, k, 3, dims, strides, box_kv) ||
       !encode_tmap_16bit(&tv, v, 3, dims, strides, box_kv) || !encode_tmap_16bit(&to, o, 3, dims, strides, box_o))
     return cudaErrorInvalidValue;

@@ -250,6 +250,14 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
       : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// The same for 32 registers of a load whose wait may have other work in front of it: nothing uses them any earlier.
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]),
+                 "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]),
+                 "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]),
+                 "+r"(r[31])::"memory");
+}
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // ---------------------------------------------------------------- programmatic dependent launch
@@ -295,7 +303,8 @@ __device__ __forceinline__ uint32_t sw128_offset(int row, int chunk) {
 }  // namespace tc
 
 // ---------------------------------------------------------------- host: tensor maps
-// Encodes a bf16/fp16 tiled tensor map with 128-byte swizzle through the driver entry point
+// Encodes a bf16/fp16 tiled tensor map with 128-byte swizzle (64-byte for boxes of 32 elements: the span has to be the
+// box's row, a copy with a wider span runs past the staged tile) through the driver entry point
 // obtained from the runtime (the library does not link libcuda).  dims/strides innermost first;
 // strides[i] is the byte stride of dimension i+1.
 // Launch with programmatic stream serialisation: the kernel must call tc::dependency_wait().

@@ -1159,3 +1159,30 @@ def test_global_merge_of_ragged_images_parity(toma, gh, gw, th, tw, ratio):
         assert np.abs(dense_dev[b, 0].double().cpu().numpy() - w).max() <= 6e-4
         assert_close(merged[b], O.merge(w, x_host[b]), "bf16", "merge")
         assert_close(unmerged[b], O.unmerge(w, to_host64(y_dev)[b]), "bf16", "unmerge")
+
+
+@pytest.mark.parametrize("dh", [64, 128])
+@pytest.mark.parametrize("L,split,ctas", [(1000, 0, 0), (1000, 1, 5), (130, 0, 0), (65, 0, 0), (20, 0, 0)])
+def test_attention_scores_that_outgrow_every_headroom(toma, tuning, dh, L, split, ctas):
+    """Scores jump by hundreds of log2 units from key tile to key tile, at different tiles for different rows and in either of
+    the two pipelines a row's tiles are dealt to: the reference has to be moved again and again, also while the other
+    pipeline's probabilities lie ready against the old one."""
+    B, h = 1, 3
+    rng = np.random.default_rng(dh + L)
+    u = rng.normal(size=(4, dh))
+    u /= np.linalg.norm(u, axis=1, keepdims=True)
+    rows = rng.integers(0, 4, size=L)   # a query's direction: four kinds of rows side by side in every warp
+    q = 0.2 * rng.normal(size=(B, L, h, dh)) + 16.0 * u[rows][None, :, None]
+    tiles = (L + 63) // 64
+    level = np.stack([np.cumsum(rng.random(tiles) * rng.integers(0, 2, tiles)) for _ in range(4)], 1)  # per tile and direction
+    k = 0.2 * rng.normal(size=(B, L, h, dh)) + (np.sqrt(dh) * 3.0 * level @ u)[np.arange(L) // 64][None, :, None]
+    v = rng.normal(size=(B, L, h, dh))
+    host = [gen.round_to_dtype(a.reshape(B, L, h * dh).astype(np.float32), "bf16") for a in (q, k, v)]
+    dq, dk, dv = (to_dev(a, "bf16") for a in host)
+    o = torch.empty_like(dq)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    tuning(attention_split=split, attention_ctas=ctas)
+    toma.toma_attention(B, L, h, dh, "bf16", dq, dk, dv, o, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert_close(to_host64(o)[0], O.attention(host[0][0], host[1][0], host[2][0], h), "bf16", "attention with jumping scores")
