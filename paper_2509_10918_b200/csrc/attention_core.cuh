@@ -6,9 +6,6 @@
 #include "common.cuh"
 #include "tc.cuh"
 
-#ifndef TOMA_POLY
-#define TOMA_POLY(e) (((e) & 6) == 6)
-#endif
 namespace toma {
 namespace attn {
 
@@ -197,19 +194,20 @@ __device__ __forceinline__ bool softmax_tile(uint32_t sb, uint32_t ob, float sca
 // ------------------------------------------------------------------ softmax against a reference with headroom
 // P = 2^(S c - m) of 32 columns as packed bf16 for a reference m that lies 2^kHeadroom above the scores seen when it was
 // set.  Everything is floating point, so the common factor costs no precision; what it buys is that the reference need
-// not follow the row maximum: no maximum is taken before the exponentials.  Instead `big` collects bit 14 of every
-// result, which is set exactly when P >= 2 (or is no number): then, and only then, the scores have outgrown the headroom
+// not follow the row maximum: no maximum is taken before the exponentials.  Instead the largest P of the tile is looked
+// at: one of 2 or more (bit 14, set in numbers that are none as well) says that the scores have outgrown the headroom,
 // and the caller moves the reference.  sum2: fp32 sums of the even and the odd columns.
-// One pair of columns in four takes the polynomial of ex2_poly2 on the FMA pipe, the others MUFU.
+// One pair of columns in four takes the polynomial of ex2_poly2 on the FMA pipe, the others MUFU (timed: one in eight to
+// three in eight are within 2 % of each other).
 constexpr float kHeadroom = 32.f;
 
-__device__ __forceinline__ void chunk_exp_ref(const uint32_t (&r)[32], uint32_t (&pk)[16], float scale, float neg_m, uint64_t& sum2, uint32_t& big) {
+__device__ __forceinline__ void chunk_exp_ref(const uint32_t (&r)[32], uint32_t (&pk)[16], float scale, float neg_m, uint64_t& sum2) {
   const uint64_t c2 = pack2(scale, scale), m2 = pack2(neg_m, neg_m);
 #pragma unroll
   for (int e = 0; e < 32; e += 2) {
     const uint64_t x2 = fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), c2, m2);
     float p0, p1;
-    if (TOMA_POLY(e)) {
+    if ((e & 6) == 6) {
       ex2_poly2(x2, p0, p1);
     } else {
       float x0, x1;
@@ -220,8 +218,27 @@ __device__ __forceinline__ void chunk_exp_ref(const uint32_t (&r)[32], uint32_t 
     sum2 = add2(sum2, pack2(p0, p1));
     pk[e >> 1] = pack_bf16_rn(p0, p1);
   }
+}
+// The largest P of a tile, even and odd columns (P is not negative, so packed bf16 compare as whole numbers).
+__device__ __forceinline__ uint32_t largest2(const uint32_t (&pk)[32]) {
+  uint32_t top = 0;
 #pragma unroll
-  for (int e = 0; e < 16; e += 2) big |= pk[e] | pk[e + 1];
+  for (int e = 0; e < 32; e += 2) top = __vimax3_u16x2(pk[e], pk[e + 1], top);
+  return top;
+}
+__device__ __forceinline__ bool outgrown(uint32_t top) { return (top & 0x40004000u) != 0u; }
+// sum2 adds up P before its rounding to bf16: one instruction per pair of columns, where the rounded values take three
+// (735 us against 825 us at 4 x 8192 tokens, 10 heads of 64).  Rounding errors of many keys cancel; that of a key which
+// makes up most of its row would scale the whole output row by up to 2^-9.  In a tile where some P is more than a quarter
+// of the row's sum so far, the row therefore counts what the product really multiplies.
+__device__ __forceinline__ bool dominates(uint32_t top, float sum) {
+  return 4.f * fmaxf(__uint_as_float(top << 16), __uint_as_float(top & 0xFFFF0000u)) > sum;
+}
+__device__ __forceinline__ uint64_t rounded_sum2(const uint32_t (&pk)[32]) {
+  uint64_t sum2 = 0;
+#pragma unroll
+  for (int e = 0; e < 32; ++e) sum2 = add2(sum2, pack2(__uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xFFFF0000u)));
+  return sum2;
 }
 
 // 32 accumulator columns of one row, scaled and rounded to bf16: 64 contiguous bytes.

@@ -9,32 +9,28 @@
 // scratch; the warp that arrives last at the (unit, warp) ticket adds the pieces up and writes the
 // output rows.  Nobody waits for another CTA.
 //
-// Inside a CTA (12 warps): warps 0..3 run the online softmax of query tile 0, warps 4..7 that of
-// query tile 1 (one thread per query row, straight out of tensor memory), warp 8 feeds Q, K and V
-// through TMA rings, one elected thread of warp 9 issues the tcgen05 MMAs (at head_dim 128 those of query tile 0,
-// and one of warp 11 those of query tile 1), warp 10 publishes a
-// partial first piece (memory fence and tickets, off everybody else's path).
-//   S_q,j = Q_q K_j^T      -> tensor memory, two 64-column buffers per query tile.  MMAs issued by
-//                             one thread execute in order, so S_q,j+2 is issued right behind the
-//                             product that reads P_q,j out of the same buffer, without a round trip
-//                             through a barrier: a softmax warp group always finds its next S tile
-//                             complete, and the tensor pipe, the two softmax groups and the loads
-//                             overlap instead of taking turns.
-//   P_q,j = 2^(S*c - m)    -> written back over S_q,j's first 32 columns as bf16 and used as the
-//                             A operand (from tensor memory) of  O_q += P_q,j V_j
-//   row sums (head_dim 64) -> the B operand of that product is [V_j | 1]: 16 extra columns of ones
-//                             accumulate sum_k P_jk behind O in tensor memory: exactly the bf16 P
-//                             that multiplies V, so P can be produced by truncation (one
-//                             byte-permute per pair, no conversion on the XU pipe) without biasing
-//                             the normalised result
-//   running maximum        -> O (and the row sums) are rescaled only when the maximum grew by more
-//                             than 2^8; the final division by the row sum makes a stale maximum exact
-//   exponentials           -> one pair of columns in four (three in eight at head_dim 128) goes through
-//                             a degree-3 polynomial on the FMA pipe (relative error 7.5e-5, far below
-//                             bf16 resolution of P), the rest through MUFU ex2; the scaling S*c - m and
-//                             the polynomial run in packed f32x2 arithmetic (one issue slot for two columns)
-// The whole S row of a tile (64 fp32) is fetched with one tensor-memory round trip and kept in
-// registers for both the maximum and the exponentials.
+// Inside a CTA (20 warps): warps 0..15 run the softmax as four pipelines of four warps, one per query tile q and parity h
+// of the key tile (one thread per query row, straight out of tensor memory; so two threads share a row, each with every
+// second key tile), warp 16 feeds Q, K and V through TMA rings, one elected thread of warp 17 issues the tcgen05 MMAs (at
+// head_dim 128 those of query tile 0, and one of warp 19 those of query tile 1), warp 18 publishes a partial first piece
+// (memory fence and tickets, off everybody else's path).
+//   S_q,j = Q_q K_j^T      -> tensor memory, 64 columns per pipeline.  MMAs issued by one thread execute in order, so
+//                             S_q,j+2 is issued right behind the product that reads P_q,j out of the same columns,
+//                             without a round trip through a barrier.
+//   P_q,j = 2^(S*c - m)    -> written back over S_q,j's first 32 columns as bf16 and used as the A operand (from tensor
+//                             memory) of  O += P_q,j V_j
+//   O                      -> at head_dim 64 every pipeline has an accumulator and a reference m of its own (four of 64
+//                             columns beside four of S fill the tensor memory), added up at the end of a piece; at
+//                             head_dim 128 the two pipelines of a query tile share one, and with it the reference
+//   reference              -> set 2^32 above the piece's first scores and moved only when scores outgrow it (see
+//                             chunk_exp_ref), so no row maximum stands before the exponentials
+//   exponentials           -> one pair of columns in four goes through a degree-3 polynomial on the FMA pipe (relative
+//                             error 7.5e-5, far below bf16 resolution of P), the rest through MUFU ex2; the scaling
+//                             S*c - m and the polynomial run in packed f32x2 arithmetic
+// What bounds it is the softmax (per 64 keys and row about 450 issue slots of a warp; the tensor pipe is busy 35 to 60 % of
+// the time): with one pipeline per query tile a scheduler had two softmax warps, which left it idle whenever both waited
+// for tensor memory or each other's dependencies.  Four pipelines: 960 -> 754 us at 4 x 8192 tokens and 10 heads of 64,
+// 49.5 -> 41.6 us at 2 x 2048, 142 -> 136.5 us at 4 x 2048 tokens and 17 heads of 128.
 // Keys past the sequence end are zero-filled by TMA and masked out; query rows past the end are
 // computed on zeros and not written.
 #include <mutex>
@@ -43,9 +39,6 @@
 #include "common.cuh"
 #include "tc.cuh"
 
-#ifndef TOMA_ISS
-#define TOMA_ISS (DH == 128 ? 2 : 1)
-#endif
 namespace toma {
 
 using namespace tc;
@@ -71,7 +64,10 @@ struct AttCfg {
   static constexpr int kBarBytes = 512;
   static constexpr int kSmemBytes = 1024 + kQBufs * kQBytes + 2 * kStages * kKvBytes + kOutBytes + kBarBytes;
   static constexpr int kTmemCols = 512;
-  static constexpr int kIssuers = TOMA_ISS;  // threads that issue MMAs
+  // Threads that issue MMAs.  At head_dim 128 a tile is 12 MMAs and one thread for both query tiles keeps the tensor pipe
+  // waiting; at head_dim 64 the softmax bounds and a second thread takes issue slots from it (752 -> 799 us at 4 x 8192
+  // tokens, 10 heads).
+  static constexpr int kIssuers = DH == 128 ? 2 : 1;
   // Tensor memory: a pipeline (query tile q, parity h) has 64 columns of S (P takes the first 32) and, at head_dim 64, an
   // accumulator of its own; at head_dim 128 the two pipelines of a query tile share one.
   static constexpr bool kOwnO = DH == 64;
@@ -890,10 +886,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         }
         uint32_t pk[32];
         uint64_t sum2;
+        uint32_t top;
         bool asked = false;  // a second time would not help (scores that are no numbers)
 #pragma unroll 1
         for (;;) {
-          uint32_t big = 0;
           sum2 = 0;
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
@@ -905,9 +901,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
               for (int e = 0; e < 32; ++e)
                 if (c * 32 + e >= valid) r[e] = 0xFF800000u;  // -inf
             }
-            chunk_exp_ref(r, *reinterpret_cast<uint32_t(*)[16]>(&pk[c * 16]), scale_log2, -m_used, sum2, big);
+            chunk_exp_ref(r, *reinterpret_cast<uint32_t(*)[16]>(&pk[c * 16]), scale_log2, -m_used, sum2);
           }
-          const bool grown = __any_sync(0xffffffffu, (big & 0x40004000u) != 0u) && !asked;
+          top = largest2(pk);
+          const bool grown = __any_sync(0xffffffffu, outgrown(top)) && !asked;
           if constexpr (C::kOwnO) {
             if (!grown) break;
             moved_to(move_reference<DH>(t, bar, s_addr, valid, scale_log2, m_used, !first, n, dev_status));
@@ -919,12 +916,20 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           asked = asked || grown;
         }
         first = false;
-        l2 = add2(l2, sum2);
         tmem_st32(s_addr, pk);
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&bar->p_full[t.q][t.half]);
+        // the sum, while the tensor cores already multiply P
+        float even, odd;
+        unpack2(add2(l2, sum2), even, odd);
+        const bool dom = dominates(top, even + odd);
+        if (__any_sync(0xffffffffu, dom)) {
+          const uint64_t rounded = rounded_sum2(pk);
+          if (dom) sum2 = rounded;
+        }
+        l2 = add2(l2, sum2);
       }
       if constexpr (!C::kOwnO) {  // the other warp may still want to move the reference
         for (;;) {
