@@ -2,16 +2,14 @@
 // accumulation in tensor memory, bf16 out): the QKV and output projections of the attention module
 // that ToMA wraps (Algorithm 3's core module F; App. C counts them as the 4 d^2 N term).
 //
-// Rows of A (tokens) sit on the MMA M dimension, 128 per CTA; a CTA covers up to 320 output columns
-// (two MMAs along N, at most 192 + 128).  A is the K-major operand exactly as stored ([m][k] row-major),
-// W the MN-major one exactly as stored ([k][n] row-major), so neither is transposed or copied.
-// blockIdx.z selects one of up to three weight / output pairs that share A (Q, K and V in one
-// launch).  Warp 0 feeds a TMA ring, warp 1 issues the MMAs, warps 2..5 take the accumulators out of tensor
-// memory (through the activation when one is asked for: the first layer of the MLP, the other module ToMA
-// wraps), stage each warp's 32 rows in shared memory as 64-column slabs in the layout of the output tensor
-// map's box (the ring is free by then) and store them with one TMA store per warp and slab: whole lines,
-// asynchronous, instead of 16-byte stores to 32 different rows per warp instruction.
-#include <cstdlib>
+// Rows of A (tokens) sit on the MMA M dimension.  A is the K-major operand exactly as stored ([m][k] row-major),
+// W the MN-major one exactly as stored ([k][n] row-major), so neither is transposed or copied.  Up to three weight /
+// output pairs share A (Q, K and V in one launch).  Warp 0 feeds a TMA ring, warp 1 issues the MMAs, the other warps take
+// the accumulators out of tensor memory (through the activation when one is asked for: the first layer of the MLP, the
+// other module ToMA wraps), stage their 32 rows in shared memory as 64-column slabs in the layout of the output tensor
+// map's box and store them with one TMA store per warp and slab: whole lines, asynchronous, instead of 16-byte stores to
+// 32 different rows per warp instruction.
+#include <climits>
 
 #include "common.cuh"
 #include "tc.cuh"
@@ -26,46 +24,78 @@ constexpr int kKC = 64;                  // contraction elements per stage
 constexpr int kSlab = kKC * 128;         // [64 k][64 n] slab of W, 128-byte rows
 constexpr int kABytes = 128 * 128;       // [128 m][64 k] slab of A
 
-struct GemmBars {
-  uint64_t full[4], empty[4], done;
+// GELU(v) = v Phi(v) = max(v, 0) - |v| Phi(-|v|) of two values, for results that are rounded to bf16.
+// Phi(-a) = erfcx(a / sqrt 2) / 2 * 2^(-a^2 log2(e) / 2), and erfcx(x) / 2 = t (c0 + c1 t + ... + c7 t^7) with
+// t = 1 / (1 + 0.33 x): the coefficients are the minimax fit of the relative error on x in [0, 10] (9.4e-8; with fp32
+// arithmetic the result is within 5e-7 of the exact one for v > -1 and 8e-6 down to -13, where v (1 + erff) loses all
+// digits).  Eleven issue slots and two MUFU operations per value against about 45 slots with erff, which made the first
+// layer of an MLP of 4096 x 2560 x 640 a matter of its epilogue (34 us of which 13 us the activation).
+__device__ __forceinline__ float rcp_mufu(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float min_nan(float a, float b) {  // a number that is none stays one
+  float d;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t both(float v) { return pack2(v, v); }
+__device__ __forceinline__ void gelu2(uint32_t& v0, uint32_t& v1) {
+  const float x0 = __uint_as_float(v0), x1 = __uint_as_float(v1);
+  const uint64_t a = pack2(min_nan(fabsf(x0), 30.f), min_nan(fabsf(x1), 30.f));
+  float d0, d1, e0, e1;
+  unpack2(fma2(a, both(0.233345238f), both(1.f)), d0, d1);
+  const uint64_t t = pack2(rcp_mufu(d0), rcp_mufu(d1));
+  uint64_t q = fma2(both(-0.0676728131f), t, both(0.230118425f));
+  q = fma2(q, t, both(-0.175574611f));
+  q = fma2(q, t, both(0.204249755f));
+  q = fma2(q, t, both(0.0236104601f));
+  q = fma2(q, t, both(0.100611901f));
+  q = fma2(q, t, both(0.0914779779f));
+  q = fma2(q, t, both(0.0931789011f));
+  unpack2(mul2(mul2(a, both(-0.72134752f)), a), e0, e1);
+  q = mul2(mul2(mul2(q, t), a), pack2(ex2_mufu(e0), ex2_mufu(e1)));
+  float g0, g1;
+  unpack2(sub2(pack2(fmaxf(x0, 0.f), fmaxf(x1, 0.f)), q), g0, g1);
+  v0 = __float_as_uint(g0);
+  v1 = __float_as_uint(g1);
+}
+
+// ------------------------------------------------------------------------------------------------
+// Tiles of 256 rows x 256 columns, one per CTA: two 128-row blocks share every W slab, so a CTA moves 64 KB per
+// 256 x 256 x 64 multiply-adds instead of 48 KB per 128 x 256 x 64.  For long contractions, which are bound by the
+// operands' traffic from L2 and hide the prologue and the epilogue this form does not overlap.
+// ------------------------------------------------------------------------------------------------
+constexpr int kPairRows = 256, kPairCols = 256, kPairStages = 3;
+constexpr int kPairRing = 2 * 4 * 128 * 128;  // the output tile is staged where the ring was
+struct PairBars {
+  uint64_t full[kPairStages], empty[kPairStages], done;
   uint32_t tmem_base;
   int abort_flag;
 };
 
-
-// kCols = 320: two accumulators (192 + 128 columns), 512 tensor-memory columns, one CTA per SM, deep ring.
-// kCols = 256: one accumulator, 256 tensor-memory columns, two CTAs per SM, for grids that would otherwise
-// spill into a second wave or leave most SMs idle.
-// kCols = 128: 128 tensor-memory columns and 32 KB stages, two CTAs per SM, for narrow outputs with a long
-// contraction (the second layer of the MLP: 4096 x 640 x 2560 is 64 tiles of 128 x 320 but 160 of 128 x 128).
-// kRowBlocks = 2 (with kCols = 256): two 128-row blocks per CTA share every W slab, so a CTA moves 64 KB
-// per 256 x 256 x 64 multiply-adds instead of 48 KB per 128 x 256 x 64 (these shapes re-read their operands
-// from L2 many times and are bound by that traffic); one CTA per SM.
-template <int kCols, int kRowBlocks = 1>
 __global__ void __launch_bounds__(192, 1)
-linear_rows_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w0,
+linear_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w0,
                    const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__ CUtensorMap tm_w2,
                    const __grid_constant__ CUtensorMap tm_c0, const __grid_constant__ CUtensorMap tm_c1,
-                   const __grid_constant__ CUtensorMap tm_c2, int M, int N, int K, int stages, int ring_bytes, int act,
-                   uint32_t* dev_status) {
+                   const __grid_constant__ CUtensorMap tm_c2, int M, int N, int K, int act, uint32_t* dev_status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int kFirst = kCols == 320 ? 3 : 4;  // 64-column slabs of the first accumulator
-  const int m0 = blockIdx.x * 128 * kRowBlocks, n0 = blockIdx.y * kCols;
+  const int m0 = blockIdx.x * kPairRows, n0 = blockIdx.y * kPairCols;
   const CUtensorMap* tm_w = blockIdx.z == 0 ? &tm_w0 : blockIdx.z == 1 ? &tm_w1 : &tm_w2;
   const CUtensorMap* tm_c = blockIdx.z == 0 ? &tm_c0 : blockIdx.z == 1 ? &tm_c1 : &tm_c2;
-  const int n_cols = min(kCols, N - n0);         // columns of this CTA (multiple of 8)
+  const int n_cols = min(kPairCols, N - n0);     // columns of this CTA (multiple of 8)
   const int slabs = (n_cols + 63) / 64;
-  const int n_a = min(slabs, kFirst) * 64, n_b = (slabs - min(slabs, kFirst)) * 64;
-  const int stage_bytes = kRowBlocks * kABytes + slabs * kSlab;
-  GemmBars* bar = reinterpret_cast<GemmBars*>(smem + ring_bytes);  // behind the ring and the output's staging area, whichever is larger
+  constexpr int kStageBytes = 2 * kABytes + kPairCols / 64 * kSlab;
+  PairBars* bar = reinterpret_cast<PairBars*>(smem + kPairStages * kStageBytes);
   const int nk = (K + kKC - 1) / kKC;
-  constexpr uint32_t ncols = (kCols == 320 || kRowBlocks == 2) ? 512 : kCols == 128 ? 128 : 256;
-  static_assert(kRowBlocks == 1 || kCols == 256, "two row blocks need the one-accumulator column form");
+  constexpr uint32_t ncols = 512;
+  static_assert(kPairStages * kStageBytes >= kPairRing, "the output's staging area outgrew the ring");
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < stages; ++s) {
+    for (int s = 0; s < kPairStages; ++s) {
       mbar_init(&bar->full[s], 1);
       mbar_init(&bar->empty[s], 1);
     }
@@ -88,34 +118,31 @@ linear_rows_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
   if (warp == 0) {
     if (elect_one()) {
       for (int k = 0; k < nk; ++k) {
-        const int s = k % stages;
-        if (k >= stages && !mbar_wait(&bar->empty[s], ((k / stages) - 1) & 1, dev_status, abort_flag)) break;
-        uint8_t* sa = smem + s * stage_bytes;
-        mbar_expect_tx(&bar->full[s], stage_bytes);
-        for (int rb = 0; rb < kRowBlocks; ++rb) tma_load_2d(sa + rb * kABytes, &tm_a, &bar->full[s], k * kKC, m0 + rb * 128);
+        const int s = k % kPairStages;
+        if (k >= kPairStages && !mbar_wait(&bar->empty[s], ((k / kPairStages) - 1) & 1, dev_status, abort_flag)) break;
+        uint8_t* sa = smem + s * kStageBytes;
+        mbar_expect_tx(&bar->full[s], 2 * kABytes + slabs * kSlab);
+        for (int rb = 0; rb < 2; ++rb) tma_load_2d(sa + rb * kABytes, &tm_a, &bar->full[s], k * kKC, m0 + rb * 128);
         for (int j = 0; j < slabs; ++j)
-          tma_load_2d(sa + kRowBlocks * kABytes + j * kSlab, tm_w, &bar->full[s], n0 + j * 64, k * kKC);
+          tma_load_2d(sa + 2 * kABytes + j * kSlab, tm_w, &bar->full[s], n0 + j * 64, k * kKC);
       }
     }
   } else if (warp == 1) {
     if (elect_one()) {
-      const uint32_t idesc_a = idesc_f16(kFmtBF16, kFmtBF16, false, true, 128, n_a);
-      const uint32_t idesc_b = idesc_f16(kFmtBF16, kFmtBF16, false, true, 128, n_b > 0 ? n_b : 64);
+      const uint32_t idesc = idesc_f16(kFmtBF16, kFmtBF16, false, true, 128, slabs * 64);
       bool ok = true;
       for (int k = 0; k < nk; ++k) {
-        const int s = k % stages;
-        if (!mbar_wait(&bar->full[s], (k / stages) & 1, dev_status, abort_flag)) { ok = false; break; }
+        const int s = k % kPairStages;
+        if (!mbar_wait(&bar->full[s], (k / kPairStages) & 1, dev_status, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t aa = smem_u32(smem + s * stage_bytes), wa = aa + kRowBlocks * kABytes;
+        const uint32_t aa = smem_u32(smem + s * kStageBytes), wa = aa + 2 * kABytes;
         const int ksteps = min(kKC, K - k * kKC + 15) / 16;  // 16 contraction elements per MMA (zero filled past K)
         for (int kk = 0; kk < ksteps; ++kk) {
           const uint64_t wd = smem_desc_sw128(wa + kk * 2048, kSlab, 1024);
 #pragma unroll
-          for (int rb = 0; rb < kRowBlocks; ++rb) {
+          for (int rb = 0; rb < 2; ++rb) {
             const uint64_t ad = smem_desc_sw128(aa + rb * kABytes + kk * 32, 16, 1024);
-            mma_ss(tmem + rb * 256, ad, wd, idesc_a, k > 0 || kk > 0);
-            if (kRowBlocks == 1 && n_b > 0)
-              mma_ss(tmem + kFirst * 64, ad, smem_desc_sw128(wa + kFirst * kSlab + kk * 2048, kSlab, 1024), idesc_b, k > 0 || kk > 0);
+            mma_ss(tmem + rb * 256, ad, wd, idesc, k > 0 || kk > 0);
           }
         }
         mma_commit(&bar->empty[s]);
@@ -130,7 +157,7 @@ linear_rows_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
       // every load has been consumed: slab j of row block rb goes to smem + (rb * slabs + j) * 16 KB as
       // [128 rows][128 B], 128-byte swizzled; a warp's 32 rows are 4 KB of it
 #pragma unroll 1
-      for (int rb = 0; rb < kRowBlocks; ++rb) {
+      for (int rb = 0; rb < 2; ++rb) {
         const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + rb * 256;
         for (int j = 0; j < n_cols; j += 32) {
           uint32_t r[32];
@@ -138,7 +165,7 @@ linear_rows_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
           tmem_wait_ld();
           if (act == kActGelu) {
 #pragma unroll
-            for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(gelu(__uint_as_float(r[e])));
+            for (int e = 0; e < 32; e += 2) gelu2(r[e], r[e + 1]);
           }
           uint8_t* slab = smem + (rb * slabs + (j >> 6)) * (128 * 128);
 #pragma unroll
@@ -154,7 +181,7 @@ linear_rows_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
       fence_proxy_async();  // the staged rows are read by the TMA engine
       __syncwarp();
       if (lane == 0) {
-        for (int rb = 0; rb < kRowBlocks; ++rb) {
+        for (int rb = 0; rb < 2; ++rb) {
           const int row0 = m0 + rb * 128 + quarter * 32;
           if (row0 >= M) continue;  // rows past M and columns past N inside a box are clipped by the store
           for (int j = 0; j < slabs; ++j)
@@ -171,6 +198,185 @@ linear_rows_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
     tc_fence_after();
     tmem_dealloc(tmem, ncols);
   }
+}
+
+// ------------------------------------------------------------------------------------------------
+// Persistent form: one CTA per SM walks over tiles of 128 rows x kCols columns.  The ring runs on across tiles, and two
+// accumulators in tensor memory alternate, so that a tile's epilogue (eight warps: a GELU per element is as long as the
+// tile's MMAs at K = 640) runs under the next tile's loads and MMAs.  Against one tile per CTA, four epilogue warps and
+// nothing overlapped: 4096 x 2560 x 640 with GELU 34 -> 22 us, without 20.3 -> 15.9 us, 4096 x 640 x 2560
+// 20.5 -> 16.1 us, 8192 x 4096 x 1024 64 -> 53.9 us, 6144 x 640 x 640 8.1 -> 7.8 us (rows x columns x contraction).
+// ------------------------------------------------------------------------------------------------
+constexpr int kMaxStages = 6;
+constexpr int kEpiWarps = 8;
+
+struct PersistBars {
+  uint64_t full[kMaxStages], empty[kMaxStages];
+  uint64_t acc_full[2], acc_empty[2];
+  uint32_t tmem_base;
+  int abort_flag;
+};
+
+template <int kCols>
+struct PersistCfg {
+  static constexpr int kStageBytes = kABytes + kCols / 64 * kSlab;
+  static constexpr int kStages = kCols == 128 ? 6 : 4;
+  static constexpr int kStaging = kEpiWarps * 32 * 128;  // per epilogue warp: 32 rows of a 64-column slab
+  static constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kStaging + 256;
+  static constexpr uint32_t kAccCols = kCols == 128 ? 128 : 256;
+};
+
+template <int kCols>
+__global__ void __launch_bounds__((2 + kEpiWarps) * 32, 1)
+linear_persistent_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w0,
+                         const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__ CUtensorMap tm_w2,
+                         const __grid_constant__ CUtensorMap tm_c0, const __grid_constant__ CUtensorMap tm_c1,
+                         const __grid_constant__ CUtensorMap tm_c2, int M, int N, int K, int n_items, int act, uint32_t* dev_status) {
+  using C = PersistCfg<kCols>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* staging = smem + C::kStages * C::kStageBytes;
+  PersistBars* bar = reinterpret_cast<PersistBars*>(staging + C::kStaging);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nk = (K + kKC - 1) / kKC;
+  const int mb = (M + 127) / 128, nb = (N + kCols - 1) / kCols;
+  // item -> row block (fastest: CTAs that run together share W slabs), column block, matrix
+  auto m_of = [&](int item) { return item % mb * 128; };
+  auto n_of = [&](int item) { return item / mb % nb * kCols; };
+  auto z_of = [&](int item) { return item / mb / nb; };
+  auto slabs_at = [&](int n0) { return (min(kCols, N - n0) + 63) / 64; };
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < C::kStages; ++s) {
+      mbar_init(&bar->full[s], 1);
+      mbar_init(&bar->empty[s], 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(&bar->acc_full[a], 1);
+      mbar_init(&bar->acc_empty[a], kEpiWarps);
+    }
+    bar->abort_flag = 0;
+    mbar_fence_init();
+    prefetch_tmap(&tm_a);
+    prefetch_tmap(&tm_w0);
+    prefetch_tmap(&tm_c0);
+  }
+  dependency_wait();
+  if (threadIdx.x == 0) release_dependents();
+  if (warp == 1) tmem_alloc(&bar->tmem_base, 2 * C::kAccCols);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = bar->tmem_base;
+  volatile int* abort_flag = &bar->abort_flag;
+
+  if (warp == 0) {
+    if (elect_one()) {
+      int kc = 0;  // k-steps so far, over all items: ring slot and phase follow it
+      bool ok = true;
+      for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
+        const int m0 = m_of(item), n0 = n_of(item), z = z_of(item), slabs = slabs_at(n0);
+        const CUtensorMap* tm_w = z == 0 ? &tm_w0 : z == 1 ? &tm_w1 : &tm_w2;
+        for (int k = 0; k < nk; ++k, ++kc) {
+          const int s = kc % C::kStages;
+          if (kc >= C::kStages && !mbar_wait(&bar->empty[s], ((kc / C::kStages) - 1) & 1, dev_status, abort_flag)) { ok = false; break; }
+          uint8_t* sa = smem + s * C::kStageBytes;
+          mbar_expect_tx(&bar->full[s], kABytes + slabs * kSlab);
+          tma_load_2d(sa, &tm_a, &bar->full[s], k * kKC, m0);
+          for (int j = 0; j < slabs; ++j) tma_load_2d(sa + kABytes + j * kSlab, tm_w, &bar->full[s], n0 + j * 64, k * kKC);
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (elect_one()) {
+      int kc = 0, n = 0;
+      bool ok = true;
+      for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++n) {
+        const int a = n & 1;
+        if (n >= 2 && !mbar_wait(&bar->acc_empty[a], ((n >> 1) - 1) & 1, dev_status, abort_flag)) break;
+        tc_fence_after();
+        const uint32_t t_acc = tmem + a * C::kAccCols;
+        const uint32_t idesc = idesc_f16(kFmtBF16, kFmtBF16, false, true, 128, slabs_at(n_of(item)) * 64);
+        for (int k = 0; k < nk; ++k, ++kc) {
+          const int s = kc % C::kStages;
+          if (!mbar_wait(&bar->full[s], (kc / C::kStages) & 1, dev_status, abort_flag)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t aa = smem_u32(smem + s * C::kStageBytes), wa = aa + kABytes;
+          const int ksteps = min(kKC, K - k * kKC + 15) / 16;  // 16 contraction elements per MMA (zero filled past K)
+          for (int kk = 0; kk < ksteps; ++kk)
+            mma_ss(t_acc, smem_desc_sw128(aa + kk * 32, 16, 1024), smem_desc_sw128(wa + kk * 2048, kSlab, 1024), idesc, k > 0 || kk > 0);
+          mma_commit(&bar->empty[s]);
+        }
+        if (!ok) break;
+        mma_commit(&bar->acc_full[a]);
+      }
+    }
+  } else {
+    // two warps per quarter of the rows, each with every second 64-column slab
+    const int quarter = warp & 3, half = (warp - 2) >> 2;
+    uint8_t* mine = staging + (warp - 2) * 4096;
+    int n = 0;
+    for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++n) {
+      const int a = n & 1, m0 = m_of(item) + quarter * 32, n0 = n_of(item), z = z_of(item), slabs = slabs_at(n0);
+      const CUtensorMap* tm_c = z == 0 ? &tm_c0 : z == 1 ? &tm_c1 : &tm_c2;
+      // one answer per warp: the tensor-memory loads below are warp-wide operations
+      if (!__all_sync(0xffffffffu, mbar_wait(&bar->acc_full[a], (n >> 1) & 1, dev_status, abort_flag))) break;
+      tc_fence_after();
+      const uint32_t taddr = tmem + a * C::kAccCols + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll 1
+      for (int j = half; j < slabs; j += 2) {
+        if (lane == 0) tma_store_wait_read();  // the slab staged before has been read
+        __syncwarp();
+#pragma unroll 1
+        for (int c = 0; c < 64; c += 32) {
+          uint32_t r[32];
+          tmem_ld32(taddr + j * 64 + c, r);
+          tmem_wait_ld();
+          if (act == kActGelu) {
+#pragma unroll
+            for (int e = 0; e < 32; e += 2) gelu2(r[e], r[e + 1]);
+          }
+#pragma unroll
+          for (int e = 0; e < 32; e += 8) {
+            __align__(16) __nv_bfloat162 q[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              q[u] = __floats2bfloat162_rn(__uint_as_float(r[e + 2 * u]), __uint_as_float(r[e + 2 * u + 1]));
+            *reinterpret_cast<uint4*>(mine + sw128_offset(lane, (c + e) >> 3)) = *reinterpret_cast<const uint4*>(q);
+          }
+        }
+        fence_proxy_async();  // the staged rows are read by the TMA engine
+        __syncwarp();
+        if (lane == 0 && m0 < M) {  // rows past M and columns past N inside a box are clipped by the store
+          tma_store_2d(tm_c, mine, n0 + j * 64, m0);
+          tma_store_commit();
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar->acc_empty[a]);
+    }
+    if (lane == 0) tma_store_wait_read();  // shared memory must outlive the engine's reads
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, 2 * C::kAccCols);
+  }
+}
+
+template <int kCols>
+cudaError_t run_persistent(int M, int N, int K, int n_mats, const CUtensorMap& ta, const CUtensorMap (&tw)[3], const CUtensorMap (&tc)[3], int act,
+                           uint32_t* dev_status, cudaStream_t s) {
+  using C = PersistCfg<kCols>;
+  static std::atomic<unsigned long long> raised{0};
+  if (cudaError_t e = raise_dynamic_smem(linear_persistent_kernel<kCols>, C::kSmemBytes, raised); e != cudaSuccess) return e;
+  const long long items = (long long)((M + 127) / 128) * ((N + kCols - 1) / kCols) * n_mats;
+  if (items > INT32_MAX / 2) return cudaErrorInvalidValue;
+  const int grid = items < sm_count() ? (int)items : sm_count();
+  return launch_dependent(linear_persistent_kernel<kCols>, dim3(grid), dim3((2 + kEpiWarps) * 32), (size_t)C::kSmemBytes, s, ta, tw[0], tw[1], tw[2],
+                          tc[0], tc[1], tc[2], M, N, K, (int)items, act, dev_status);
 }
 
 }  // namespace
@@ -195,57 +401,35 @@ cudaError_t launch_linear_tc(int M, int N, int K, const void* a, const void* con
     if (!encode_tmap_16bit(&tw[i], w[j], 2, wdims, wstr, wbox) || !encode_tmap_16bit(&tc_[i], c[j], 2, cdims, wstr, cbox))
       return cudaErrorInvalidValue;
   }
-  // Tile form: the one with the least serial work per SM, counted as CTAs per SM (rounded up) times the
-  // multiply-adds of a tile, the 256 x 256 form credited with the 1.3x it gains from moving fewer operand
-  // bytes per multiply-add (timed on eleven shapes from 4096 x 640 x 640 to 16384 x 8192 x 4096; the
-  // model picks the faster form on each).  The 128 x 256 form keeps two CTAs per SM resident and is only
-  // considered while its grid fits them.
+  // Tile form: the one with the least serial work per SM, i.e. tiles per SM (rounded up) times the time of one, which was
+  // timed on fourteen shapes between 200 x 640 x 640 and 32768 x 2560 x 640: a tile of 128 x 192 takes 1.2 times, one of
+  // 128 x 256 1.35 times as long as one of 128 x 128 (they read fewer operand bytes per multiply-add, and L2's rate is
+  // what bounds these shapes), one of 256 x 256 2.5 times - 4 % less than two of 128 x 256 from about 2048 contraction
+  // elements on, more below, where its epilogue shows.
   const int sms = sm_count();
-  const int mb = (M + 127) / 128;
-  const long long ctas320 = (long long)mb * ((N + 319) / 320) * n_mats, ctas256 = (long long)mb * ((N + 255) / 256) * n_mats;
-  const long long ctas_pair = (long long)((M + 255) / 256) * ((N + 255) / 256) * n_mats;
-  const long long cost320 = ((ctas320 + sms - 1) / sms) * (128 * 320) * 13;
-  const long long cost256 = ctas256 <= 2 * sms ? ((ctas256 + sms - 1) / sms) * (128 * 256) * 13 : cost320 + 1;
-  const long long cost_pair = M > 128 ? ((ctas_pair + sms - 1) / sms) * (256 * 256) * 10 : cost320 + 1;
-  // 128 x 128 tiles, two CTAs per SM sharing its tensor pipe: serial work = CTAs per SM (rounded up) tiles
-  const long long ctas128 = (long long)mb * ((N + 127) / 128) * n_mats;
-  const long long cost128 = ctas128 <= 2 * sms ? ((ctas128 + sms - 1) / sms) * (128 * 128) * 13 : cost320 + 1;
-  // ties go to the form with more, smaller CTAs (more SMs take in operands at once)
-  bool small = cost128 <= cost256 && cost128 <= cost_pair && cost128 < cost320;
-  bool narrow = !small && cost256 <= cost_pair && cost256 < cost320;
-  int pair = !small && !narrow && cost_pair < cost320;
-  if (const int v = g_tune_linear_tile.load(std::memory_order_relaxed)) {  // test-only override: 128 x 256 (1), 128 x 320 (2), 256 x 256 (3) or 128 x 128 (4) tiles
-    pair = v == 3 && M > 128;
-    narrow = v == 1;
-    small = v == 4;
+  auto cost = [&](int rows, int cols, int tile) {
+    const long long tiles = (long long)((M + rows - 1) / rows) * ((N + cols - 1) / cols) * n_mats;
+    return (tiles + sms - 1) / sms * tile;
+  };
+  const long long cost128 = cost(128, 128, 20), cost192 = cost(128, 192, 24), cost256 = cost(128, 256, 27);
+  const long long cost_pair = M > 128 && K >= 2048 ? cost(kPairRows, kPairCols, 50) : LLONG_MAX;
+  int form = cost128 <= cost192 && cost128 <= cost256 ? 4 : cost192 <= cost256 ? 2 : 1;
+  if (cost_pair < cost128 && cost_pair < cost192 && cost_pair < cost256) form = 3;
+  // test-only override: 128 x 256 (1), 128 x 192 (2), 256 x 256 (3) or 128 x 128 (4) tiles
+  if (const int v = g_tune_linear_tile.load(std::memory_order_relaxed); v && (v != 3 || M > 128)) form = v;
+  cudaError_t e;
+  if (form == 3) {
+    constexpr int smem = 1024 + kPairStages * (2 * kABytes + kPairCols / 64 * kSlab) + 256;
+    static std::atomic<unsigned long long> raised{0};
+    if (e = raise_dynamic_smem(linear_pair_kernel, smem, raised); e != cudaSuccess) return e;
+    const dim3 grid((M + kPairRows - 1) / kPairRows, (N + kPairCols - 1) / kPairCols, n_mats);
+    e = launch_dependent(linear_pair_kernel, grid, dim3(192), (size_t)smem, s, ta, tw[0], tw[1], tw[2], tc_[0], tc_[1], tc_[2], M, N, K, act,
+                         dev_status);
+  } else {
+    e = form == 4   ? run_persistent<128>(M, N, K, n_mats, ta, tw, tc_, act, dev_status, s)
+        : form == 2 ? run_persistent<192>(M, N, K, n_mats, ta, tw, tc_, act, dev_status, s)
+                    : run_persistent<256>(M, N, K, n_mats, ta, tw, tc_, act, dev_status, s);
   }
-  const int cols = small ? 128 : (narrow || pair) ? 256 : 320;
-  const int slabs = ((N < cols ? N : cols) + 63) / 64;
-  const int stage_bytes = (pair ? 2 : 1) * kABytes + slabs * kSlab;
-  int stages = (((narrow && !pair) || small ? 110 : 222) * 1024) / stage_bytes;
-  stages = stages > 4 ? 4 : stages < 1 ? 1 : stages;
-  const int nk = (K + kKC - 1) / kKC;
-  if (stages > nk) stages = nk;
-  const int staging = (pair ? 2 : 1) * slabs * 128 * 128;  // the output tile, staged where the ring was
-  const int ring_bytes = stages * stage_bytes > staging ? stages * stage_bytes : staging;
-  const int smem = 1024 + ring_bytes + 256;
-  {
-    static std::atomic<unsigned long long> r320{0}, r256{0}, rpair{0}, r128{0};
-    cudaError_t e = raise_dynamic_smem(linear_rows_kernel<320>, 227 * 1024, r320);
-    if (e == cudaSuccess) e = raise_dynamic_smem(linear_rows_kernel<128>, 227 * 1024, r128);
-    if (e == cudaSuccess) e = raise_dynamic_smem(linear_rows_kernel<256>, 227 * 1024, r256);
-    if (e == cudaSuccess) e = raise_dynamic_smem(linear_rows_kernel<256, 2>, 227 * 1024, rpair);
-    if (e != cudaSuccess) return e;
-  }
-  dim3 grid(pair ? (M + 255) / 256 : mb, (N + cols - 1) / cols, n_mats);
-  cudaError_t e = pair ? launch_dependent(linear_rows_kernel<256, 2>, grid, dim3(192), (size_t)smem, s, ta, tw[0], tw[1], tw[2], tc_[0], tc_[1],
-                                          tc_[2], M, N, K, stages, ring_bytes, act, dev_status)
-                  : small ? launch_dependent(linear_rows_kernel<128>, grid, dim3(192), (size_t)smem, s, ta, tw[0], tw[1], tw[2], tc_[0], tc_[1],
-                                            tc_[2], M, N, K, stages, ring_bytes, act, dev_status)
-                  : narrow ? launch_dependent(linear_rows_kernel<256>, grid, dim3(192), (size_t)smem, s, ta, tw[0], tw[1], tw[2], tc_[0], tc_[1],
-                                            tc_[2], M, N, K, stages, ring_bytes, act, dev_status)
-                         : launch_dependent(linear_rows_kernel<320>, grid, dim3(192), (size_t)smem, s, ta, tw[0], tw[1], tw[2], tc_[0], tc_[1],
-                                            tc_[2], M, N, K, stages, ring_bytes, act, dev_status);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -710,6 +710,25 @@ def test_linear_every_tile_form(toma, tuning, tile, m, n, k):
     assert_close(to_host64(c), O.linear(a_host, w_host), "bf16", f"linear, tile form {tile}")
 
 
+@pytest.mark.parametrize("tile", [0, 1, 3], ids=["128x256", "128x192", "128x128"])
+@pytest.mark.parametrize("m,n,k", [(9000, 1016, 72), (20000, 64, 200)])
+def test_linear_several_tiles_per_cta(toma, tuning, tile, m, n, k):
+    """More tiles than SMs: a CTA's ring and accumulators run on across tiles, the last of a row block ragged in both
+    directions, with fewer and with more tiles than accumulators per CTA."""
+    tuning(linear_tile=tile + 1)
+    rng = np.random.default_rng(m)
+    a = torch.from_numpy(rng.standard_normal((m, k)).astype(np.float32)).cuda().to(torch.bfloat16)
+    w = torch.from_numpy((rng.standard_normal((k, n)) / np.sqrt(k)).astype(np.float32)).cuda().to(torch.bfloat16)
+    c = torch.full((m, n), float("nan"), dtype=a.dtype, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    toma.toma_linear(a, w, c, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    rows = np.unique(np.concatenate([[0, 127, 128, m - 1], rng.choice(m, size=300, replace=False)]))
+    assert not torch.isnan(c).any()
+    assert_close(to_host64(c)[rows], O.linear(to_host64(a)[rows], to_host64(w)), "bf16", "linear")
+
+
 def _proj_weights(cfg, seed=93):
     """Four [d, d] projection matrices N(0, 1/d), rounded to the storage dtype."""
     d = cfg.dim
