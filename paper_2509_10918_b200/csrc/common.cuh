@@ -155,4 +155,11 @@ __device__ __forceinline__ int tile_token(int p, int l, int tiles_x, int th, int
   return (ty * th + ly) * W + tx * tw + lx;
 }
 
+// 32 bytes to a 32-byte aligned address: a thread that writes a row of its own fills whole sectors.
+__device__ __forceinline__ void st_global_32(void* p, const uint32_t (&v)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]),
+               "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+
 }  // namespace toma

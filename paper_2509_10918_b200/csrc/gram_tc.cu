@@ -16,29 +16,29 @@ using namespace tc;
 namespace {
 
 constexpr int kKC = 64;  // channels per stage
-constexpr int kStages = 4;
+constexpr int kMaxStages = 4;
 
 struct GramBars {
-  uint64_t full[kStages], empty[kStages], done;
+  uint64_t full[kMaxStages], empty[kMaxStages], done;
   uint32_t tmem_base;
   int abort_flag;
 };
 
 __global__ void __launch_bounds__(192, 1)
 gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
-               uint16_t* __restrict__ sq, int Nloc, int d, int n_cols, uint32_t* dev_status) {
+               uint16_t* __restrict__ sq, int Nloc, int d, int n_cols, int stages, uint32_t* dev_status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int a_bytes = 128 * 128, b_bytes = n_cols * 128;
   const int stage_bytes = a_bytes + b_bytes;
-  GramBars* bar = reinterpret_cast<GramBars*>(smem + kStages * stage_bytes);
+  GramBars* bar = reinterpret_cast<GramBars*>(smem + stages * stage_bytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tile = blockIdx.x, m0 = blockIdx.y * 128, n0 = blockIdx.z * n_cols;
   const int nk = (d + kKC - 1) / kKC;
   const uint32_t ncols = n_cols > 128 ? 256u : n_cols > 64 ? 128u : n_cols > 32 ? 64u : 32u;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < stages; ++s) {
       mbar_init(&bar->full[s], 1);
       mbar_init(&bar->empty[s], 1);
     }
@@ -60,8 +60,8 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   if (warp == 0) {
     if (elect_one()) {
       for (int k = 0; k < nk; ++k) {
-        const int s = k % kStages;
-        if (k >= kStages && !mbar_wait(&bar->empty[s], ((k / kStages) - 1) & 1, dev_status, abort_flag)) break;
+        const int s = k % stages;
+        if (k >= stages && !mbar_wait(&bar->empty[s], ((k / stages) - 1) & 1, dev_status, abort_flag)) break;
         uint8_t* sa = smem + s * stage_bytes;
         mbar_expect_tx(&bar->full[s], stage_bytes);
         tma_load_3d(sa, &tm_a, &bar->full[s], k * kKC, m0, tile);
@@ -73,8 +73,8 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       const uint32_t idesc = idesc_f16(kFmtBF16, kFmtBF16, false, false, 128, n_cols);
       bool ok = true;
       for (int k = 0; k < nk; ++k) {
-        const int s = k % kStages;
-        if (!mbar_wait(&bar->full[s], (k / kStages) & 1, dev_status, abort_flag)) { ok = false; break; }
+        const int s = k % stages;
+        if (!mbar_wait(&bar->full[s], (k / stages) & 1, dev_status, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t aa = smem_u32(smem + s * stage_bytes), ba = aa + a_bytes;
 #pragma unroll
@@ -92,6 +92,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     if (mbar_wait(&bar->done, 0, dev_status, abort_flag)) {
       tc_fence_after();
       const int pitch = sq_pitch(Nloc);
+      const bool wide = pitch % 16 == 0;
       uint16_t* row = sq + ((size_t)tile * Nloc + (i < Nloc ? i : 0)) * pitch + n0;
       for (int j0 = 0; j0 < n_cols; j0 += 32) {
         uint32_t r[32];
@@ -99,11 +100,11 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         tmem_wait_ld();
         if (i < Nloc) {
 #pragma unroll
-          for (int e = 0; e < 32; e += 8) {
+          for (int e = 0; e < 32; e += 16) {
             if (j0 + e >= n_cols || n0 + j0 + e >= pitch) break;
-            uint32_t pk[4];
+            uint32_t pk[8];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < 8; ++u) {
               const int ja = n0 + j0 + e + 2 * u;
               int lo = __float2int_rn(__uint_as_float(r[e + 2 * u]) * 4096.f) + kSqBias;
               int hi = __float2int_rn(__uint_as_float(r[e + 2 * u + 1]) * 4096.f) + kSqBias;
@@ -113,7 +114,13 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
               if (ja + 1 >= Nloc) hi = 0;
               pk[u] = ((uint32_t)hi << 16) | (uint32_t)lo;
             }
-            *reinterpret_cast<uint4*>(row + j0 + e) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            if (wide) {
+              st_global_32(row + j0 + e, pk);
+            } else {
+              *reinterpret_cast<uint4*>(row + j0 + e) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+              if (j0 + e + 8 < n_cols && n0 + j0 + e + 8 < pitch)
+                *reinterpret_cast<uint4*>(row + j0 + e + 8) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+            }
           }
         }
       }
@@ -138,11 +145,15 @@ cudaError_t launch_gram_tc(const Geom& g, const __nv_bfloat16* y, uint16_t* sq, 
   const uint32_t box_b[3] = {64, (uint32_t)n_cols, 1};
   if (!encode_tmap_16bit(&ta, y, 3, dims, strides, box_a) || !encode_tmap_16bit(&tb, y, 3, dims, strides, box_b))
     return cudaErrorInvalidValue;
-  const int smem = 1024 + kStages * (128 * 128 + n_cols * 128) + 256;
+  // One wave of CTAs: a deep ring.  More than one: rings of two stages, so that two CTAs of 256 columns fit an SM and one
+  // multiplies while the other converts and stores (64 tiles of 1024 tokens, 640 channels: 127 -> 101 us).
+  const long long ctas = (long long)g.B * g.P * ((g.Nloc + 127) / 128) * ((g.Nloc + n_cols - 1) / n_cols);
+  const int stages = ctas <= sm_count() ? kMaxStages : 2;
+  const int smem = 1024 + stages * (128 * 128 + n_cols * 128) + 256;
   static std::atomic<unsigned long long> smem_raised{0};
   if (cudaError_t e = raise_dynamic_smem(gram_tc_kernel, 200 * 1024, smem_raised); e != cudaSuccess) return e;
   dim3 grid(g.B * g.P, (g.Nloc + 127) / 128, (g.Nloc + n_cols - 1) / n_cols);
-  const cudaError_t le = launch_dependent(gram_tc_kernel, grid, dim3(192), (size_t)smem, s, ta, tb, sq, g.Nloc, g.d, n_cols, dev_status);
+  const cudaError_t le = launch_dependent(gram_tc_kernel, grid, dim3(192), (size_t)smem, s, ta, tb, sq, g.Nloc, g.d, n_cols, stages, dev_status);
   count_launch();
   return le != cudaSuccess ? le : cudaGetLastError();
 }

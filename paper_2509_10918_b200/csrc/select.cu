@@ -211,6 +211,13 @@ static cudaError_t run_greedy(const Geom& g, const uint16_t* sq, int32_t* idx, c
   if (kSmem)
     if (cudaError_t e = raise_dynamic_smem(greedy_kernel<kOne, kSmem>, kOne ? 64 * 64 * 2 : kGreedySmemTok * kGreedySmemTok * 2, raised); e != cudaSuccess)
       return e;
+  // Rows in global memory: not launched before its predecessor ends.  CTAs placed then are spread over the chip, those
+  // placed beside the predecessor's last ones crowd where there is room first, and share the paths to L2 that bound the
+  // rounds (64 tiles of 1024 tokens: 600 us against 543 us).
+  if (!kSmem) {
+    greedy_kernel<kOne, kSmem><<<g.B * g.P, kGreedyThreads, smem, s>>>(sq, idx, g.Nloc, g.Dloc);
+    return cudaGetLastError();
+  }
   return launch_dependent(greedy_kernel<kOne, kSmem>, dim3(g.B * g.P), dim3(kGreedyThreads), smem, s, sq, idx, g.Nloc, g.Dloc);
 }
 
