@@ -411,10 +411,10 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
       }
     }
     asm volatile("bar.sync 1, %0;" ::"n"(128 * kMB) : "memory");
-    if (ok && valid) {
+    if (ok && quarter * 32 < p.m_tok) {  // whole warps: tensor-memory loads are warp-wide, whoever has a row to write
       // pass 4: A~_ik = A_ik / Z_i, written as row k of A~^T [N_loc][D_loc], hi plane then lo plane
       const size_t plane = (size_t)p.Nloc * Dl;
-      const size_t row = (size_t)((mb + half) * p.m_tok + k_loc) * Dl;
+      const size_t row = (size_t)((mb + half) * p.m_tok + (valid ? k_loc : 0)) * Dl;
       __nv_bfloat16* t_hi = w + (size_t)batch * 2 * plane + row;
       __nv_bfloat16* u_hi = wu ? wu + (size_t)batch * 2 * plane + row : nullptr;
       for (int i0 = 0; i0 < Dl; i0 += 32) {
@@ -423,7 +423,7 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         tmem_wait_ld();
 #pragma unroll
         for (int e0 = 0; e0 < 32; e0 += 8) {
-          if (i0 + e0 >= Dl) break;  // D_loc is a multiple of 8
+          if (!valid || i0 + e0 >= Dl) break;  // D_loc is a multiple of 8
           __align__(16) __nv_bfloat16 hi[8], lo[8], uh[8], ul[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e) {

@@ -1157,6 +1157,13 @@ def test_regions_of_any_shape_parity(toma, th, tw, ratio, dim, heads, unmerge):
         assert np.array_equal(unmerged[b, cfg.n_tokens:], y_host[b, cfg.n_tiles * d_loc:])
 
 
+@pytest.mark.parametrize("th,tw,ratio", [(8, 6, 0.5), (4, 4, 0.5), (5, 8, 0.4), (10, 12, 0.6), (7, 8, 0.0)])
+def test_tiles_of_partial_warps_parity(toma, th, tw, ratio):
+    """Tiles whose token count is a multiple of 8 but not of 32, with D_loc a multiple of 8: the last warp of source tokens
+    of the weights kernel is only partly filled."""
+    test_regions_of_any_shape_parity(toma, th, tw, ratio, 64, 1, "shares")
+
+
 @pytest.mark.parametrize("gh,gw,th,tw,ratio", [(18, 28, 9, 14, 0.5), (30, 42, 10, 21, 0.5), (15, 26, 15, 13, 0.43)])
 def test_global_merge_of_ragged_images_parity(toma, gh, gw, th, tw, ratio):
     """The image as one region of any shape: the same kernels with up to 630 destinations, which is past the 512 of a block."""
