@@ -10,9 +10,11 @@
 //     TMA stride.  They are gathered instead: eight warps read the aligned 16-byte packets that cover eight weights,
 //     shift them into place and write the 128-byte-swizzled operand tile; the same warps are the epilogue later.
 // The weights are the A operand of both (destinations on M for the merge, MN-major; tokens on M for the unmerge,
-// K-major), the tokens / attended rows the MN-major B operand with 128 or 256 channels: a weight block is then
-// gathered once per 128 or 256 channels, and every thread of the epilogue holds one output row.
+// K-major), the tokens / attended rows the MN-major B operand with up to 320 channels: a weight block is then
+// gathered once per 320 channels, and every thread of the epilogue holds one output row.
 // Per CTA: warp 0 TMA, warp 1 MMA, warps 2..9 gather and epilogue.
+#include <climits>
+
 #include "common.cuh"
 #include "tc.cuh"
 
@@ -34,7 +36,7 @@ struct RgBars {
 struct RgParams {
   int P, tiles_x, th, tw, Nloc, Dloc, d;
   int rows;        // tile rows of a full box
-  int nch;         // channels per CTA (a multiple of 64, at most 256)
+  int nch;         // channels per CTA (a multiple of 64, at most 320)
   int stages;
   int kc;          // contraction rows of a stage (64 or 128; unmerge: 64)
   const __nv_bfloat16* w;
@@ -62,30 +64,28 @@ __device__ __forceinline__ void funnel8(const uint4& lo, const uint4& hi, uint32
   }
 }
 
-// One weight block into its swizzled operand tile(s): kRows rows starting at plane row `row0` (rows >= n_rows become
-// 0), kChunks groups of eight columns starting at `col0` (columns >= D_loc become 0), both planes.  Slab s holds
-// columns 64 s .. 64 s + 63; `slab_bytes` apart, planes `plane_bytes` apart.
+// One weight block into its swizzled operand tile(s): `rows_total` rows starting at plane row `row0` (rows >= n_rows
+// become 0), kChunks groups of eight columns starting at `col0` (columns >= D_loc become 0), both planes.  Slab s holds
+// columns 64 s .. 64 s + 63; `slab_bytes` apart, planes `plane_bytes` apart.  In two halves, so that a block's packets
+// are in flight while the block before waits for its buffer: load() takes four of the thread's rows, store() writes them.
 template <int kChunks>
-__device__ __forceinline__ void gather_block(const RgParams& p, const uint8_t* plane0, int t, int rows_total, int row0, int n_rows, int col0,
-                                             uint8_t* dst, int slab_bytes, int plane_bytes) {
-  constexpr int kRowStep = kWorkers / kChunks;
-  const int ch = t % kChunks, r0 = t / kChunks;
-  const int n = min(8, p.Dloc - (col0 + ch * 8));
-  if (n <= 0) return;  // zero since the start
-  uint8_t* out = dst + (ch >> 3) * slab_bytes;
-  const size_t plane_stride = (size_t)p.Nloc * p.Dloc * 2;
-  const bool aligned = ((p.Dloc & 7) == 0);  // then every packet starts on 16 bytes
-  for (int rb = r0; rb < rows_total; rb += 4 * kRowStep) {
-    uint4 lo[2][4], hi[2][4];
-    uint32_t sh[2][4];
+struct Gather {
+  static constexpr int kRowStep = kWorkers / kChunks, kPass = 4 * kRowStep;  // rows between a thread's, rows of a pass
+  uint4 lo[2][4], hi[2][4];
+  uint32_t sh[2][4];
+
+  __device__ __forceinline__ void load(const RgParams& p, const uint8_t* plane0, int t, int first, int row0, int n_rows, int col0) {
+    const int ch = t % kChunks, n = min(8, p.Dloc - (col0 + ch * 8));
+    const size_t plane_stride = (size_t)p.Nloc * p.Dloc * 2;
+    const bool aligned = ((p.Dloc & 7) == 0);  // then every packet starts on 16 bytes
 #pragma unroll
     for (int pl = 0; pl < 2; ++pl)
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int row = rb + u * kRowStep;
+        const int row = first + t / kChunks + u * kRowStep;
         lo[pl][u] = hi[pl][u] = make_uint4(0u, 0u, 0u, 0u);
         sh[pl][u] = 0u;
-        if (row < n_rows) {
+        if (row < n_rows && n > 0) {
           const uint8_t* a = plane0 + pl * plane_stride + ((size_t)(row0 + row) * p.Dloc + col0 + ch * 8) * 2;
           const uint32_t s = (uint32_t)(reinterpret_cast<uintptr_t>(a) & 15);
           const uint4* q = reinterpret_cast<const uint4*>(a - s);
@@ -103,11 +103,17 @@ __device__ __forceinline__ void gather_block(const RgParams& p, const uint8_t* p
           }
         }
       }
+  }
+  __device__ __forceinline__ void store(const RgParams& p, int t, int first, int rows_total, int col0, uint8_t* dst, int slab_bytes,
+                                        int plane_bytes) const {
+    const int ch = t % kChunks, n = min(8, p.Dloc - (col0 + ch * 8));
+    if (n <= 0) return;  // zero since the start
+    uint8_t* out = dst + (ch >> 3) * slab_bytes;
 #pragma unroll
     for (int pl = 0; pl < 2; ++pl)
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int row = rb + u * kRowStep;
+        const int row = first + t / kChunks + u * kRowStep;
         if (row < rows_total) {
           uint32_t v[4];
           funnel8(lo[pl][u], hi[pl][u], sh[pl][u], n, v);
@@ -115,7 +121,7 @@ __device__ __forceinline__ void gather_block(const RgParams& p, const uint8_t* p
         }
       }
   }
-}
+};
 
 // Epilogue: this warp's 32 accumulator rows (tensor-memory lanes 32 (warp & 3) ..), columns [c_lo, c_hi), as bf16 into
 // the staged slabs [128 rows][64 channels], the layout of the output map's box.
@@ -158,7 +164,7 @@ ragged_kernel(const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ 
   const int stage_bytes = 2 * a_plane + (p.nch / 64) * b_slab;
   RgBars* bar = reinterpret_cast<RgBars*>(smem + p.stages * stage_bytes);
   const int nk = kMerge ? n_boxes : (p.Dloc + 63) / 64;
-  const uint32_t ncols = p.nch > 128 ? 256u : p.nch > 64 ? 128u : 64u;
+  const uint32_t ncols = p.nch > 256 ? 512u : p.nch > 128 ? 256u : p.nch > 64 ? 128u : 64u;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
@@ -209,7 +215,9 @@ ragged_kernel(const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ 
     }
   } else if (warp == 1) {
     if (elect_one()) {
-      const uint32_t idesc = idesc_f16(kFmtBF16, kFmtBF16, kMerge, true, 128, n_mma);
+      const int n_a = min(n_mma, 256), n_b = n_mma - n_a;
+      const uint32_t idesc_a = idesc_f16(kFmtBF16, kFmtBF16, kMerge, true, 128, n_a);
+      const uint32_t idesc_b = idesc_f16(kFmtBF16, kFmtBF16, kMerge, true, 128, n_b > 0 ? n_b : 64);
       bool ok = true;
       for (int k = 0; k < nk; ++k) {
         const int s = k % p.stages;
@@ -224,7 +232,8 @@ ragged_kernel(const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ 
           for (int pl = 0; pl < 2; ++pl) {
             const uint64_t ad = kMerge ? smem_desc_sw128(aa + pl * a_plane + kk * 2048, a_slab, 1024)
                                        : smem_desc_sw128(aa + pl * a_plane + kk * 32, 16, 1024);
-            mma_ss(tmem, ad, bd, idesc, k > 0 || kk > 0 || pl > 0);
+            mma_ss(tmem, ad, bd, idesc_a, k > 0 || kk > 0 || pl > 0);
+            if (n_b > 0) mma_ss(tmem + 256, ad, smem_desc_sw128(ba + 4 * b_slab + kk * 2048, b_slab, 1024), idesc_b, k > 0 || kk > 0 || pl > 0);
           }
         }
         mma_commit(&bar->empty[s]);
@@ -235,6 +244,15 @@ ragged_kernel(const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ 
     const int t = threadIdx.x - 64;
     const uint8_t* plane0 = reinterpret_cast<const uint8_t*>(p.w) + (size_t)batch * 2 * p.Nloc * p.Dloc * 2;
     const int box_tok = p.rows * p.tw;
+    // block k of the weights: its first row, rows, padded rows and first column
+    const int m_len = (mb == n_boxes - 1 ? tail_rows : p.rows) * p.tw;
+    auto row0_of = [&](int k) { return kMerge ? k * box_tok : mb * box_tok; };
+    auto rows_of = [&](int k) { return kMerge ? (k == n_boxes - 1 ? tail_rows : p.rows) * p.tw : m_len; };
+    auto col0_of = [&](int k) { return kMerge ? mb * 128 : k * 64; };
+    const int rows_total = kMerge ? (box_tok + 15) & ~15 : m_len;
+    Gather<kMerge ? 16 : 8> gather;
+    constexpr int kPass = Gather<kMerge ? 16 : 8>::kPass;
+    gather.load(p, plane0, t, 0, row0_of(0), rows_of(0), col0_of(0));
     bool ok = true;
     for (int k = 0; k < nk; ++k) {
       const int s = k % p.stages;
@@ -242,12 +260,13 @@ ragged_kernel(const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ 
       if (k >= p.stages) ok = __all_sync(0xffffffffu, mbar_wait(&bar->empty[s], ((k / p.stages) - 1) & 1, dev_status, abort_flag));
       if (!ok) break;
       uint8_t* sa = smem + s * stage_bytes;
-      if (kMerge) {
-        const int len = (k == n_boxes - 1 ? tail_rows : p.rows) * p.tw;
-        gather_block<16>(p, plane0, t, (box_tok + 15) & ~15, k * box_tok, len, mb * 128, sa, a_slab, a_plane);
-      } else {
-        const int len = (mb == n_boxes - 1 ? tail_rows : p.rows) * p.tw;
-        gather_block<8>(p, plane0, t, len, mb * box_tok, len, k * 64, sa, a_slab, a_plane);
+      gather.store(p, t, 0, rows_total, col0_of(k), sa, a_slab, a_plane);
+      for (int first = kPass; first < rows_total; first += kPass) {
+        gather.load(p, plane0, t, first, row0_of(k), rows_of(k), col0_of(k));
+        gather.store(p, t, first, rows_total, col0_of(k), sa, a_slab, a_plane);
+      }
+      if (k + 1 < nk) gather.load(p, plane0, t, 0, row0_of(k + 1), rows_of(k + 1), col0_of(k + 1));
+      if (!kMerge) {
         if (k == nk - 1 && k >= p.stages) {  // columns past D_loc still hold an earlier block's weights
           const int first = (p.Dloc - k * 64 + 7) / 8, last = ((p.Dloc - k * 64 + 15) / 16) * 2;
           for (int e = t; e < (last - first) * 256; e += kWorkers) {
@@ -313,10 +332,17 @@ cudaError_t launch_ragged(const Geom& g, const void* w, const void* in, void* ou
   p.rows = box_max / g.tw < g.th ? box_max / g.tw : g.th;
   const int n_boxes = (g.th + p.rows - 1) / p.rows, tail = g.th - (n_boxes - 1) * p.rows;
   const int m_blocks = kMerge ? (g.Dloc + 127) / 128 : n_boxes;
-  // 256 channels per CTA halve how often the weights are gathered; 128 where that would leave SMs without a CTA
-  const long long wide = (long long)g.B * g.P * m_blocks * ((g.d + 255) / 256);
-  p.nch = g.d > 128 && wide >= sm_count() ? 256 : 128;
-  if (g.d <= 64) p.nch = 64;
+  // Channels per CTA: the fewer CTAs per SM (rounded up) the better, then the fewer channels - a CTA's time is that of
+  // gathering its weights, about what 600 channels' multiplications take, plus that of its channels (timed with 64 to 320
+  // channels on nine shapes: one wave of 320 takes 42 us where one of 192 takes 35; 2 x 4032 tokens in regions of 18 x 14,
+  // 640 channels: merge 22.0 -> 13.3 us, unmerge 17.9 -> 9.9 us against 128 and 256 channels without the prefetch).
+  long long best = LLONG_MAX;
+  for (int nch = 64; nch <= 320; nch += 64) {
+    if (nch > 64 && nch - 64 >= g.d) break;
+    const long long ctas = (long long)g.B * g.P * m_blocks * ((g.d + nch - 1) / nch);
+    const long long cost = (ctas + sm_count() - 1) / sm_count() * (600 + nch);
+    if (cost < best) best = cost, p.nch = nch;
+  }
   p.w = (const __nv_bfloat16*)w;
   p.w_end = (const uint8_t*)w + (size_t)g.B * g.P * g.Nloc * g.Dloc * 4;
   p.zero = (uint32_t*)zero;
@@ -331,8 +357,7 @@ cudaError_t launch_ragged(const Geom& g, const void* w, const void* in, void* ou
   const int a_plane = kMerge ? 2 * p.kc * 128 : 128 * 128;
   const int stage_bytes = 2 * a_plane + (p.nch / 64) * p.kc * 128;
   const int nk = kMerge ? n_boxes : (g.Dloc + 63) / 64;
-  // two stages of the narrow form leave room for a second CTA on the SM; the wide form runs alone
-  p.stages = p.nch > 128 || p.kc > 64 ? (220 * 1024) / stage_bytes : 2;
+  p.stages = (220 * 1024) / stage_bytes;
   p.stages = p.stages > 3 ? 3 : p.stages;
   if (p.stages > nk) p.stages = nk;
   int ring = p.stages * stage_bytes;
