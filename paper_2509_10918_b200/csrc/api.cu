@@ -139,7 +139,7 @@ static cudaError_t do_merge(const Geom& g_sel, const void* w, const void* x, voi
     cudaError_t e = linear_tc_supported(g) ? launch_merge_tc(g, w, x, xm, zero, zero_bytes, dev_status, s)
                                            : launch_merge_ragged(g, w, x, xm, zero, zero_bytes, dev_status, s);
     if (zeroed) *zeroed = e == cudaSuccess && zero_bytes > 0;
-    return e != cudaSuccess ? e : launch_copy_extra(g, x, xm, true, s);
+    return e;
   }
   return launch_merge_simt(g, w, x, xm, s);
 }
@@ -150,7 +150,7 @@ static cudaError_t do_unmerge(const Geom& g_sel, const void* w, const void* y, v
   w = unmerge_matrix(g_sel, w);
   if (linear_tc_supported(g) || ragged_tc_supported(g)) {
     cudaError_t e = linear_tc_supported(g) ? launch_unmerge_tc(g, w, y, out, dev_status, s) : launch_unmerge_ragged(g, w, y, out, dev_status, s);
-    return e != cudaSuccess ? e : launch_copy_extra(g, y, out, false, s);
+    return e;
   }
   return launch_unmerge_simt(g, w, y, out, s);
 }

@@ -99,7 +99,6 @@ bool ragged_tc_supported(const Geom& g);
 cudaError_t launch_merge_ragged(const Geom& g, const void* w, const void* x, void* xm, void* zero, size_t zero_bytes, uint32_t* dev_status,
                                 cudaStream_t s);
 cudaError_t launch_unmerge_ragged(const Geom& g, const void* w, const void* y, void* out, uint32_t* dev_status, cudaStream_t s);
-cudaError_t launch_copy_extra(const Geom& g, const void* src, void* dst, bool merging, cudaStream_t s);
 // Scratch of the tensor-core attention (tickets and partial results of split work units).
 size_t attention_tc_workspace_bytes(int B, int L, int heads, int dh);
 // The scratch starts with the tickets (attention_tc_ticket_bytes()), which must be zero when the
@@ -153,6 +152,36 @@ __device__ __forceinline__ int tile_token(int p, int l, int tiles_x, int th, int
   const int ty = p / tiles_x, tx = p - ty * tiles_x;
   const int ly = l / tw, lx = l - ly * tw;
   return (ty * th + ly) * W + tx * tw + lx;
+}
+
+// Rows that pass a merge or an unmerge unchanged (a sequence's text tokens), copied by warps that wait for their
+// first product anyway: `per` 16-byte packets in each of `batches` batch items.
+struct RowCopy {
+  const uint4* src = nullptr;
+  uint4* dst = nullptr;
+  size_t src_stride = 0, dst_stride = 0;
+  int per = 0, batches = 0;
+};
+__device__ __forceinline__ void copy_part(const RowCopy& c, int thread, int n_threads) {
+  for (int b = 0; b < c.batches; ++b) {
+    const uint4* src = c.src + b * c.src_stride;
+    uint4* dst = c.dst + b * c.dst_stride;
+#pragma unroll 4
+    for (int e = thread; e < c.per; e += n_threads) dst[e] = src[e];
+  }
+}
+// bf16, d a multiple of 8: the un-merged trailing tokens of x -> merged rows (merging) or of attended rows -> output.
+inline RowCopy extra_rows(const Geom& g, const void* src, void* dst, bool merging) {
+  RowCopy c;
+  if (g.n_extra == 0) return c;
+  const size_t full = (size_t)g.tokens_all(), mrg = (size_t)g.Lm, vec = (size_t)g.d / 8;
+  c.src = (const uint4*)src + (merging ? (size_t)g.N : (size_t)g.D) * vec;
+  c.dst = (uint4*)dst + (merging ? (size_t)g.D : (size_t)g.N) * vec;
+  c.src_stride = (merging ? full : mrg) * vec;
+  c.dst_stride = (merging ? mrg : full) * vec;
+  c.per = (int)(g.n_extra * vec);
+  c.batches = g.B;
+  return c;
 }
 
 // 32 bytes to a 32-byte aligned address: a thread that writes a row of its own fills whole sectors.

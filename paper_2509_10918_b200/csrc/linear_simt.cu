@@ -553,12 +553,6 @@ static void copy_extra(const Geom& g, const T* src, T* dst, bool merging, cudaSt
   count_launch();
 }
 
-cudaError_t launch_copy_extra(const Geom& g, const void* src, void* dst, bool merging, cudaStream_t s) {
-  if (g.f32) copy_extra<float>(g, (const float*)src, (float*)dst, merging, s);
-  else copy_extra<__nv_bfloat16>(g, (const __nv_bfloat16*)src, (__nv_bfloat16*)dst, merging, s);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_merge_simt(const Geom& g, const void* w, const void* x, void* xm, cudaStream_t s) {
   const int batches = g.B * g.P;
   if (g.f32) {

@@ -43,6 +43,7 @@ struct RgParams {
   const uint8_t* w_end;
   uint32_t* zero;  // merge only: words cleared on the side (the attention kernel's tickets)
   int zero_words;
+  RowCopy extra;
 };
 
 // Eight consecutive weights starting `off` elements into a plane, the first `n` of them real and the rest 0.
@@ -279,6 +280,8 @@ ragged_kernel(const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ 
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar->full[s]);
     }
+    copy_part(p.extra, (int)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * kWorkers + t,
+              (int)(gridDim.x * gridDim.y * gridDim.z) * kWorkers);
     if (ok && __all_sync(0xffffffffu, mbar_wait(&bar->done, 0, dev_status, abort_flag))) {
       tc_fence_after();
       // every load has been consumed: the stages are the output's staging area
@@ -347,6 +350,7 @@ cudaError_t launch_ragged(const Geom& g, const void* w, const void* in, void* ou
   p.w_end = (const uint8_t*)w + (size_t)g.B * g.P * g.Nloc * g.Dloc * 4;
   p.zero = (uint32_t*)zero;
   p.zero_words = (int)(zero_bytes / 4);
+  p.extra = extra_rows(g, in, out, kMerge);
   CUtensorMap tb, tbt, to, tot;
   bool ok;
   if (kMerge) ok = token_map(g, in, p.rows, &tb) && token_map(g, in, tail, &tbt) && merged_map(g, out, 128, &to);
