@@ -92,7 +92,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     if (mbar_wait(&bar->done, 0, dev_status, abort_flag)) {
       tc_fence_after();
       const int pitch = sq_pitch(Nloc);
-      const bool wide = pitch % 16 == 0;
+      const bool wide = pitch % 16 == 0 && (reinterpret_cast<uintptr_t>(sq) & 31) == 0;  // a workspace need only be 16-byte aligned
       uint16_t* row = sq + ((size_t)tile * Nloc + (i < Nloc ? i : 0)) * pitch + n0;
       for (int j0 = 0; j0 < n_cols; j0 += 32) {
         uint32_t r[32];

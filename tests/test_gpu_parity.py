@@ -1119,6 +1119,22 @@ def test_selection_at_the_edges_of_its_kernels(toma, th, tw, ratio):
             assert np.array_equal(idx[b, p], want)
 
 
+def test_selection_in_a_workspace_aligned_to_16_bytes(toma):
+    """The similarity matrix is stored 32 bytes at a time where its address allows; a workspace promises 16."""
+    cfg = gen.config("cfg2", batch=1, grid_h=16, grid_w=32, tile_h=16, tile_w=16, dim=64, n_heads=1)
+    x = to_dev(gen.features(cfg), cfg.dtype)
+    desc = toma.desc_from_config(cfg)
+    ws = toma.alloc_workspace(desc)
+    shifted = torch.empty(ws.numel() * ws.element_size() + 64, dtype=torch.uint8, device="cuda")
+    shifted = shifted[(16 - shifted.data_ptr()) % 32:][: ws.numel() * ws.element_size()]
+    assert shifted.data_ptr() % 32 == 16
+    idx = [toma.alloc_idx(desc) for _ in range(2)]
+    for out, scratch in zip(idx, (ws, shifted)):
+        toma.toma_select(desc, x, out, scratch)
+    torch.cuda.synchronize()
+    assert torch.equal(idx[0], idx[1])
+
+
 RAGGED = [  # tile_h, tile_w, ratio, dim, heads: boxes of whole tile rows with a tail, D_loc of every alignment, rows over 64 tokens
     (18, 14, 0.5, 640, 10), (19, 13, 0.5, 128, 2), (9, 7, 0.4, 64, 1), (5, 27, 0.3, 72, 1), (3, 65, 0.5, 128, 2), (2, 100, 0.25, 320, 5),
     (1, 128, 0.5, 64, 1), (24, 25, 0.75, 192, 3), (17, 3, 0.9, 328, 1), (16, 16, 0.41, 640, 10), (28, 28, 0.2, 64, 1), (1, 1, 0.0, 64, 1),
