@@ -344,7 +344,7 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     const bool valid = k_loc < p.m_tok;
     const uint32_t taddr = tmem + mb * ncols_mb + ((uint32_t)(quarter * 32) << 16);
     float* zrow = zw + (mb * 4 + quarter) * Dl;
-    float neg_m = 0.f, inv = 0.f;
+    float inv = 0.f;
     const bool ok = mbar_wait(&bar->done, 0, dev_status, abort_flag);
     if (ok) {
       tc_fence_after();
@@ -358,7 +358,7 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         for (int e = 0; e < 32; ++e)
           if (i0 + e < Dl) mx = fmaxf(mx, __uint_as_float(r[e]));
       }
-      neg_m = -mx * p.scale_log2;
+      const float neg_m = -mx * p.scale_log2;
       // pass 2: denominator of the token's softmax
       float sum = 0.f;
       for (int i0 = 0; i0 < Dl; i0 += 32) {
@@ -366,9 +366,14 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         tmem_ld32(taddr + i0, r);
         tmem_wait_ld();
 #pragma unroll
-        for (int e = 0; e < 32; ++e)
-          if (i0 + e < Dl) sum += fast_exp2(fmaf(__uint_as_float(r[e]), p.scale_log2, neg_m));
+        for (int e = 0; e < 32; ++e) {
+          const float v = fast_exp2(fmaf(__uint_as_float(r[e]), p.scale_log2, neg_m));
+          if (i0 + e < Dl) sum += v;
+          r[e] = __float_as_uint(v);
+        }
+        tmem_st32(taddr + i0, r);  // for the passes below
       }
+      tmem_wait_st();
       inv = valid ? 1.f / sum : 0.f;
       // pass 3: the shares' sums over this warp's 32 source tokens, per destination
       for (int i0 = 0; i0 < Dl; i0 += 32) {
@@ -378,7 +383,7 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         float a[32];
 #pragma unroll
         for (int e = 0; e < 32; ++e) {
-          const float v = fast_exp2(fmaf(__uint_as_float(r[e]), p.scale_log2, neg_m)) * inv;
+          const float v = __uint_as_float(r[e]) * inv;
           a[e] = (valid && i0 + e < Dl) ? v : 0.f;
         }
         // transpose-reduce: afterwards lane c holds the sum over the warp's 32 rows of column i0 + c
@@ -442,7 +447,7 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
           __align__(16) __nv_bfloat16 hi[8], lo[8], uh[8], ul[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
-            const float a = fast_exp2(fmaf(__uint_as_float(r[e0 + e]), p.scale_log2, neg_m)) * inv;
+            const float a = __uint_as_float(r[e0 + e]) * inv;
             const float v = a * zinv[i0 + e0 + e];
             hi[e] = __float2bfloat16_rn(v);
             lo[e] = __float2bfloat16_rn(v - __bfloat162float(hi[e]));
