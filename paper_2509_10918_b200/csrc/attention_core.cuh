@@ -15,8 +15,9 @@ constexpr int kBM = 128;  // rows of one query tile = threads of one softmax war
 constexpr int kBN = 64;   // keys per tile
 constexpr float kRescaleThreshold = 8.0f;
 
-// 2^x for x <= ~9 on the FMA pipe, two at a time: round to nearest integer with the 1.5*2^23 trick, degree-3
-// near-minimax polynomial for 2^f on [-0.5, 0.5], exponent patched in with an integer add.
+// 2^x for x <= 127 on the FMA pipe, two at a time: round to nearest integer with the 1.5*2^23 trick, degree-3
+// near-minimax polynomial for 2^f on [-0.5, 0.5], exponent patched in with an integer add.  Below -126 the result is
+// 2^-126; above 127 the add runs into the sign bit and wraps, so callers whose x has no upper bound clamp it.
 __device__ __forceinline__ void ex2_poly2(uint64_t x2, float& p0, float& p1) {
   float x0, x1;
   unpack2(x2, x0, x1);
@@ -159,9 +160,9 @@ __device__ __forceinline__ bool softmax_tile(uint32_t sb, uint32_t ob, float sca
 // ------------------------------------------------------------------ softmax against a reference with headroom
 // P = 2^(S c - m) of 32 columns as packed bf16 for a reference m that lies 2^kHeadroom above the scores seen when it was
 // set.  Everything is floating point, so the common factor costs no precision; what it buys is that the reference need
-// not follow the row maximum: no maximum is taken before the exponentials.  Instead the largest P of the tile is looked
-// at: one of 2 or more (bit 14, set in numbers that are none as well) says that the scores have outgrown the headroom,
-// and the caller moves the reference.  sum2: fp32 sums of the even and the odd columns.
+// not follow the row maximum: no maximum is taken before the exponentials.  Instead the sum of the tile's P is looked at
+// (sum2: fp32 sums of the even and the odd columns): one of 2 or more, or none at all, says that the scores have outgrown
+// the headroom, and the caller moves the reference.
 // One pair of columns in four takes the polynomial of ex2_poly2 on the FMA pipe, the others MUFU (timed: one in eight to
 // three in eight are within 2 % of each other).
 constexpr float kHeadroom = 32.f;
@@ -171,12 +172,12 @@ __device__ __forceinline__ void chunk_exp_ref(const uint32_t (&r)[32], uint32_t 
 #pragma unroll
   for (int e = 0; e < 32; e += 2) {
     const uint64_t x2 = fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), c2, m2);
-    float p0, p1;
+    float p0, p1, x0, x1;
+    unpack2(x2, x0, x1);
     if ((e & 6) == 6) {
-      ex2_poly2(x2, p0, p1);
+      // a score may lie any distance above the reference: 2^126 stands for all that is larger, for outgrown() to see
+      ex2_poly2(pack2(fminf(x0, 126.f), fminf(x1, 126.f)), p0, p1);
     } else {
-      float x0, x1;
-      unpack2(x2, x0, x1);
       p0 = ex2_mufu(x0);
       p1 = ex2_mufu(x1);
     }
@@ -191,11 +192,21 @@ __device__ __forceinline__ uint32_t largest2(const uint32_t (&pk)[32]) {
   for (int e = 0; e < 32; e += 2) top = __vimax3_u16x2(pk[e], pk[e + 1], top);
   return top;
 }
-__device__ __forceinline__ bool outgrown(uint32_t top) { return (top & 0x40004000u) != 0u; }
+__device__ __forceinline__ bool outgrown(uint64_t sum2) {
+  float even, odd;
+  unpack2(sum2, even, odd);
+  return !(even + odd < 2.f);
+}
 // sum2 adds up P before its rounding to bf16: one instruction per pair of columns, where the rounded values take three
 // (735 us against 825 us at 4 x 8192 tokens, 10 heads of 64).  Rounding errors of many keys cancel; that of a key which
 // makes up most of its row would scale the whole output row by up to 2^-9.  In a tile where some P is more than a quarter
-// of the row's sum so far, the row therefore counts what the product really multiplies.
+// of the row's sum so far, the row therefore counts what the product really multiplies.  Where the whole tile is less than
+// a quarter no P can be: the largest is looked for in the other tiles only, a row's first few and the odd one later.
+__device__ __forceinline__ bool may_dominate(uint64_t sum2, float sum) {
+  float even, odd;
+  unpack2(sum2, even, odd);
+  return 4.f * (even + odd) > sum;
+}
 __device__ __forceinline__ bool dominates(uint32_t top, float sum) {
   return 4.f * fmaxf(__uint_as_float(top << 16), __uint_as_float(top & 0xFFFF0000u)) > sum;
 }

@@ -886,7 +886,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         }
         uint32_t pk[32];
         uint64_t sum2;
-        uint32_t top;
         bool asked = false;  // a second time would not help (scores that are no numbers)
 #pragma unroll 1
         for (;;) {
@@ -903,8 +902,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             }
             chunk_exp_ref(r, *reinterpret_cast<uint32_t(*)[16]>(&pk[c * 16]), scale_log2, -m_used, sum2);
           }
-          top = largest2(pk);
-          const bool grown = __any_sync(0xffffffffu, outgrown(top)) && !asked;
+          const bool grown = __any_sync(0xffffffffu, outgrown(sum2)) && !asked;
           if constexpr (C::kOwnO) {
             if (!grown) break;
             moved_to(move_reference<DH>(t, bar, s_addr, valid, scale_log2, m_used, !first, n, dev_status));
@@ -924,10 +922,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         // the sum, while the tensor cores already multiply P
         float even, odd;
         unpack2(add2(l2, sum2), even, odd);
-        const bool dom = dominates(top, even + odd);
-        if (__any_sync(0xffffffffu, dom)) {
-          const uint64_t rounded = rounded_sum2(pk);
-          if (dom) sum2 = rounded;
+        if (__any_sync(0xffffffffu, may_dominate(sum2, even + odd))) {
+          const bool dom = dominates(largest2(pk), even + odd);
+          if (__any_sync(0xffffffffu, dom)) {
+            const uint64_t rounded = rounded_sum2(pk);
+            if (dom) sum2 = rounded;
+          }
         }
         l2 = add2(l2, sum2);
       }

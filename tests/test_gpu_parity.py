@@ -1206,7 +1206,7 @@ def test_global_merge_of_ragged_images_parity(toma, gh, gw, th, tw, ratio):
 @pytest.mark.parametrize("dh", [64, 128])
 @pytest.mark.parametrize("L,split,ctas", [(1000, 0, 0), (1000, 1, 5), (130, 0, 0), (65, 0, 0), (20, 0, 0)])
 def test_attention_scores_that_outgrow_every_headroom(toma, tuning, dh, L, split, ctas):
-    """Scores jump by hundreds of log2 units from key tile to key tile, at different tiles for different rows and in either of
+    """Scores climb by up to 69 log2 units from key tile to key tile, at different tiles for different rows and in either of
     the two pipelines a row's tiles are dealt to: the reference has to be moved again and again, also while the other
     pipeline's probabilities lie ready against the old one."""
     B, h = 1, 3
@@ -1228,3 +1228,44 @@ def test_attention_scores_that_outgrow_every_headroom(toma, tuning, dh, L, split
     torch.cuda.synchronize()
     assert int(status.item()) == 0
     assert_close(to_host64(o)[0], O.attention(host[0][0], host[1][0], host[2][0], h), "bf16", "attention with jumping scores")
+
+
+def _scores_of(rng, rows, levels, dh):
+    """q, k, v [L][dh] whose score of query r and key c is about rows[r] * levels[c] nats (each +- 1)."""
+    u = rng.normal(size=dh)
+    u /= np.linalg.norm(u)
+    q = 0.1 * rng.normal(size=(len(rows), dh)) + 16.0 * rows[:, None] * u
+    k = 0.1 * rng.normal(size=(len(levels), dh)) + np.sqrt(dh) / 16.0 * levels[:, None] * u
+    return q, k, rng.normal(size=(len(levels), dh))
+
+
+@pytest.mark.parametrize("dh", [64, 128])
+@pytest.mark.parametrize("split,ctas", [(0, 0), (1, 5)])
+@pytest.mark.parametrize("jump", [85, 100, 115, 150, 180, 200, 260, 300, 400, 1000])
+@pytest.mark.parametrize("kind", ["tiles", "one_key_first_tile", "one_key_later_tile"])
+def test_attention_scores_far_above_the_reference(toma, tuning, dh, split, ctas, jump, kind):
+    """Scores `jump` nats above everything the row's reference was set from: whole key tiles (a jump in every second tile, so
+    that each pipeline sees it against its own earlier tiles), or one key alone at each column residue mod 8 (a pair of
+    columns in four takes another exponential), behind the 32 columns that set the first reference or in a later tile.
+    All rows agree in the even heads; in the odd ones only every third row sees the jump.  One head per residue and kind."""
+    rng = np.random.default_rng(jump + dh)
+    L, h = 450, 16
+    q, k, v = (np.empty((1, L, h, dh)) for _ in range(3))
+    for n in range(h):
+        rows = np.where(np.arange(L) % 3 == 0, 1.0, 0.0) if n & 1 else np.ones(L)
+        levels = np.zeros(L)
+        if kind == "tiles":
+            levels += jump * ((np.arange(L) // 64 + n // 2 % 2) // 2 % 2)
+        else:
+            at = (32 if kind == "one_key_first_tile" else 64 * (2 + n // 2 % 4)) + 8 * (n // 4) + n // 2
+            levels[at] = jump
+        q[0, :, n], k[0, :, n], v[0, :, n] = _scores_of(rng, rows, levels, dh)
+    host = [gen.round_to_dtype(a.reshape(1, L, h * dh).astype(np.float32), "bf16") for a in (q, k, v)]
+    dq, dk, dv = (to_dev(a, "bf16") for a in host)
+    o = torch.empty_like(dq)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    tuning(attention_split=split, attention_ctas=ctas)
+    toma.toma_attention(1, L, h, dh, "bf16", dq, dk, dv, o, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert_close(to_host64(o)[0], O.attention(host[0][0], host[1][0], host[2][0], h), "bf16", "attention with scores far above the reference")
