@@ -103,7 +103,7 @@ __device__ __forceinline__ float chunk_exp(const uint32_t (&r)[32], uint32_t (&p
 
 // One 64-key tile of the online softmax for one query row.
 template <int DH, bool kSumMma, bool kMask>
-__device__ __forceinline__ bool softmax_tile(uint32_t sb, uint32_t ob, float scale_log2, int valid, int j, float& m_used,
+__device__ __forceinline__ void softmax_tile(uint32_t sb, uint32_t ob, float scale_log2, int valid, int j, float& m_used,
                                              float& l, uint64_t* pv_done, uint32_t pv_parity, uint32_t* dev_status, volatile int* abort_flag) {
   uint32_t sr[64];
   tmem_ld32(sb, sub32<0>(sr));
@@ -124,7 +124,7 @@ __device__ __forceinline__ bool softmax_tile(uint32_t sb, uint32_t ob, float sca
   }
   if (__any_sync(0xffffffffu, rescale)) {
     // O holds every PV product issued so far; the last one (tile j-1) must have landed
-    if (!mbar_wait(pv_done, pv_parity, dev_status, abort_flag)) return false;
+    mbar_wait(pv_done, pv_parity, dev_status, abort_flag);  // ran out: the results are void, but all lanes go the same way
     tc_fence_after();
     l *= factor;
 #pragma unroll
@@ -154,7 +154,6 @@ __device__ __forceinline__ bool softmax_tile(uint32_t sb, uint32_t ob, float sca
   l += chunk_exp<kMask, kRegSum, DH == 128>(sub32<32>(sr), pk, scale_log2, neg_m, 32, valid);
   tmem_st16(sb + 16, pk);
   tmem_wait_st();
-  return true;
 }
 
 // ------------------------------------------------------------------ softmax against a reference with headroom

@@ -338,9 +338,8 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       const uint32_t sb = tmem + lane_addr + (2 * q + bb) * kBN;
       if (!mbar_wait(&bar->s_full[q][bb], (n >> 1) & 1, dev_status, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      ok = softmax_tile<64, true, false>(sb, ob, p.scale_log2, kBN, n, m_used, l, &bar->pv_done[(n + 3) & 3], (uint32_t)(((n - 1) >> 2) & 1),
-                                         dev_status, abort_flag);
-      if (!ok) break;
+      softmax_tile<64, true, false>(sb, ob, p.scale_log2, kBN, n, m_used, l, &bar->pv_done[(n + 3) & 3], (uint32_t)(((n - 1) >> 2) & 1), dev_status,
+                                    abort_flag);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar->p_full[q][bb]);

@@ -1269,3 +1269,20 @@ def test_attention_scores_far_above_the_reference(toma, tuning, dh, split, ctas,
     torch.cuda.synchronize()
     assert int(status.item()) == 0
     assert_close(to_host64(o)[0], O.attention(host[0][0], host[1][0], host[2][0], h), "bf16", "attention with scores far above the reference")
+
+
+@pytest.mark.parametrize("dh,B,L,h", [(128, 2, 28, 12), (128, 1, 300, 4), (128, 2, 1100, 3), (64, 2, 130, 4)])
+def test_attention_error_on_flat_scores(toma, dh, B, L, h):
+    """Scores within a few binades of each other: the error is the result's rounding to bf16 (relative 1.66e-3) and that of
+    the probabilities, whose 8 significant bits are worth most where the row's largest lie just below a power of two (relative
+    1.13e-3 there, 2.26e-3 just above one: 2.2e-3 in all against 2.4e-3 where the reference leaves that to chance)."""
+    rng = np.random.default_rng(L)
+    host = [gen.round_to_dtype((s * rng.normal(size=(B, L, h * dh))).astype(np.float32), "bf16") for s in (0.3, 0.3, 1.0)]
+    q, k, v = (to_dev(a, "bf16") for a in host)
+    o = torch.empty_like(q)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    toma.toma_attention(B, L, h, dh, "bf16", q, k, v, o, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    want = np.stack([O.attention(host[0][b], host[1][b], host[2][b], h) for b in range(B)])
+    assert np.linalg.norm(to_host64(o) - want) / np.linalg.norm(want) < 2.3e-3
