@@ -157,8 +157,9 @@ __device__ __forceinline__ void softmax_tile(uint32_t sb, uint32_t ob, float sca
 }
 
 // ------------------------------------------------------------------ softmax against a reference with headroom
-// P = 2^(S c - m) of 32 columns as packed bf16 for a reference m that lies 2^kHeadroom above the scores seen when it was
-// set.  Everything is floating point, so the common factor costs no precision; what it buys is that the reference need
+// P = 2^(S c - m) of 32 columns as packed bf16 for a reference m that lies 2^kHeadroom above the largest score seen when it
+// was set.  Everything is floating point, so the common factor costs no precision (a power of two exactly: the largest P
+// stay just below a power of two, where their 8 bits are worth most); what it buys is that the reference need
 // not follow the row maximum: no maximum is taken before the exponentials.  Instead the sum of the tile's P is looked at
 // (sum2: fp32 sums of the even and the odd columns): one of 2 or more, or none at all, says that the scores have outgrown
 // the headroom, and the caller moves the reference.

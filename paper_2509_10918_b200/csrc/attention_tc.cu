@@ -2,7 +2,7 @@
 // softmax and accumulation: four softmax pipelines per CTA, for head_dim 64 (units, spans and pieces: attention_span.cuh),
 // and the work plan and the choice between this kernel and attention_two_tc.cu's for every call.
 //
-// Inside a CTA (19 warps): warps 0..15 run the softmax as four pipelines of four warps, one per query tile q and parity h
+// Inside a CTA (20 warps, the last one idle): warps 0..15 run the softmax as four pipelines of four warps, one per query tile q and parity h
 // of the key tile (one thread per query row, straight out of tensor memory; so two threads share a row, each with every
 // second key tile), warp 16 feeds Q, K and V through TMA rings, one elected thread of warp 17 issues the tcgen05 MMAs,
 // warp 18 publishes a partial first piece (memory fence and tickets, off everybody else's path).
@@ -13,7 +13,7 @@
 //                             memory) of  O += P_q,j V_j
 //   O                      -> every pipeline has an accumulator and a reference m of its own (four of 64 columns beside four
 //                             of S fill the tensor memory), added up at the end of a piece
-//   reference              -> set 2^32 above the piece's first scores and moved only when scores outgrow it (see
+//   reference              -> set 2^32 above the piece's first tile and moved only when scores outgrow it (see
 //                             chunk_exp_ref), so no row maximum stands before the exponentials
 //   exponentials           -> one pair of columns in four goes through a degree-3 polynomial on the FMA pipe (relative
 //                             error 7.5e-5, far below bf16 resolution of P), the rest through MUFU ex2; the scaling
@@ -39,7 +39,7 @@ namespace {
 
 constexpr int DH = 64;
 constexpr int kSoftWarps = 16;
-constexpr int kThreads = (kSoftWarps + 3) * 32;
+constexpr int kThreads = (kSoftWarps + 4) * 32;  // the last warp idles: a block of 19 was 0.5 % slower
 static_assert(kSoftWarps <= kTicketCols, "tickets per unit");
 
 constexpr int kStages = 8;                       // K/V ring depth (S runs two tiles ahead of P V)
@@ -321,23 +321,31 @@ __device__ __noinline__ void settle_first_piece(Barriers* bar, int it_begin, int
 
 // Largest score (log2 domain) of this row in a tile, the first `valid` of its columns counting.
 __device__ __noinline__ float tile_max(uint32_t s_addr, int valid, float scale_log2) {
-  float mx = -INFINITY;
+  float even = -INFINITY, odd = -INFINITY;
 #pragma unroll 1
-  for (int c = 0; c < valid; c += 16) {
-    uint32_t r[16];
-    tmem_ld16(s_addr + c, r);
+  for (int c = 0; c < valid; c += 32) {
+    uint32_t r[32];
+    tmem_ld32(s_addr + c, r);
     tmem_wait_ld();
+    if (valid - c < 32) {
 #pragma unroll
-    for (int e = 0; e < 16; ++e) mx = c + e < valid ? fmaxf(mx, __uint_as_float(r[e])) : mx;
+      for (int e = 0; e < 32; ++e)
+        if (c + e >= valid) r[e] = 0xFF800000u;  // -inf
+    }
+#pragma unroll
+    for (int e = 0; e < 32; e += 4) {
+      even = max3(even, __uint_as_float(r[e]), __uint_as_float(r[e + 2]));
+      odd = max3(odd, __uint_as_float(r[e + 1]), __uint_as_float(r[e + 3]));
+    }
   }
-  return mx * scale_log2;
+  return fmaxf(even, odd) * scale_log2;
 }
 // The reference for a row whose scores have reached `mx`.
-__device__ __forceinline__ float reference(float mx, float m_used) { return mx > m_used + 1.f ? ceilf(mx) + kHeadroom : m_used; }
-// Columns [c0, c1) of this row's accumulator times `factor` (a power of two: exact).
-__device__ __forceinline__ void scale_o(uint32_t o_addr, int c0, int c1, float factor) {
+__device__ __forceinline__ float reference(float mx, float m_used) { return mx > m_used + 1.f ? mx + kHeadroom : m_used; }
+// This row's accumulator times `factor`.
+__device__ __forceinline__ void scale_o(uint32_t o_addr, float factor) {
 #pragma unroll 1
-  for (int c = c0; c < c1; c += 16) {
+  for (int c = 0; c < DH; c += 16) {
     uint32_t r[16];
     tmem_ld16(o_addr + c, r);
     tmem_wait_ld();
@@ -348,16 +356,16 @@ __device__ __forceinline__ void scale_o(uint32_t o_addr, int c0, int c1, float f
   tmem_wait_st();
 }
 
-// Some row of this warp has scores that outgrew its reference.  Such rows get a new one,
-// kHeadroom above the tile's largest score, and the pipeline's accumulator is multiplied by the power of two between the
-// two (references are whole numbers).  Out of line, it hardly ever runs.  Returns the new reference.
+// Some row of this warp has scores that outgrew its reference.  Such rows get a new one, kHeadroom above the tile's largest
+// score, and the pipeline's accumulator is multiplied by what lies between the two.  Out of line, it hardly ever runs.
+// Returns the new reference.
 __device__ __noinline__ float move_reference(Row t, Barriers* bar, uint32_t s_addr, int valid, float scale_log2, float m_used, bool have_o, int n,
                                              uint32_t* dev_status) {
   const float m_new = reference(tile_max(s_addr, valid, scale_log2), m_used);
   // every product issued so far must have landed
   if (have_o && __all_sync(0xffffffffu, mbar_wait(&bar->pv_done[t.q][t.half], ((n >> 1) - 1) & 1, dev_status, &bar->abort_flag))) {
     tc_fence_after();
-    scale_o(t.tm + o_col(t.q, t.half), 0, DH, ex2_mufu(m_used - m_new));
+    scale_o(t.tm + o_col(t.q, t.half), ex2_mufu(m_used - m_new));
   }
   return m_new;
 }
@@ -583,7 +591,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         ok = ok && mbar_wait(s_bar, (n >> 1) & 1, dev_status, abort_flag);
         __syncwarp();
         tc_fence_after();
-        if (first) m_used = ceilf(tile_max(s_addr, min(valid, 32), scale_log2)) + kHeadroom;
+        if (first) m_used = tile_max(s_addr, valid, scale_log2) + kHeadroom;
         uint32_t pk[32];
         uint64_t sum2;
         bool asked = false;  // a second time would not help (scores that are no numbers)
@@ -605,7 +613,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           const bool grown = __any_sync(0xffffffffu, outgrown(sum2)) && !asked;
           if (!grown) break;
           moved_to(move_reference(t, bar, s_addr, valid, scale_log2, m_used, !first, n, dev_status));
-          asked = true;
+          asked = asked || grown;
         }
         first = false;
         tmem_st32(s_addr, pk);

@@ -1271,7 +1271,7 @@ def test_attention_scores_far_above_the_reference(toma, tuning, dh, split, ctas,
     assert_close(to_host64(o)[0], O.attention(host[0][0], host[1][0], host[2][0], h), "bf16", "attention with scores far above the reference")
 
 
-@pytest.mark.parametrize("dh,B,L,h", [(128, 2, 28, 12), (128, 1, 300, 4), (128, 2, 1100, 3), (64, 2, 130, 4)])
+@pytest.mark.parametrize("dh,B,L,h", [(128, 2, 28, 12), (128, 1, 300, 4), (128, 2, 1100, 3), (64, 2, 130, 4), (64, 1, 1000, 8), (64, 1, 2300, 30)])
 def test_attention_error_on_flat_scores(toma, dh, B, L, h):
     """Scores within a few binades of each other: the error is the result's rounding to bf16 (relative 1.66e-3) and that of
     the probabilities, whose 8 significant bits are worth most where the row's largest lie just below a power of two (relative
