@@ -133,13 +133,15 @@ __device__ __noinline__ void combine_rows(const float* pieces, const Spans& sp, 
       const float mb = __ldcg(sb + kM + row), lb = __ldcg(sb + kL + row);
       const float wa = ex2_mufu(ma - M), wb = g < g_last ? ex2_mufu(mb - M) : 0.f;
       denom = fmaf(wb, lb, fmaf(wa, la, denom));
+      const float4* pa = reinterpret_cast<const float4*>(sa) + (size_t)(c0 >> 2) * kUM + row;  // the loads below at constant offsets
+      const float4* pb = reinterpret_cast<const float4*>(sb) + (size_t)(c0 >> 2) * kUM + row;
 #pragma unroll
       for (int s = 0; s < kStep; s += 4 * kQuads) {
         float4 va[kQuads], vb[kQuads];
 #pragma unroll
         for (int q = 0; q < kQuads; ++q) {
-          va[q] = __ldcg(reinterpret_cast<const float4*>(sa) + (size_t)((c0 + s) / 4 + q) * kUM + row);
-          vb[q] = __ldcg(reinterpret_cast<const float4*>(sb) + (size_t)((c0 + s) / 4 + q) * kUM + row);
+          va[q] = __ldcg(pa + (size_t)(s / 4 + q) * kUM);
+          vb[q] = __ldcg(pb + (size_t)(s / 4 + q) * kUM);
         }
 #pragma unroll
         for (int q = 0; q < kQuads; ++q) {
