@@ -341,7 +341,7 @@ __device__ __noinline__ float tile_max(uint32_t s_addr, int valid, float scale_l
   return fmaxf(even, odd) * scale_log2;
 }
 // The reference for a row whose scores have reached `mx`.
-__device__ __forceinline__ float reference(float mx, float m_used) { return mx > m_used + 1.f ? mx + kHeadroom : m_used; }
+__device__ __forceinline__ float reference(float mx, float m_used) { return mx > m_used ? mx + kHeadroom : m_used; }
 // This row's accumulator times `factor`.
 __device__ __forceinline__ void scale_o(uint32_t o_addr, float factor) {
 #pragma unroll 1
