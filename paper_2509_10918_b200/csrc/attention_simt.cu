@@ -82,19 +82,28 @@ __global__ void __launch_bounds__(BQ * 4) attention_simt_kernel(const T* __restr
     __syncthreads();
     const float* Kt = Ks + st * C::kTile + tx * C::kPitch;
     const float* Qt = Qs + r0 * C::kPitch;
+    // four chains of DH / 4 channels instead of one of DH: half the rounding error of a score
     float s[4][4] = {};
+#pragma unroll 1
+    for (int c0 = 0; c0 < DH; c0 += DH / 4) {
+      float part[4][4] = {};
 #pragma unroll 4
-    for (int c = 0; c < DH; c += 4) {
-      float4 a[4], w[4];
+      for (int c = c0; c < c0 + DH / 4; c += 4) {
+        float4 a[4], w[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(Qt + i * C::kPitch + c);
+        for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(Qt + i * C::kPitch + c);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const float4*>(Kt + j * 16 * C::kPitch + c);
+        for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const float4*>(Kt + j * 16 * C::kPitch + c);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            part[i][j] = fmaf(a[i].w, w[j].w, fmaf(a[i].z, w[j].z, fmaf(a[i].y, w[j].y, fmaf(a[i].x, w[j].x, part[i][j]))));
+      }
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          s[i][j] = fmaf(a[i].w, w[j].w, fmaf(a[i].z, w[j].z, fmaf(a[i].y, w[j].y, fmaf(a[i].x, w[j].x, s[i][j]))));
+        for (int j = 0; j < 4; ++j) s[i][j] += part[i][j];
     }
     if (k0 + kKeys > L) {
 #pragma unroll

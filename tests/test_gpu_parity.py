@@ -1286,3 +1286,21 @@ def test_attention_error_on_flat_scores(toma, dh, B, L, h):
     assert int(status.item()) == 0
     want = np.stack([O.attention(host[0][b], host[1][b], host[2][b], h) for b in range(B)])
     assert np.linalg.norm(to_host64(o) - want) / np.linalg.norm(want) < 2.3e-3
+
+
+@pytest.mark.parametrize("dh,L", [(128, 32), (64, 182)])
+def test_f32_attention_score_rounding(toma, dh, L):
+    """Scores of some tens of nats in fp32 mode: their rounding is what the result's error is made of.  A chain of n products
+    errs in proportion to sqrt(n), so four chains of dh / 4 half as much as one of dh (here 3.0e-7 and 4.6e-7 against 5.9e-7
+    and 7.0e-7)."""
+    B, h = 3, 14
+    rng = np.random.default_rng(dh)
+    host = [(s * rng.normal(size=(B, L, h * dh))).astype(np.float32) for s in (2.0, 2.0, 1.0)]
+    q, k, v = (to_dev(a, "f32") for a in host)
+    o = torch.empty_like(q)
+    toma.toma_attention(B, L, h, dh, "f32", q, k, v, o)
+    torch.cuda.synchronize()
+    host = [a.astype(np.float64) for a in host]
+    want = np.stack([O.attention(host[0][b], host[1][b], host[2][b], h) for b in range(B)])
+    got = o.double().cpu().numpy()
+    assert np.linalg.norm(got - want) / np.linalg.norm(want) < (4.2e-7 if dh == 128 else 5.7e-7)
