@@ -159,15 +159,15 @@ __device__ __forceinline__ int tile_token(int p, int l, int tiles_x, int th, int
 struct RowCopy {
   const uint4* src = nullptr;
   uint4* dst = nullptr;
-  size_t src_stride = 0, dst_stride = 0;
-  int per = 0, batches = 0;
+  size_t src_stride = 0, dst_stride = 0, per = 0;
+  int batches = 0;
 };
-__device__ __forceinline__ void copy_part(const RowCopy& c, int thread, int n_threads) {
+__device__ __forceinline__ void copy_part(const RowCopy& c, size_t thread, size_t n_threads) {
   for (int b = 0; b < c.batches; ++b) {
     const uint4* src = c.src + b * c.src_stride;
     uint4* dst = c.dst + b * c.dst_stride;
 #pragma unroll 4
-    for (int e = thread; e < c.per; e += n_threads) dst[e] = src[e];
+    for (size_t e = thread; e < c.per; e += n_threads) dst[e] = src[e];
   }
 }
 // bf16, d a multiple of 8: the un-merged trailing tokens of x -> merged rows (merging) or of attended rows -> output.
@@ -179,7 +179,7 @@ inline RowCopy extra_rows(const Geom& g, const void* src, void* dst, bool mergin
   c.dst = (uint4*)dst + (merging ? (size_t)g.D : (size_t)g.N) * vec;
   c.src_stride = (merging ? full : mrg) * vec;
   c.dst_stride = (merging ? mrg : full) * vec;
-  c.per = (int)(g.n_extra * vec);
+  c.per = (size_t)g.n_extra * vec;
   c.batches = g.B;
   return c;
 }

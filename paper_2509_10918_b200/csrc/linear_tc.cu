@@ -46,8 +46,8 @@ struct LinParams {
 // text tokens of 3072 channels.
 // Out of line: sequences without text tokens should not fetch its instructions (0.2 us per launch).
 __device__ __noinline__ void copy_extra(const RowCopy c) {
-  const int cta = (int)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
-  copy_part(c, cta * 128 + (int)threadIdx.x - 64, (int)(gridDim.x * gridDim.y * gridDim.z) * 128);
+  const size_t cta = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  copy_part(c, cta * 128 + threadIdx.x - 64, (size_t)gridDim.x * gridDim.y * gridDim.z * 128);
 }
 
 __device__ __forceinline__ uint32_t tmem_cols_for(int n) { return n > 128 ? 256u : n > 64 ? 128u : 64u; }

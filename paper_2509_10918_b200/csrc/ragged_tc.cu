@@ -280,8 +280,9 @@ ragged_kernel(const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ 
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar->full[s]);
     }
-    copy_part(p.extra, (int)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * kWorkers + t,
-              (int)(gridDim.x * gridDim.y * gridDim.z) * kWorkers);
+    if (p.extra.per)
+      copy_part(p.extra, (((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * kWorkers + t,
+                (size_t)gridDim.x * gridDim.y * gridDim.z * kWorkers);
     if (ok && __all_sync(0xffffffffu, mbar_wait(&bar->done, 0, dev_status, abort_flag))) {
       tc_fence_after();
       // every load has been consumed: the stages are the output's staging area

@@ -1304,3 +1304,20 @@ def test_f32_attention_score_rounding(toma, dh, L):
     want = np.stack([O.attention(host[0][b], host[1][b], host[2][b], h) for b in range(B)])
     got = o.double().cpu().numpy()
     assert np.linalg.norm(got - want) / np.linalg.norm(want) < (4.2e-7 if dh == 128 else 5.7e-7)
+
+
+def test_text_rows_of_more_than_2_31_packets(toma):
+    """34 GB of text tokens: their 16-byte packets do not count in 31 bits."""
+    extra, d = (1 << 22) + 40, 4096
+    desc = toma.make_desc(batch=1, grid_h=8, grid_w=8, dim=d, tile_h=8, tile_w=8, merge_ratio=0.5, tau=0.1, n_heads=32, head_dim=128, dtype="bf16",
+                          n_extra=extra)
+    w = toma.alloc_weights(desc).zero_()
+    x = torch.empty((1, 64 + extra, d), dtype=torch.bfloat16, device="cuda")
+    x.view(torch.int16).random_()
+    xm = torch.empty((1, 32 + extra, d), dtype=torch.bfloat16, device="cuda")
+    toma.toma_merge(desc, w, x, xm)
+    same = all(torch.equal(x.view(torch.int16)[0, 64 + r: 64 + r + (1 << 19)], xm.view(torch.int16)[0, 32 + r: 32 + r + (1 << 19)])
+               for r in range(0, extra, 1 << 19))
+    del x, xm
+    torch.cuda.empty_cache()
+    assert same
