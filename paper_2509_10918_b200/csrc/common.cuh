@@ -170,6 +170,17 @@ __device__ __forceinline__ void copy_part(const RowCopy& c, size_t thread, size_
     for (size_t e = thread; e < c.per; e += n_threads) dst[e] = src[e];
   }
 }
+cudaError_t launch_copy_rows(const RowCopy& c, cudaStream_t s);
+// Whether `threads` copying threads are done about when the first products are: four packets are in flight per thread and
+// microsecond.  With more to do (few regions, many text tokens) the contraction would wait for its copies: 2 x 256 tokens
+// of 576 channels and 4096 text tokens, merge 89 us beside the contraction and 17 us behind it.
+inline bool copied_beside(const RowCopy& c, long long threads) { return (double)c.per * c.batches <= 16.0 * (double)threads; }
+// The end of a launch: what could not be copied beside it is copied behind it.
+inline cudaError_t finish_launch(cudaError_t e, const RowCopy& rows, const RowCopy& beside, cudaStream_t s) {
+  count_launch();
+  if (e == cudaSuccess) e = cudaGetLastError();
+  return e == cudaSuccess && rows.per != beside.per ? launch_copy_rows(rows, s) : e;
+}
 // bf16, d a multiple of 8: the un-merged trailing tokens of x -> merged rows (merging) or of attended rows -> output.
 inline RowCopy extra_rows(const Geom& g, const void* src, void* dst, bool merging) {
   RowCopy c;

@@ -6,6 +6,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "tc.cuh"
 
 namespace toma {
 
@@ -538,6 +539,19 @@ __global__ void copy_rows_kernel(const T* __restrict__ src, T* __restrict__ dst,
   if (e >= per) return;
   const int b = blockIdx.y;
   dst[(size_t)b * dst_stride + dst_row0 * d + e] = src[(size_t)b * src_stride + src_row0 * d + e];
+}
+
+// Rows of bf16 packets (the tensor-core kernels' text tokens), where too few threads of theirs would copy them.
+__global__ void __launch_bounds__(256) copy_packets_kernel(const RowCopy c) {
+  tc::dependency_wait();  // launched with programmatic stream serialisation
+  if (threadIdx.x == 0) tc::release_dependents();
+  copy_part(c, (size_t)blockIdx.x * 256 + threadIdx.x, (size_t)gridDim.x * 256);
+}
+cudaError_t launch_copy_rows(const RowCopy& c, cudaStream_t s) {
+  const size_t want = (c.per + 4 * 256 - 1) / (4 * 256), most = (size_t)sm_count() * 8;  // four packets per thread, a full chip at most
+  const cudaError_t e = launch_dependent(copy_packets_kernel, dim3((unsigned)(want < most ? want : most)), dim3(256), 0, s, c);
+  count_launch();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename T>

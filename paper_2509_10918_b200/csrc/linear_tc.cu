@@ -44,10 +44,11 @@ struct LinParams {
 
 // The epilogue warps' first work: two launches less per step, 6 us of 125 on joint sequences of 4096 image and 512
 // text tokens of 3072 channels.
+constexpr long long kCopyThreads = 128;  // of a CTA: the four epilogue warps
 // Out of line: sequences without text tokens should not fetch its instructions (0.2 us per launch).
 __device__ __noinline__ void copy_extra(const RowCopy c) {
   const size_t cta = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  copy_part(c, cta * 128 + threadIdx.x - 64, (size_t)gridDim.x * gridDim.y * gridDim.z * 128);
+  copy_part(c, cta * kCopyThreads + threadIdx.x - 64, (size_t)gridDim.x * gridDim.y * gridDim.z * kCopyThreads);
 }
 
 __device__ __forceinline__ uint32_t tmem_cols_for(int n) { return n > 128 ? 256u : n > 64 ? 128u : 64u; }
@@ -781,7 +782,7 @@ cudaError_t launch_merge_tc(const Geom& g, const void* w, const void* x, void* x
   const uint32_t box[4] = {64, (uint32_t)g.tw, (uint32_t)(64 / g.tw), 1};
   if (!encode_tmap_16bit(&tx, x, 4, dims, strides, box) || !encode_w(g, w, &tw, 64)) return cudaErrorInvalidValue;
   LinParams p = make_params(g);
-  p.extra = extra_rows(g, x, xm, true);
+  const RowCopy rows = extra_rows(g, x, xm, true);
   // merged rows as (channel, destination, tile, batch): a store that runs past a tile's D_loc rows is clipped
   CUtensorMap to;
   // Destinations per CTA.  A tile's destinations normally fit one CTA (<= 256).  When they do not (global
@@ -828,15 +829,16 @@ cudaError_t launch_merge_tc(const Geom& g, const void* w, const void* x, void* x
       if (e == cudaSuccess) e = raise_dynamic_smem(merge_persistent_kernel<true>, 227 * 1024, raised_pb);
       if (e != cudaSuccess) return e;
       const int ctas = n_items < sm_count() ? n_items : sm_count();
+      if (copied_beside(rows, ctas * kCopyThreads)) p.extra = rows;
       e = n_blocks > 1 ? launch_dependent(merge_persistent_kernel<true>, dim3(ctas), dim3(192), (size_t)smem_p, s, tx, tw, to, p, n_items, n_chunks,
                                           n_blocks, dev_status)
                        : launch_dependent(merge_persistent_kernel<false>, dim3(ctas), dim3(192), (size_t)smem_p, s, tx, tw, to, p, n_items, n_chunks,
                                           n_blocks, dev_status);
-      count_launch();
-      return e != cudaSuccess ? e : cudaGetLastError();
+      return finish_launch(e, rows, p.extra, s);
     }
     p.stages = 2;
   }
+  if (copied_beside(rows, grid.x * grid.y * grid.z * kCopyThreads)) p.extra = rows;
   if (g.Dloc > kMaxCols) {
     static std::atomic<unsigned long long> raised_b{0};
     e = raise_dynamic_smem(merge_tc_kernel<true>, 200 * 1024, raised_b);
@@ -848,8 +850,7 @@ cudaError_t launch_merge_tc(const Geom& g, const void* w, const void* x, void* x
     if (e != cudaSuccess) return e;
     e = launch_dependent(merge_tc_kernel<false>, grid, dim3(192), (size_t)smem, s, tx, tw, to, p, dev_status);
   }
-  count_launch();
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return finish_launch(e, rows, p.extra, s);
 }
 
 cudaError_t launch_unmerge_tc(const Geom& g, const void* w, const void* y, void* out, uint32_t* dev_status,
@@ -862,7 +863,7 @@ cudaError_t launch_unmerge_tc(const Geom& g, const void* w, const void* y, void*
   if (!encode_tmap_16bit(&ty, y, 3, dims, strides, box) || !encode_w(g, w, &tw, (uint32_t)n_tok))
     return cudaErrorInvalidValue;
   LinParams p = make_params(g);
-  p.extra = extra_rows(g, y, out, false);
+  const RowCopy rows = extra_rows(g, y, out, false);
   // Tokens on M when a region has many destinations, and also when that form fits the SMs in one wave while
   // the channels-on-M grid would spill into a second one (64x64 tokens: 128 CTAs against 320 on 296 slots).
   const int sms = sm_count();
@@ -886,10 +887,10 @@ cudaError_t launch_unmerge_tc(const Geom& g, const void* w, const void* y, void*
       static std::atomic<unsigned long long> raised_rp{0};
       if (cudaError_t e = raise_dynamic_smem(unmerge_rows_persistent_kernel, 227 * 1024, raised_rp); e != cudaSuccess) return e;
       const int ch_blocks = (g.d + kRowsChBlock - 1) / kRowsChBlock;
+      if (copied_beside(rows, sms * kCopyThreads)) p.extra = rows;
       cudaError_t e = launch_dependent(unmerge_rows_persistent_kernel, dim3(sms), dim3(192), (size_t)smem, s, ty, tw128, to, p, rows_ctas,
                                        ch_blocks, dev_status);
-      count_launch();
-      return e != cudaSuccess ? e : cudaGetLastError();
+      return finish_launch(e, rows, p.extra, s);
     }
   }
   if ((g.Dloc > kMaxCols || one_wave) && g.Nloc % 128 == 0) {
@@ -911,9 +912,9 @@ cudaError_t launch_unmerge_tc(const Geom& g, const void* w, const void* y, void*
     const uint32_t obox[4] = {64, (uint32_t)g.tw, (uint32_t)(128 / g.tw), 1};
     if (!encode_tmap_16bit(&to, out, 4, odims, ostrides, obox)) return cudaErrorInvalidValue;
     dim3 grid(g.B * g.P * (g.Nloc / 128), (g.d + kRowsChBlock - 1) / kRowsChBlock);
+    if (copied_beside(rows, grid.x * grid.y * kCopyThreads)) p.extra = rows;
     cudaError_t e = launch_dependent(unmerge_rows_kernel, grid, dim3(192), (size_t)smem, s, ty, tw128, to, p, dev_status);
-    count_launch();
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return finish_launch(e, rows, p.extra, s);
   }
   // output tokens as (channel, x, y, batch): a CTA's token block is n_tok / tile_w whole tile rows
   CUtensorMap to;
@@ -929,9 +930,9 @@ cudaError_t launch_unmerge_tc(const Geom& g, const void* w, const void* y, void*
   cudaError_t e = raise_dynamic_smem(unmerge_tc_kernel, 200 * 1024, raised);
   if (e != cudaSuccess) return e;
   dim3 grid(g.B * g.P, (g.d + 127) / 128, g.Nloc / n_tok);
+  if (copied_beside(rows, grid.x * grid.y * grid.z * kCopyThreads)) p.extra = rows;
   e = launch_dependent(unmerge_tc_kernel, grid, dim3(192), (size_t)smem, s, ty, tw, to, p, n_tok, dev_status);
-  count_launch();
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return finish_launch(e, rows, p.extra, s);
 }
 
 }  // namespace toma

@@ -351,7 +351,7 @@ cudaError_t launch_ragged(const Geom& g, const void* w, const void* in, void* ou
   p.w_end = (const uint8_t*)w + (size_t)g.B * g.P * g.Nloc * g.Dloc * 4;
   p.zero = (uint32_t*)zero;
   p.zero_words = (int)(zero_bytes / 4);
-  p.extra = extra_rows(g, in, out, kMerge);
+  const RowCopy rows = extra_rows(g, in, out, kMerge);
   CUtensorMap tb, tbt, to, tot;
   bool ok;
   if (kMerge) ok = token_map(g, in, p.rows, &tb) && token_map(g, in, tail, &tbt) && merged_map(g, out, 128, &to);
@@ -375,9 +375,9 @@ cudaError_t launch_ragged(const Geom& g, const void* w, const void* in, void* ou
   static std::atomic<unsigned long long> raised{0};
   if (cudaError_t e = raise_dynamic_smem(ragged_kernel<kMerge>, 227 * 1024, raised); e != cudaSuccess) return e;
   const dim3 grid((unsigned)((g.d + p.nch - 1) / p.nch), (unsigned)m_blocks, (unsigned)(g.B * g.P));
+  if (copied_beside(rows, (long long)grid.x * grid.y * grid.z * kWorkers)) p.extra = rows;
   const cudaError_t e = launch_dependent(ragged_kernel<kMerge>, grid, dim3(64 + kWorkers), (size_t)smem, s, tb, tbt, to, tot, p, dev_status);
-  count_launch();
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return finish_launch(e, rows, p.extra, s);
 }
 
 }  // namespace

@@ -1321,3 +1321,22 @@ def test_text_rows_of_more_than_2_31_packets(toma):
     del x, xm
     torch.cuda.empty_cache()
     assert same
+
+
+@pytest.mark.parametrize("th,tw,dim,extra", [(8, 16, 64, 1), (8, 16, 64, 515), (16, 16, 320, 700), (7, 9, 72, 333), (32, 32, 640, 2000)])
+def test_text_rows_beside_and_behind_the_contraction(toma, th, tw, dim, extra):
+    """Few regions and many text tokens: copied by the contraction's own threads or, where those are too few, behind it."""
+    desc = toma.make_desc(batch=2, grid_h=th, grid_w=tw, dim=dim, tile_h=th, tile_w=tw, merge_ratio=0.5, tau=0.1, n_heads=dim // 8, head_dim=8,
+                          dtype="bf16", n_extra=extra)
+    w = toma.alloc_weights(desc).zero_()
+    d_loc = toma.toma_dest_per_tile(desc)
+    x = torch.randn(2, th * tw + extra, dim, device="cuda").to(torch.bfloat16)
+    xm = torch.full((2, d_loc + extra, dim), float("nan"), dtype=x.dtype, device="cuda")
+    out = torch.full_like(x, float("nan"))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    toma.toma_merge(desc, w, x, xm, status)
+    toma.toma_unmerge(desc, w, xm, out, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert torch.equal(xm[:, d_loc:], x[:, th * tw:]) and torch.equal(out[:, th * tw:], x[:, th * tw:])
+    assert not xm[:, :d_loc].any() and not out[:, :th * tw].any()
