@@ -812,7 +812,9 @@ cudaError_t launch_four(int B, int L, int heads, const void* q, const void* k, c
 // Key tiles of the longest span from which on four pipelines win at head_dim 64: their join at the end of a piece and the
 // larger block cost a CTA what it gains in about six tiles (timed on 260 shapes: one to four tiles 0.85 to 1.0 times as
 // fast, eight 1.01 to 1.12, sixteen 1.08, a hundred 1.15 to 1.2).
-constexpr int kFourFrom = 8;
+// Spans cut inside units end in pieces, whose reading and adding up costs four pipelines more: there it takes fourteen (4 x
+// 512 tokens, 23 heads, spans of eleven: 24 us against 20).
+constexpr int kFourFrom = 8, kFourFromSplit = 14;
 
 }  // namespace
 
@@ -852,7 +854,7 @@ cudaError_t launch_attention_tc(int B, int L, int heads, int dh, const void* q, 
   plan_spans((int)units, nblk, &sp);
   if (sp.split && !tickets_clean)  // units are split: their tickets start at zero
     if (cudaError_t e = cudaMemsetAsync(ws, 0, ticket_bytes(B, L, heads), s); e != cudaSuccess) return e;
-  if (dh == 64 && sp.longest >= kFourFrom) return launch_four(B, L, heads, q, k, v, o, ws, sp, dev_status, s);
+  if (dh == 64 && sp.longest >= (sp.split ? kFourFromSplit : kFourFrom)) return launch_four(B, L, heads, q, k, v, o, ws, sp, dev_status, s);
   return launch_attention_two(B, L, heads, dh, q, k, v, o, ws, sp, dev_status, s);
 }
 
