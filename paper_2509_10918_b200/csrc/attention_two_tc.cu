@@ -333,7 +333,7 @@ __device__ __noinline__ void settle_first_piece(Barriers* bar, int it_begin, int
   const bool first_partial = it_begin > u * nblk || it_end < (u + 1) * nblk;
   if (!first_partial || it_end <= (u + 1) * nblk) return;  // whole, or also the span's last piece: settled already
   const int g_first = sp.unit_lo[0][blockIdx.x], g_last = sp.unit_hi[0][blockIdx.x];
-  if (!mbar_wait(&bar->pub_done, 0, dev_status, &bar->abort_flag)) return;
+  if (!mbar_wait_warp(&bar->pub_done, 0, dev_status, &bar->abort_flag)) return;
   if (bar->first_ticket[t.warp] != (uint32_t)(g_last - g_first)) return;
   __threadfence();
   combine_rows<DH, DH, 64, 8>(pieces, sp, u, g_first, g_last, t.row, 0, out_row<DH>(o, u, t.row, L, heads));

@@ -301,7 +301,7 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         const SlabRow cur = w0;
         w0 = w1;
         if (i + 2 < n_build) w1 = load_slab_row(p, b, unit * 8 + 2 * ((i + 2) % n_pairs), r);
-        if (i >= 2 && !mbar_wait(&bar->slab_empty[s], ((i >> 1) - 1) & 1, dev_status, abort_flag)) { ok = false; break; }
+        if (i >= 2 && !mbar_wait_warp(&bar->slab_empty[s], ((i >> 1) - 1) & 1, dev_status, abort_flag)) { ok = false; break; }
         store_slab_row(sA + 2 * s * kPairBytes, cur, r);
         fence_proxy_async();
         __syncwarp();
@@ -311,7 +311,7 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       // merged rows of every group of four tiles: tensor memory -> bf16 rows of the shared matrix
       const uint32_t peer = (uint32_t)(unit ^ 1);
       for (int g = 0; g < n_pairs / 2; ++g) {
-        if (!mbar_wait(&bar->acc_full[g], 0, dev_status, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(&bar->acc_full[g], 0, dev_status, abort_flag)) { ok = false; break; }
         tc_fence_after();
         uint8_t* rows = sKV + (unit * 2 + g) * kPairBytes + quarter * 4096;  // this warp's 32 rows
         row_to_smem(tmem + lane_addr + g * 64, sKV + (unit * 2 + g) * kPairBytes, r, 1.f);
@@ -336,7 +336,7 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     for (int n = 0; ok && n < nblk; ++n) {
       const int bb = n & 1;
       const uint32_t sb = tmem + lane_addr + (2 * q + bb) * kBN;
-      if (!mbar_wait(&bar->s_full[q][bb], (n >> 1) & 1, dev_status, abort_flag)) { ok = false; break; }
+      if (!mbar_wait_warp(&bar->s_full[q][bb], (n >> 1) & 1, dev_status, abort_flag)) { ok = false; break; }
       tc_fence_after();
       softmax_tile<64, true, false>(sb, ob, p.scale_log2, kBN, n, m_used, l, &bar->pv_done[(n + 3) & 3], (uint32_t)(((n - 1) >> 2) & 1), dev_status,
                                     abort_flag);
@@ -347,7 +347,7 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     // normalised accumulator -> bf16 rows in shared memory (the unmerge's B operand)
     SlabRow w3;
     if (q == 1) w3 = load_slab_row(p, b, unit * 8 + 6, r);  // the unmerge's fourth pair; needed after the next wait
-    if (ok) ok = mbar_wait(&bar->o_done[q], 0, dev_status, abort_flag);
+    if (ok) ok = mbar_wait_warp(&bar->o_done[q], 0, dev_status, abort_flag);
     if (ok) {
       tc_fence_after();
       uint32_t rs[16];
@@ -362,7 +362,7 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     // ------------------------------------------------------------------ C
     if (ok && q == 1) {  // the fourth pair's slab takes the stage of the first once its MMAs are done
       const int gi = n_pairs + 2, s = gi & 1;
-      ok = mbar_wait(&bar->slab_empty[s], ((gi >> 1) - 1) & 1, dev_status, abort_flag);
+      ok = mbar_wait_warp(&bar->slab_empty[s], ((gi >> 1) - 1) & 1, dev_status, abort_flag);
       if (ok) {
         store_slab_row(sA + 2 * s * kPairBytes, w3, r);
         fence_proxy_async();
@@ -371,9 +371,9 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       }
     }
     // the rows of K and V become the staging area of the output; the peer must have received its copy of them
-    if (ok && p.units == 2) ok = mbar_wait_cluster(&bar->kv_sent, 0, dev_status, abort_flag);
+    if (ok && p.units == 2) ok = __all_sync(0xffffffffu, mbar_wait_cluster(&bar->kv_sent, 0, dev_status, abort_flag));
     for (int c = 2 * q; ok && c < 2 * q + 2; ++c) {
-      if (!mbar_wait(&bar->c_full[q][c & 1], 0, dev_status, abort_flag)) { ok = false; break; }
+      if (!mbar_wait_warp(&bar->c_full[q][c & 1], 0, dev_status, abort_flag)) { ok = false; break; }
       tc_fence_after();
       uint8_t* stage = sKV + c * kPairBytes;  // K and V are no longer read: every MMA before this accumulator's has completed
       row_to_smem(tmem + lane_addr + (2 * q + (c & 1)) * kBN, stage, r, 1.f);

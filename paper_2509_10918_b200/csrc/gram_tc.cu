@@ -88,7 +88,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     const int quarter = warp & 3;
     const int i = m0 + quarter * 32 + lane;
     const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
-    if (mbar_wait(&bar->done, 0, dev_status, abort_flag)) {
+    if (mbar_wait_warp(&bar->done, 0, dev_status, abort_flag)) {
       tc_fence_after();
       const int pitch = sq_pitch(Nloc);
       const bool wide = pitch % 16 == 0 && (reinterpret_cast<uintptr_t>(sq) & 31) == 0;  // a workspace need only be 16-byte aligned

@@ -176,7 +176,7 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
     if (p.extra.per) copy_extra(p.extra);
     const int quarter = warp & 3, cl = quarter * 32 + lane;
     const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
-    if (mbar_wait(&bar->done, 0, dev_status, abort_flag)) {  // every load has been consumed: the stages are free
+    if (mbar_wait_warp(&bar->done, 0, dev_status, abort_flag)) {  // every load has been consumed: the stages are free
       tc_fence_after();
       stage_and_store(smem, bar, taddr, cl, n_dest, p.out_rows, dev_status, [&] {
         for (int c = 0; c < 2; ++c)
@@ -429,7 +429,7 @@ unmerge_tc_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_constan
     if (p.extra.per) copy_extra(p.extra);
     const int quarter = warp & 3, cl = quarter * 32 + lane;
     const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
-    if (mbar_wait(&bar->done, 0, dev_status, abort_flag)) {
+    if (mbar_wait_warp(&bar->done, 0, dev_status, abort_flag)) {
       tc_fence_after();
       // rows of the staged tile = the CTA's token slots in tile order = the (x, y) box of the output map
       const int ty = tile / p.tiles_x, tx = tile - ty * p.tiles_x;
@@ -538,7 +538,7 @@ unmerge_rows_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_const
     if (p.extra.per) copy_extra(p.extra);
     const int quarter = warp & 3, row = quarter * 32 + lane;  // token slot t0 + row = tensor-memory lane
     const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
-    if (mbar_wait(&bar->done, 0, dev_status, abort_flag)) {
+    if (mbar_wait_warp(&bar->done, 0, dev_status, abort_flag)) {
       tc_fence_after();
       // every load has been consumed: slab c of the output, [128 tokens][128 B] swizzled, goes to smem + c * 16 KB
       for (int c = 0; c < n_ch; c += 32) {  // accumulator column = channel (the second accumulator starts at 192)

@@ -102,6 +102,11 @@ __device__ __forceinline__ void copy_to_peer(uint32_t peer_dst, const void* src,
 __device__ __forceinline__ void mbar_arrive_peer(uint32_t addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
+// One answer for the warp, which a branch around warp-wide operations (tensor-memory loads and stores, votes, shuffles)
+// needs: lanes poll on their own, and at the limit one may see the phase complete that another gave up on.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, uint32_t* dev_status, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, dev_status, abort_flag));
+}
 // mbar_wait() whose acquire spans the cluster: the barrier also counts bytes the peer CTA sends.
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, uint32_t* dev_status, volatile int* abort_flag) {
   for (uint32_t it = 0; it < kSpinLimit; ++it) {

@@ -233,7 +233,7 @@ weights_gram_kernel(const float* __restrict__ G, const int32_t* __restrict__ idx
       mbar_arrive_peer(peer_addr(smem_u32(&bar->z_in), (uint32_t)q));
     }
   }
-  const bool got = n_cta == 1 || mbar_wait_cluster(&bar->z_in, 0, dev_status, &bar->abort_flag);
+  const bool got = n_cta == 1 || __all_sync(0xffffffffu, mbar_wait_cluster(&bar->z_in, 0, dev_status, &bar->abort_flag));
   for (int i = t; i < Dl; i += blockDim.x) {
     float z = 0.f;
     for (int q = 0; q < n_cta; ++q) z += zpart[q * Dl + i];  // strips in rank order, in every CTA

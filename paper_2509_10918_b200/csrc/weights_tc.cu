@@ -157,7 +157,7 @@ weights_logits_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     const bool valid = k_loc < p.m_tok;
     const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
     float* zrow = zw + quarter * Dl;
-    if (mbar_wait(&bar->done, 0, dev_status, abort_flag)) {
+    if (mbar_wait_warp(&bar->done, 0, dev_status, abort_flag)) {
       tc_fence_after();
       const bool wide = p.Dloc % 8 == 0 && (reinterpret_cast<uintptr_t>(shares) & 31) == 0;
       if (p.raw) {  // scaled logits only: the row's other destination blocks are in other CTAs
@@ -345,7 +345,7 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     const uint32_t taddr = tmem + mb * ncols_mb + ((uint32_t)(quarter * 32) << 16);
     float* zrow = zw + (mb * 4 + quarter) * Dl;
     float inv = 0.f;
-    const bool ok = mbar_wait(&bar->done, 0, dev_status, abort_flag);
+    const bool ok = mbar_wait_warp(&bar->done, 0, dev_status, abort_flag);
     if (ok) {
       tc_fence_after();
       // pass 1: maximum logit over the destinations
@@ -414,7 +414,7 @@ weights_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         st_peer_f32(peer_z + 4u * (uint32_t)i, z);
       }
       mbar_arrive_peer(peer_addr(smem_u32(&bar->z_in), peer));
-      const bool got = mbar_wait_cluster(&bar->z_in, 0, dev_status, abort_flag);
+      const bool got = __all_sync(0xffffffffu, mbar_wait_cluster(&bar->z_in, 0, dev_status, abort_flag));
       for (int i = threadIdx.x - 64; i < Dl; i += 128) {
         const float z = !got ? 0.f : half == 0 ? zinv[i] + zpeer[i] : zpeer[i] + zinv[i];
         zinv[i] = z > 0.f ? 1.f / z : 0.f;
