@@ -853,6 +853,22 @@ cudaError_t launch_merge_tc(const Geom& g, const void* w, const void* x, void* x
   return finish_launch(e, rows, p.extra, s);
 }
 
+// Whether the SMs, each taking every sms-th item, end about when they would if every SM took the next item as it comes free.
+// Channel blocks are not alike where the last is narrow: 78 token blocks x 1664 channels (five blocks of 320 and one of 64)
+// give some SMs 1280 channels and others 768, which made the walk 159 us where one CTA per item takes 132.
+static bool walks_evenly(int items, int d, int sms) {
+  const int ch_blocks = (d + kRowsChBlock - 1) / kRowsChBlock, last = d - (ch_blocks - 1) * kRowsChBlock;
+  long long most = 0;
+  for (int c = 0; c < sms && c < items; ++c) {
+    long long load = 0;
+    for (int item = c; item < items; item += sms) load += item % ch_blocks == ch_blocks - 1 ? last : kRowsChBlock;
+    most = load > most ? load : most;
+  }
+  const int full = items / ch_blocks * (ch_blocks - 1);
+  const long long rounds = (long long)((full + sms - 1) / sms) * kRowsChBlock, even = (long long)(items / ch_blocks) * d / sms;
+  return 5 * most <= 6 * (rounds > even ? rounds : even) || ch_blocks == 1;
+}
+
 cudaError_t launch_unmerge_tc(const Geom& g, const void* w, const void* y, void* out, uint32_t* dev_status,
                               cudaStream_t s) {
   CUtensorMap ty, tw;
@@ -870,7 +886,7 @@ cudaError_t launch_unmerge_tc(const Geom& g, const void* w, const void* y, void*
   const int rows_ctas = g.B * g.P * (g.Nloc / 128) * ((g.d + kRowsChBlock - 1) / kRowsChBlock);
   const int classic_ctas = g.B * g.P * ((g.d + 127) / 128) * (g.Nloc / n_tok);
   const bool one_wave = rows_ctas <= sms && classic_ctas > 2 * sms;
-  if (g.Nloc % 128 == 0 && rows_ctas > sms) {
+  if (g.Nloc % 128 == 0 && rows_ctas > sms && (g.Dloc <= kMaxCols || walks_evenly(rows_ctas, g.d, sms))) {
     // many more items than SMs: tokens on M, one CTA per SM walking its items
     CUtensorMap tw128, to;
     if (!encode_w(g, w, &tw128, 128)) return cudaErrorInvalidValue;
