@@ -16,8 +16,10 @@ namespace toma {
 // Fixed-point cosine similarity constants (see toma_select in toma.h).
 constexpr double kCosScaleTimesOne = 0.99 * 4096.0;  // token length 0.99 in units of 2^-12
 constexpr int kDiagQ = 4014;                          // rint(0.99^2 * 4096)
-// The similarity matrix in the workspace: entry S + kSqBias (unsigned, below 2^13: |S| <= 4014), rows of sq_pitch()
-// entries (16-byte aligned), 0 behind the tile's tokens.
+// The similarity matrix in the workspace: entry S + kSqBias (unsigned, below 2^13), rows of sq_pitch() entries (16-byte
+// aligned), 0 behind the tile's tokens.  |S| <= 4095: rounding a token's d <= 4096 components to whole units adds at most
+// sqrt(d) / 2 <= 32 units to its length of 4055, rounding those to 8 bits a factor of 1 + 2^-9, so it stays below 4096
+// units and |S| below 4096^2 / 4096.  (Equal tokens exceed the diagonal's 4014: 4076 at 3952 equal components.)
 constexpr int kSqBias = 4096;
 __host__ __device__ constexpr int sq_pitch(int nloc) { return (nloc + 7) & ~7; }
 constexpr int kMaxNloc = 1024;

@@ -16,8 +16,8 @@
 // that makes 55 rounds out of 127, on 1024 tokens with 512 destinations 176 out of 511; the picks are the same.
 //
 // Thread = two tokens = one 32-bit word of every row (entries biased to be >= 0, see sq_pitch() in common.cuh): the
-// update of both for one changed column is two 16x2 maxima.  The differences are non-negative and at most 8028, so
-// eight columns add up in a word without a carry between the halves.  Every warp posts its two best keys and its
+// update of both for one changed column is two 16x2 maxima.  The differences are non-negative and at most 8190 (|S| <=
+// 4095), so eight columns add up in a word without a carry between the halves (65520).  Every warp posts its two best keys and its
 // third; the four best of all posted keys are the four best of all as long as they exceed every third.
 #pragma once
 
@@ -38,7 +38,7 @@ __device__ __forceinline__ uint32_t max_u16x2(uint32_t a, uint32_t b) {
 
 // Gain and candidate in one key, 0 = none: the largest key is the largest gain with the lowest index.  A gain is
 // below 2^22: sum_j relu(S_ij - m_j) = (sum |S_ij - m_j| + sum (S_ij - m_j)) / 2, the second sum is not positive
-// for the first pick's m (the largest row sum) and m only grows, so a gain is at most N_loc * 8028 / 2.
+// for the first pick's m (the largest row sum) and m only grows, so a gain is at most N_loc * 8190 / 2 < 2^22.
 constexpr int kIdxBits = 10;
 __device__ __forceinline__ uint32_t make_key(uint32_t gain, int i) { return ((gain << kIdxBits) | (uint32_t)(kMaxNloc - 1 - i)) + 1u; }
 __device__ __forceinline__ int key_index(uint32_t key) { return kMaxNloc - 1 - (int)((key - 1u) & (kMaxNloc - 1)); }

@@ -1340,3 +1340,17 @@ def test_text_rows_beside_and_behind_the_contraction(toma, th, tw, dim, extra):
     assert int(status.item()) == 0
     assert torch.equal(xm[:, d_loc:], x[:, th * tw:]) and torch.equal(out[:, th * tw:], x[:, th * tw:])
     assert not xm[:, :d_loc].any() and not out[:, :th * tw].any()
+
+
+@pytest.mark.parametrize("d", [1024, 2048, 3952])
+@pytest.mark.parametrize("kind", ["one", "opposite"])
+def test_selection_of_equal_tokens_past_unit_similarity(toma, d, kind):
+    """Rounding each component lengthens a token beyond 0.99: equal tokens have a similarity above that of a token with
+    itself (4032, 4050 and 4076 of 4096 at these dims, against 4014), which is what the packed sums of the rounds have to hold."""
+    x = np.ones((1, 1024, d), np.float32)
+    if kind == "opposite":
+        x[0, 1::2] = -1.0
+    cfg = gen.config("cfg2", batch=1, grid_h=32, grid_w=32, tile_h=32, tile_w=32, dim=d, n_heads=d // 16, head_dim=16)
+    idx = Run(toma, cfg, x).select()
+    want, _ = O.select_tile(x[0].astype(np.float64), od(cfg))
+    assert np.array_equal(idx[0, 0], want)
