@@ -151,8 +151,14 @@ def _ptr(t: Optional[torch.Tensor]):
 
 
 def _stream():
-    # the raw handle of torch.cuda.current_stream(), without building a Stream object on every call
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    # the raw handle of torch.cuda.current_stream(), where this torch has it without building a Stream object on every call
+    if _raw_stream is None or _device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_device())
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _check(status: int, where: str):

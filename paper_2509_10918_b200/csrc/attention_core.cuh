@@ -1,6 +1,6 @@
-// Device helpers of the tensor-core attention kernels: the online softmax of one 64-key tile for one
-// query row straight out of tensor memory (see attention_tc.cu for the scheme), and the scaled bf16
-// store of accumulator rows.
+// Device helpers of the tensor-core attention kernels, for one query row straight out of tensor memory: the online softmax
+// of a 64-key tile (attention_two_tc.cu and, in its one instance without a mask at head_dim 64, block_fused_tc.cu) and the
+// exponentials against a reference with headroom (attention_tc.cu).
 #pragma once
 
 #include "common.cuh"
@@ -218,19 +218,6 @@ __device__ __forceinline__ uint64_t rounded_sum2(const uint32_t (&pk)[32]) {
 #pragma unroll
   for (int e = 0; e < 32; ++e) sum2 = add2(sum2, pack2(__uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xFFFF0000u)));
   return sum2;
-}
-
-// 32 accumulator columns of one row, scaled and rounded to bf16: 64 contiguous bytes.
-__device__ __forceinline__ void store_row32(__nv_bfloat16* dst, const uint32_t (&r)[32], float inv) {
-#pragma unroll
-  for (int e = 0; e < 32; e += 8) {
-    uint4 v;
-    v.x = pack_bf16_rn(__uint_as_float(r[e]) * inv, __uint_as_float(r[e + 1]) * inv);
-    v.y = pack_bf16_rn(__uint_as_float(r[e + 2]) * inv, __uint_as_float(r[e + 3]) * inv);
-    v.z = pack_bf16_rn(__uint_as_float(r[e + 4]) * inv, __uint_as_float(r[e + 5]) * inv);
-    v.w = pack_bf16_rn(__uint_as_float(r[e + 6]) * inv, __uint_as_float(r[e + 7]) * inv);
-    *reinterpret_cast<uint4*>(dst + e) = v;
-  }
 }
 
 }  // namespace attn

@@ -199,8 +199,10 @@ cudaError_t run_dtype(int B, int L, int heads, int dh, const void* q, const void
   switch (dh) {
     case 16: return run<T, 16>(B, L, heads, q, k, v, o, s);
     case 32: return run<T, 32>(B, L, heads, q, k, v, o, s);
-    case 64: return run<T, 64>(B, L, heads, q, k, v, o, s);
-    case 128: return run<T, 128>(B, L, heads, q, k, v, o, s);
+  }
+  if constexpr (sizeof(T) == 4) {  // bf16: on the tensor cores
+    if (dh == 64) return run<T, 64>(B, L, heads, q, k, v, o, s);
+    if (dh == 128) return run<T, 128>(B, L, heads, q, k, v, o, s);
   }
   return cudaErrorInvalidValue;
 }
