@@ -81,7 +81,7 @@ cudaError_t launch_quantise(const Geom& g, const void* x, __nv_bfloat16* y, cuda
 
 // ---------------------------------------------------------------------------
 // Greedy (Algorithm 2), one CTA per tile; the rounds are greedy.cuh's.  The two passes over the whole matrix (row
-// sums for the first pick, initial gains) run on all 16 warps with 16-byte reads; then the warps that own tokens
+// sums for the first pick, initial gains) run on all warps with 16-byte reads; then the warps that own tokens
 // (64 each) go on.  kSmem: the matrix is copied to shared memory during the first pass (up to 336 tokens), which
 // turns the two dependent reads of a round from an L2 round trip into a shared-memory latency.
 // Measured against one pick per round and one thread per token (kernel time, launch included): 32 tiles of 256
@@ -89,11 +89,11 @@ cudaError_t launch_quantise(const Geom& g, const void* x, __nv_bfloat16* y, cuda
 // destinations 1783 -> 695 us (there the rows come from L2 and DRAM, 32 of them in flight per thread; with 8 it
 // was 837 us).
 // ---------------------------------------------------------------------------
-constexpr int kGreedyThreads = 512;
+constexpr int kGreedyThreads = 512;  // at most
 constexpr int kGreedySmemTok = 336;  // 336 x 336 entries and the lists below fill an SM's shared memory
 
 template <bool kOne, bool kSmem>
-__global__ void __launch_bounds__(kGreedyThreads, 1) greedy_kernel(const uint16_t* __restrict__ sq, int32_t* __restrict__ idx, int Nloc,
+__global__ void __launch_bounds__(kOne ? 64 : kGreedyThreads, 1) greedy_kernel(const uint16_t* __restrict__ sq, int32_t* __restrict__ idx, int Nloc,
                                                                 int Dloc) {
   constexpr int kTok = kOne ? 64 : kSmem ? kGreedySmemTok : kMaxNloc;
   extern __shared__ __align__(16) uint32_t greedy_smem[];
@@ -101,15 +101,16 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) greedy_kernel(const uint16_
   __shared__ int total[kTok];  // row sums (biased alike), then initial gains + msum
   __shared__ int msum;
   __shared__ int2 best[16];
+  const int threads = blockDim.x;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int pitch = sq_pitch(Nloc), vecs = pitch / 8;  // 16-byte packets per row
   const uint4* src = reinterpret_cast<const uint4*>(sq + (size_t)blockIdx.x * Nloc * pitch);
-  for (int e = tid; e < kTok; e += kGreedyThreads) total[e] = 0;
+  for (int e = tid; e < kTok; e += threads) total[e] = 0;
   if (tid == 0) msum = 0;
   tc::dependency_wait();  // launched with programmatic stream serialisation
   if (tid == 0) tc::release_dependents();
   __syncthreads();
-  const int v = tid % vecs, n_rg = kGreedyThreads / vecs, rg = tid / vecs;  // this thread's packet of a row, and its rows
+  const int v = tid % vecs, n_rg = threads / vecs, rg = tid / vecs;  // this thread's packet of a row, and its rows
   const uint4* S4 = kSmem ? reinterpret_cast<const uint4*>(greedy_smem) : src;
   int acc[8];
   auto add8 = [&](const uint32_t (&t)[4]) {
@@ -146,7 +147,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) greedy_kernel(const uint16_
   // ---- first pick: the largest row sum, the lowest index on ties
   {
     int s = -1, i = kMaxNloc;
-    for (int e = tid; e < Nloc; e += kGreedyThreads)
+    for (int e = tid; e < Nloc; e += threads)
       if (total[e] > s) s = total[e], i = e;
     const int bs = __reduce_max_sync(0xffffffffu, s);
     const int bi = __reduce_min_sync(0xffffffffu, s == bs ? i : kMaxNloc);
@@ -155,11 +156,11 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) greedy_kernel(const uint16_
   __syncthreads();
   int first;
   {
-    const int2 b = lane < 16 ? best[lane] : make_int2(-1, kMaxNloc);
+    const int2 b = lane < threads / 32 ? best[lane] : make_int2(-1, kMaxNloc);
     const int bs = __reduce_max_sync(0xffffffffu, b.x);
     first = __reduce_min_sync(0xffffffffu, b.x == bs ? b.y : kMaxNloc);
   }
-  for (int e = tid; e < kTok; e += kGreedyThreads) total[e] = 0;
+  for (int e = tid; e < kTok; e += threads) total[e] = 0;
   __syncthreads();
 
   // ---- initial gains: g_i = sum_j max(S[j][i], m_j) - sum_j m_j with m = the first pick's row
@@ -189,7 +190,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) greedy_kernel(const uint16_
   post8();
   {
     int ms = 0;
-    for (int e = tid; e < Nloc; e += kGreedyThreads) ms += mrow[e];
+    for (int e = tid; e < Nloc; e += threads) ms += mrow[e];
     ms = __reduce_add_sync(0xffffffffu, ms);
     if (lane == 0 && ms) atomicAdd(&msum, ms);
   }
@@ -211,14 +212,18 @@ static cudaError_t run_greedy(const Geom& g, const uint16_t* sq, int32_t* idx, c
   if (kSmem)
     if (cudaError_t e = raise_dynamic_smem(greedy_kernel<kOne, kSmem>, kOne ? 64 * 64 * 2 : kGreedySmemTok * kGreedySmemTok * 2, raised); e != cudaSuccess)
       return e;
-  // Rows in global memory: not launched before its predecessor ends.  CTAs placed then are spread over the chip, those
-  // placed beside the predecessor's last ones crowd where there is room first, and share the paths to L2 that bound the
-  // rounds (64 tiles of 1024 tokens: 600 us against 543 us).
-  if (!kSmem) {
-    greedy_kernel<kOne, kSmem><<<g.B * g.P, kGreedyThreads, smem, s>>>(sq, idx, g.Nloc, g.Dloc);
+  // A region's threads: enough for its two passes over the matrix, few enough that many small regions share an SM (with 512
+  // for every size selection of 408 regions of 64 tokens took 53 us and takes 34, of 644 regions of 16 tokens 33 and 16).
+  const int threads = g.Nloc <= 64 ? 64 : g.Nloc <= 128 ? 128 : g.Nloc <= 192 ? 256 : kGreedyThreads;
+  // Rows in global memory, and few threads in no more regions than there are SMs: not launched before the predecessor ends.
+  // CTAs placed then are spread over the chip, those placed beside the predecessor's last ones crowd where there is room
+  // first, and share the paths to L2 that bound the rounds (64 tiles of 1024 tokens: 600 us against 543 us), or an SM's
+  // issue slots (144 of 128 tokens: 90 us against 60).
+  if (!kSmem || (threads < kGreedyThreads && g.B * g.P <= sm_count())) {
+    greedy_kernel<kOne, kSmem><<<g.B * g.P, threads, smem, s>>>(sq, idx, g.Nloc, g.Dloc);
     return cudaGetLastError();
   }
-  return launch_dependent(greedy_kernel<kOne, kSmem>, dim3(g.B * g.P), dim3(kGreedyThreads), smem, s, sq, idx, g.Nloc, g.Dloc);
+  return launch_dependent(greedy_kernel<kOne, kSmem>, dim3(g.B * g.P), dim3(threads), smem, s, sq, idx, g.Nloc, g.Dloc);
 }
 
 cudaError_t launch_greedy(const Geom& g, const uint16_t* sq, int32_t* idx, cudaStream_t s) {
