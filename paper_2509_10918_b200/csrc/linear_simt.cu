@@ -70,6 +70,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, KG > 1 || BM == 12
   __shared__ __align__(16) float Bs[2][kBK][BN];
   const int batch = blockIdx.z, m0 = blockIdx.y * BM, n0 = blockIdx.x * BN, tid = threadIdx.x;
   const int in_group = tid % kGroup, kg = tid / kGroup;
+  tc::dependency_wait();  // launched with programmatic stream serialisation
+  if (tid == 0) tc::release_dependents();
   const int tn = in_group % (BN / TN) * 4, tm = in_group / (BN / TN) * TM;  // columns tn .. + 3, and with TN = 8 BN / 2 further on
   // packet e of an operand: k along the line: line e / 4, k 4 (e % 4); else: k e / (rows / 4), rows 4 (e % (rows / 4))
   float4 ra[kVecA], rb[kVecB];
@@ -359,7 +361,7 @@ struct UnmergeOp {
 template <class Op, typename AccT, int BM, int BN, int TM, int TN, int KG = 1>
 static void run_tile(const Op& op, int batches, cudaStream_t s) {
   const dim3 grid((op.N + BN - 1) / BN, (op.M + BM - 1) / BM, batches);
-  simt_gemm_kernel<Op, AccT, BM, BN, TM, TN, KG><<<grid, (BM / TM) * (BN / TN) * KG, 0, s>>>(op);
+  launch_dependent(simt_gemm_kernel<Op, AccT, BM, BN, TM, TN, KG>, grid, dim3((BM / TM) * (BN / TN) * KG), 0, s, op);  // errors: cudaGetLastError
   count_launch();
 }
 
@@ -411,6 +413,8 @@ __global__ void __launch_bounds__(kSoftThreads) softmax_dest_kernel(float* __res
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = blockIdx.x * kSoftTok + lane;
   constexpr int kWarps = kSoftThreads / 32;
   const bool live = k < Nloc;
+  tc::dependency_wait();
+  if (threadIdx.x == 0) tc::release_dependents();
   float* L = logits + (size_t)blockIdx.y * Dloc * Nloc + (live ? k : 0);
   float mx = -INFINITY;
 #pragma unroll 8
@@ -442,6 +446,8 @@ __global__ void __launch_bounds__(kSoftThreads) softmax_dest_kernel(float* __res
 // The same without shared memory for more destinations than it holds (global merge): one thread per source token.
 __global__ void __launch_bounds__(128) softmax_dest_long_kernel(float* __restrict__ logits, int Nloc, int Dloc) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  tc::dependency_wait();
+  if (threadIdx.x == 0) tc::release_dependents();
   if (k >= Nloc) return;
   float* L = logits + (size_t)blockIdx.y * Dloc * Nloc + k;
   float mx = -INFINITY;
@@ -470,25 +476,34 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const float* __restrict__ 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int batch = blockIdx.y, i0 = blockIdx.x * 32;
   const int ni = min(32, Dloc - i0);
+  tc::dependency_wait();
+  if (threadIdx.x == 0) tc::release_dependents();
   const float* a = A + ((size_t)batch * Dloc + i0) * Nloc;
-  for (int r = warp; r < ni; r += 8) {
-    float z = 0.f;
-#pragma unroll 8
-    for (int k = lane; k < Nloc; k += 32) z += a[(size_t)r * Nloc + k];
+  {  // a warp's four rows side by side
+    const int r0 = warp * 4;
+    float z[4] = {};
+#pragma unroll 4
+    for (int k = lane; k < Nloc; k += 32)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-    if (lane == 0) inv[r] = z > 0.f ? 1.f / z : 0.f;
+      for (int u = 0; u < 4; ++u)
+        if (r0 + u < ni) z[u] += a[(size_t)(r0 + u) * Nloc + k];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) z[u] += __shfl_xor_sync(0xffffffffu, z[u], o);
+      if (lane == 0 && r0 + u < ni) inv[r0 + u] = z[u] > 0.f ? 1.f / z[u] : 0.f;
+    }
   }
   __syncthreads();
   const size_t plane = (size_t)Nloc * Dloc;
   for (int k0 = (blockIdx.z * 8 + warp) * 32; k0 < Nloc; k0 += gridDim.z * 256) {
     const int nk = min(32, Nloc - k0);
-#pragma unroll 16
+#pragma unroll
     for (int r = 0; r < 32; ++r) tr[warp][lane][r] = r < ni && lane < nk ? a[(size_t)r * Nloc + k0 + lane] : 0.f;
     __syncwarp();
     if (lane < ni) {
       const float f = inv[lane];
-#pragma unroll 4
+#pragma unroll 8
       for (int k = 0; k < nk; ++k) {
         const float v = tr[warp][k][lane];
         const size_t off = (size_t)(k0 + k) * Dloc + i0 + lane;
@@ -500,34 +515,156 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const float* __restrict__ 
   }
 }
 
+// Logits of bf16 tokens, <X[idx_i], X_k> * scale, every sum one chain of fused multiply-adds in ascending channels: the same
+// bits as the general kernel above gives.  What bounds it is the FMA pipe (a product is 2 N_loc D_loc d operations of the
+// 75 TFLOP/s it has) as long as operands keep coming, and the general kernel's did not: its stages of 16 channels, one
+// ahead, cover a third of a load's latency, and it converts and transposes them on the way.  Here the rows travel as they
+// are, by cp.async, kStages - 1 stages of 64 channels ahead, and are widened in registers as they are read (a shift or a mask,
+// on the ALU pipe beside the FMAs).  Rows lie 144 bytes apart, so that eight threads read eight rows' 16 bytes at once.
+// Thread = TM x TN outputs, rows tm + u BM / TM and columns tn + u BN / TN.  Logits, softmax and normalisation of 384 regions of
+// 96 tokens of 1280 channels 355 -> 163 us, of 32 of 252 tokens of 640 channels 92 -> 55, of 3 of 126 tokens 53 -> 18.
+constexpr int kLogitK = 64, kLogitPitch = kLogitK * 2 + 16;
+template <int BM, int BN>
+constexpr int logit_stages() { return BM + BN > 64 ? 4 : 6; }
+template <int BM, int BN>
+constexpr int logit_smem() { return logit_stages<BM, BN>() * (BM + BN) * kLogitPitch + (BM + BN) * 8; }
+
+__device__ __forceinline__ void cp_async16(uint32_t smem, const void* src, bool real) {  // zeros where nothing is read
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem), "l"(src), "r"(real ? 16 : 0) : "memory");
+}
+
+template <int BM, int BN, int TM, int TN>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN)) logits_kernel(const LogitsOp<__nv_bfloat16> op) {
+  constexpr int kStages = logit_stages<BM, BN>(), kRows = BM + BN, kStageBytes = kRows * kLogitPitch;
+  constexpr int kGm = BM / TM, kGn = BN / TN, kThreads = kGm * kGn, kPackets = kRows * 8 / kThreads;
+  static_assert(kRows * 8 % kThreads == 0, "tile form");
+  extern __shared__ __align__(16) uint8_t logit_smem_raw[];
+  const __nv_bfloat16** row = reinterpret_cast<const __nv_bfloat16**>(logit_smem_raw + kStages * kStageBytes);
+  const int tid = threadIdx.x, batch = blockIdx.z, m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const int tn = tid % kGn, tm = tid / kGn;
+  tc::dependency_wait();  // launched with programmatic stream serialisation
+  if (tid == 0) tc::release_dependents();
+  for (int e = tid; e < kRows; e += kThreads) {
+    const int i = e < BM ? m0 + e : n0 + e - BM;
+    row[e] = i < (e < BM ? op.M : op.N) ? (e < BM ? op.a_ptr(batch, i) : op.b_ptr(batch, i)) : nullptr;
+  }
+  __syncthreads();
+  const uint32_t base = tc::smem_u32(logit_smem_raw);
+  const int nk = (op.K + kLogitK - 1) / kLogitK;
+  auto fetch = [&](int ks) {
+    if (ks < nk) {
+#pragma unroll
+      for (int v = 0; v < kPackets; ++v) {
+        const int e = tid + v * kThreads, r = e >> 3, c = ks * kLogitK + (e & 7) * 8;
+        const __nv_bfloat16* p = row[r];
+        const bool real = p != nullptr && c < op.K;
+        cp_async16(base + (ks % kStages) * kStageBytes + r * kLogitPitch + (e & 7) * 16, real ? p + c : op.x, real);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  Sum2f acc[TM][TN / 2] = {};
+#pragma unroll 1
+  for (int ks = 0; ks < kStages - 1; ++ks) fetch(ks);
+#pragma unroll 1
+  for (int ks = 0; ks < nk; ++ks) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+    __syncthreads();         // stage ks is there for all, stage ks - 1 read by all
+    fetch(ks + kStages - 1);
+    const uint8_t* st = logit_smem_raw + (ks % kStages) * kStageBytes;
+#pragma unroll 2
+    for (int c = 0; c < 8; ++c) {
+      uint4 a[TM], b[TN];
+#pragma unroll
+      for (int u = 0; u < TM; ++u) a[u] = *reinterpret_cast<const uint4*>(st + (tm + u * kGm) * kLogitPitch + c * 16);
+#pragma unroll
+      for (int u = 0; u < TN; ++u) b[u] = *reinterpret_cast<const uint4*>(st + (BM + tn + u * kGn) * kLogitPitch + c * 16);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        auto wide = [&](const uint4& q) {
+          const uint32_t h = (e >> 1) == 0 ? q.x : (e >> 1) == 1 ? q.y : (e >> 1) == 2 ? q.z : q.w;
+          return __uint_as_float(e & 1 ? h & 0xFFFF0000u : h << 16);
+        };
+        uint64_t b2[TN / 2];
+#pragma unroll
+        for (int u = 0; u < TN / 2; ++u) b2[u] = tc::pack2(wide(b[2 * u]), wide(b[2 * u + 1]));
+#pragma unroll
+        for (int u = 0; u < TM; ++u) {
+          const float av = wide(a[u]);
+          const uint64_t a2 = tc::pack2(av, av);
+#pragma unroll
+          for (int q = 0; q < TN / 2; ++q) acc[u][q].fma(a2, b2[q]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < TM; ++u) {
+    const int m = m0 + tm + u * kGm;
+    if (m >= op.M) break;
+    float* dst = op.logits + ((size_t)batch * op.M + m) * op.N;
+#pragma unroll
+    for (int q = 0; q < TN / 2; ++q) {
+      float v[2];
+      acc[u][q].get(v);
+      const int n = n0 + tn + 2 * q * kGn;
+      if (n < op.N) dst[n] = v[0] * op.scale;
+      if (n + kGn < op.N) dst[n + kGn] = v[1] * op.scale;
+    }
+  }
+}
+
+template <int BM, int BN, int TM, int TN>
+static cudaError_t run_logits(const LogitsOp<__nv_bfloat16>& op, int batches, cudaStream_t s) {
+  static std::atomic<unsigned long long> raised{0};
+  if (cudaError_t e = raise_dynamic_smem(logits_kernel<BM, BN, TM, TN>, logit_smem<BM, BN>(), raised); e != cudaSuccess) return e;
+  const dim3 grid((op.N + BN - 1) / BN, (op.M + BM - 1) / BM, batches);
+  count_launch();
+  return launch_dependent(logits_kernel<BM, BN, TM, TN>, grid, dim3((BM / TM) * (BN / TN)), logit_smem<BM, BN>(), s, op);
+}
+// The form that is through first.  Timed on thirteen shapes (microseconds per tile and 640 channels on the fullest SM): 64 x 64
+// takes 18 while an SM has few of them and 14.5 among many; 64 x 32 by 64 threads takes 8, but 18 where there is nothing
+// beside it; 32 x 32 by 128 threads 5.3, alone as well.
+static cudaError_t launch_logits(const LogitsOp<__nv_bfloat16>& op, int batches, cudaStream_t s) {
+  auto on_an_sm = [&](int bm, int bn) {
+    const long long ctas = (long long)((op.M + bm - 1) / bm) * ((op.N + bn - 1) / bn) * batches;
+    return (double)((ctas + sm_count() - 1) / sm_count());
+  };
+  const double n = on_an_sm(64, 64), large = n * (n > 4 ? 14.5 : 18.0), tall = fmax(18.0, 8.0 * on_an_sm(64, 32)), small = 5.3 * on_an_sm(32, 32);
+  if (large <= tall && large <= small) return run_logits<64, 64, 4, 8>(op, batches, s);
+  return tall <= small ? run_logits<64, 32, 4, 8>(op, batches, s) : run_logits<32, 32, 2, 4>(op, batches, s);
+}
+
 cudaError_t launch_weights_simt(const Geom& g, const void* x, const int32_t* idx, void* w, void* wu, float* logits,
                                 cudaStream_t s) {
   const int batches = g.B * g.P;
+  cudaError_t e;
   if (g.f32) {  // fp32 mode sums the logits in double: a logit of some hundreds has to be right to its last fp32 bit
     LogitsOp<float> op{g.Dloc, g.Nloc, g.d, true, true, make_map(g), (const float*)x, idx, logits, g.logit_scale};
     run_gemm<LogitsOp<float>, double>(op, batches, s);
   } else {
     LogitsOp<__nv_bfloat16> op{g.Dloc, g.Nloc, g.d, true, true, make_map(g), (const __nv_bfloat16*)x, idx, logits, g.logit_scale};
-    run_gemm<LogitsOp<__nv_bfloat16>, float>(op, batches, s);
+    if ((e = launch_logits(op, batches, s)) != cudaSuccess) return e;
   }
   const size_t smem = (size_t)g.Dloc * kSoftTok * 4;
   if (smem <= 200 * 1024) {
     static std::atomic<unsigned long long> raised{0};
-    if (cudaError_t e = raise_dynamic_smem(softmax_dest_kernel, 200 * 1024, raised); e != cudaSuccess) return e;
-    softmax_dest_kernel<<<dim3((g.Nloc + kSoftTok - 1) / kSoftTok, batches), kSoftThreads, smem, s>>>(logits, g.Nloc, g.Dloc);
+    if ((e = raise_dynamic_smem(softmax_dest_kernel, 200 * 1024, raised)) != cudaSuccess) return e;
+    e = launch_dependent(softmax_dest_kernel, dim3((g.Nloc + kSoftTok - 1) / kSoftTok, batches), dim3(kSoftThreads), smem, s, logits, g.Nloc, g.Dloc);
   } else {
-    softmax_dest_long_kernel<<<dim3((g.Nloc + 127) / 128, batches), 128, 0, s>>>(logits, g.Nloc, g.Dloc);
+    e = launch_dependent(softmax_dest_long_kernel, dim3((g.Nloc + 127) / 128, batches), dim3(128), 0, s, logits, g.Nloc, g.Dloc);
   }
+  if (e != cudaSuccess) return e;
   count_launch();
   // a CTA per 32 destinations, their source tokens split further where that leaves SMs idle (each part sums the rows anew)
   const int blocks = (g.Dloc + 31) / 32;
-  int parts = 1;
-  while (parts < 8 && (long long)blocks * batches * parts < sm_count() && parts * 256 < g.Nloc) parts *= 2;
-  const dim3 grid(blocks, batches, parts);
-  if (g.f32) rownorm_kernel<float><<<grid, 256, 0, s>>>(logits, (float*)w, (float*)wu, g.Nloc, g.Dloc);
-  else rownorm_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(logits, (__nv_bfloat16*)w, (__nv_bfloat16*)wu, g.Nloc, g.Dloc);
+  int row_parts = 1;
+  while (row_parts < 8 && (long long)blocks * batches * row_parts < sm_count() && row_parts * 256 < g.Nloc) row_parts *= 2;
+  const dim3 grid(blocks, batches, row_parts);
+  e = g.f32 ? launch_dependent(rownorm_kernel<float>, grid, dim3(256), 0, s, logits, (float*)w, (float*)wu, g.Nloc, g.Dloc)
+            : launch_dependent(rownorm_kernel<__nv_bfloat16>, grid, dim3(256), 0, s, logits, (__nv_bfloat16*)w, (__nv_bfloat16*)wu, g.Nloc, g.Dloc);
   count_launch();
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // Copy of the un-merged trailing tokens (rows [src_row0, src_row0 + n_extra) of every batch item).
@@ -634,6 +771,8 @@ cudaError_t launch_linear_simt(int M, int N, int K, bool f32, const void* a, con
 __global__ void global_idx_kernel(const int32_t* __restrict__ idx, int32_t* __restrict__ gidx, int P, int Dloc, int tiles_x,
                                   int th, int tw, int W, int total) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  tc::dependency_wait();  // launched with programmatic stream serialisation
+  if (threadIdx.x == 0) tc::release_dependents();
   if (e >= total) return;
   const int p = (e / Dloc) % P;
   gidx[e] = tile_token(p, idx[e], tiles_x, th, tw, W);
@@ -641,9 +780,8 @@ __global__ void global_idx_kernel(const int32_t* __restrict__ idx, int32_t* __re
 
 cudaError_t launch_global_idx(const Geom& g, const int32_t* idx, int32_t* gidx, cudaStream_t s) {
   const int total = g.B * g.D;
-  global_idx_kernel<<<(total + 255) / 256, 256, 0, s>>>(idx, gidx, g.P, g.Dloc, g.tiles_x, g.th, g.tw, g.W, total);
   count_launch();
-  return cudaGetLastError();
+  return launch_dependent(global_idx_kernel, dim3((total + 255) / 256), dim3(256), 0, s, idx, gidx, g.P, g.Dloc, g.tiles_x, g.th, g.tw, g.W, total);
 }
 
 // Dense fp32 A~ [batch][P][D_loc][N_loc]  <->  stored A~^T [batch][P][N_loc][D_loc].

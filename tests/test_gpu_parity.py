@@ -1354,3 +1354,29 @@ def test_selection_of_equal_tokens_past_unit_similarity(toma, d, kind):
     idx = Run(toma, cfg, x).select()
     want, _ = O.select_tile(x[0].astype(np.float64), od(cfg))
     assert np.array_equal(idx[0, 0], want)
+
+
+def _regions(cfg, x):
+    """Tokens of every region, fp64 on the device: [batch, tiles, N_loc, dim]."""
+    ids = torch.from_numpy(np.ascontiguousarray(O.tile_token_ids(cfg.grid_h, cfg.grid_w, cfg.tile_h, cfg.tile_w))).cuda()
+    return x.double()[:, ids.reshape(-1).long()].reshape(cfg.batch, cfg.n_tiles, cfg.n_loc, cfg.dim)
+
+
+@pytest.mark.parametrize("batch,gy,gx,th,tw,dim,ratio", [
+    (2, 6, 6, 20, 20, 72, 0.5),    # logits in tiles of 64 x 64, many per SM; a last stage of 8 channels
+    (2, 4, 4, 18, 14, 640, 0.5),   # 64 x 32, partial in both directions
+    (1, 1, 1, 7, 5, 8, 0.0),       # 32 x 32: one region of one stage of 8 channels
+    (1, 3, 1, 21, 6, 200, 0.97),   # ... four destinations
+    (3, 2, 2, 11, 3, 64, 0.5),     # ... a tile of one token
+])
+def test_ffma_weights_of_every_tile_form(toma, batch, gy, gx, th, tw, dim, ratio):
+    """Merge weights of regions the tensor cores do not serve, every region of the launch, against 64-bit arithmetic."""
+    cfg = gen.config("cfg2", batch=batch, grid_h=gy * th, grid_w=gx * tw, tile_h=th, tile_w=tw, dim=dim, n_heads=dim // 8, head_dim=8,
+                     merge_ratio=ratio)
+    run = Run(toma, cfg, gen.features(cfg))
+    run.select()
+    dense = torch.from_numpy(run.weights()).cuda()
+    xt = _regions(cfg, run.x)
+    dest = torch.gather(xt, 2, run.idx.reshape(batch, cfg.n_tiles, run.d_loc, 1).long().expand(-1, -1, -1, dim))
+    shares = torch.softmax(dest @ xt.transpose(2, 3) / (cfg.tau * dim ** 0.5), dim=2)
+    assert float((dense - shares / shares.sum(3, keepdim=True)).abs().max()) <= 6e-4  # as in the parity tests above
