@@ -9,24 +9,96 @@ namespace toma {
 
 // ---------------------------------------------------------------------------
 // Quantise: one warp per image token.  y = bf16(rint(x * 0.99*4096/|x|) * 2^-12)
-// written tile-major: row (b*P + p)*N_loc + l.  fp64 arithmetic so that the CPU
-// definition can be matched bit for bit.
+// written tile-major: row (b*P + p)*N_loc + l.  Defined in fp64 (the squares added up per lane in channel order, then by
+// the tree below; scale, product and rounding), so that the CPU definition can be matched bit for bit.
+// The fp64 pipe and its conversions bounded this kernel (4 x 16384 tokens of 640 channels: 65 us, where reading and writing
+// them takes 26; now 50).  bf16 tokens therefore get their squares' sum from the same fp64 additions, but of doubles put together
+// from the bits, and the products as pairs of floats: x * scale = hi + lo to about 2^-45 of it, and what is not within 2^-20
+// of the middle between two integers rounds as the fp64 product does.  A token with a channel that is (one in some
+// thousands), or with a norm far from 1, is done again in fp64.
 // ---------------------------------------------------------------------------
 // Eight consecutive elements as floats (16-byte aligned source).
 __device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&v)[8]) {
   const uint4 raw = *reinterpret_cast<const uint4*>(p);
-  const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&raw);
+  const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    const float2 f = __bfloat1622float2(h[e]);
-    v[2 * e] = f.x;
-    v[2 * e + 1] = f.y;
+    v[2 * e] = __uint_as_float(w[e] << 16);
+    v[2 * e + 1] = __uint_as_float(w[e] & 0xFFFF0000u);
   }
 }
 __device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
   const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
   v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
   v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+__device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&k)[8]) {  // k: integers of up to 13 bits
+  __align__(16) __nv_bfloat162 q[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) q[e] = __floats2bfloat162_rn(k[2 * e] * (1.0f / 4096.0f), k[2 * e + 1] * (1.0f / 4096.0f));
+  *reinterpret_cast<uint4*>(p) = *reinterpret_cast<const uint4*>(q);
+}
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+// The definition, eight channels (16 or 32 contiguous bytes) per lane and trip; dim is a multiple of 8.
+template <typename T>
+__device__ __forceinline__ void quantise_f64(const T* row, __nv_bfloat16* out, int d, int lane) {
+  double ss = 0.0;
+  for (int c = lane * 8; c < d; c += 256) {
+    float v[8];
+    load8(row + c, v);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) ss += (double)v[e] * (double)v[e];
+  }
+  const double scale = kCosScaleTimesOne / fmax(sqrt(warp_sum(ss)), 1e-30);
+  for (int c = lane * 8; c < d; c += 256) {  // second read of the row: an L1/L2 hit
+    float v[8];
+    load8(row + c, v);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = (float)rint((double)v[e] * scale);
+    store8(out + c, v);
+  }
+}
+// A bf16 value (as a float's bits) as the same double; 2^-127 or so instead of zero and of denormals.
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = __float_as_uint(v);
+  return __hiloint2double((int)(((b & 0x7FFFFFFFu) >> 3) + 0x38000000u), 0);  // without the sign: it is squared
+}
+// False: not this way.
+__device__ __forceinline__ bool quantise_fast(const __nv_bfloat16* row, __nv_bfloat16* out, int d, int lane) {
+  double ss = 0.0;
+  for (int c = lane * 8; c < d; c += 256) {
+    float v[8];
+    load8(row + c, v);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const double x = widen(v[e]);
+      ss = fma(x, x, ss);  // the square is exact
+    }
+  }
+  ss = warp_sum(ss);
+  // no infinities, no sum that 2^-254 for a zero could change, no scale whose parts leave the range of floats
+  if (!(ss > 1e-40 && ss < 1e40)) return false;
+  const double scale = kCosScaleTimesOne / sqrt(ss);
+  const float s_hi = (float)scale, s_lo = (float)(scale - (double)s_hi);
+  float off = 0.f;  // largest distance from an integer
+  for (int c = lane * 8; c < d; c += 256) {
+    float v[8];
+    load8(row + c, v);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const float p = v[e] * s_hi;
+      const float lo = fmaf(v[e], s_lo, fmaf(v[e], s_hi, -p));
+      const float k = (p + 12582912.f) - 12582912.f;  // |p| <= 4056: the nearest integer
+      off = fmaxf(off, fabsf((p - k) + lo));
+      v[e] = k;
+    }
+    store8(out + c, v);
+  }
+  return !__any_sync(0xffffffffu, off > 0.5f - 0x1p-20f);
 }
 
 template <typename T>
@@ -44,25 +116,10 @@ __global__ void __launch_bounds__(256) quantise_kernel(const T* __restrict__ x, 
   const int l = (yy % th) * tw + xx % tw;
   const T* row = x + ((size_t)b * n_all + n) * d;
   __nv_bfloat16* out = y + ((size_t)(b * P + p) * Nloc + l) * d;
-  // eight channels (16 or 32 contiguous bytes) per lane and trip; dim is a multiple of 8
-  double ss = 0.0;
-  for (int c = lane * 8; c < d; c += 256) {
-    float v[8];
-    load8(row + c, v);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) ss += (double)v[e] * (double)v[e];
+  if constexpr (sizeof(T) == 2) {
+    if (quantise_fast(row, out, d, lane)) return;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-  const double scale = kCosScaleTimesOne / fmax(sqrt(ss), 1e-30);
-  for (int c = lane * 8; c < d; c += 256) {  // second read of the row: an L1/L2 hit
-    float v[8];
-    load8(row + c, v);
-    __align__(16) __nv_bfloat16 q[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) q[e] = __float2bfloat16_rn((float)rint((double)v[e] * scale) * (1.0f / 4096.0f));
-    *reinterpret_cast<uint4*>(out + c) = *reinterpret_cast<const uint4*>(q);
-  }
+  quantise_f64(row, out, d, lane);
 }
 
 cudaError_t launch_quantise(const Geom& g, const void* x, __nv_bfloat16* y, cudaStream_t s) {

@@ -1380,3 +1380,21 @@ def test_ffma_weights_of_every_tile_form(toma, batch, gy, gx, th, tw, dim, ratio
     dest = torch.gather(xt, 2, run.idx.reshape(batch, cfg.n_tiles, run.d_loc, 1).long().expand(-1, -1, -1, dim))
     shares = torch.softmax(dest @ xt.transpose(2, 3) / (cfg.tau * dim ** 0.5), dim=2)
     assert float((dense - shares / shares.sum(3, keepdim=True)).abs().max()) <= 6e-4  # as in the parity tests above
+
+
+@pytest.mark.parametrize("d", [8, 264, 640])
+def test_selection_of_tokens_at_the_edges_of_the_quantisation(toma, d):
+    """Tokens whose quantised channels are computed by floats and by doubles in turn: norms from 2^-133 to 2^120, channels
+    of 2^-133 beside ones of unit size, zeros, and one channel that holds a token's whole norm."""
+    cfg = gen.config("cfg2", batch=1, grid_h=16, grid_w=8, tile_h=16, tile_w=8, dim=d, n_heads=d // 8, head_dim=8)
+    x = gen.features(cfg).astype(np.float32)
+    scale = 2.0 ** np.linspace(-110, 110, cfg.n_loc).astype(np.int64).astype(np.float64)
+    x[0] = (x[0] * scale[:, None]).astype(np.float32)
+    x[0, 3] = 0.0
+    x[0, 5, 1:] = 0.0
+    x[0, 64:80, ::3] = 2.0 ** -133  # the smallest bf16 number
+    x[0, 66] = x[0, 65]
+    x = gen.round_to_dtype(x, "bf16")
+    idx = Run(toma, cfg, x).select()
+    want, _ = O.select_tile(x[0].astype(np.float64), od(cfg))
+    assert np.array_equal(idx[0, 0], want)
