@@ -66,13 +66,14 @@ __device__ __forceinline__ float chunk_max(const uint32_t (&r)[32], float mx, in
   return mx;
 }
 
-// P for 32 columns as packed bf16 pairs in pk[16]; returns their fp32 sum when sums stay in registers.
+// P for 32 columns as packed bf16 pairs in pk[16]; sum2: fp32 sums of the even and the odd columns, when sums stay in
+// registers (one packed addition per pair, and two chains; one sum of single values was 1 instruction in 9 of the tile's:
+// 4608 tokens, 24 heads of 128 channels 225.9 -> 221.8 us).
 // kMorePoly: three pairs of columns in eight instead of two take the polynomial (timed: 1-2 % faster at head_dim
 // 128, where the sums add to the FMA pipe's load anyway, 4 % slower at head_dim 64).
 template <bool kMask, bool kRegSum, bool kMorePoly>
-__device__ __forceinline__ float chunk_exp(const uint32_t (&r)[32], uint32_t (&pk)[16], float scale, float neg_m,
-                                           int first, int valid) {
-  float l = 0.f;
+__device__ __forceinline__ void chunk_exp(const uint32_t (&r)[32], uint32_t (&pk)[16], float scale, float neg_m, int first, int valid,
+                                          uint64_t& sum2) {
 #pragma unroll
   for (int e = 0; e < 32; e += 2) {
     // S * c - m for a pair of columns in one packed multiply-add
@@ -92,13 +93,12 @@ __device__ __forceinline__ float chunk_exp(const uint32_t (&r)[32], uint32_t (&p
       if (first + e + 1 >= valid) p1 = 0.f;
     }
     if (kRegSum) {
-      l += p0 + p1;
+      sum2 = add2(sum2, pack2(p0, p1));
       pk[e >> 1] = pack_bf16_rn(p0, p1);
     } else {
       pk[e >> 1] = pack_bf16_trunc(p0, p1);
     }
   }
-  return l;
 }
 
 // One 64-key tile of the online softmax for one query row.
@@ -149,11 +149,17 @@ __device__ __forceinline__ void softmax_tile(uint32_t sb, uint32_t ob, float sca
   const float neg_m = -m_used;
   constexpr bool kRegSum = !kSumMma;
   uint32_t pk[16];
-  l += chunk_exp<kMask, kRegSum, DH == 128>(sub32<0>(sr), pk, scale_log2, neg_m, 0, valid);
+  uint64_t sum2 = 0;
+  chunk_exp<kMask, kRegSum, DH == 128>(sub32<0>(sr), pk, scale_log2, neg_m, 0, valid, sum2);
   tmem_st16(sb, pk);
-  l += chunk_exp<kMask, kRegSum, DH == 128>(sub32<32>(sr), pk, scale_log2, neg_m, 32, valid);
+  chunk_exp<kMask, kRegSum, DH == 128>(sub32<32>(sr), pk, scale_log2, neg_m, 32, valid, sum2);
   tmem_st16(sb + 16, pk);
   tmem_wait_st();
+  if (kRegSum) {
+    float even, odd;
+    unpack2(sum2, even, odd);
+    l += even + odd;
+  }
 }
 
 // ------------------------------------------------------------------ softmax against a reference with headroom
