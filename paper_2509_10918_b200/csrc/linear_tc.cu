@@ -24,6 +24,7 @@ constexpr int kKC = 64;           // contraction elements per pipeline stage
 constexpr int kSlab = kKC * 128;  // bytes of a 64-row x 128-byte slab
 constexpr int kMaxCols = 256;     // output columns (MMA N) per merge CTA
 constexpr int kUnmergeTok = 128;  // tokens per unmerge CTA: small enough that two CTAs share an SM
+constexpr int kRowsEpiWarps = 8, kRowsThreads = (2 + kRowsEpiWarps) * 32;  // of the kernels with tokens on M
 
 struct PipeBars {
   uint64_t full[4], empty[4], done;
@@ -44,11 +45,11 @@ struct LinParams {
 
 // The epilogue warps' first work: two launches less per step, 8 us of 124 on joint sequences of 4096 image and 512 text
 // tokens of 3072 channels (a reuse step; a refresh step gains nothing).
-constexpr long long kCopyThreads = 128;  // of a CTA: the four epilogue warps
+constexpr long long kCopyThreads = 128, kRowsCopyThreads = 32 * kRowsEpiWarps;  // of a CTA: the epilogue warps
 // Out of line: sequences without text tokens should not fetch its instructions (0.2 us per launch).
 __device__ __noinline__ void copy_extra(const RowCopy c) {
-  const size_t cta = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  copy_part(c, cta * kCopyThreads + threadIdx.x - 64, (size_t)gridDim.x * gridDim.y * gridDim.z * kCopyThreads);
+  const size_t cta = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x, threads = blockDim.x - 64;
+  copy_part(c, cta * threads + threadIdx.x - 64, (size_t)gridDim.x * gridDim.y * gridDim.z * threads);
 }
 
 __device__ __forceinline__ uint32_t tmem_cols_for(int n) { return n > 128 ? 256u : n > 64 ? 128u : 64u; }
@@ -92,6 +93,43 @@ __device__ __forceinline__ void stage_and_store(uint8_t* so, PipeBars* bar, uint
     tma_store_commit();
     tma_store_wait_read();  // shared memory must outlive the engine's reads
   }
+}
+
+// Epilogue with tokens on M.  Thread = token slot `row` (0..127) of the CTA's block, channels on the columns; two warps of a
+// quarter take every second 64-channel slab.  A warp's 32 rows of a slab are a box of the output map and are stored as soon as
+// the warp has staged them: with four warps and one store of the whole tile behind them all, the epilogue was a third of a
+// launch (32 tiles of 256 tokens, 128 destinations, 640 channels: 3.2 of 8 us).  `so`: slabs of [128 rows][128 B], 128-byte
+// swizzled; store(slab).
+template <typename Store>
+__device__ __forceinline__ void stage_rows_and_store(uint8_t* so, uint32_t taddr, int row, int half, int n_ch, Store store) {
+  for (int c0 = half * 64; c0 < n_ch; c0 += 128) {
+    uint8_t* slab = so + (c0 >> 6) * (128 * 128);
+#pragma unroll 1
+    for (int c = c0; c < c0 + 64 && c < n_ch; c += 32) {
+      uint32_t r[32];
+      tmem_ld32(taddr + c, r);
+      tmem_wait_ld();
+#pragma unroll
+      for (int e = 0; e < 32; e += 8) {
+        __align__(16) __nv_bfloat162 q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) q[u] = __floats2bfloat162_rn(__uint_as_float(r[e + 2 * u]), __uint_as_float(r[e + 2 * u + 1]));
+        *reinterpret_cast<uint4*>(slab + sw128_offset(row, ((c & 63) + e) >> 3)) = *reinterpret_cast<const uint4*>(q);
+      }
+    }
+    fence_proxy_async();  // the staged rows are read by the TMA engine
+    __syncwarp();
+    if ((row & 31) == 0) {  // a slab cut short by the channel count is clipped by the store
+      store(c0 >> 6);
+      tma_store_commit();
+    }
+  }
+}
+// Where the 32 tokens from slot `t` of a tile on start.
+__device__ __forceinline__ void token_at(const LinParams& p, int tx, int ty, int t, int& x, int& y) {
+  y = t / p.tw;
+  x = tx * p.tw + t - y * p.tw;
+  y += ty * p.th;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -461,7 +499,7 @@ unmerge_tc_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_constan
 // ------------------------------------------------------------------------------------------------
 constexpr int kRowsChBlock = 320;  // channels per CTA (five 64-channel slabs)
 
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(kRowsThreads, 1)
 unmerge_rows_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_w,
                     const __grid_constant__ CUtensorMap tm_o, const LinParams p, uint32_t* dev_status) {
   extern __shared__ uint8_t smem_raw[];
@@ -487,8 +525,25 @@ unmerge_rows_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_const
     prefetch_tmap(&tm_w);
     prefetch_tmap(&tm_o);
   }
+  // k-step k of the operands into its stage
+  auto load = [&](int k) {
+    const int s = k % p.stages;
+    uint8_t* sw = smem + s * stage_bytes;
+    uint8_t* sy = sw + 2 * w_plane;
+    mbar_expect_tx(&bar->full[s], stage_bytes);
+    for (int pl = 0; pl < 2; ++pl) tma_load_3d(sw + pl * w_plane, &tm_w, &bar->full[s], k * kKC, t0, 2 * batch + pl);
+    for (int c = 0; c < slabs; ++c)
+      tma_load_3d(sy + c * kSlab, &tm_y, &bar->full[s], c0 + c * 64, tile * p.Dloc + k * kKC, b);
+  };
+  const int early = min(nk, p.stages);
   dependency_wait();
   if (threadIdx.x == 0) release_dependents();
+  if (warp == 0) {  // the first loads do not wait for the others' preparations: 0.35 us of a launch
+    __syncwarp();
+    if (elect_one())
+      for (int k = 0; k < early; ++k) load(k);
+    __syncwarp();
+  }
   if (warp == 1) tmem_alloc(&bar->tmem_base, ncols);
   tc_fence_before();
   __syncthreads();
@@ -498,15 +553,9 @@ unmerge_rows_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_const
 
   if (warp == 0) {
     if (elect_one()) {
-      for (int k = 0; k < nk; ++k) {
-        const int s = k % p.stages;
-        if (k >= p.stages && !mbar_wait(&bar->empty[s], ((k / p.stages) - 1) & 1, dev_status, abort_flag)) break;
-        uint8_t* sw = smem + s * stage_bytes;
-        uint8_t* sy = sw + 2 * w_plane;
-        mbar_expect_tx(&bar->full[s], stage_bytes);
-        for (int pl = 0; pl < 2; ++pl) tma_load_3d(sw + pl * w_plane, &tm_w, &bar->full[s], k * kKC, t0, 2 * batch + pl);
-        for (int c = 0; c < slabs; ++c)
-          tma_load_3d(sy + c * kSlab, &tm_y, &bar->full[s], c0 + c * 64, tile * p.Dloc + k * kKC, b);
+      for (int k = early; k < nk; ++k) {
+        if (!mbar_wait(&bar->empty[k % p.stages], ((k / p.stages) - 1) & 1, dev_status, abort_flag)) break;
+        load(k);
       }
     }
   } else if (warp == 1) {
@@ -536,38 +585,18 @@ unmerge_rows_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_const
     }
   } else {
     if (p.extra.per) copy_extra(p.extra);
-    const int quarter = warp & 3, row = quarter * 32 + lane;  // token slot t0 + row = tensor-memory lane
-    const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
-    if (mbar_wait_warp(&bar->done, 0, dev_status, abort_flag)) {
-      tc_fence_after();
-      // every load has been consumed: slab c of the output, [128 tokens][128 B] swizzled, goes to smem + c * 16 KB
-      for (int c = 0; c < n_ch; c += 32) {  // accumulator column = channel (the second accumulator starts at 192)
-        uint32_t r[32];
-        tmem_ld32(taddr + c, r);
-        tmem_wait_ld();
-        uint8_t* slab = smem + (c >> 6) * (128 * 128);
-#pragma unroll
-        for (int e = 0; e < 32; e += 8) {
-          if (c + e < n_ch) {
-            __align__(16) __nv_bfloat162 q[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-              q[u] = __floats2bfloat162_rn(__uint_as_float(r[e + 2 * u]), __uint_as_float(r[e + 2 * u + 1]));
-            *reinterpret_cast<uint4*>(slab + sw128_offset(row, ((c & 63) + e) >> 3)) = *reinterpret_cast<const uint4*>(q);
-          }
-        }
-      }
-      fence_proxy_async();  // the staged rows are read by the TMA engine
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bar->epi);
-      if (row == 0 && mbar_wait(&bar->epi, 0, dev_status, abort_flag)) {
-        const int ty = tile / p.tiles_x, tx = tile - ty * p.tiles_x;
-        for (int c = 0; c < slabs; ++c)  // a slab cut short by the channel count is clipped by the store
-          tma_store_4d(&tm_o, smem + c * (128 * 128), c0 + c * 64, tx * p.tw, ty * p.th + t0 / p.tw, b);
-        tma_store_commit();
-        tma_store_wait_read();  // shared memory must outlive the engine's reads
-      }
-    }
+    const int quarter = warp & 3, row = quarter * 32 + lane, half = (warp - 2) >> 2;  // token slot t0 + row = tensor-memory lane
+    // every load has been consumed: the stages are free (a wait that ran out: the results are void, the way is the same)
+    mbar_wait_warp(&bar->done, 0, dev_status, abort_flag);
+    tc_fence_after();
+    const int ty = tile / p.tiles_x, tx = tile - ty * p.tiles_x;
+    int x, y;
+    token_at(p, tx, ty, t0 + quarter * 32, x, y);
+    // accumulator column = channel (the second accumulator starts at 192)
+    stage_rows_and_store(smem, tmem + ((uint32_t)(quarter * 32) << 16), row, half, n_ch, [&](int c) {
+      tma_store_4d(&tm_o, smem + c * (128 * 128) + quarter * 4096, c0 + c * 64, x, y, b);
+    });
+    if (lane == 0) tma_store_wait_read();  // shared memory must outlive the engine's reads
   }
   tc_fence_before();
   __syncthreads();
@@ -584,7 +613,7 @@ unmerge_rows_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_const
 // under the next item's MMAs.  One accumulator set (up to 320 columns of tensor memory): the next item's MMAs
 // wait only until the epilogue warps have read the accumulators out.
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(kRowsThreads, 1)
 unmerge_rows_persistent_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_w,
                                const __grid_constant__ CUtensorMap tm_o, const LinParams p, int n_items, int ch_blocks,
                                uint32_t* dev_status) {
@@ -606,23 +635,13 @@ unmerge_rows_persistent_kernel(const __grid_constant__ CUtensorMap tm_y, const _
       mbar_init(&bar->empty[s], 1);
     }
     mbar_init(&bar->acc_full[0], 1);
-    mbar_init(&bar->acc_empty[0], 4);
-    mbar_init(&bar->staged, 4);
-    mbar_init(&bar->stored, 1);
+    mbar_init(&bar->acc_empty[0], kRowsEpiWarps);
     bar->abort_flag = 0;
     mbar_fence_init();
     prefetch_tmap(&tm_y);
     prefetch_tmap(&tm_w);
     prefetch_tmap(&tm_o);
   }
-  dependency_wait();
-  if (threadIdx.x == 0) release_dependents();
-  if (warp == 1) tmem_alloc(&bar->tmem_base, ncols);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = bar->tmem_base;
-  volatile int* abort_flag = &bar->abort_flag;
   // item -> (tile of the batch, 128-token block, channel block); channel blocks of one token block are neighbours,
   // so that concurrently running CTAs share its weights in L2
   auto decode = [&](int item, int& batch, int& t0, int& c0) {
@@ -632,24 +651,40 @@ unmerge_rows_persistent_kernel(const __grid_constant__ CUtensorMap tm_y, const _
     c0 = cb * kRowsChBlock;
   };
 
+  auto load = [&](int item, int k, int kc) {
+    int batch, t0, c0;
+    decode(item, batch, t0, c0);
+    const int b = batch / p.P, tile = batch - b * p.P;
+    const int slabs = (min(kRowsChBlock, p.d - c0) + 63) / 64, s = kc % p.stages;
+    uint8_t* sw = smem + s * stage_bytes;
+    uint8_t* sy = sw + 2 * w_plane;
+    mbar_expect_tx(&bar->full[s], 2 * w_plane + slabs * kSlab);
+    for (int pl = 0; pl < 2; ++pl) tma_load_3d(sw + pl * w_plane, &tm_w, &bar->full[s], k * kKC, t0, 2 * batch + pl);
+    for (int c = 0; c < slabs; ++c) tma_load_3d(sy + c * kSlab, &tm_y, &bar->full[s], c0 + c * 64, tile * p.Dloc + k * kKC, b);
+  };
+  const int early = min(nk, p.stages);
+  dependency_wait();
+  if (threadIdx.x == 0) release_dependents();
+  if (warp == 0) {
+    __syncwarp();
+    if (elect_one())
+      for (int k = 0; k < early; ++k) load(blockIdx.x, k, k);
+    __syncwarp();
+  }
+  if (warp == 1) tmem_alloc(&bar->tmem_base, ncols);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = bar->tmem_base;
+  volatile int* abort_flag = &bar->abort_flag;
   if (warp == 0) {
     if (elect_one()) {
-      int kc = 0;
+      int kc = early;
       bool ok = true;
       for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
-        int batch, t0, c0;
-        decode(item, batch, t0, c0);
-        const int b = batch / p.P, tile = batch - b * p.P;
-        const int slabs = (min(kRowsChBlock, p.d - c0) + 63) / 64;
-        for (int k = 0; k < nk; ++k, ++kc) {
-          const int s = kc % p.stages;
-          if (kc >= p.stages && !mbar_wait(&bar->empty[s], ((kc / p.stages) - 1) & 1, dev_status, abort_flag)) { ok = false; break; }
-          uint8_t* sw = smem + s * stage_bytes;
-          uint8_t* sy = sw + 2 * w_plane;
-          mbar_expect_tx(&bar->full[s], 2 * w_plane + slabs * kSlab);
-          for (int pl = 0; pl < 2; ++pl) tma_load_3d(sw + pl * w_plane, &tm_w, &bar->full[s], k * kKC, t0, 2 * batch + pl);
-          for (int c = 0; c < slabs; ++c)
-            tma_load_3d(sy + c * kSlab, &tm_y, &bar->full[s], c0 + c * 64, tile * p.Dloc + k * kKC, b);
+        for (int k = item == (int)blockIdx.x ? early : 0; k < nk; ++k, ++kc) {
+          if (kc >= p.stages && !mbar_wait(&bar->empty[kc % p.stages], ((kc / p.stages) - 1) & 1, dev_status, abort_flag)) { ok = false; break; }
+          load(item, k, kc);
         }
       }
     }
@@ -690,52 +725,29 @@ unmerge_rows_persistent_kernel(const __grid_constant__ CUtensorMap tm_y, const _
     }
   } else {
     if (p.extra.per) copy_extra(p.extra);
-    const int quarter = warp & 3, row = quarter * 32 + lane;  // token slot t0 + row = tensor-memory lane
-    const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
+    const int quarter = warp & 3, row = quarter * 32 + lane, half = (warp - 2) >> 2;  // token slot t0 + row = tensor-memory lane
     int n = 0;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++n) {
       int batch, t0, c0;
       decode(item, batch, t0, c0);
       const int b = batch / p.P, tile = batch - b * p.P;
-      const int n_ch = min(kRowsChBlock, p.d - c0), slabs = (n_ch + 63) / 64;
-      // the accumulators are complete, and the previous item's store has read the staging area; one answer per
-      // warp (the tensor-memory loads are warp-wide operations)
-      const bool go = mbar_wait(&bar->acc_full[0], n & 1, dev_status, abort_flag) &&
-                      (n == 0 || mbar_wait(&bar->stored, (n - 1) & 1, dev_status, abort_flag));
-      if (!__all_sync(0xffffffffu, go)) break;
-      tc_fence_after();
-      for (int c = 0; c < n_ch; c += 32) {  // accumulator column = channel (the second accumulator starts at 192)
-        uint32_t r[32];
-        tmem_ld32(taddr + c, r);
-        tmem_wait_ld();
-        uint8_t* slab = so + (c >> 6) * (128 * 128);
-#pragma unroll
-        for (int e = 0; e < 32; e += 8) {
-          if (c + e < n_ch) {
-            __align__(16) __nv_bfloat162 q[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-              q[u] = __floats2bfloat162_rn(__uint_as_float(r[e + 2 * u]), __uint_as_float(r[e + 2 * u + 1]));
-            *reinterpret_cast<uint4*>(slab + sw128_offset(row, ((c & 63) + e) >> 3)) = *reinterpret_cast<const uint4*>(q);
-          }
-        }
-      }
-      tc_fence_before();
-      fence_proxy_async();  // the staged rows are read by the TMA engine
+      const int n_ch = min(kRowsChBlock, p.d - c0), ty = tile / p.tiles_x, tx = tile - ty * p.tiles_x;
+      int x, y;
+      token_at(p, tx, ty, t0 + quarter * 32, x, y);
+      // the accumulators are complete, and this warp's stores of the previous item have read its part of the staging area
+      if (!mbar_wait_warp(&bar->acc_full[0], n & 1, dev_status, abort_flag)) break;
+      if (lane == 0) tma_store_wait_read();
       __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(&bar->acc_empty[0]);  // the next item's products may overwrite the accumulators
-        mbar_arrive(&bar->staged);
-      }
-      if (row == 0 && mbar_wait(&bar->staged, n & 1, dev_status, abort_flag)) {  // a wait that ran out ends the loop at its top
-        const int ty = tile / p.tiles_x, tx = tile - ty * p.tiles_x;
-        for (int c = 0; c < slabs; ++c)  // a slab cut short by the channel count is clipped by the store
-          tma_store_4d(&tm_o, so + c * (128 * 128), c0 + c * 64, tx * p.tw, ty * p.th + t0 / p.tw, b);
-        tma_store_commit();
-        tma_store_wait_read();  // shared memory must outlive the engine's reads
-        mbar_arrive(&bar->stored);
-      }
+      tc_fence_after();
+      // accumulator column = channel (the second accumulator starts at 192)
+      stage_rows_and_store(so, tmem + ((uint32_t)(quarter * 32) << 16), row, half, n_ch, [&](int c) {
+        tma_store_4d(&tm_o, so + c * (128 * 128) + quarter * 4096, c0 + c * 64, x, y, b);
+      });
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar->acc_empty[0]);  // the next item's products may overwrite the accumulators
     }
+    if (lane == 0) tma_store_wait_read();  // shared memory must outlive the engine's reads
   }
   tc_fence_before();
   __syncthreads();
@@ -892,7 +904,7 @@ cudaError_t launch_unmerge_tc(const Geom& g, const void* w, const void* y, void*
     if (!encode_w(g, w, &tw128, 128)) return cudaErrorInvalidValue;
     const uint64_t odims[4] = {(uint64_t)g.d, (uint64_t)g.W, (uint64_t)g.H, (uint64_t)g.B};
     const uint64_t ostrides[3] = {(uint64_t)g.d * 2, (uint64_t)g.W * g.d * 2, (uint64_t)g.tokens_all() * g.d * 2};
-    const uint32_t obox[4] = {64, (uint32_t)g.tw, (uint32_t)(128 / g.tw), 1};
+    const uint32_t obox[4] = {64, (uint32_t)(g.tw < 32 ? g.tw : 32), (uint32_t)(g.tw < 32 ? 32 / g.tw : 1), 1};  // a warp's 32 tokens
     if (!encode_tmap_16bit(&to, out, 4, odims, ostrides, obox)) return cudaErrorInvalidValue;
     const int max_slabs = ((g.d < kRowsChBlock ? g.d : kRowsChBlock) + 63) / 64;
     const int stage_bytes = 2 * 128 * 128 + max_slabs * kSlab, staging = max_slabs * 128 * 128;
@@ -903,8 +915,8 @@ cudaError_t launch_unmerge_tc(const Geom& g, const void* w, const void* y, void*
       static std::atomic<unsigned long long> raised_rp{0};
       if (cudaError_t e = raise_dynamic_smem(unmerge_rows_persistent_kernel, 227 * 1024, raised_rp); e != cudaSuccess) return e;
       const int ch_blocks = (g.d + kRowsChBlock - 1) / kRowsChBlock;
-      if (copied_beside(rows, sms * kCopyThreads)) p.extra = rows;
-      cudaError_t e = launch_dependent(unmerge_rows_persistent_kernel, dim3(sms), dim3(192), (size_t)smem, s, ty, tw128, to, p, rows_ctas,
+      if (copied_beside(rows, sms * kRowsCopyThreads)) p.extra = rows;
+      cudaError_t e = launch_dependent(unmerge_rows_persistent_kernel, dim3(sms), dim3(kRowsThreads), (size_t)smem, s, ty, tw128, to, p, rows_ctas,
                                        ch_blocks, dev_status);
       return finish_launch(e, rows, p.extra, s);
     }
@@ -921,15 +933,15 @@ cudaError_t launch_unmerge_tc(const Geom& g, const void* w, const void* y, void*
     const int smem = 1024 + p.stages * stage_bytes + 256;
     static std::atomic<unsigned long long> raised_r{0};
     if (cudaError_t e = raise_dynamic_smem(unmerge_rows_kernel, 227 * 1024, raised_r); e != cudaSuccess) return e;
-    // output tokens as (channel, x, y, batch): a CTA's 128 tokens are 128 / tile_w whole tile rows
+    // output tokens as (channel, x, y, batch)
     CUtensorMap to;
     const uint64_t odims[4] = {(uint64_t)g.d, (uint64_t)g.W, (uint64_t)g.H, (uint64_t)g.B};
     const uint64_t ostrides[3] = {(uint64_t)g.d * 2, (uint64_t)g.W * g.d * 2, (uint64_t)g.tokens_all() * g.d * 2};
-    const uint32_t obox[4] = {64, (uint32_t)g.tw, (uint32_t)(128 / g.tw), 1};
+    const uint32_t obox[4] = {64, (uint32_t)(g.tw < 32 ? g.tw : 32), (uint32_t)(g.tw < 32 ? 32 / g.tw : 1), 1};  // a warp's 32 tokens
     if (!encode_tmap_16bit(&to, out, 4, odims, ostrides, obox)) return cudaErrorInvalidValue;
     dim3 grid(g.B * g.P * (g.Nloc / 128), (g.d + kRowsChBlock - 1) / kRowsChBlock);
-    if (copied_beside(rows, grid.x * grid.y * kCopyThreads)) p.extra = rows;
-    cudaError_t e = launch_dependent(unmerge_rows_kernel, grid, dim3(192), (size_t)smem, s, ty, tw128, to, p, dev_status);
+    if (copied_beside(rows, grid.x * grid.y * kRowsCopyThreads)) p.extra = rows;
+    cudaError_t e = launch_dependent(unmerge_rows_kernel, grid, dim3(kRowsThreads), (size_t)smem, s, ty, tw128, to, p, dev_status);
     return finish_launch(e, rows, p.extra, s);
   }
   // output tokens as (channel, x, y, batch): a CTA's token block is n_tok / tile_w whole tile rows

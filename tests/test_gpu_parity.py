@@ -1398,3 +1398,32 @@ def test_selection_of_tokens_at_the_edges_of_the_quantisation(toma, d):
     idx = Run(toma, cfg, x).select()
     want, _ = O.select_tile(x[0].astype(np.float64), od(cfg))
     assert np.array_equal(idx[0, 0], want)
+
+
+@pytest.mark.parametrize("th,tw,ratio,dim", [
+    (8, 8, 0.75, 640),    # 16 destinations; one load of tokens
+    (16, 16, 0.6875, 72),  # 80: two slabs of weights, three of a warp's four parts; a last channel block of 72
+    (32, 2, 0.0, 136),    # 64 destinations; boxes of two tokens a row; 8 channels in the second block
+    (64, 1, 0.5, 64),     # rows of one token
+    (4, 64, 0.5, 320),    # 128: one whole block; rows of 64 tokens
+    (32, 16, 0.71875, 200),  # 144: a second block of 16
+    (16, 32, 0.5, 328),   # 256
+])
+@pytest.mark.parametrize("batch", [1, 40])  # a launch that the SMs hold at once, one that they walk
+def test_merge_and_unmerge_of_box_regions(toma, th, tw, ratio, dim, batch):
+    """Contractions with destinations or tokens on the rows of the product, at the edges of their blocks and of their
+    output boxes, every region against the same sums of the exported weights in 64 bits; the rows behind stay as they were."""
+    cfg = gen.config("cfg2", batch=batch, grid_h=2 * th, grid_w=3 * tw, tile_h=th, tile_w=tw, dim=dim, n_heads=dim // 8, head_dim=8,
+                     merge_ratio=ratio)
+    run = Run(toma, cfg, gen.features(cfg))
+    run.select()
+    dense = torch.from_numpy(run.weights()).cuda()
+    xt = _regions(cfg, run.x)
+    guard = torch.full((4096,), 7.0, dtype=run.x.dtype, device="cuda")
+    merged = run.merge().reshape(batch, cfg.n_tiles, run.d_loc, dim)
+    assert_close(merged, (dense @ xt).cpu().numpy(), "bf16", "merge")
+    y = (run.xm.float() * 0.25).to(run.xm.dtype)  # as in test_edge_shapes: keeps the outputs below 8
+    out = torch.from_numpy(run.unmerge(y)).cuda()
+    want = dense.transpose(2, 3) @ y.double().reshape(batch, cfg.n_tiles, run.d_loc, dim)
+    assert_close(_regions(cfg, out).cpu().numpy(), want.cpu().numpy(), "bf16", "unmerge")
+    assert bool((guard == 7.0).all())
