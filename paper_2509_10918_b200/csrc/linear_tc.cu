@@ -2,15 +2,13 @@
 // tensor cores: bf16 tokens, weights as a hi + lo pair of bf16 planes (two MMAs per step, ~16
 // mantissa bits), fp32 accumulation in tensor memory.
 //
-// Both are computed transposed, with 128 feature channels on the MMA M dimension:
-//   merge:    X_m^T [ch x D_loc] = X^T  [ch x N_loc] * A~^T [N_loc x D_loc]
-//   unmerge:  Y^T   [ch x N_loc] = X'^T [ch x D_loc] * A~   [D_loc x N_loc]
-// so the one stored weight layout A~^T [N_loc][D_loc] is the B operand of both (MN-major for the
-// merge, K-major for the unmerge) and the token tensors are MN-major A operands that TMA fetches
-// straight from their row-major [token][channel] storage: a spatial tile is one 4-D box of the
-// (channel, x, y, batch) view of X, so no gather/reshape pass exists.
-// One CTA = one (tile, 128-channel chunk, block of <= 256 output columns); warp 0 TMA, warp 1
-// MMA, warps 2..5 epilogue (one thread per channel).
+// The one stored weight layout A~^T [N_loc][D_loc] serves both, K-major for the unmerge and MN-major for the merge, and the
+// token tensors are MN-major operands that TMA fetches straight from their row-major [token][channel] storage: a spatial tile
+// is one 4-D box of the (channel, x, y, batch) view of X, so no gather/reshape pass exists.  Which side lies on the MMA's M
+// dimension decides what an epilogue thread holds:
+//   merge_rows_kernel, unmerge_rows_*: destinations or tokens on M; a thread owns an output row and stages 16 bytes at a time
+//   merge_tc, merge_persistent, unmerge_tc: 128 channels on M; a thread owns a channel of <= 256 output columns, 2 bytes at a time
+// Warp 0 issues the loads, warp 1 the MMAs, the others (eight with rows on M, four with channels) the epilogue.
 #include "common.cuh"
 #include "tc.cuh"
 
@@ -135,17 +133,15 @@ __device__ __forceinline__ void token_at(const LinParams& p, int tx, int ty, int
 // ------------------------------------------------------------------------------------------------
 // merge: grid (tile, channel chunk, destination block); K loop over the tile's tokens.
 // ------------------------------------------------------------------------------------------------
-// kBlocked: the destinations of a region are split into blocks of p.dest_block (global merge); otherwise a
-// region's destinations (<= kMaxCols) belong to one CTA and the block size is a compile-time constant.
-template <bool kBlocked>
+// For regions with more than kMaxCols destinations (global merge), in blocks of p.dest_block of them.
 __global__ void __launch_bounds__(192, 1)
 merge_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                 const __grid_constant__ CUtensorMap tm_o, const LinParams p, uint32_t* dev_status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int batch = blockIdx.x, c0 = blockIdx.y * 128, i_base = blockIdx.z * (kBlocked ? p.dest_block : kMaxCols);
-  const int n_dest = min(kBlocked ? p.dest_block : kMaxCols, p.Dloc - i_base);  // destinations this CTA produces
+  const int batch = blockIdx.x, c0 = blockIdx.y * 128, i_base = blockIdx.z * p.dest_block;
+  const int n_dest = min(p.dest_block, p.Dloc - i_base);  // destinations this CTA produces
   const int slabs = (n_dest + 63) / 64;               // 64-destination slabs per weight plane
   const int n_mma = slabs * 64;                       // MMA N (zero padded by TMA)
   const int stage_bytes = (2 + 2 * slabs) * kSlab;
@@ -227,6 +223,115 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, ncols);
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
+// merge with destinations on M: X_m [D_loc x ch] = A~ [D_loc x N_loc] * X [N_loc x ch], for launches that the SMs hold at once.
+// One CTA = (128 destinations, 128 channels); both operands MN-major as they lie in memory.  The same bytes and products per
+// CTA as with channels on M, but a thread then owns an output row and stages 16 bytes at a time where the other form stages 2:
+// the epilogue was 2.3 us of a launch of 8 (32 tiles of 256 tokens, 128 destinations, 640 channels).
+// A block of 64 destinations or fewer loads one slab of a weight plane: the rows of the product that the other one would have
+// made are made of whatever lies there, and not stored.
+// ------------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(kRowsThreads, 2)
+merge_rows_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
+                  const __grid_constant__ CUtensorMap tm_o, const LinParams p, uint32_t* dev_status) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  constexpr int kStage = 6 * kSlab;  // two planes of two slabs of weights, two slabs of tokens
+  PipeBars* bar = reinterpret_cast<PipeBars*>(smem + p.stages * kStage);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int batch = blockIdx.x, c0 = blockIdx.y * 128, i_base = blockIdx.z * 128;
+  const int w_slabs = p.Dloc - i_base > 64 ? 2 : 1, x_slabs = p.d - c0 > 64 ? 2 : 1;
+  const int b = batch / p.P, tile = batch - b * p.P;
+  const int ty = tile / p.tiles_x, tx = tile - ty * p.tiles_x;
+  const int rows_per_chunk = kKC / p.tw;
+  const int nk = p.Nloc / kKC;
+
+  if (threadIdx.x == 0) {
+    pipe_init(bar, p.stages);
+    prefetch_tmap(&tm_x);
+    prefetch_tmap(&tm_w);
+    prefetch_tmap(&tm_o);
+  }
+  // k-step k of the operands into its stage
+  auto load = [&](int k) {
+    const int s = k % p.stages;
+    uint8_t* sw = smem + s * kStage;
+    uint8_t* sx = sw + 4 * kSlab;
+    mbar_expect_tx(&bar->full[s], (2 * w_slabs + x_slabs) * kSlab);
+    for (int pl = 0; pl < 2; ++pl)
+      for (int c = 0; c < w_slabs; ++c)
+        tma_load_3d(sw + (2 * pl + c) * kSlab, &tm_w, &bar->full[s], i_base + c * 64, k * kKC, 2 * batch + pl);
+    for (int c = 0; c < x_slabs; ++c)
+      tma_load_4d(sx + c * kSlab, &tm_x, &bar->full[s], c0 + c * 64, tx * p.tw, ty * p.th + k * rows_per_chunk, b);
+  };
+  const int early = min(nk, p.stages);
+  dependency_wait();
+  if (threadIdx.x == 0) release_dependents();
+  if (warp == 0) {
+    __syncwarp();
+    if (elect_one())
+      for (int k = 0; k < early; ++k) load(k);
+    __syncwarp();
+  }
+  if (warp == 1) tmem_alloc(&bar->tmem_base, 128);
+  if (p.zero_words > 0) {
+    const int cta = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    const int n_thr = gridDim.x * gridDim.y * gridDim.z * blockDim.x;
+    for (int i = cta * blockDim.x + threadIdx.x; i < p.zero_words; i += n_thr) p.zero[i] = 0u;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = bar->tmem_base;
+  volatile int* abort_flag = &bar->abort_flag;
+
+  if (warp == 0) {
+    if (elect_one()) {
+      for (int k = early; k < nk; ++k) {
+        if (!mbar_wait(&bar->empty[k % p.stages], ((k / p.stages) - 1) & 1, dev_status, abort_flag)) break;
+        load(k);
+      }
+    }
+  } else if (warp == 1) {
+    if (elect_one()) {
+      const uint32_t idesc = idesc_f16(kFmtBF16, kFmtBF16, true, true, 128, x_slabs * 64);
+      bool ok = true;
+      for (int k = 0; k < nk; ++k) {
+        const int s = k % p.stages;
+        if (!mbar_wait(&bar->full[s], (k / p.stages) & 1, dev_status, abort_flag)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t wa = smem_u32(smem + s * kStage), xa = wa + 4 * kSlab;
+#pragma unroll
+        for (int kk = 0; kk < kKC / 16; ++kk) {  // 16 tokens per MMA: 16 rows of 128 B in every slab
+          const uint64_t xd = smem_desc_sw128(xa + kk * 2048, kSlab, 1024);
+          mma_ss(tmem, smem_desc_sw128(wa + kk * 2048, kSlab, 1024), xd, idesc, k > 0 || kk > 0);
+          mma_ss(tmem, smem_desc_sw128(wa + 2 * kSlab + kk * 2048, kSlab, 1024), xd, idesc, true);
+        }
+        mma_commit(&bar->empty[s]);
+      }
+      if (ok) mma_commit(&bar->done);
+    }
+  } else {
+    if (p.extra.per) copy_extra(p.extra);
+    const int quarter = warp & 3, row = quarter * 32 + lane, half = (warp - 2) >> 2;  // destination i_base + row = tensor-memory lane
+    // every load has been consumed: the stages are free (a wait that ran out: the results are void, the way is the same)
+    mbar_wait_warp(&bar->done, 0, dev_status, abort_flag);
+    tc_fence_after();
+    if (i_base + quarter * 32 < p.Dloc) {
+      stage_rows_and_store(smem, tmem + ((uint32_t)(quarter * 32) << 16), row, half, min(128, p.d - c0), [&](int c) {
+        tma_store_4d(&tm_o, smem + c * (128 * 128) + quarter * 4096, c0 + c * 64, i_base + quarter * 32, tile, b);
+      });
+      if (lane == 0) tma_store_wait_read();  // shared memory must outlive the engine's reads
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, 128);
   }
 }
 
@@ -819,11 +924,8 @@ cudaError_t launch_merge_tc(const Geom& g, const void* w, const void* x, void* x
   const int stage_bytes = (2 + 2 * slabs) * kSlab;
   p.zero = (uint32_t*)zero;
   p.zero_words = (int)(zero_bytes / 4);
-  p.stages = 2;  // two stages keep a CTA below ~100 KB so that two or three CTAs share an SM and hide each other's latencies
-  if (g.Dloc > kMaxCols) {  // one CTA per SM anyway: as deep as shared memory allows
-    p.stages = (198 * 1024) / stage_bytes;
-    p.stages = p.stages > 4 ? 4 : p.stages < 2 ? 2 : p.stages;
-  }
+  p.stages = (198 * 1024) / stage_bytes;  // one CTA per SM: as deep as shared memory allows
+  p.stages = p.stages > 4 ? 4 : p.stages < 2 ? 2 : p.stages;
   if (p.stages > g.Nloc / kKC) p.stages = g.Nloc / kKC;
   const int smem = 1024 + p.stages * stage_bytes + 256;
   dim3 grid(g.B * g.P, (g.d + 127) / 128, (g.Dloc + p.dest_block - 1) / p.dest_block);
@@ -850,18 +952,22 @@ cudaError_t launch_merge_tc(const Geom& g, const void* w, const void* x, void* x
     }
     p.stages = 2;
   }
-  if (copied_beside(rows, grid.x * grid.y * grid.z * kCopyThreads)) p.extra = rows;
-  if (g.Dloc > kMaxCols) {
-    static std::atomic<unsigned long long> raised_b{0};
-    e = raise_dynamic_smem(merge_tc_kernel<true>, 200 * 1024, raised_b);
-    if (e != cudaSuccess) return e;
-    e = launch_dependent(merge_tc_kernel<true>, grid, dim3(192), (size_t)smem, s, tx, tw, to, p, dev_status);
-  } else {
-    static std::atomic<unsigned long long> raised{0};
-    e = raise_dynamic_smem(merge_tc_kernel<false>, 200 * 1024, raised);
-    if (e != cudaSuccess) return e;
-    e = launch_dependent(merge_tc_kernel<false>, grid, dim3(192), (size_t)smem, s, tx, tw, to, p, dev_status);
+  if (g.Dloc <= kMaxCols) {
+    const uint32_t rbox[4] = {64, 32, 1, 1};  // a warp's 32 destinations
+    if (!encode_tmap_16bit(&to, xm, 4, odims, ostrides, rbox)) return cudaErrorInvalidValue;
+    constexpr int kStage = 6 * kSlab;
+    p.stages = g.Nloc / kKC < 2 ? g.Nloc / kKC : 2;  // two CTAs per SM hide each other's latencies
+    const dim3 rgrid(g.B * g.P, (g.d + 127) / 128, (g.Dloc + 127) / 128);
+    if (copied_beside(rows, rgrid.x * rgrid.y * rgrid.z * kRowsCopyThreads)) p.extra = rows;
+    static std::atomic<unsigned long long> raised_m{0};
+    if (e = raise_dynamic_smem(merge_rows_kernel, 1024 + 2 * kStage + 256, raised_m); e != cudaSuccess) return e;
+    e = launch_dependent(merge_rows_kernel, rgrid, dim3(kRowsThreads), (size_t)(1024 + p.stages * kStage + 256), s, tx, tw, to, p, dev_status);
+    return finish_launch(e, rows, p.extra, s);
   }
+  if (copied_beside(rows, grid.x * grid.y * grid.z * kCopyThreads)) p.extra = rows;
+  static std::atomic<unsigned long long> raised{0};
+  if (e = raise_dynamic_smem(merge_tc_kernel, 200 * 1024, raised); e != cudaSuccess) return e;
+  e = launch_dependent(merge_tc_kernel, grid, dim3(192), (size_t)smem, s, tx, tw, to, p, dev_status);
   return finish_launch(e, rows, p.extra, s);
 }
 
