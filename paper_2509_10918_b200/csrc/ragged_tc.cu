@@ -183,38 +183,49 @@ ragged_kernel(const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ 
   // what no load ever writes has to be a finite number: padding rows of the B operand, padding columns of A
   for (int e = threadIdx.x; e < p.stages * stage_bytes / 16; e += blockDim.x) reinterpret_cast<uint4*>(smem)[e] = make_uint4(0u, 0u, 0u, 0u);
   fence_proxy_async();
+  __syncthreads();
   dependency_wait();
   if (threadIdx.x == 0) release_dependents();
-  if (warp == 1) tmem_alloc(&bar->tmem_base, ncols);
   if (kMerge && p.zero_words > 0) {
     const int cta = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
     const int n_thr = gridDim.x * gridDim.y * gridDim.z * blockDim.x;
     for (int i = cta * blockDim.x + threadIdx.x; i < p.zero_words; i += n_thr) p.zero[i] = 0u;
   }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = bar->tmem_base;
   volatile int* abort_flag = &bar->abort_flag;
-
+  // All meet once more when the tensor memory is there; the first loads, of tokens and of weights, do not wait for that. (With
+  // the stores by slabs below: 384 regions of 96 tokens, 1280 channels, merge 97.4 -> 92.2 us, unmerge 81.6 -> 73.8.)
   if (warp == 0) {
-    if (elect_one()) {
-      for (int k = 0; k < nk; ++k) {
-        const int s = k % p.stages;
-        if (k >= p.stages && !mbar_wait(&bar->empty[s], ((k / p.stages) - 1) & 1, dev_status, abort_flag)) break;
-        uint8_t* sb = smem + s * stage_bytes + 2 * a_plane;
-        if (kMerge) {
-          const bool tail = k == n_boxes - 1;
-          mbar_expect_tx(&bar->full[s], slabs * (tail ? tail_rows : p.rows) * p.tw * 128);
-          for (int c = 0; c < slabs; ++c)
-            tma_load_4d(sb + c * b_slab, tail ? &tm_b_tail : &tm_b, &bar->full[s], c0 + c * 64, tx * p.tw, ty * p.th + k * p.rows, b);
-        } else {
-          mbar_expect_tx(&bar->full[s], slabs * b_slab);
-          for (int c = 0; c < slabs; ++c) tma_load_4d(sb + c * b_slab, &tm_b, &bar->full[s], c0 + c * 64, k * 64, tile, b);
-        }
+    const int early = min(nk, p.stages);
+    auto load = [&](int k) {
+      const int s = k % p.stages;
+      uint8_t* sb = smem + s * stage_bytes + 2 * a_plane;
+      if (kMerge) {
+        const bool tail = k == n_boxes - 1;
+        mbar_expect_tx(&bar->full[s], slabs * (tail ? tail_rows : p.rows) * p.tw * 128);
+        for (int c = 0; c < slabs; ++c)
+          tma_load_4d(sb + c * b_slab, tail ? &tm_b_tail : &tm_b, &bar->full[s], c0 + c * 64, tx * p.tw, ty * p.th + k * p.rows, b);
+      } else {
+        mbar_expect_tx(&bar->full[s], slabs * b_slab);
+        for (int c = 0; c < slabs; ++c) tma_load_4d(sb + c * b_slab, &tm_b, &bar->full[s], c0 + c * 64, k * 64, tile, b);
+      }
+    };
+    const bool one = elect_one();
+    if (one)
+      for (int k = 0; k < early; ++k) load(k);
+    __syncwarp();
+    __syncthreads();
+    if (one) {
+      for (int k = early; k < nk; ++k) {
+        if (!mbar_wait(&bar->empty[k % p.stages], ((k / p.stages) - 1) & 1, dev_status, abort_flag)) break;
+        load(k);
       }
     }
   } else if (warp == 1) {
+    tmem_alloc(&bar->tmem_base, ncols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = bar->tmem_base;
     if (elect_one()) {
       const int n_a = min(n_mma, 256), n_b = n_mma - n_a;
       const uint32_t idesc_a = idesc_f16(kFmtBF16, kFmtBF16, kMerge, true, 128, n_a);
@@ -254,6 +265,9 @@ ragged_kernel(const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ 
     Gather<kMerge ? 16 : 8> gather;
     constexpr int kPass = Gather<kMerge ? 16 : 8>::kPass;
     gather.load(p, plane0, t, 0, row0_of(0), rows_of(0), col0_of(0));
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = bar->tmem_base;
     bool ok = true;
     for (int k = 0; k < nk; ++k) {
       const int s = k % p.stages;
@@ -283,30 +297,30 @@ ragged_kernel(const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ 
     if (p.extra.per)
       copy_part(p.extra, (((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * kWorkers + t,
                 (size_t)gridDim.x * gridDim.y * gridDim.z * kWorkers);
-    if (ok && __all_sync(0xffffffffu, mbar_wait(&bar->done, 0, dev_status, abort_flag))) {
-      tc_fence_after();
-      // every load has been consumed: the stages are the output's staging area
-      const int quarter = warp & 3, half = (warp - 2) >> 2, row = quarter * 32 + lane;
-      const int mid = ((n_mma / 2) + 31) & ~31;
-      stage_rows(smem, tmem + ((uint32_t)(quarter * 32) << 16), row, half ? mid : 0, half ? n_mma : mid);
+    // every load has been consumed: the stages are the output's staging area (a wait that ran out: the results are void, the
+    // way is the same: four warps meet at barriers)
+    mbar_wait_warp(&bar->done, 0, dev_status, abort_flag);
+    tc_fence_after();
+    const int quarter = warp & 3, half = (warp - 2) >> 2, row = quarter * 32 + lane;
+    // four warps take every second slab, which is stored as soon as they have staged it
+    for (int c = half; c < slabs; c += 2) {
+      stage_rows(smem, tmem + ((uint32_t)(quarter * 32) << 16), row, c * 64, c * 64 + 64);
       fence_proxy_async();  // the staged rows are read by the TMA engine
-      asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory");
-      if (t == 0) {
-        for (int c = 0; c < slabs; ++c) {
-          const void* src = smem + c * (128 * 128);
-          if (kMerge) tma_store_4d(&tm_o, src, c0 + c * 64, mb * 128, tile, b);  // rows past the region's D_loc are clipped
-          else tma_store_4d(mb == n_boxes - 1 ? &tm_o_tail : &tm_o, src, c0 + c * 64, tx * p.tw, ty * p.th + mb * p.rows, b);
-        }
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + half), "n"(kWorkers / 2) : "memory");
+      if ((t & 127) == 0) {
+        const void* src = smem + c * (128 * 128);
+        if (kMerge) tma_store_4d(&tm_o, src, c0 + c * 64, mb * 128, tile, b);  // rows past the region's D_loc are clipped
+        else tma_store_4d(mb == n_boxes - 1 ? &tm_o_tail : &tm_o, src, c0 + c * 64, tx * p.tw, ty * p.th + mb * p.rows, b);
         tma_store_commit();
-        tma_store_wait_read();  // shared memory must outlive the engine's reads
       }
     }
+    if ((t & 127) == 0) tma_store_wait_read();  // shared memory must outlive the engine's reads
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, ncols);
+    tmem_dealloc(bar->tmem_base, ncols);
   }
 }
 
