@@ -63,144 +63,6 @@ __device__ __forceinline__ void gelu2(uint32_t& v0, uint32_t& v1) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// Tiles of 256 rows x 256 columns, one per CTA: two 128-row blocks share every W slab, so a CTA moves 64 KB per
-// 256 x 256 x 64 multiply-adds instead of 48 KB per 128 x 256 x 64.  For long contractions, which are bound by the
-// operands' traffic from L2 and hide the prologue and the epilogue this form does not overlap.
-// ------------------------------------------------------------------------------------------------
-constexpr int kPairRows = 256, kPairCols = 256, kPairStages = 3;
-constexpr int kPairRing = 2 * 4 * 128 * 128;  // the output tile is staged where the ring was
-struct PairBars {
-  uint64_t full[kPairStages], empty[kPairStages], done;
-  uint32_t tmem_base;
-  int abort_flag;
-};
-
-__global__ void __launch_bounds__(192, 1)
-linear_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w0,
-                   const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__ CUtensorMap tm_w2,
-                   const __grid_constant__ CUtensorMap tm_c0, const __grid_constant__ CUtensorMap tm_c1,
-                   const __grid_constant__ CUtensorMap tm_c2, int M, int N, int K, int act, uint32_t* dev_status) {
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.x * kPairRows, n0 = blockIdx.y * kPairCols;
-  const CUtensorMap* tm_w = blockIdx.z == 0 ? &tm_w0 : blockIdx.z == 1 ? &tm_w1 : &tm_w2;
-  const CUtensorMap* tm_c = blockIdx.z == 0 ? &tm_c0 : blockIdx.z == 1 ? &tm_c1 : &tm_c2;
-  const int n_cols = min(kPairCols, N - n0);     // columns of this CTA (multiple of 8)
-  const int slabs = (n_cols + 63) / 64;
-  constexpr int kStageBytes = 2 * kABytes + kPairCols / 64 * kSlab;
-  PairBars* bar = reinterpret_cast<PairBars*>(smem + kPairStages * kStageBytes);
-  const int nk = (K + kKC - 1) / kKC;
-  constexpr uint32_t ncols = 512;
-  static_assert(kPairStages * kStageBytes >= kPairRing, "the output's staging area outgrew the ring");
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kPairStages; ++s) {
-      mbar_init(&bar->full[s], 1);
-      mbar_init(&bar->empty[s], 1);
-    }
-    mbar_init(&bar->done, 1);
-    bar->abort_flag = 0;
-    mbar_fence_init();
-    prefetch_tmap(&tm_a);
-    prefetch_tmap(tm_w);
-    prefetch_tmap(tm_c);
-  }
-  dependency_wait();
-  if (threadIdx.x == 0) release_dependents();
-  if (warp == 1) tmem_alloc(&bar->tmem_base, ncols);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = bar->tmem_base;
-  volatile int* abort_flag = &bar->abort_flag;
-
-  if (warp == 0) {
-    if (elect_one()) {
-      for (int k = 0; k < nk; ++k) {
-        const int s = k % kPairStages;
-        if (k >= kPairStages && !mbar_wait(&bar->empty[s], ((k / kPairStages) - 1) & 1, dev_status, abort_flag)) break;
-        uint8_t* sa = smem + s * kStageBytes;
-        mbar_expect_tx(&bar->full[s], 2 * kABytes + slabs * kSlab);
-        for (int rb = 0; rb < 2; ++rb) tma_load_2d(sa + rb * kABytes, &tm_a, &bar->full[s], k * kKC, m0 + rb * 128);
-        for (int j = 0; j < slabs; ++j)
-          tma_load_2d(sa + 2 * kABytes + j * kSlab, tm_w, &bar->full[s], n0 + j * 64, k * kKC);
-      }
-    }
-  } else if (warp == 1) {
-    if (elect_one()) {
-      const uint32_t idesc = idesc_f16(kFmtBF16, kFmtBF16, false, true, 128, slabs * 64);
-      bool ok = true;
-      for (int k = 0; k < nk; ++k) {
-        const int s = k % kPairStages;
-        if (!mbar_wait(&bar->full[s], (k / kPairStages) & 1, dev_status, abort_flag)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t aa = smem_u32(smem + s * kStageBytes), wa = aa + 2 * kABytes;
-        const int ksteps = min(kKC, K - k * kKC + 15) / 16;  // 16 contraction elements per MMA (zero filled past K)
-        for (int kk = 0; kk < ksteps; ++kk) {
-          const uint64_t wd = smem_desc_sw128(wa + kk * 2048, kSlab, 1024);
-#pragma unroll
-          for (int rb = 0; rb < 2; ++rb) {
-            const uint64_t ad = smem_desc_sw128(aa + rb * kABytes + kk * 32, 16, 1024);
-            mma_ss(tmem + rb * 256, ad, wd, idesc, k > 0 || kk > 0);
-          }
-        }
-        mma_commit(&bar->empty[s]);
-      }
-      if (ok) mma_commit(&bar->done);
-    }
-  } else {
-    const int quarter = warp & 3, r_in = quarter * 32 + lane;  // row inside a 128-row block = tensor-memory lane
-    // one answer per warp: the tensor-memory loads below are warp-wide operations
-    if (__all_sync(0xffffffffu, mbar_wait(&bar->done, 0, dev_status, abort_flag))) {
-      tc_fence_after();
-      // every load has been consumed: slab j of row block rb goes to smem + (rb * slabs + j) * 16 KB as
-      // [128 rows][128 B], 128-byte swizzled; a warp's 32 rows are 4 KB of it
-#pragma unroll 1
-      for (int rb = 0; rb < 2; ++rb) {
-        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + rb * 256;
-        for (int j = 0; j < n_cols; j += 32) {
-          uint32_t r[32];
-          tmem_ld32(taddr + j, r);
-          tmem_wait_ld();
-          if (act == kActGelu) {
-#pragma unroll
-            for (int e = 0; e < 32; e += 2) gelu2(r[e], r[e + 1]);
-          }
-          uint8_t* slab = smem + (rb * slabs + (j >> 6)) * (128 * 128);
-#pragma unroll
-          for (int e = 0; e < 32; e += 8) {
-            __align__(16) __nv_bfloat162 q[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-              q[u] = __floats2bfloat162_rn(__uint_as_float(r[e + 2 * u]), __uint_as_float(r[e + 2 * u + 1]));
-            *reinterpret_cast<uint4*>(slab + sw128_offset(r_in, ((j & 63) + e) >> 3)) = *reinterpret_cast<const uint4*>(q);
-          }
-        }
-      }
-      fence_proxy_async();  // the staged rows are read by the TMA engine
-      __syncwarp();
-      if (lane == 0) {
-        for (int rb = 0; rb < 2; ++rb) {
-          const int row0 = m0 + rb * 128 + quarter * 32;
-          if (row0 >= M) continue;  // rows past M and columns past N inside a box are clipped by the store
-          for (int j = 0; j < slabs; ++j)
-            tma_store_2d(tm_c, smem + (rb * slabs + j) * (128 * 128) + quarter * 4096, n0 + j * 64, row0);
-        }
-        tma_store_commit();
-        tma_store_wait_read();  // shared memory must outlive the engine's reads
-      }
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    tmem_dealloc(tmem, ncols);
-  }
-}
-
-// ------------------------------------------------------------------------------------------------
 // Persistent form: one CTA per SM walks over tiles of 128 rows x kCols columns.  The ring runs on across tiles, and two
 // accumulators in tensor memory alternate, so that a tile's epilogue (eight warps: a GELU per element is as long as the
 // tile's MMAs at K = 640) runs under the next tile's loads and MMAs.  Against one tile per CTA, four epilogue warps and
@@ -225,6 +87,40 @@ struct PersistCfg {
   static constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kStaging + 256;
   static constexpr uint32_t kAccCols = kCols == 128 ? 128 : 256;
 };
+
+// A warp's 32 rows of a tile, every second 64-column slab from `half` on: out of tensor memory, through the activation, staged
+// in `mine` (32 rows of 128 B) and stored.
+__device__ __forceinline__ void tile_out(uint32_t taddr, uint8_t* mine, int lane, const CUtensorMap* tm_c, int half, int slabs, int n0, int m0, int M,
+                                         int act) {
+#pragma unroll 1
+  for (int j = half; j < slabs; j += 2) {
+    if (lane == 0) tma_store_wait_read();  // the slab staged before has been read
+    __syncwarp();
+#pragma unroll 1
+    for (int c = 0; c < 64; c += 32) {
+      uint32_t r[32];
+      tmem_ld32(taddr + j * 64 + c, r);
+      tmem_wait_ld();
+      if (act == kActGelu) {
+#pragma unroll
+        for (int e = 0; e < 32; e += 2) gelu2(r[e], r[e + 1]);
+      }
+#pragma unroll
+      for (int e = 0; e < 32; e += 8) {
+        __align__(16) __nv_bfloat162 q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) q[u] = __floats2bfloat162_rn(__uint_as_float(r[e + 2 * u]), __uint_as_float(r[e + 2 * u + 1]));
+        *reinterpret_cast<uint4*>(mine + sw128_offset(lane, (c + e) >> 3)) = *reinterpret_cast<const uint4*>(q);
+      }
+    }
+    fence_proxy_async();  // the staged rows are read by the TMA engine
+    __syncwarp();
+    if (lane == 0 && m0 < M) {  // rows past M and columns past N inside a box are clipped by the store
+      tma_store_2d(tm_c, mine, n0 + j * 64, m0);
+      tma_store_commit();
+    }
+  }
+}
 
 template <int kCols>
 __global__ void __launch_bounds__((2 + kEpiWarps) * 32, 1)
@@ -323,35 +219,7 @@ linear_persistent_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_
       if (!__all_sync(0xffffffffu, mbar_wait(&bar->acc_full[a], (n >> 1) & 1, dev_status, abort_flag))) break;
       tc_fence_after();
       const uint32_t taddr = tmem + a * C::kAccCols + ((uint32_t)(quarter * 32) << 16);
-#pragma unroll 1
-      for (int j = half; j < slabs; j += 2) {
-        if (lane == 0) tma_store_wait_read();  // the slab staged before has been read
-        __syncwarp();
-#pragma unroll 1
-        for (int c = 0; c < 64; c += 32) {
-          uint32_t r[32];
-          tmem_ld32(taddr + j * 64 + c, r);
-          tmem_wait_ld();
-          if (act == kActGelu) {
-#pragma unroll
-            for (int e = 0; e < 32; e += 2) gelu2(r[e], r[e + 1]);
-          }
-#pragma unroll
-          for (int e = 0; e < 32; e += 8) {
-            __align__(16) __nv_bfloat162 q[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-              q[u] = __floats2bfloat162_rn(__uint_as_float(r[e + 2 * u]), __uint_as_float(r[e + 2 * u + 1]));
-            *reinterpret_cast<uint4*>(mine + sw128_offset(lane, (c + e) >> 3)) = *reinterpret_cast<const uint4*>(q);
-          }
-        }
-        fence_proxy_async();  // the staged rows are read by the TMA engine
-        __syncwarp();
-        if (lane == 0 && m0 < M) {  // rows past M and columns past N inside a box are clipped by the store
-          tma_store_2d(tm_c, mine, n0 + j * 64, m0);
-          tma_store_commit();
-        }
-      }
+      tile_out(taddr, mine, lane, tm_c, half, slabs, n0, m0, M, act);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar->acc_empty[a]);
@@ -364,6 +232,140 @@ linear_persistent_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_
     tc_fence_after();
     tmem_dealloc(tmem, 2 * C::kAccCols);
   }
+}
+
+// ------------------------------------------------------------------------------------------------
+// The same by pairs of SMs: a cluster of two CTAs walks over tiles of 256 rows x 256 columns.  Each CTA loads and keeps 128 of
+// the rows of A and 128 of the columns of W, the first one's thread issues the MMAs of both (cta_group::2).  An SM then takes
+// in 32 KB and reads 32 KB out of shared memory per 128 x 256 x 64 multiply-adds (512 cycles) where one working alone takes in
+// and reads 48 KB each, which is more than the 128 bytes a cycle that shared memory has.  4096 x 2560 x 640 16.5 -> 15.0 us,
+// 8192 x 1280 x 1280 25.6 -> 23.9, 16384 x 8192 x 4096 1092 -> 925 (rows x columns x contraction; against 256 x 256 by one CTA
+// for the last).  A k-step still takes about 650 cycles: six stages do not quite cover the way from a free slot to its loads.
+// Both CTAs' loads count on the first one's barrier; MMA completion is committed to both.
+// ------------------------------------------------------------------------------------------------
+constexpr int kPairRows = 256, kPairCols = 256, kPairStages = 6;
+constexpr int kPairStageBytes = kABytes + 2 * kSlab;     // a CTA's half
+constexpr int kPairStaging = kEpiWarps * 32 * 128;
+constexpr int kPairSmem = 1024 + kPairStages * kPairStageBytes + kPairStaging + 256;
+struct PairBars {
+  uint64_t full[kPairStages], empty[kPairStages];  // (full: of the first CTA)
+  uint64_t acc_full[2], acc_empty[2];
+  uint32_t tmem_base;
+  int abort_flag;
+};
+static_assert(sizeof(PairBars) <= 256, "barrier block outgrew its reservation");
+
+__global__ void __launch_bounds__((2 + kEpiWarps) * 32, 1)
+linear_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w0,
+                   const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__ CUtensorMap tm_w2,
+                   const __grid_constant__ CUtensorMap tm_c0, const __grid_constant__ CUtensorMap tm_c1,
+                   const __grid_constant__ CUtensorMap tm_c2, int M, int N, int K, int n_items, int act, uint32_t* dev_status) {
+  extern __shared__ uint8_t smem_raw[];
+  // (the same offset in both CTAs: they are launched alike)
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* staging = smem + kPairStages * kPairStageBytes;
+  PairBars* bar = reinterpret_cast<PairBars*>(staging + kPairStaging);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_rank();
+  const int nk = (K + kKC - 1) / kKC;
+  const int mb = (M + kPairRows - 1) / kPairRows, nb = (N + kPairCols - 1) / kPairCols;
+  const int pair = blockIdx.x / 2, pairs = gridDim.x / 2;
+  // item -> row block (fastest), column block, matrix; this CTA's rows and columns of it
+  auto m_of = [&](int item) { return item % mb * kPairRows; };
+  auto n_of = [&](int item) { return item / mb % nb * kPairCols; };
+  auto z_of = [&](int item) { return item / mb / nb; };
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kPairStages; ++s) {
+      mbar_init(&bar->full[s], 1);
+      mbar_init(&bar->empty[s], 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(&bar->acc_full[a], 1);
+      mbar_init(&bar->acc_empty[a], 2 * kEpiWarps);
+    }
+    bar->abort_flag = 0;
+    mbar_fence_init();
+    prefetch_tmap(&tm_a);
+    prefetch_tmap(&tm_w0);
+    prefetch_tmap(&tm_c0);
+  }
+  cluster_sync();  // both CTAs' barriers are there
+  dependency_wait();
+  if (threadIdx.x == 0) release_dependents();
+  if (warp == 1) tmem_alloc_pair(&bar->tmem_base, 512);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = bar->tmem_base;
+  volatile int* abort_flag = &bar->abort_flag;
+
+  if (warp == 0) {
+    if (elect_one()) {
+      int kc = 0;  // k-steps so far, over all items: ring slot and phase follow it
+      bool ok = true;
+      for (int item = pair; ok && item < n_items; item += pairs) {
+        const int m0 = m_of(item) + rank * 128, n0 = n_of(item) + rank * 128, z = z_of(item);
+        const CUtensorMap* tm_w = z == 0 ? &tm_w0 : z == 1 ? &tm_w1 : &tm_w2;
+        for (int k = 0; k < nk; ++k, ++kc) {
+          const int s = kc % kPairStages;
+          if (kc >= kPairStages && !mbar_wait(&bar->empty[s], ((kc / kPairStages) - 1) & 1, dev_status, abort_flag)) { ok = false; break; }
+          uint8_t* sa = smem + s * kPairStageBytes;
+          if (rank == 0) mbar_expect_tx(&bar->full[s], 2 * kPairStageBytes);  // what lies past M or N comes as zeros and counts
+          tma_load_2d_pair(sa, &tm_a, &bar->full[s], k * kKC, m0);
+          for (int j = 0; j < 2; ++j) tma_load_2d_pair(sa + kABytes + j * kSlab, tm_w, &bar->full[s], n0 + j * 64, k * kKC);
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (rank == 0) {
+      if (elect_one()) {
+        constexpr uint32_t idesc = idesc_f16(kFmtBF16, kFmtBF16, false, true, kPairRows, kPairCols);
+        int kc = 0, n = 0;
+        bool ok = true;
+        for (int item = pair; ok && item < n_items; item += pairs, ++n) {
+          const int a = n & 1;
+          if (n >= 2 && !mbar_wait(&bar->acc_empty[a], ((n >> 1) - 1) & 1, dev_status, abort_flag)) break;
+          tc_fence_after();
+          for (int k = 0; k < nk; ++k, ++kc) {
+            const int s = kc % kPairStages;
+            if (!mbar_wait(&bar->full[s], (kc / kPairStages) & 1, dev_status, abort_flag)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t aa = smem_u32(smem + s * kPairStageBytes), wa = aa + kABytes;
+            const int ksteps = min(kKC, K - k * kKC + 15) / 16;  // 16 contraction elements per MMA (zero filled past K)
+            for (int kk = 0; kk < ksteps; ++kk)
+              mma_ss_pair(tmem + a * 256, smem_desc_sw128(aa + kk * 32, 16, 1024), smem_desc_sw128(wa + kk * 2048, kSlab, 1024), idesc, k > 0 || kk > 0);
+            mma_commit_pair(&bar->empty[s]);
+          }
+          if (ok) mma_commit_pair(&bar->acc_full[a]);
+        }
+      }
+    }
+  } else {
+    // two warps per quarter of the CTA's rows, each with every second 64-column slab
+    const int quarter = warp & 3, half = (warp - 2) >> 2;
+    uint8_t* mine = staging + (warp - 2) * 4096;
+    int n = 0;
+    for (int item = pair; item < n_items; item += pairs, ++n) {
+      const int a = n & 1, m0 = m_of(item) + rank * 128 + quarter * 32, n0 = n_of(item), z = z_of(item), slabs = (min(kPairCols, N - n0) + 63) / 64;
+      const CUtensorMap* tm_c = z == 0 ? &tm_c0 : z == 1 ? &tm_c1 : &tm_c2;
+      // one answer per warp: the tensor-memory loads below are warp-wide operations
+      if (!__all_sync(0xffffffffu, mbar_wait(&bar->acc_full[a], (n >> 1) & 1, dev_status, abort_flag))) break;
+      tc_fence_after();
+      tile_out(tmem + a * 256 + ((uint32_t)(quarter * 32) << 16), mine, lane, tm_c, half, slabs, n0, m0, M, act);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_at(peer_addr(smem_u32(&bar->acc_empty[a]), 0));  // of the issuing CTA, which may be this one
+    }
+    if (lane == 0) tma_store_wait_read();  // shared memory must outlive the engine's reads
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem, 512);
+  }
+  cluster_sync();  // neither leaves while the other's MMAs read its shared memory or its arrivals are under way
 }
 
 template <int kCols>
@@ -402,29 +404,29 @@ cudaError_t launch_linear_tc(int M, int N, int K, const void* a, const void* con
       return cudaErrorInvalidValue;
   }
   // Tile form: the one with the least serial work per SM, i.e. tiles per SM (rounded up) times the time of one, which was
-  // timed on fourteen shapes between 200 x 640 x 640 and 32768 x 2560 x 640: a tile of 128 x 192 takes 1.2 times, one of
-  // 128 x 256 1.35 times as long as one of 128 x 128 (they read fewer operand bytes per multiply-add, and L2's rate is
-  // what bounds these shapes), one of 256 x 256 2.5 times - 4 % less than two of 128 x 256 from about 2048 contraction
-  // elements on, more below, where its epilogue shows.
+  // timed on seventeen shapes between 200 x 640 x 640 and 16384 x 8192 x 4096: a tile of 128 x 192 takes 1.2 times, one of
+  // 128 x 256 1.35 times as long as one of 128 x 128 (they read fewer operand bytes per multiply-add), a pair's of 256 x 256
+  // 1.25 times - 1.1 from about 2048 contraction elements on - and a fifth more per launch for the cluster's start and end.
   const int sms = sm_count();
-  auto cost = [&](int rows, int cols, int tile) {
+  auto cost = [&](int rows, int cols, int tile, int at_once) {
     const long long tiles = (long long)((M + rows - 1) / rows) * ((N + cols - 1) / cols) * n_mats;
-    return (tiles + sms - 1) / sms * tile;
+    return (tiles + at_once - 1) / at_once * tile;
   };
-  const long long cost128 = cost(128, 128, 20), cost192 = cost(128, 192, 24), cost256 = cost(128, 256, 27);
-  const long long cost_pair = M > 128 && K >= 2048 ? cost(kPairRows, kPairCols, 50) : LLONG_MAX;
+  const long long cost128 = cost(128, 128, 20, sms), cost192 = cost(128, 192, 24, sms), cost256 = cost(128, 256, 27, sms);
+  const long long cost_pair = M > 128 && sms >= 2 ? cost(kPairRows, kPairCols, K >= 2048 ? 22 : 25, sms / 2) + 4 : LLONG_MAX;
   int form = cost128 <= cost192 && cost128 <= cost256 ? 4 : cost192 <= cost256 ? 2 : 1;
   if (cost_pair < cost128 && cost_pair < cost192 && cost_pair < cost256) form = 3;
   // test-only override: 128 x 256 (1), 128 x 192 (2), 256 x 256 (3) or 128 x 128 (4) tiles
   if (const int v = g_tune_linear_tile.load(std::memory_order_relaxed); v && (v != 3 || M > 128)) form = v;
   cudaError_t e;
   if (form == 3) {
-    constexpr int smem = 1024 + kPairStages * (2 * kABytes + kPairCols / 64 * kSlab) + 256;
     static std::atomic<unsigned long long> raised{0};
-    if (e = raise_dynamic_smem(linear_pair_kernel, smem, raised); e != cudaSuccess) return e;
-    const dim3 grid((M + kPairRows - 1) / kPairRows, (N + kPairCols - 1) / kPairCols, n_mats);
-    e = launch_dependent(linear_pair_kernel, grid, dim3(192), (size_t)smem, s, ta, tw[0], tw[1], tw[2], tc_[0], tc_[1], tc_[2], M, N, K, act,
-                         dev_status);
+    if (e = raise_dynamic_smem(linear_pair_kernel, kPairSmem, raised); e != cudaSuccess) return e;
+    const long long items = (long long)((M + kPairRows - 1) / kPairRows) * ((N + kPairCols - 1) / kPairCols) * n_mats;
+    if (items > INT32_MAX / 2) return cudaErrorInvalidValue;
+    const int pairs = items < sms / 2 ? (int)items : sms / 2;
+    e = launch_dependent_cluster(linear_pair_kernel, dim3(2 * pairs), dim3((2 + kEpiWarps) * 32), (size_t)kPairSmem, 2, s, ta, tw[0], tw[1], tw[2],
+                                 tc_[0], tc_[1], tc_[2], M, N, K, (int)items, act, dev_status);
   } else {
     e = form == 4   ? run_persistent<128>(M, N, K, n_mats, ta, tw, tc_, act, dev_status, s)
         : form == 2 ? run_persistent<192>(M, N, K, n_mats, ta, tw, tc_, act, dev_status, s)

@@ -1427,3 +1427,20 @@ def test_merge_and_unmerge_of_box_regions(toma, th, tw, ratio, dim, batch):
     want = dense.transpose(2, 3) @ y.double().reshape(batch, cfg.n_tiles, run.d_loc, dim)
     assert_close(_regions(cfg, out).cpu().numpy(), want.cpu().numpy(), "bf16", "unmerge")
     assert bool((guard == 7.0).all())
+
+
+@pytest.mark.parametrize("m,n,k", [(9000, 1016, 72), (20000, 64, 200), (40000, 520, 24), (257, 256, 512), (256, 264, 640)])
+def test_linear_several_tiles_per_pair(toma, tuning, m, n, k):
+    """The form of two SMs per 256 x 256 tile, forced: more tiles than pairs, so that its ring runs on across them; a second
+    CTA without rows, a second column half without columns; as many k-steps as stages, and more."""
+    tuning(linear_tile=3)
+    rng = np.random.default_rng(m)
+    a = torch.from_numpy(rng.standard_normal((m, k)).astype(np.float32)).cuda().to(torch.bfloat16)
+    w = torch.from_numpy((rng.standard_normal((k, n)) / np.sqrt(k)).astype(np.float32)).cuda().to(torch.bfloat16)
+    c = torch.full((m, n), float("nan"), dtype=a.dtype, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    toma.toma_linear(a, w, c, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert not torch.isnan(c).any()
+    assert_close(to_host64(c), (a.double() @ w.double()).cpu().numpy(), "bf16", "linear")
