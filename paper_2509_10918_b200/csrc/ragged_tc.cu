@@ -209,12 +209,11 @@ ragged_kernel(const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ 
         for (int c = 0; c < slabs; ++c) tma_load_4d(sb + c * b_slab, &tm_b, &bar->full[s], c0 + c * 64, k * 64, tile, b);
       }
     };
-    const bool one = elect_one();
-    if (one)
+    if (elect_one())
       for (int k = 0; k < early; ++k) load(k);
     __syncwarp();
     __syncthreads();
-    if (one) {
+    if (elect_one()) {
       for (int k = early; k < nk; ++k) {
         if (!mbar_wait(&bar->empty[k % p.stages], ((k / p.stages) - 1) & 1, dev_status, abort_flag)) break;
         load(k);
