@@ -7,9 +7,15 @@
 // tx + 32, tx + 48, whose rows of DH + 4 floats fall into different banks) and 4 x DH / 16 outputs, four contraction
 // steps per 16-byte shared read, so that 64 multiply-adds go with eight reads.  Scores become probabilities in
 // registers (row maxima and sums by shuffles within the sixteen lanes) and pass through shared memory once, between
-// lanes of one half warp.  Bound by the FMA pipe; 10 heads x 512 tokens x 64 channels, fp32: 159 us with one thread
-// per query and quarter row before.
+// lanes of one half warp.  Bound by the FMA pipe where there are queries enough to fill it (16 warps per SM).  Where there are
+// not, the four warps of 32 queries wait for their own latencies - 10 heads x 512 tokens x 64 channels, fp32: 46 us, 9 of
+// them multiply-adds -, and so three or four groups of warps share the queries, each with every third or fourth key tile, a
+// reference and sums of its own, added up at the end (KG): 28 us.  512 tokens of 20 heads of 128 223 -> 206, bound by reads of
+// shared memory, as are all (2.8 cycles for each of them, eight for 32 packed multiply-adds).
+#include <float.h>
+
 #include "common.cuh"
+#include "tc.cuh"
 
 namespace toma {
 
@@ -30,80 +36,112 @@ __device__ __forceinline__ void copy16(float* dst, const __nv_bfloat16* src, boo
   *reinterpret_cast<float4*>(dst) = v;
 }
 
-template <int DH, int BQ>
+// KG groups of BQ * 4 threads.  One group: K and V double buffered; several: one buffer of each per group, the next K on its
+// way from the scores on, the next V from the outputs on.
+template <int DH, int BQ, int KG>
 struct SimtCfg {
   static constexpr int kPitch = DH + 4;
   static constexpr int kTile = kKeys * kPitch;
   static constexpr int kPPitch = kKeys + 4;
-  static constexpr size_t kSmem = ((size_t)BQ * kPitch + 4 * kTile + (size_t)BQ * kPPitch) * 4;
+  static constexpr int kBufs = KG == 1 ? 2 : 1;
+  static constexpr int kGroup = 2 * kBufs * kTile + BQ * kPPitch;
+  static constexpr size_t kSmem = ((size_t)BQ * kPitch + (size_t)KG * kGroup) * 4;
+  static_assert(BQ * DH <= kTile && 2 * BQ <= kPPitch * BQ, "a group's outputs and sums fit where its tiles were");
 };
 
-template <typename T, int DH, int BQ>
-__global__ void __launch_bounds__(BQ * 4) attention_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-                                                                T* __restrict__ o, int L, int heads, float scale) {
-  using C = SimtCfg<DH, BQ>;
+template <typename T, int DH, int BQ, int KG>
+__global__ void __launch_bounds__(BQ * 4 * KG) attention_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
+                                                                     T* __restrict__ o, int L, int heads, float scale) {
+  using C = SimtCfg<DH, BQ, KG>;
   constexpr int kThreads = BQ * 4, DV = DH / 16;
   extern __shared__ __align__(16) float att_smem[];
-  float* Qs = att_smem;                  // [BQ][pitch], scaled
-  float* Ks = Qs + BQ * C::kPitch;       // [2][64][pitch]
-  float* Vs = Ks + 2 * C::kTile;         // [2][64][pitch]
-  float* Ps = Vs + 2 * C::kTile;         // [BQ][64 + 4]
-  const int b = blockIdx.z, h = blockIdx.y, q0 = blockIdx.x * BQ, tid = threadIdx.x;
+  const int group = KG == 1 ? 0 : threadIdx.x / kThreads, tid = KG == 1 ? threadIdx.x : threadIdx.x % kThreads;
+  float* Qs = att_smem;                                // [BQ][pitch], scaled
+  float* Ks = Qs + BQ * C::kPitch + group * C::kGroup; // [bufs][64][pitch]
+  float* Vs = Ks + C::kBufs * C::kTile;                // [bufs][64][pitch]
+  float* Ps = Vs + C::kBufs * C::kTile;                // [BQ][64 + 4]
+  const int b = blockIdx.z, h = blockIdx.y, q0 = blockIdx.x * BQ;
   const int tx = tid & 15, r0 = (tid >> 4) * 4;
   const size_t row_stride = (size_t)heads * DH;
   const size_t base = (size_t)b * L * row_stride + (size_t)h * DH;
-  auto load_tile = [&](int k0, int st) {
+  auto load_one = [&](float* dst, const T* src, int k0) {
 #pragma unroll 4
     for (int e = tid; e < kKeys * (DH / 4); e += kThreads) {
       const int r = e / (DH / 4), c = (e % (DH / 4)) * 4;
       const bool in = k0 + r < L;
-      const size_t off = base + (size_t)(in ? k0 + r : 0) * row_stride + c;
-      copy16(Ks + st * C::kTile + r * C::kPitch + c, k + off, in);
-      copy16(Vs + st * C::kTile + r * C::kPitch + c, v + off, in);
+      copy16(dst + r * C::kPitch + c, src + base + (size_t)(in ? k0 + r : 0) * row_stride + c, in);
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  load_tile(0, 0);
-  for (int e = tid; e < BQ * DH; e += kThreads) {
+  auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+  auto load_tile = [&](int k0, int st) {
+    load_one(Ks + st * C::kTile, k, k0);
+    load_one(Vs + st * C::kTile, v, k0);
+    commit();
+  };
+  auto group_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(kThreads) : "memory"); };
+  tc::dependency_wait();  // launched with programmatic stream serialisation
+  if (threadIdx.x == 0) tc::release_dependents();
+  if constexpr (KG == 1) {
+    load_tile(0, 0);
+  } else {
+    load_one(Ks, k, group * kKeys);
+    commit();
+    load_one(Vs, v, group * kKeys);
+    commit();
+  }
+  for (int e = threadIdx.x; e < BQ * DH; e += kThreads * KG) {
     const int r = e / DH, c = e % DH;
     Qs[r * C::kPitch + c] = q0 + r < L ? to_f32(q[base + (size_t)(q0 + r) * row_stride + c]) * scale : 0.f;
   }
-  float acc[4][DV] = {}, m[4], l[4];
+  // outputs of two channels in a register pair (one for DV = 1: the second of the pair is not used)
+  constexpr int kPairs = (DV + 1) / 2;
+  uint64_t acc[4][kPairs] = {};
+  float m[4], l[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) m[i] = -INFINITY, l[i] = 0.f;
+  for (int i = 0; i < 4; ++i) m[i] = KG > 1 ? -FLT_MAX : -INFINITY, l[i] = 0.f;  // one group's keys may all be at -infinity
   int st = 0;
-  for (int k0 = 0; k0 < L; k0 += kKeys, st ^= 1) {
-    if (k0 + kKeys < L) {
-      load_tile(k0 + kKeys, st ^ 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
+  if constexpr (KG > 1) __syncthreads();  // the queries
+  for (int k0 = group * kKeys; k0 < L; k0 += KG * kKeys, st ^= C::kBufs - 1) {
+    if constexpr (KG > 1) {
+      asm volatile("cp.async.wait_group 1;" ::: "memory");  // K; V may still be on its way
+      group_sync();
     } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      if (k0 + kKeys < L) {
+        load_tile(k0 + kKeys, st ^ 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+      } else {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+      }
+      __syncthreads();
     }
-    __syncthreads();
     const float* Kt = Ks + st * C::kTile + tx * C::kPitch;
     const float* Qt = Qs + r0 * C::kPitch;
-    // four chains of DH / 4 channels instead of one of DH: half the rounding error of a score
+    // eight chains of DH / 8 channels instead of one of DH (a third of the rounding error of a score), the even and the odd
+    // channels of a quarter in one packed multiply-add
     float s[4][4] = {};
 #pragma unroll 1
     for (int c0 = 0; c0 < DH; c0 += DH / 4) {
-      float part[4][4] = {};
-#pragma unroll 4
+      uint64_t part[4][4] = {};
+#pragma unroll 8
       for (int c = c0; c < c0 + DH / 4; c += 4) {
-        float4 a[4], w[4];
+        ulonglong2 a[4], w[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(Qt + i * C::kPitch + c);
+        for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const ulonglong2*>(Qt + i * C::kPitch + c);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const float4*>(Kt + j * 16 * C::kPitch + c);
+        for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const ulonglong2*>(Kt + j * 16 * C::kPitch + c);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            part[i][j] = fmaf(a[i].w, w[j].w, fmaf(a[i].z, w[j].z, fmaf(a[i].y, w[j].y, fmaf(a[i].x, w[j].x, part[i][j]))));
+          for (int j = 0; j < 4; ++j) part[i][j] = tc::fma2(a[i].y, w[j].y, tc::fma2(a[i].x, w[j].x, part[i][j]));
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) s[i][j] += part[i][j];
+        for (int j = 0; j < 4; ++j) {
+          float even, odd;
+          tc::unpack2(part[i][j], even, odd);
+          s[i][j] += even + odd;
+        }
     }
     if (k0 + kKeys > L) {
 #pragma unroll
@@ -129,11 +167,19 @@ __global__ void __launch_bounds__(BQ * 4) attention_simt_kernel(const T* __restr
       }
       l[i] = l[i] * corr + sum;  // this lane's keys; the sixteen lanes' sums meet at the end
 #pragma unroll
-      for (int c = 0; c < DV; ++c) acc[i][c] *= corr;
+      for (int c = 0; c < kPairs; ++c) acc[i][c] = tc::mul2(acc[i][c], tc::pack2(corr, corr));
     }
-    __syncwarp();  // a row's probabilities are written and read by the same half warp
+    if constexpr (KG > 1) {
+      group_sync();  // K has been read
+      if (k0 + KG * kKeys < L) load_one(Ks, k, k0 + KG * kKeys);
+      commit();
+      asm volatile("cp.async.wait_group 1;" ::: "memory");  // V
+      group_sync();
+    } else {
+      __syncwarp();  // a row's probabilities are written and read by the same half warp
+    }
     const float* Vt = Vs + st * C::kTile;
-#pragma unroll 2
+#pragma unroll 4
     for (int kk = 0; kk < kKeys; kk += 4) {
       float4 p[4];
 #pragma unroll
@@ -141,57 +187,119 @@ __global__ void __launch_bounds__(BQ * 4) attention_simt_kernel(const T* __restr
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const float* vr = Vt + (kk + u) * C::kPitch;
-        float vv[DV];  // channels tx DV .. (DV <= 4), or tx 4 .. and 64 + tx 4 ..
+        uint64_t vv[kPairs];  // channels tx DV .. (DV <= 4), or tx 4 .. and 64 + tx 4 ..
         if constexpr (DV >= 4) {
 #pragma unroll
           for (int g = 0; g < DV / 4; ++g) {
-            const float4 t = *reinterpret_cast<const float4*>(vr + g * 64 + tx * 4);
-            vv[4 * g] = t.x; vv[4 * g + 1] = t.y; vv[4 * g + 2] = t.z; vv[4 * g + 3] = t.w;
+            const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(vr + g * 64 + tx * 4);
+            vv[2 * g] = t.x, vv[2 * g + 1] = t.y;
           }
+        } else if constexpr (DV == 2) {
+          vv[0] = *reinterpret_cast<const uint64_t*>(vr + tx * 2);
         } else {
-#pragma unroll
-          for (int c = 0; c < DV; ++c) vv[c] = vr[tx * DV + c];
+          vv[0] = tc::pack2(vr[tx], 0.f);
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float pu = u == 0 ? p[i].x : u == 1 ? p[i].y : u == 2 ? p[i].z : p[i].w;
+          const uint64_t p2 = tc::pack2(pu, pu);
 #pragma unroll
-          for (int c = 0; c < DV; ++c) acc[i][c] = fmaf(pu, vv[c], acc[i][c]);
+          for (int c = 0; c < kPairs; ++c) acc[i][c] = tc::fma2(p2, vv[c], acc[i][c]);
         }
       }
     }
-    __syncthreads();  // this stage's tiles are overwritten next
+    if constexpr (KG > 1) {
+      group_sync();  // V and the probabilities have been read
+      if (k0 + KG * kKeys < L) load_one(Vs, v, k0 + KG * kKeys);
+      commit();
+    } else {
+      __syncthreads();  // this stage's tiles are overwritten next
+    }
   }
+  float out[4][2 * kPairs];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float sum = l[i];
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int x = 8; x > 0; x >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, x);
-    const float inv = 1.f / sum;
-    if (q0 + r0 + i < L) {
-      T* dst = o + base + (size_t)(q0 + r0 + i) * row_stride;
+    for (int c = 0; c < kPairs; ++c) tc::unpack2(acc[i][c], out[i][2 * c], out[i][2 * c + 1]);
+  if constexpr (KG > 1) {
+    // the groups' outputs and sums, to where their tiles were, and from there into one
+    asm volatile("cp.async.wait_group 0;" ::: "memory");  // a group without a tile has fetched zeros
+    group_sync();
+    float* mine = Ks;  // [BQ][DH]
+    float* ml = Ps;    // m[BQ], l[BQ]
 #pragma unroll
-      for (int c = 0; c < DV; ++c) from_f32(dst[DV >= 4 ? (c / 4) * 64 + tx * 4 + c % 4 : tx * DV + c], acc[i][c] * inv);
+    for (int i = 0; i < 4; ++i) {
+      float sum = l[i];
+#pragma unroll
+      for (int x = 8; x > 0; x >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, x);
+      if (tx == 0) ml[r0 + i] = m[i], ml[BQ + r0 + i] = sum;
+#pragma unroll
+      for (int c = 0; c < DV; ++c) mine[(r0 + i) * DH + (DV >= 4 ? (c / 4) * 64 + tx * 4 + c % 4 : tx * DV + c)] = out[i][c];
+    }
+    __syncthreads();
+    const float* all = att_smem + BQ * C::kPitch;
+    for (int e = threadIdx.x; e < BQ * DH / 4; e += kThreads * KG) {
+      const int r = e / (DH / 4), c = (e % (DH / 4)) * 4;
+      float M = -INFINITY, sum = 0.f;
+#pragma unroll
+      for (int g = 0; g < KG; ++g) M = fmaxf(M, all[g * C::kGroup + 2 * C::kBufs * C::kTile + r]);
+      float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int g = 0; g < KG; ++g) {
+        const float* p = all + g * C::kGroup;
+        const float w = expf(p[2 * C::kBufs * C::kTile + r] - M);  // a group without a tile: 0
+        sum = fmaf(w, p[2 * C::kBufs * C::kTile + BQ + r], sum);
+        const float4 a = *reinterpret_cast<const float4*>(p + r * DH + c);
+        t.x = fmaf(w, a.x, t.x), t.y = fmaf(w, a.y, t.y), t.z = fmaf(w, a.z, t.z), t.w = fmaf(w, a.w, t.w);
+      }
+      const float inv = 1.f / sum;
+      if (q0 + r < L) {
+        T* dst = o + base + (size_t)(q0 + r) * row_stride + c;
+        from_f32(dst[0], t.x * inv), from_f32(dst[1], t.y * inv), from_f32(dst[2], t.z * inv), from_f32(dst[3], t.w * inv);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float sum = l[i];
+#pragma unroll
+      for (int x = 8; x > 0; x >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, x);
+      const float inv = 1.f / sum;
+      if (q0 + r0 + i < L) {
+        T* dst = o + base + (size_t)(q0 + r0 + i) * row_stride;
+#pragma unroll
+        for (int c = 0; c < DV; ++c) from_f32(dst[DV >= 4 ? (c / 4) * 64 + tx * 4 + c % 4 : tx * DV + c], out[i][c] * inv);
+      }
     }
   }
 }
 
-template <typename T, int DH, int BQ>
+template <typename T, int DH, int BQ, int KG>
 cudaError_t run_one(int B, int L, int heads, const void* q, const void* k, const void* v, void* o, cudaStream_t s) {
+  using C = SimtCfg<DH, BQ, KG>;
   static std::atomic<unsigned long long> raised{0};
-  if (cudaError_t e = raise_dynamic_smem(attention_simt_kernel<T, DH, BQ>, (int)SimtCfg<DH, BQ>::kSmem, raised); e != cudaSuccess) return e;
+  if (cudaError_t e = raise_dynamic_smem(attention_simt_kernel<T, DH, BQ, KG>, (int)C::kSmem, raised); e != cudaSuccess) return e;
   const dim3 grid((L + BQ - 1) / BQ, heads, B);
-  attention_simt_kernel<T, DH, BQ><<<grid, BQ * 4, SimtCfg<DH, BQ>::kSmem, s>>>((const T*)q, (const T*)k, (const T*)v, (T*)o, L, heads,
-                                                                              1.0f / sqrtf((float)DH));
   count_launch();
-  return cudaGetLastError();
+  return launch_dependent(attention_simt_kernel<T, DH, BQ, KG>, grid, dim3(BQ * 4 * KG), C::kSmem, s, (const T*)q, (const T*)k, (const T*)v, (T*)o, L,
+                          heads, 1.0f / sqrtf((float)DH));
 }
 
 template <typename T, int DH>
 cudaError_t run(int B, int L, int heads, const void* q, const void* k, const void* v, void* o, cudaStream_t s) {
-  // 64 queries per CTA read K and V half as often; 32 while that would not give every SM two CTAs
+  // 64 queries per CTA read K and V half as often and two CTAs fill an SM.  Where that would not give every SM two CTAs, 32 or
+  // 40, one CTA per SM, their keys dealt out to as many groups of warps as shared memory and registers hold: whichever leaves
+  // the fullest SM fewer queries (512 tokens of 10 heads are 160 CTAs of 32 on 148 SMs, and 130 of 40).
   const long long ctas64 = (long long)((L + 63) / 64) * heads * B;
-  return ctas64 >= 2LL * sm_count() ? run_one<T, DH, 64>(B, L, heads, q, k, v, o, s) : run_one<T, DH, 32>(B, L, heads, q, k, v, o, s);
+  if (ctas64 >= 2LL * sm_count()) return run_one<T, DH, 64, 1>(B, L, heads, q, k, v, o, s);
+  auto fullest = [&](int bq) { return ((long long)((L + bq - 1) / bq) * heads * B + sm_count() - 1) / sm_count() * bq; };
+  if constexpr (DH == 128) {
+    // bound by shared-memory reads, and two groups would not have a second K and V: one group, 64 queries where the fullest SM
+    // has no more of them so (3 x 300 tokens, 7 heads: 60 us with 32, 46 with 64)
+    return fullest(64) <= fullest(32) ? run_one<T, DH, 64, 1>(B, L, heads, q, k, v, o, s) : run_one<T, DH, 32, 1>(B, L, heads, q, k, v, o, s);
+  } else {
+    return fullest(40) < fullest(32) ? run_one<T, DH, 40, 3>(B, L, heads, q, k, v, o, s) : run_one<T, DH, 32, 4>(B, L, heads, q, k, v, o, s);
+  }
 }
 
 template <typename T>

@@ -1444,3 +1444,41 @@ def test_linear_several_tiles_per_pair(toma, tuning, m, n, k):
     assert int(status.item()) == 0
     assert not torch.isnan(c).any()
     assert_close(to_host64(c), (a.double() @ w.double()).cpu().numpy(), "bf16", "linear")
+
+
+@pytest.mark.parametrize("dtype,B,L,h,dh", [
+    ("f32", 1, 1, 1, 64), ("f32", 1, 63, 2, 64), ("f32", 1, 64, 2, 16), ("f32", 1, 65, 2, 64), ("f32", 2, 129, 3, 32),
+    ("f32", 1, 257, 3, 64), ("f32", 1, 512, 10, 64), ("f32", 1, 1025, 4, 64), ("f32", 2, 300, 3, 128), ("f32", 1, 33, 1, 128), ("f32", 3, 300, 7, 128),
+    ("f32", 3, 839, 17, 64), ("bf16", 1, 700, 6, 32), ("bf16", 2, 130, 5, 16),
+])
+def test_ffma_attention_with_its_keys_dealt_out(toma, dtype, B, L, h, dh):
+    """One to four groups of warps share the queries' keys: groups without a key tile, with a partial last one, 32 and 40 and
+    64 queries per CTA.  Scores of each group's own range, so that the groups' references differ."""
+    rng = np.random.default_rng(L)
+    q, k, v = (torch.from_numpy(rng.standard_normal((B, L, h * dh)).astype(np.float32)).cuda() for _ in range(3))
+    k = k * (1 + torch.arange(L, device="cuda").div(64, rounding_mode="floor") % 5)[None, :, None]
+    q, k, v = (t.to(torch.float32 if dtype == "f32" else torch.bfloat16) for t in (q, k, v))
+    o = torch.full_like(q, float("nan"))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    toma.toma_attention(B, L, h, dh, dtype, q, k, v, o, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    qd, kd, vd = (t.double().reshape(B, L, h, dh).transpose(1, 2) for t in (q, k, v))
+    want = torch.softmax(qd @ kd.transpose(2, 3) / dh ** 0.5, dim=3) @ vd
+    assert_close(to_host64(o), want.transpose(1, 2).reshape(B, L, h * dh).cpu().numpy(), dtype, "attention")
+
+
+def test_ffma_attention_of_keys_at_minus_infinity(toma):
+    """Sixty-four keys, all that one group of warps has, whose scores overflow to minus infinity: they weigh nothing."""
+    L, dh = 256, 64
+    rng = np.random.default_rng(5)
+    q, k, v = (torch.from_numpy(rng.standard_normal((1, L, dh)).astype(np.float32)).cuda() for _ in range(3))
+    q = q.abs() * 1e20
+    k[:, 64:128] = -1e20
+    k[:, :64] *= 1e-20
+    k[:, 128:] *= 1e-20
+    o = torch.empty_like(q)
+    toma.toma_attention(1, L, 1, dh, "f32", q, k, v, o)
+    rest = torch.cat([torch.arange(64), torch.arange(128, L)]).cuda()
+    want = torch.softmax(q[0].double() @ k[0, rest].double().T / dh ** 0.5, dim=1) @ v[0, rest].double()
+    assert_close(to_host64(o)[0], want.cpu().numpy(), "f32", "attention")
