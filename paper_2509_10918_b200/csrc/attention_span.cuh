@@ -45,6 +45,25 @@ struct Spans {
   }
 };
 
+// What the ends of a CTA's span need of the plan, in shared memory: at the end of a piece the parameter memory is cold, and
+// its reads, one behind the other, cost a microsecond.  Filled in by lanes 0 and 1 of a warp at the start.
+struct Edges {
+  int lo[2], hi[2];  // lowest and highest CTA with key tiles of the unit the span starts in, and of the one it ends in
+  int first_unit;    // the unit the span starts in
+  int other_slot;    // scratch slot of the last unit's other contributor, where it has one
+  __device__ __forceinline__ void fill(const Spans& sp, int it_begin, int it_end, int lane) {
+    const int u = (lane ? it_end - 1 : it_begin) / sp.nblk;
+    lo[lane] = sp.unit_lo[lane][blockIdx.x];
+    hi[lane] = sp.unit_hi[lane][blockIdx.x];
+    if (lane == 0) {
+      first_unit = u;
+    } else {  // a CTA's first piece sits in slot 0 of its two, a later partial piece in slot 1
+      const int g = lo[1] == (int)blockIdx.x ? hi[1] : lo[1];
+      other_slot = 2 * g + (u > sp.bound(g) / sp.nblk ? 1 : 0);
+    }
+  }
+};
+
 // One piece = the part of a span inside one unit: key tiles [k0, k0 + cnt) of unit u.
 struct Piece {
   int u, k0, cnt;
@@ -163,10 +182,21 @@ __device__ __noinline__ void combine_rows(const float* pieces, const Spans& sp, 
   }
 }
 
-__device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
+// Whether each of the kN tickets (a multiple of four, 16-byte aligned) has been drawn once; if so, what their drawers had
+// written before is visible from here on.  (One fence behind all the loads: loads that acquire each wait for the one before,
+// 10 us for sixteen.)
+template <int kN>
+__device__ __forceinline__ bool all_drawn_once(const uint32_t* tk) {
+  uint32_t off = 0;
+#pragma unroll
+  for (int w = 0; w < kN; w += 4) {
+    uint32_t v[4];
+    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "l"(tk + w) : "memory");
+    off |= (v[0] ^ 1u) | (v[1] ^ 1u) | (v[2] ^ 1u) | (v[3] ^ 1u);
+  }
+  if (off) return false;
+  __threadfence();
+  return true;
 }
 
 __device__ __forceinline__ void st_release_cta(uint32_t* smem_word, uint32_t v) {

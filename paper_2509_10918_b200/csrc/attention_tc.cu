@@ -67,6 +67,7 @@ struct Barriers {
   uint32_t first_ticket[kSoftWarps];    // per softmax warp: ticket its first (partial) piece drew
   uint32_t others_done;                 // set by the publisher when the span's last unit has all its other pieces in scratch
   uint32_t poll_stop[2];                // set by each softmax group when the answer is no longer needed
+  Edges edge;
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -158,15 +159,18 @@ __device__ __forceinline__ void stage16(const OutStage& os, int lane, int part, 
     *reinterpret_cast<uint4*>(os.stage + lane * 64 + (((part * 2 + (e >> 3)) ^ ((lane >> 1) & 3)) << 4)) = v;
   }
 }
-// Whole warp.  (ch0, row0, b): first channel of the slab, first token of the warp's 32 rows, batch item.
+// Whole warp.  (ch0, row0, b): first channel of the slab, first token of the warp's 32 rows, batch item.  The slab is being
+// read until staging_free().
 __device__ __forceinline__ void flush_slab(const OutStage& os, int lane, int ch0, int row0, int b, int L) {
   fence_proxy_async();  // the staged rows are read by the TMA engine
   __syncwarp();
   if (lane == 0 && row0 < L) {
     tma_store_3d(os.tm_o, os.stage, ch0, row0, b);
     tma_store_commit();
-    tma_store_wait_read();  // the slab is staged again right away
   }
+}
+__device__ __forceinline__ void staging_free(int lane) {
+  if (lane == 0) tma_store_wait_read();
   __syncwarp();
 }
 // End of a piece that covers all keys of its unit (the only kind when units are kept whole), run by
@@ -181,20 +185,16 @@ __device__ __noinline__ bool finish_whole(Row t, Barriers* bar, Piece p, int las
   const OutStage os{stage_of(bar, t.warp), tm_o};
   const float inv = 1.f / jn.l;
   const int c0 = t.half * (DH / 2);
-#pragma unroll 1
-  for (int c = c0; c < c0 + DH / 2; c += 32) {
-    uint32_t r[16];
-    read_o16(t, jn, c, r);
-    stage16(os, t.lane, 0, r, inv);
-    read_o16(t, jn, c + 16, r);
-    stage16(os, t.lane, 1, r, inv);
-    if (c + 32 >= c0 + DH / 2) {
-      tc_fence_before();
-      __syncwarp();
-      if (t.lane == 0) mbar_arrive(&bar->o_free[t.q]);  // the next piece's first PV product may overwrite the accumulator
-    }
-    flush_slab(os, t.lane, ch0 + c, row0, b, L);
-  }
+  static_assert(DH / 2 == 32, "a slab per warp and piece");
+  uint32_t r[2][16];
+  read_o16(t, jn, c0, r[0]);
+  read_o16(t, jn, c0 + 16, r[1]);
+  tc_fence_before();
+  __syncwarp();
+  if (t.lane == 0) mbar_arrive(&bar->o_free[t.q]);  // the next piece's first PV product may overwrite the accumulator
+  stage16(os, t.lane, 0, r[0], inv);
+  stage16(os, t.lane, 1, r[1], inv);
+  flush_slab(os, t.lane, ch0 + c0, row0, b, L);
   return true;
 }
 
@@ -219,8 +219,8 @@ __device__ __noinline__ bool finish_partial(Row t, Barriers* bar, Piece p, int p
   const int row = t.row, lane = t.lane, c0 = t.half * (DH / 2);
   uint32_t* ticket = tickets + (size_t)p.u * kTicketCols + t.warp;
   // a partial piece lies in the unit the span starts in or in the one it ends in
-  const int which = p.u == sp.bound(blockIdx.x) / sp.nblk ? 0 : 1;
-  const int g_first = sp.unit_lo[which][blockIdx.x], g_last = sp.unit_hi[which][blockIdx.x];
+  const int which = p.u == bar->edge.first_unit ? 0 : 1;
+  const int g_first = bar->edge.lo[which], g_last = bar->edge.hi[which];
   bool own_first = false;  // this CTA is the lower of the two contributors
   const float4* other = nullptr;
   float m_o = 0.f, l_o = 0.f;
@@ -237,7 +237,7 @@ __device__ __noinline__ bool finish_partial(Row t, Barriers* bar, Piece p, int p
   if (last_of_span && (row & (kBM - 1)) == 0 && t.half == 0) *(volatile uint32_t*)&bar->poll_stop[t.q] = 1u;
   if (direct) {
     own_first = (int)blockIdx.x == g_first;
-    const float* slot = slot_of<DH>(pieces, sp, own_first ? g_last : g_first, p.u);
+    const float* slot = pieces + (size_t)bar->edge.other_slot * piece_floats<DH>();
     m_o = __ldcg(slot + kM + row);
     l_o = __ldcg(slot + kL + row);
     other = reinterpret_cast<const float4*>(slot) + row;
@@ -312,7 +312,7 @@ __device__ __noinline__ void settle_first_piece(Barriers* bar, int it_begin, int
   const int nblk = sp.nblk, u = it_begin / nblk;
   const bool first_partial = it_begin > u * nblk || it_end < (u + 1) * nblk;
   if (!first_partial || it_end <= (u + 1) * nblk) return;  // whole, or also the span's last piece: settled already
-  const int g_first = sp.unit_lo[0][blockIdx.x], g_last = sp.unit_hi[0][blockIdx.x];
+  const int g_first = bar->edge.lo[0], g_last = bar->edge.hi[0];
   if (!mbar_wait_warp(&bar->pub_done, 0, dev_status, &bar->abort_flag)) return;
   if (bar->first_ticket[t.warp] != (uint32_t)(g_last - g_first)) return;
   __threadfence();
@@ -411,6 +411,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     bar->abort_flag = 0;
     mbar_fence_init();
   }
+  if (warp == kSoftWarps + 3 && lane < 2) bar->edge.fill(sp, it_begin, it_end, lane);
   if (threadIdx.x == kSoftWarps * 32) {  // descriptor fetches overlap the previous kernel's tail
     prefetch_tmap(&tm_q);
     prefetch_tmap(&tm_k);
@@ -550,10 +551,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const uint32_t* tk = tickets + (size_t)ul * kTicketCols;
         for (uint32_t spin = 0; spin < kSpinLimit; ++spin) {
           if ((*(volatile uint32_t*)&bar->poll_stop[0] && *(volatile uint32_t*)&bar->poll_stop[1]) || *abort_flag) break;
-          bool all = true;
-#pragma unroll
-          for (int w = 0; w < kSoftWarps; ++w) all = all && ld_acquire_gpu(tk + w) == 1u;
-          if (all) {
+          if (all_drawn_once<kSoftWarps>(tk)) {
             st_release_cta(&bar->others_done, 1u);
             break;
           }
@@ -635,6 +633,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       }
       float l, l_odd;
       unpack2(l2, l, l_odd);
+      staging_free(lane);
       const Joint jn = join_halves(t, bar, m_used, l + l_odd);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) continue;
@@ -642,6 +641,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       else ok = finish_partial(t, bar, p, pc, last_n, it >= it_end, jn, o, &tm_o, L, heads, sp, tickets, pieces, dev_status);
     }
     if (__all_sync(0xffffffffu, ok)) settle_first_piece(bar, it_begin, it_end, t, o, L, heads, sp, pieces, dev_status);
+    staging_free(lane);  // shared memory must outlive the engine's reads
   }
   tc_fence_before();
   __syncthreads();

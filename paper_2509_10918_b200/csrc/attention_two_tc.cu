@@ -74,6 +74,7 @@ struct Barriers {
   uint32_t others_done;               // set by the publisher when the span's last unit has all its other pieces in scratch
   uint32_t poll_stop[2];              // set by each softmax group when the answer is no longer needed
   uint32_t tmem_base;
+  Edges edge;
   int abort_flag;
 };
 static_assert(sizeof(Barriers) <= 512, "barrier block outgrew its reservation");
@@ -131,8 +132,11 @@ __device__ __forceinline__ void flush_slab(const OutStage& os, int lane, int ch0
   if (lane == 0 && row0 < L) {
     tma_store_3d(os.tm_o, os.stage, ch0, row0, b);
     tma_store_commit();
-    tma_store_wait_read();  // the slab is staged again right away
   }
+}
+// Before the slab is staged again, and before the block ends.
+__device__ __forceinline__ void staging_free(int lane) {
+  if (lane == 0) tma_store_wait_read();
   __syncwarp();
 }
 // End of a piece that covers all keys of its unit (the only kind when units are kept whole), run by
@@ -159,6 +163,7 @@ __device__ __forceinline__ void finish_whole(const Row& t, Barriers* bar, int un
     uint32_t r[32];
     tmem_ld32(t.ob + c * 32, r);
     tmem_wait_ld();
+    if (!(c & 1)) staging_free(t.lane);
     stage_half(os, t.lane, c & 1, r, inv);
     if (c & 1) flush_slab(os, t.lane, ch0 + (c >> 1) * 64, row0, b, L);
   }
@@ -188,8 +193,8 @@ __device__ __noinline__ void finish_partial(Row t, Barriers* bar, Piece p, int p
   const int row = t.row, lane = t.lane;
   uint32_t* ticket = tickets + (size_t)p.u * kTicketCols + t.warp;
   // a partial piece lies in the unit the span starts in or in the one it ends in
-  const int which = p.u == sp.bound(blockIdx.x) / sp.nblk ? 0 : 1;
-  const int g_first = sp.unit_lo[which][blockIdx.x], g_last = sp.unit_hi[which][blockIdx.x];
+  const int which = p.u == bar->edge.first_unit ? 0 : 1;
+  const int g_first = bar->edge.lo[which], g_last = bar->edge.hi[which];
   bool own_first = false;  // this CTA is the lower of the two contributors
   // The direct path comes in two forms.  The wide one holds 64 columns of the other piece in registers (the
   // function then spills); the lean one takes 16 columns at a time with the next 16 on their way.  Timed as a
@@ -211,7 +216,7 @@ __device__ __noinline__ void finish_partial(Row t, Barriers* bar, Piece p, int p
   if (last_of_span && (row & (kBM - 1)) == 0) *(volatile uint32_t*)&bar->poll_stop[t.q] = 1u;
   if (direct) {
     own_first = (int)blockIdx.x == g_first;
-    other = slot_of<DH>(pieces, sp, own_first ? g_last : g_first, p.u);
+    other = pieces + (size_t)bar->edge.other_slot * piece_floats<DH>();
     m_o = __ldcg(other + kM + row);
     l_o = __ldcg(other + kL + row);
 #pragma unroll
@@ -268,6 +273,7 @@ __device__ __noinline__ void finish_partial(Row t, Barriers* bar, Piece p, int p
             r[4 * q + e] = __float_as_uint(own_first ? fmaf(w_o, vv[e], w_own * own) : fmaf(w_own, own, w_o * vv[e]));
           }
         }
+        if ((c & 3) == 0) staging_free(lane);
         stage_quarter(os, t.lane, c & 3, r, inv);
         if ((c & 3) == 3) flush_slab(os, t.lane, ch0 + (c >> 2) * 64, row0, b_item, L);
       }
@@ -301,6 +307,7 @@ __device__ __noinline__ void finish_partial(Row t, Barriers* bar, Piece p, int p
             r[4 * q + e] = __float_as_uint(own_first ? fmaf(w_o, vv[e], w_own * own) : fmaf(w_own, own, w_o * vv[e]));
           }
         }
+        if (!(c & 1)) staging_free(lane);
         stage_half(os, t.lane, c & 1, r, inv);
         if (c & 1) flush_slab(os, t.lane, ch0 + (c >> 1) * 64, row0, b_item, L);
       } else {
@@ -332,7 +339,7 @@ __device__ __noinline__ void settle_first_piece(Barriers* bar, int it_begin, int
   const int nblk = sp.nblk, u = it_begin / nblk;
   const bool first_partial = it_begin > u * nblk || it_end < (u + 1) * nblk;
   if (!first_partial || it_end <= (u + 1) * nblk) return;  // whole, or also the span's last piece: settled already
-  const int g_first = sp.unit_lo[0][blockIdx.x], g_last = sp.unit_hi[0][blockIdx.x];
+  const int g_first = bar->edge.lo[0], g_last = bar->edge.hi[0];
   if (!mbar_wait_warp(&bar->pub_done, 0, dev_status, &bar->abort_flag)) return;
   if (bar->first_ticket[t.warp] != (uint32_t)(g_last - g_first)) return;
   __threadfence();
@@ -402,6 +409,7 @@ attention_two_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     prefetch_tmap(&tm_v);
     prefetch_tmap(&tm_o);
   }
+  if (warp == 10 && lane < 2) bar->edge.fill(sp, it_begin, it_end, lane);
   dependency_wait();
   if (threadIdx.x == 0) release_dependents();
   if (warp == 9) tmem_alloc(&bar->tmem_base, C::kTmemCols);
@@ -552,10 +560,7 @@ attention_two_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         const uint32_t* tk = tickets + (size_t)ul * kTicketCols;
         for (uint32_t spin = 0; spin < kSpinLimit; ++spin) {
           if ((*(volatile uint32_t*)&bar->poll_stop[0] && *(volatile uint32_t*)&bar->poll_stop[1]) || *abort_flag) break;
-          bool all = true;
-#pragma unroll
-          for (int w = 0; w < 8; ++w) all = all && ld_acquire_gpu(tk + w) == 1u;
-          if (all) {
+          if (all_drawn_once<8>(tk)) {
             st_release_cta(&bar->others_done, 1u);
             break;
           }
@@ -595,6 +600,7 @@ attention_two_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
       else finish_partial<DH>(t, bar, p, pc, it >= it_end, m_used, l, o, &tm_o, L, heads, sp, tickets, pieces, dev_status);
     }
     settle_first_piece<DH>(bar, it_begin, it_end, t, o, L, heads, sp, pieces, dev_status);
+    staging_free(lane);  // shared memory must outlive the engine's reads
   }
   tc_fence_before();
   __syncthreads();
