@@ -25,8 +25,8 @@
 // nothing else to do at that time.  A merge MMA has M = 128 = two such 64-destination slabs; the
 // pair that belongs to the other half of the accumulator's rows reads a block of zeros instead.
 //
-// Warps 0..3 / 4..7: softmax of query tile 0 / 1; in A warps 0..3 build slabs and warps 4..7 move
-// merged rows from tensor memory to shared memory; in C each group builds and stores its own pairs.
+// Warps 0..3 / 4..7: softmax of query tile 0 / 1; in A each group builds every second pair's slab and moves a group of merged
+// rows from tensor memory to shared memory; in C each group builds and stores its own pairs.
 // Warp 8: TMA producer of the token tiles (A only; the four pairs have a stage each).  Warp 9: one elected thread issues every MMA.
 #include "attention_core.cuh"
 #include "common.cuh"
@@ -68,33 +68,36 @@ struct FParams {
   float scale_log2;
 };
 
-// A thread's row of a pair's slab: the 32 weights (hi and lo plane) of one token of tile ta or ta + 1.
-struct SlabRow {
+// A warp's 32 rows of a pair's slab, the 32 weights (hi and lo plane) of a token each, all of one tile: 2 KB of either plane
+// without a gap, read as such (a row per thread would touch four times the cache lines: 2.3 us until the first slab stood, of
+// which a microsecond was that).  Lane l has 16 bytes l % 4 of the rows 8 i + l / 4.
+struct SlabRows {
   uint4 v[2][4];
 };
-__device__ __forceinline__ SlabRow load_slab_row(const FParams& p, int b, int ta, int r /*0..127*/) {
-  const int tile = r < kTileTok ? ta : ta + 1, k = r & (kTileTok - 1);
-  const size_t row = ((size_t)(2 * (b * (p.D / kTileDest) + tile)) * kTileTok + k) * kTileDest;
-  SlabRow w;
+__device__ __forceinline__ SlabRows load_slab_rows(const FParams& p, int b, int ta, int quarter, int lane) {
+  const size_t tile = b * (p.D / kTileDest) + ta + (quarter >> 1);
+  SlabRows w;
 #pragma unroll
   for (int pl = 0; pl < 2; ++pl) {
-    const uint4* src = reinterpret_cast<const uint4*>(p.w + row + (size_t)pl * kTileTok * kTileDest);
+    const uint4* src = reinterpret_cast<const uint4*>(p.w + ((2 * tile + pl) * kTileTok + (quarter & 1) * 32) * kTileDest);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) w.v[pl][c] = __ldg(src + c);
+    for (int i = 0; i < 4; ++i) w.v[pl][i] = __ldg(src + i * 32 + lane);
   }
   return w;
 }
-// Writes it into `slab` (hi plane, then lo plane kPairBytes further): data in the half of the row that belongs to the
-// token's tile, zeros in the other.
-__device__ __forceinline__ void store_slab_row(uint8_t* slab, const SlabRow& w, int r) {
-  const int side = r >> 6;
+// Writes them into `slab` (hi plane, then lo plane kPairBytes further): data in the half of a row that belongs to the token's
+// tile, zeros in the other; odd rows the other way round, so that neighbours' stores fall into different banks.
+__device__ __forceinline__ void store_slab_rows(uint8_t* slab, const SlabRows& w, int quarter, int lane) {
+  const int side = quarter >> 1, odd = (lane >> 2) & 1;
 #pragma unroll
   for (int pl = 0; pl < 2; ++pl) {
     uint8_t* dst = slab + pl * kPairBytes;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      *reinterpret_cast<uint4*>(dst + sw128_offset(r, side * 4 + c)) = w.v[pl][c];
-      *reinterpret_cast<uint4*>(dst + sw128_offset(r, (side ^ 1) * 4 + c)) = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 0; i < 4; ++i) {
+      const int row = quarter * 32 + i * 8 + (lane >> 2), c = lane & 3;
+      const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(dst + sw128_offset(row, (side ^ odd) * 4 + c)) = odd ? zero : w.v[pl][i];
+      *reinterpret_cast<uint4*>(dst + sw128_offset(row, (side ^ odd ^ 1) * 4 + c)) = odd ? w.v[pl][i] : zero;
     }
   }
 }
@@ -154,7 +157,7 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       }
     }
     for (int s = 0; s < 4; ++s) mbar_init(&bar->pv_done[s], 1);
-    mbar_init(&bar->kv_ready, p.units == 2 ? 5 : 4);  // own warps; the peer's rows arrive as bytes
+    mbar_init(&bar->kv_ready, p.units == 2 ? 9 : 8);  // own warps; the peer's rows arrive as bytes
     bar->abort_flag = 0;
     mbar_fence_init();
     mbar_init(&bar->kv_sent, 1);
@@ -174,7 +177,7 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (p.units == 2) cluster_sync();  // the peer's barriers are initialised before anything is sent to it
+  if (p.units == 2) cluster_arrive();  // barriers initialised; the peer waits for that before it sends anything here
   const uint32_t tmem = bar->tmem_base;
   volatile int* abort_flag = &bar->abort_flag;
   // tensor memory: columns 0..255 the four S buffers (the merge accumulators before, the unmerge accumulators
@@ -195,6 +198,7 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     }
   } else if (warp == 9) {
     // ------------------------------------------------------------------ every MMA, in program order
+    if (p.units == 2) cluster_wait();
     if (elect_one()) {
       bool ok = true;
       // ---- A: X_m rows of four tiles = (pair 0 | zeros) and (zeros | pair 1) times the tokens of the pairs
@@ -224,7 +228,6 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       // ---- B: attention of the unit's two query tiles over all D keys of the resident matrix
       if (ok) ok = mbar_wait_cluster(&bar->kv_ready, 0, dev_status, abort_flag);
       if (ok) {
-        if (p.units == 2) mbar_arrive_peer(peer_addr(smem_u32(&bar->kv_sent), (uint32_t)(unit ^ 1)));
         tc_fence_after();
         constexpr uint32_t idesc_s = idesc_f16(kFmtBF16, kFmtBF16, false, false, kBM, kBN);
         constexpr uint32_t idesc_o = idesc_f16(kFmtBF16, kFmtBF16, false, true, kBM, 64 + 16);
@@ -242,6 +245,7 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
           issue_s(n, 0);
           issue_s(n, 1);
         }
+        if (p.units == 2) mbar_arrive_at(peer_addr(smem_u32(&bar->kv_sent), (uint32_t)(unit ^ 1)));
         for (int n = 0; ok && n < nblk; ++n) {
           const int bb = n & 1;
           const uint32_t va = kv + n * kBN * 128;
@@ -290,28 +294,29 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     bool ok = true;
     // ------------------------------------------------------------------ A
-    if (q == 0) {
-      // slabs of all pairs, then (same stages, same barriers) of the first two pairs of the unmerge; a pair's
-      // weights are requested before the wait for its stage, so that their latency passes under it
-      constexpr int n_build = n_pairs + 2;
-      SlabRow w0 = load_slab_row(p, b, unit * 8, r), w1 = load_slab_row(p, b, unit * 8 + 2, r);
-#pragma unroll
-      for (int i = 0; i < n_build; ++i) {
-        const int s = i & 1;
-        const SlabRow cur = w0;
-        w0 = w1;
-        if (i + 2 < n_build) w1 = load_slab_row(p, b, unit * 8 + 2 * ((i + 2) % n_pairs), r);
-        if (i >= 2 && !mbar_wait_warp(&bar->slab_empty[s], ((i >> 1) - 1) & 1, dev_status, abort_flag)) { ok = false; break; }
-        store_slab_row(sA + 2 * s * kPairBytes, cur, r);
+    {
+      // Group q builds the slabs of stage q: pairs q and q + 2 of the merge, then pair q of the unmerge.
+      const SlabRows w0 = load_slab_rows(p, b, unit * 8 + 2 * q, quarter, lane), w1 = load_slab_rows(p, b, unit * 8 + 2 * (q + 2), quarter, lane);
+      uint8_t* stage = sA + 2 * q * kPairBytes;
+      auto built = [&](uint64_t* full) {
         fence_proxy_async();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&bar->slab_full[s]);
+        if (lane == 0) mbar_arrive(full);
+      };
+      store_slab_rows(stage, w0, quarter, lane);
+      built(&bar->slab_full[q]);
+      ok = mbar_wait_warp(&bar->slab_empty[q], 0, dev_status, abort_flag);
+      if (ok) {
+        store_slab_rows(stage, w1, quarter, lane);
+        built(&bar->slab_full[q]);
       }
-    } else {
-      // merged rows of every group of four tiles: tensor memory -> bf16 rows of the shared matrix
+      if (p.units == 2) cluster_wait();  // the peer's barriers are there
+      // Merged rows of a group of four tiles, the first of them by the second group of warps (which is done with its slabs when
+      // they are there): tensor memory -> bf16 rows of the shared matrix, and of the peer's.
+      const int g = q ^ 1;
       const uint32_t peer = (uint32_t)(unit ^ 1);
-      for (int g = 0; g < n_pairs / 2; ++g) {
-        if (!mbar_wait_warp(&bar->acc_full[g], 0, dev_status, abort_flag)) { ok = false; break; }
+      if (ok) ok = mbar_wait_warp(&bar->acc_full[g], 0, dev_status, abort_flag);
+      if (ok) {
         tc_fence_after();
         uint8_t* rows = sKV + (unit * 2 + g) * kPairBytes + quarter * 4096;  // this warp's 32 rows
         row_to_smem(tmem + lane_addr + g * 64, sKV + (unit * 2 + g) * kPairBytes, r, 1.f);
@@ -320,14 +325,18 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         if (p.units == 2 && lane == 0) copy_to_peer(peer_addr(smem_u32(rows), peer), rows, 4096, peer_addr(smem_u32(&bar->kv_ready), peer));
       }
       tc_fence_before();
+      __syncwarp();
       if (lane == 0) mbar_arrive(&bar->kv_ready);
-      // the unmerge's third pair, into the token stages 2 and 3: every merge MMA has completed (the last group's
-      // accumulator was complete), so nothing reads them any more
+      if (ok) ok = mbar_wait_warp(&bar->slab_empty[q], 1, dev_status, abort_flag);
       if (ok) {
-        store_slab_row(sX + 2 * kPairBytes, load_slab_row(p, b, unit * 8 + 4, r), r);
-        fence_proxy_async();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bar->slab2_full);
+        store_slab_rows(stage, w0, quarter, lane);
+        built(&bar->slab_full[q]);
+        // the unmerge's third pair, into the token stages 2 and 3: every merge MMA has completed (the last group's accumulator
+        // was complete), so nothing reads them any more
+        if (q == 0) {
+          store_slab_rows(sX + 2 * kPairBytes, w1, quarter, lane);
+          built(&bar->slab2_full);
+        }
       }
     }
     // ------------------------------------------------------------------ B
@@ -345,8 +354,8 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       if (lane == 0) mbar_arrive(&bar->p_full[q][bb]);
     }
     // normalised accumulator -> bf16 rows in shared memory (the unmerge's B operand)
-    SlabRow w3;
-    if (q == 1) w3 = load_slab_row(p, b, unit * 8 + 6, r);  // the unmerge's fourth pair; needed after the next wait
+    SlabRows w3;
+    if (q == 1) w3 = load_slab_rows(p, b, unit * 8 + 6, quarter, lane);  // the unmerge's fourth pair; needed after the next wait
     if (ok) ok = mbar_wait_warp(&bar->o_done[q], 0, dev_status, abort_flag);
     if (ok) {
       tc_fence_after();
@@ -364,14 +373,15 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       const int gi = n_pairs + 2, s = gi & 1;
       ok = mbar_wait_warp(&bar->slab_empty[s], ((gi >> 1) - 1) & 1, dev_status, abort_flag);
       if (ok) {
-        store_slab_row(sA + 2 * s * kPairBytes, w3, r);
+        store_slab_rows(sA + 2 * s * kPairBytes, w3, quarter, lane);
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) mbar_arrive(&bar->slab_full[s]);
       }
     }
     // the rows of K and V become the staging area of the output; the peer must have received its copy of them
-    if (ok && p.units == 2) ok = __all_sync(0xffffffffu, mbar_wait_cluster(&bar->kv_sent, 0, dev_status, abort_flag));
+    if (ok && p.units == 2) ok = mbar_wait_warp(&bar->kv_sent, 0, dev_status, abort_flag);
+    if (p.units == 2) cluster_arrive();
     for (int c = 2 * q; ok && c < 2 * q + 2; ++c) {
       if (!mbar_wait_warp(&bar->c_full[q][c & 1], 0, dev_status, abort_flag)) { ok = false; break; }
       tc_fence_after();
@@ -387,13 +397,17 @@ block_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     }
     if (lane == 0) tma_store_wait_read();  // shared memory must outlive the engine's reads
   }
+  if (warp >= 8 && p.units == 2) {
+    if (warp != 9) cluster_wait();  // the issuer's warp has
+    cluster_arrive();
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == 9) {
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
-  if (p.units == 2) cluster_sync();  // neither CTA's shared memory goes away while the other could still write to it
+  if (p.units == 2) cluster_wait();  // neither CTA's shared memory goes away while the other could still write to it
 }
 
 constexpr int kFusedSmem = 1024 + kMaxD * 128 + 4 * kPairBytes + 2 * kZeroBytes + 4 * kPairBytes + kOnesBytes + 512;
