@@ -24,28 +24,12 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p, int n, bool vec)
   return make_float4(n > 0 ? to_f32(p[0]) : 0.f, n > 1 ? to_f32(p[1]) : 0.f, n > 2 ? to_f32(p[2]) : 0.f, n > 3 ? to_f32(p[3]) : 0.f);
 }
 
-// Two columns of a row of sums: two floats in a 64-bit register, so that one packed fma (one issue slot) serves both,
-// or two doubles.
+// Two columns of a row of sums: two floats in a 64-bit register, so that one packed fma (one issue slot) serves both.
 struct Sum2f {
   unsigned long long v;
   __device__ __forceinline__ void fma(unsigned long long a2, unsigned long long b2) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(v) : "l"(a2), "l"(b2)); }
   __device__ __forceinline__ void get(float* o) const { asm("mov.b64 {%0, %1}, %2;" : "=f"(o[0]), "=f"(o[1]) : "l"(v)); }
 };
-struct Sum2d {
-  double x, y;
-  __device__ __forceinline__ void fma(unsigned long long a2, unsigned long long b2) {
-    float a, b0, b1;
-    asm("{\n\t.reg .f32 t;\n\tmov.b64 {%0, t}, %1;\n\t}" : "=f"(a) : "l"(a2));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(b0), "=f"(b1) : "l"(b2));
-    x = ::fma((double)a, (double)b0, x);
-    y = ::fma((double)a, (double)b1, y);
-  }
-  __device__ __forceinline__ void get(double* o) const { o[0] = x; o[1] = y; }
-  __device__ __forceinline__ void add(double a, double b) { x += a, y += b; }
-};
-
-template <typename AccT> struct SumOf { typedef Sum2f Pair; };
-template <> struct SumOf<double> { typedef Sum2d Pair; };
 
 // C[m][n] = sum_k A(m,k) B(k,n) for one batch entry (blockIdx.z), every sum one chain of fused multiply-adds in
 // ascending k (the result does not depend on the tile form).  Tile BM x BN, TM x TN outputs per thread, 16
@@ -53,45 +37,32 @@ template <> struct SumOf<double> { typedef Sum2d Pair; };
 // operand's contiguous axis) while the current one is multiplied out of shared memory, two stages deep.  Both
 // operands lie there as [k][row], rows swizzled by 8 ((k / 4) % 4), which keeps groups of eight together for the
 // 16-byte reads and the transposing stores free of bank conflicts.
-// KG > 1 (double sums only, where the order of addition does not show): that many thread groups share a tile, each with
-// a part of every stage's k, and add up through shared memory at the end: for products too small to fill the SMs.
 // `Op`: a_ptr / b_ptr give the contiguous line of an operand (a row m or n if k runs along it, else a row k).
 constexpr int kBK = 16;
 template <int kRows>
 __device__ __forceinline__ constexpr int swz(int k4) { return 8 * (k4 & 3 & (kRows / 8 - 1)); }
 
-template <class Op, typename AccT, int BM, int BN, int TM, int TN, int KG>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, KG > 1 || BM == 128 ? 2 : 4) simt_gemm_kernel(const Op op) {
-  using Acc = typename SumOf<AccT>::Pair;
-  constexpr int kGroup = (BM / TM) * (BN / TN), kThreads = kGroup * KG;
+template <class Op, int BM, int BN, int TM, int TN>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN), BM == 128 ? 2 : 4) simt_gemm_kernel(const Op op) {
+  constexpr int kThreads = (BM / TM) * (BN / TN);
   constexpr int kPackA = BM * kBK / 4, kPackB = BN * kBK / 4;  // 4-element packets of a stage
   constexpr int kVecA = (kPackA + kThreads - 1) / kThreads, kVecB = (kPackB + kThreads - 1) / kThreads;
   __shared__ __align__(16) float As[2][kBK][BM];
   __shared__ __align__(16) float Bs[2][kBK][BN];
   const int batch = blockIdx.z, m0 = blockIdx.y * BM, n0 = blockIdx.x * BN, tid = threadIdx.x;
-  const int in_group = tid % kGroup, kg = tid / kGroup;
   tc::dependency_wait();  // launched with programmatic stream serialisation
   if (tid == 0) tc::release_dependents();
-  const int tn = in_group % (BN / TN) * 4, tm = in_group / (BN / TN) * TM;  // columns tn .. + 3, and with TN = 8 BN / 2 further on
+  const int tn = tid % (BN / TN) * 4, tm = tid / (BN / TN) * TM;  // columns tn .. + 3, and with TN = 8 BN / 2 further on
   // packet e of an operand: k along the line: line e / 4, k 4 (e % 4); else: k e / (rows / 4), rows 4 (e % (rows / 4))
   float4 ra[kVecA], rb[kVecB];
   typename Op::APtr pa[kVecA];  // lines of an operand with k along them stay the same for the whole sum
-  typename Op::BPtr pb[kVecB];
-  bool ha[kVecA], hb[kVecB];    // ... and are there
+  bool ha[kVecA];               // ... and are there
   if (Op::a_k_contig) {
 #pragma unroll
     for (int v = 0; v < kVecA; ++v) {
       const int r = m0 + (tid + v * kThreads) / 4;
       ha[v] = r < op.M && tid + v * kThreads < kPackA;
       pa[v] = op.a_ptr(batch, ha[v] ? r : 0);
-    }
-  }
-  if (Op::b_k_contig) {
-#pragma unroll
-    for (int v = 0; v < kVecB; ++v) {
-      const int r = n0 + (tid + v * kThreads) / 4;
-      hb[v] = r < op.N && tid + v * kThreads < kPackB;
-      pb[v] = op.b_ptr(batch, hb[v] ? r : 0);
     }
   }
   auto fetch = [&](int k0) {
@@ -109,13 +80,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, KG > 1 || BM == 12
 #pragma unroll
     for (int v = 0; v < kVecB; ++v) {
       const int e = tid + v * kThreads;
-      if (Op::b_k_contig) {
-        const int k = k0 + 4 * (e & 3);
-        rb[v] = hb[v] ? load4(pb[v] + k, op.K - k, op.b_vec) : make_float4(0.f, 0.f, 0.f, 0.f);
-      } else {
-        const int k = k0 + e / (BN / 4), r = n0 + 4 * (e % (BN / 4));
-        rb[v] = e < kPackB && k < op.K && r < op.N ? load4(op.b_ptr(batch, k) + r, op.N - r, op.b_vec) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
+      const int k = k0 + e / (BN / 4), r = n0 + 4 * (e % (BN / 4));
+      rb[v] = e < kPackB && k < op.K && r < op.N ? load4(op.b_ptr(batch, k) + r, op.N - r, op.b_vec) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
   auto put = [&](int st) {
@@ -138,16 +104,11 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, KG > 1 || BM == 12
     for (int v = 0; v < kVecB; ++v) {
       const int e = tid + v * kThreads;
       if (kPackB % kThreads && e >= kPackB) continue;
-      if (Op::b_k_contig) {
-        const int r = e / 4, k = 4 * (e & 3), c = r ^ swz<BN>(e & 3);
-        Bs[st][k][c] = rb[v].x; Bs[st][k + 1][c] = rb[v].y; Bs[st][k + 2][c] = rb[v].z; Bs[st][k + 3][c] = rb[v].w;
-      } else {
-        const int k = e / (BN / 4), r = 4 * (e % (BN / 4));
-        *reinterpret_cast<float4*>(&Bs[st][k][r ^ swz<BN>(k >> 2)]) = rb[v];
-      }
+      const int k = e / (BN / 4), r = 4 * (e % (BN / 4));
+      *reinterpret_cast<float4*>(&Bs[st][k][r ^ swz<BN>(k >> 2)]) = rb[v];
     }
   };
-  Acc acc[TM][TN / 2] = {};
+  Sum2f acc[TM][TN / 2] = {};
   fetch(0);
   put(0);
   __syncthreads();
@@ -156,8 +117,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, KG > 1 || BM == 12
     const bool more = k0 + kBK < op.K;
     if (more) fetch(k0 + kBK);
 #pragma unroll
-    for (int kk = 0; kk < kBK / KG; ++kk) {
-      const int k = KG == 1 ? kk : kg * (kBK / KG) + kk;
+    for (int k = 0; k < kBK; ++k) {
       float4 a[TM / 4];
       ulonglong2 b[TN / 4];
 #pragma unroll
@@ -184,28 +144,6 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, KG > 1 || BM == 12
       __syncthreads();
     }
   }
-  if constexpr (KG > 1) {  // groups 1 .. KG - 1 hand their sums to group 0
-    __shared__ AccT part[KG - 1][TM * TN][kGroup];
-    if (kg > 0) {
-#pragma unroll
-      for (int u = 0; u < TM; ++u)
-#pragma unroll
-        for (int q = 0; q < TN / 2; ++q) {
-          AccT v[2];
-          acc[u][q].get(v);
-          part[kg - 1][u * TN + 2 * q][in_group] = v[0];
-          part[kg - 1][u * TN + 2 * q + 1][in_group] = v[1];
-        }
-    }
-    __syncthreads();
-    if (kg > 0) return;
-#pragma unroll
-    for (int u = 0; u < TM; ++u)
-#pragma unroll
-      for (int q = 0; q < TN / 2; ++q)
-#pragma unroll
-        for (int g = 0; g < KG - 1; ++g) acc[u][q].add(part[g][u * TN + 2 * q][in_group], part[g][u * TN + 2 * q + 1][in_group]);
-  }
 #pragma unroll
   for (int u = 0; u < TM; ++u) {
     const int m = m0 + tm + u;
@@ -213,7 +151,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, KG > 1 || BM == 12
 #pragma unroll
     for (int q = 0; q < TN / 4; ++q) {
       const int n = n0 + tn + q * (BN / 2);
-      AccT v[4];
+      float v[4];
       acc[u][2 * q].get(v);
       acc[u][2 * q + 1].get(v + 2);
       if (n < op.N) op.store4(batch, m, n, op.N - n, v);
@@ -299,11 +237,7 @@ template <> struct WLine<__nv_bfloat16> { typedef SplitW Ptr; };
 // logits[batch][i][k] = <X[idx_i], X_k> * scale
 template <typename T>
 struct LogitsOp {
-  static constexpr bool a_k_contig = true, b_k_contig = true;
-  typedef const T* APtr;
-  typedef const T* BPtr;
   int M, N, K;
-  bool a_vec, b_vec;
   TileMap tm;
   const T* x;
   const int32_t* idx;
@@ -311,19 +245,13 @@ struct LogitsOp {
   float scale;
   __device__ __forceinline__ const T* a_ptr(int batch, int i) const { return x + tm.x_row(batch, idx[(size_t)batch * tm.Dloc + i]) * tm.d; }
   __device__ __forceinline__ const T* b_ptr(int batch, int k) const { return x + tm.x_row(batch, k) * tm.d; }
-  template <typename AccT>
-  __device__ __forceinline__ void store4(int batch, int i, int k, int n, const AccT* v) const {
-    const float f[4] = {(float)(v[0] * (AccT)scale), (float)(v[1] * (AccT)scale), (float)(v[2] * (AccT)scale), (float)(v[3] * (AccT)scale)};
-    put4(logits + ((size_t)batch * tm.Dloc + i) * tm.Nloc + k, n, tm.Nloc % 4 == 0, f);
-  }
 };
 
 // xm[m_row(i)][c] = sum_k w[batch][k][i] x[x_row(k)][c]
 template <typename T, typename WT>
 struct MergeOp {
-  static constexpr bool a_k_contig = false, b_k_contig = false;
+  static constexpr bool a_k_contig = false;
   typedef typename WLine<WT>::Ptr APtr;
-  typedef const T* BPtr;
   int M, N, K;
   bool a_vec, b_vec;
   TileMap tm;
@@ -341,9 +269,8 @@ struct MergeOp {
 // out[x_row(k)][c] = sum_i w[batch][k][i] y[m_row(i)][c]
 template <typename T, typename WT>
 struct UnmergeOp {
-  static constexpr bool a_k_contig = true, b_k_contig = false;
+  static constexpr bool a_k_contig = true;
   typedef typename WLine<WT>::Ptr APtr;
-  typedef const T* BPtr;
   int M, N, K;
   bool a_vec, b_vec;
   TileMap tm;
@@ -358,10 +285,10 @@ struct UnmergeOp {
   }
 };
 
-template <class Op, typename AccT, int BM, int BN, int TM, int TN, int KG = 1>
+template <class Op, int BM, int BN, int TM, int TN>
 static void run_tile(const Op& op, int batches, cudaStream_t s) {
   const dim3 grid((op.N + BN - 1) / BN, (op.M + BM - 1) / BM, batches);
-  launch_dependent(simt_gemm_kernel<Op, AccT, BM, BN, TM, TN, KG>, grid, dim3((BM / TM) * (BN / TN) * KG), 0, s, op);  // errors: cudaGetLastError
+  launch_dependent(simt_gemm_kernel<Op, BM, BN, TM, TN>, grid, dim3((BM / TM) * (BN / TN)), 0, s, op);  // errors: cudaGetLastError
   count_launch();
 }
 
@@ -384,22 +311,13 @@ static int pick_form(const TileForm* f, int n, int M, int N, int batches) {
   return best;
 }
 
-template <class Op, typename AccT>
+template <class Op>
 static void run_gemm(const Op& op, int batches, cudaStream_t s) {
-  if constexpr (sizeof(AccT) == 8) {
-    static constexpr TileForm forms[] = {{64, 64, 8, 1.0}, {32, 32, 8, 0.8}, {16, 32, 4, 0.7}};
-    switch (pick_form(forms, 3, op.M, op.N, batches)) {
-      case 0: run_tile<Op, AccT, 64, 64, 4, 4>(op, batches, s); break;
-      case 1: run_tile<Op, AccT, 32, 32, 4, 4, 4>(op, batches, s); break;
-      default: run_tile<Op, AccT, 16, 32, 4, 4, 4>(op, batches, s);
-    }
-  } else {
-    static constexpr TileForm forms[] = {{128, 128, 8, 1.0}, {64, 64, 4, 0.85}, {32, 64, 4, 0.6}};
-    switch (pick_form(forms, 3, op.M, op.N, batches)) {
-      case 0: run_tile<Op, AccT, 128, 128, 8, 8>(op, batches, s); break;
-      case 1: run_tile<Op, AccT, 64, 64, 4, 8>(op, batches, s); break;
-      default: run_tile<Op, AccT, 32, 64, 4, 4>(op, batches, s);
-    }
+  static constexpr TileForm forms[] = {{128, 128, 8, 1.0}, {64, 64, 4, 0.85}, {32, 64, 4, 0.6}};
+  switch (pick_form(forms, 3, op.M, op.N, batches)) {
+    case 0: run_tile<Op, 128, 128, 8, 8>(op, batches, s); break;
+    case 1: run_tile<Op, 64, 64, 4, 8>(op, batches, s); break;
+    default: run_tile<Op, 32, 64, 4, 4>(op, batches, s);
   }
 }
 
@@ -622,6 +540,126 @@ static cudaError_t run_logits(const LogitsOp<__nv_bfloat16>& op, int batches, cu
   count_launch();
   return launch_dependent(logits_kernel<BM, BN, TM, TN>, grid, dim3((BM / TM) * (BN / TN)), logit_smem<BM, BN>(), s, op);
 }
+// The same of fp32 tokens, summed in double (the order of addition does not show in the fp32 result).  Their way into double
+// is the bound where there is enough to do (eight conversions, at a quarter of the rate, for sixteen multiply-adds); few and
+// small regions wait for loads instead, and so KG groups of threads share a tile, each with every KG-th four channels of a
+// stage of 32, and add up through shared memory at the end.  Thread = 4 x 4 outputs.
+constexpr int kLogit64K = 32, kLogit64Pitch = kLogit64K * 4 + 16;
+template <int BM, int BN>
+constexpr int logit64_stages() { return BM + BN > 32 ? 4 : 8; }
+template <int BM, int BN, int KG>
+constexpr int logit64_smem() {
+  constexpr int ring = logit64_stages<BM, BN>() * (BM + BN) * kLogit64Pitch, parts = (KG - 1) * BM * BN * 8;
+  return (ring > parts ? ring : parts) + (BM + BN) * 8;
+}
+
+template <int BM, int BN, int KG>
+__global__ void __launch_bounds__(BM / 4 * (BN / 4) * KG) logits64_kernel(const LogitsOp<float> op) {
+  constexpr int kStages = logit64_stages<BM, BN>(), kRows = BM + BN, kStageBytes = kRows * kLogit64Pitch;
+  constexpr int kGm = BM / 4, kGn = BN / 4, kGroup = kGm * kGn, kThreads = kGroup * KG, kPackets = kRows * 8 / kThreads;
+  static_assert(kRows * 8 % kThreads == 0 && 8 % KG == 0, "tile form");
+  extern __shared__ __align__(16) uint8_t logit_smem_raw[];
+  const float** row = reinterpret_cast<const float**>(logit_smem_raw + logit64_smem<BM, BN, KG>() - kRows * 8);
+  const int tid = threadIdx.x, batch = blockIdx.z, m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const int in_group = tid % kGroup, kg = tid / kGroup, tn = in_group % kGn, tm = in_group / kGn;
+  tc::dependency_wait();  // launched with programmatic stream serialisation
+  if (tid == 0) tc::release_dependents();
+  for (int e = tid; e < kRows; e += kThreads) {
+    const int i = e < BM ? m0 + e : n0 + e - BM;
+    row[e] = i < (e < BM ? op.M : op.N) ? (e < BM ? op.a_ptr(batch, i) : op.b_ptr(batch, i)) : nullptr;
+  }
+  __syncthreads();
+  const uint32_t base = tc::smem_u32(logit_smem_raw);
+  const int nk = (op.K + kLogit64K - 1) / kLogit64K;
+  auto fetch = [&](int ks) {
+    if (ks < nk) {
+#pragma unroll
+      for (int v = 0; v < kPackets; ++v) {
+        const int e = tid + v * kThreads, r = e >> 3, c = ks * kLogit64K + (e & 7) * 4;
+        const float* p = row[r];
+        const bool real = p != nullptr && c < op.K;
+        cp_async16(base + (ks % kStages) * kStageBytes + r * kLogit64Pitch + (e & 7) * 16, real ? p + c : op.x, real);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  double acc[4][4] = {};
+#pragma unroll 1
+  for (int ks = 0; ks < kStages - 1; ++ks) fetch(ks);
+#pragma unroll 1
+  for (int ks = 0; ks < nk; ++ks) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+    __syncthreads();         // stage ks is there for all, stage ks - 1 read by all
+    fetch(ks + kStages - 1);
+    const uint8_t* st = logit_smem_raw + (ks % kStages) * kStageBytes;
+#pragma unroll 1
+    for (int c = kg; c < 8; c += KG) {
+      float4 a[4], b[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[u] = *reinterpret_cast<const float4*>(st + (tm + u * kGm) * kLogit64Pitch + c * 16);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) b[u] = *reinterpret_cast<const float4*>(st + (BM + tn + u * kGn) * kLogit64Pitch + c * 16);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        auto wide = [&](const float4& q) { return (double)(e == 0 ? q.x : e == 1 ? q.y : e == 2 ? q.z : q.w); };
+        double bd[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) bd[u] = wide(b[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const double ad = wide(a[u]);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[u][q] = fma(ad, bd[q], acc[u][q]);
+        }
+      }
+    }
+  }
+  if constexpr (KG > 1) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // the last stages have been read
+    double* part = reinterpret_cast<double*>(logit_smem_raw);  // [KG - 1][16][kGroup]
+    if (kg > 0) {
+#pragma unroll
+      for (int e = 0; e < 16; ++e) part[((kg - 1) * 16 + e) * kGroup + in_group] = acc[e >> 2][e & 3];
+    }
+    __syncthreads();
+    if (kg > 0) return;
+#pragma unroll
+    for (int e = 0; e < 16; ++e)
+#pragma unroll
+      for (int g = 0; g < KG - 1; ++g) acc[e >> 2][e & 3] += part[(g * 16 + e) * kGroup + in_group];
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int m = m0 + tm + u * kGm;
+    if (m >= op.M) break;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int n = n0 + tn + q * kGn;
+      if (n < op.N) op.logits[((size_t)batch * op.M + m) * op.N + n] = (float)(acc[u][q] * (double)op.scale);
+    }
+  }
+}
+
+template <int BM, int BN, int KG>
+static cudaError_t run_logits64(const LogitsOp<float>& op, int batches, cudaStream_t s) {
+  static std::atomic<unsigned long long> raised{0};
+  if (cudaError_t e = raise_dynamic_smem(logits64_kernel<BM, BN, KG>, logit64_smem<BM, BN, KG>(), raised); e != cudaSuccess) return e;
+  const dim3 grid((op.N + BN - 1) / BN, (op.M + BM - 1) / BM, batches);
+  count_launch();
+  return launch_dependent(logits64_kernel<BM, BN, KG>, grid, dim3(BM / 4 * (BN / 4) * KG), logit64_smem<BM, BN, KG>(), s, op);
+}
+// Timed on thirteen shapes (microseconds per tile and 640 channels on the fullest SM): 16 x 16 takes 3.2 among many; 64 x 64
+// takes 44, one or two of them 90, and wins where every SM has several.  The weights as a whole (with logits in stages of 16
+// channels, one ahead, before): 16 regions of 64 tokens, 640 channels 27 -> 15 us, of 256 tokens 100 -> 65, 256 of those 769
+// -> 698.  32 x 32 in four groups was between the two, and 4 % better than both at 4 regions of 1024 tokens.
+static cudaError_t launch_logits64(const LogitsOp<float>& op, int batches, cudaStream_t s) {
+  auto on_an_sm = [&](int b) {
+    const long long ctas = (long long)((op.M + b - 1) / b) * ((op.N + b - 1) / b) * batches;
+    return (double)((ctas + sm_count() - 1) / sm_count());
+  };
+  return fmax(90.0, 44.0 * on_an_sm(64)) < 3.2 * on_an_sm(16) ? run_logits64<64, 64, 1>(op, batches, s) : run_logits64<16, 16, 8>(op, batches, s);
+}
 // The form that is through first.  Timed on thirteen shapes (microseconds per tile and 640 channels on the fullest SM): 64 x 64
 // takes 18 while an SM has few of them and 14.5 among many; 64 x 32 by 64 threads takes 8, but 18 where there is nothing
 // beside it; 32 x 32 by 128 threads 5.3, alone as well.
@@ -640,10 +678,10 @@ cudaError_t launch_weights_simt(const Geom& g, const void* x, const int32_t* idx
   const int batches = g.B * g.P;
   cudaError_t e;
   if (g.f32) {  // fp32 mode sums the logits in double: a logit of some hundreds has to be right to its last fp32 bit
-    LogitsOp<float> op{g.Dloc, g.Nloc, g.d, true, true, make_map(g), (const float*)x, idx, logits, g.logit_scale};
-    run_gemm<LogitsOp<float>, double>(op, batches, s);
+    LogitsOp<float> op{g.Dloc, g.Nloc, g.d, make_map(g), (const float*)x, idx, logits, g.logit_scale};
+    if ((e = launch_logits64(op, batches, s)) != cudaSuccess) return e;
   } else {
-    LogitsOp<__nv_bfloat16> op{g.Dloc, g.Nloc, g.d, true, true, make_map(g), (const __nv_bfloat16*)x, idx, logits, g.logit_scale};
+    LogitsOp<__nv_bfloat16> op{g.Dloc, g.Nloc, g.d, make_map(g), (const __nv_bfloat16*)x, idx, logits, g.logit_scale};
     if ((e = launch_logits(op, batches, s)) != cudaSuccess) return e;
   }
   const size_t smem = (size_t)g.Dloc * kSoftTok * 4;
@@ -708,12 +746,12 @@ cudaError_t launch_merge_simt(const Geom& g, const void* w, const void* x, void*
   const int batches = g.B * g.P;
   if (g.f32) {
     MergeOp<float, float> op{g.Dloc, g.d, g.Nloc, g.Dloc % 4 == 0, true, make_map(g), (const float*)w, (const float*)x, (float*)xm};
-    run_gemm<MergeOp<float, float>, float>(op, batches, s);
+    run_gemm<MergeOp<float, float>>(op, batches, s);
     copy_extra<float>(g, (const float*)x, (float*)xm, true, s);
   } else {
     MergeOp<__nv_bfloat16, __nv_bfloat16> op{g.Dloc, g.d, g.Nloc, false, true, make_map(g), (const __nv_bfloat16*)w, (const __nv_bfloat16*)x,
                                       (__nv_bfloat16*)xm};
-    run_gemm<MergeOp<__nv_bfloat16, __nv_bfloat16>, float>(op, batches, s);
+    run_gemm<MergeOp<__nv_bfloat16, __nv_bfloat16>>(op, batches, s);
     copy_extra<__nv_bfloat16>(g, (const __nv_bfloat16*)x, (__nv_bfloat16*)xm, true, s);
   }
   return cudaGetLastError();
@@ -723,12 +761,12 @@ cudaError_t launch_unmerge_simt(const Geom& g, const void* w, const void* y, voi
   const int batches = g.B * g.P;
   if (g.f32) {
     UnmergeOp<float, float> op{g.Nloc, g.d, g.Dloc, g.Dloc % 4 == 0, true, make_map(g), (const float*)w, (const float*)y, (float*)out};
-    run_gemm<UnmergeOp<float, float>, float>(op, batches, s);
+    run_gemm<UnmergeOp<float, float>>(op, batches, s);
     copy_extra<float>(g, (const float*)y, (float*)out, false, s);
   } else {
     UnmergeOp<__nv_bfloat16, __nv_bfloat16> op{g.Nloc, g.d, g.Dloc, false, true, make_map(g), (const __nv_bfloat16*)w, (const __nv_bfloat16*)y,
                                         (__nv_bfloat16*)out};
-    run_gemm<UnmergeOp<__nv_bfloat16, __nv_bfloat16>, float>(op, batches, s);
+    run_gemm<UnmergeOp<__nv_bfloat16, __nv_bfloat16>>(op, batches, s);
     copy_extra<__nv_bfloat16>(g, (const __nv_bfloat16*)y, (__nv_bfloat16*)out, false, s);
   }
   return cudaGetLastError();
@@ -737,9 +775,8 @@ cudaError_t launch_unmerge_simt(const Geom& g, const void* w, const void* y, voi
 // c[m][n] = sum_k a[m][k] w[k][n] (plain projection; fp32 mode and shapes the tensor-core kernel does not take).
 template <typename T>
 struct LinearOp {
-  static constexpr bool a_k_contig = true, b_k_contig = false;
+  static constexpr bool a_k_contig = true;
   typedef const T* APtr;
-  typedef const T* BPtr;
   int M, N, K;
   bool a_vec, b_vec;
   const T* a_;
@@ -759,10 +796,10 @@ struct LinearOp {
 cudaError_t launch_linear_simt(int M, int N, int K, bool f32, const void* a, const void* w, void* c, int act, cudaStream_t s) {
   if (f32) {
     LinearOp<float> op{M, N, K, K % 4 == 0, N % 4 == 0, (const float*)a, (const float*)w, (float*)c, act};
-    run_gemm<LinearOp<float>, float>(op, 1, s);
+    run_gemm<LinearOp<float>>(op, 1, s);
   } else {
     LinearOp<__nv_bfloat16> op{M, N, K, K % 4 == 0, N % 4 == 0, (const __nv_bfloat16*)a, (const __nv_bfloat16*)w, (__nv_bfloat16*)c, act};
-    run_gemm<LinearOp<__nv_bfloat16>, float>(op, 1, s);
+    run_gemm<LinearOp<__nv_bfloat16>>(op, 1, s);
   }
   return cudaGetLastError();
 }

@@ -1482,3 +1482,24 @@ def test_ffma_attention_of_keys_at_minus_infinity(toma):
     rest = torch.cat([torch.arange(64), torch.arange(128, L)]).cuda()
     want = torch.softmax(q[0].double() @ k[0, rest].double().T / dh ** 0.5, dim=1) @ v[0, rest].double()
     assert_close(to_host64(o)[0], want.cpu().numpy(), "f32", "attention")
+
+
+@pytest.mark.parametrize("batch,gy,gx,th,tw,dim,ratio", [
+    (8, 4, 4, 16, 16, 40, 0.5),   # logits in tiles of 64 x 64, many per SM; a last stage of 8 channels
+    (4, 6, 6, 19, 15, 32, 0.5),   # ... partial in both directions; one stage
+    (1, 1, 1, 1, 1, 8, 0.0),      # 16 x 16: one token
+    (2, 2, 3, 7, 5, 264, 0.5),    # ... 35 tokens, 17 destinations
+    (1, 1, 2, 16, 3, 320, 0.65),  # ... more stages than the ring holds; one tile of destinations, three of tokens
+])
+def test_f32_weights_of_every_tile_form(toma, batch, gy, gx, th, tw, dim, ratio):
+    """Merge weights of fp32 tokens, every region of the launch, against 64-bit arithmetic."""
+    cfg = gen.config("cfg2", batch=batch, grid_h=gy * th, grid_w=gx * tw, tile_h=th, tile_w=tw, dim=dim, n_heads=dim // 8, head_dim=8,
+                     merge_ratio=ratio, dtype="f32")
+    run = Run(toma, cfg, gen.features(cfg))
+    run.select()
+    dense = torch.from_numpy(run.weights()).cuda()
+    xt = _regions(cfg, run.x)
+    dest = torch.gather(xt, 2, run.idx.reshape(batch, cfg.n_tiles, run.d_loc, 1).long().expand(-1, -1, -1, dim))
+    shares = torch.softmax(dest @ xt.transpose(2, 3) / (cfg.tau * dim ** 0.5), dim=2)
+    # a logit l is rounded to 2^-24 l once more, which moves a share by as much: 6e-5 at the largest ones here (about 1000)
+    assert float((dense - shares / shares.sum(3, keepdim=True)).abs().max()) <= 1e-4
