@@ -1,9 +1,10 @@
 // Destination selection and merge weights of a 64-token tile in one kernel (Sec. 4.1, Algorithm 2 and
 // Sec. 4.2.1), for the refresh steps of the small-tile block: instead of a Gram kernel, a greedy kernel, a
 // gather and a weights kernel - four launches of a few microseconds of work each - one CTA per tile
-//   1. streams the tile's quantised tokens y and its raw tokens x (64-channel slabs, TMA ring) through two
-//      Gram products on the tensor cores: S = y y^T (exact in fp32: every partial sum is a multiple of 2^-24
-//      below 1) and G = x x^T, both 64 x 64 in tensor memory;
+//   1. streams the tile's quantised tokens y and its raw tokens x (64-channel slabs, TMA ring) through one
+//      Gram product of all 128 on the tensor cores: S = y y^T (exact in fp32: every partial sum is a multiple of 2^-24
+//      below 1) and G = x x^T are 64 x 64 each of its accumulator.  (Two products of 64 rows, with 64 more that are not
+//      there, read 12 KB of shared memory per 16 channels where this one reads 8, and took 5.7 us of 20 for 1280 channels.)
 //   2. rounds S to the fixed-point S_q in shared memory and runs the greedy rounds on it in ONE warp (two
 //      candidates and two cached maxima per lane, no block barrier; several picks per round: greedy.cuh);
 //   3. takes the logits of Sec. 4.2.1 out of G - the logit of source k and destination i is G[idx_i][k] scaled,
@@ -11,8 +12,8 @@
 //      destinations per source, row sums per destination in a fixed order, and writes A~^T as hi and lo planes.
 // The quantised tokens come from quantise_kernel (fp64 arithmetic over 148 SMs; one CTA per tile would take
 // longer over it than the kernel takes as a whole).
-// Warp 0, 1: thread = token = tensor-memory lane (warp 0 runs the greedy rounds); warp 2: TMA producer;
-// warp 3: MMA issuer.
+// Warp 2: TMA producer; warp 3: MMA issuer.  Then warps 0, 1: thread = token = tensor-memory lane of S (warp 0 runs the greedy
+// rounds); warps 2, 3: the same of G; all four write the weights.
 #include "common.cuh"
 #include "greedy.cuh"
 #include "tc.cuh"
@@ -33,7 +34,6 @@ struct RBars {
   uint64_t full[kRing], empty[kRing], done;
   uint32_t tmem_base;
   int abort_flag;
-  int go;  // the row warps' common decision to carry on after the contractions
 };
 
 struct RParams {
@@ -92,10 +92,8 @@ refresh_small_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_cons
                      uint32_t* dev_status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  // ring, then one slab of padding: an MMA reads 128 operand rows, of which only the first 64 exist; the other 64
-  // are whatever follows the slab (their accumulator rows are never read)
   uint8_t* ring = smem;
-  uint16_t* S = reinterpret_cast<uint16_t*>(ring + kRing * kStageBytes + kSlab);  // [64][64]
+  uint16_t* S = reinterpret_cast<uint16_t*>(ring + kRing * kStageBytes);        // [64][64]
   float* G = reinterpret_cast<float*>(S + kTok * kTok);                         // [64][kPitch]
   float* A = G + kTok * kPitch;                                                 // shares [D_loc][kPitch]
   float* zinv = A + kTok * kPitch;                                              // [64]
@@ -141,84 +139,105 @@ refresh_small_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_cons
     }
   } else if (warp == 3) {
     if (elect_one()) {
-      constexpr uint32_t idesc = idesc_f16(kFmtBF16, kFmtBF16, false, false, 128, kTok);
+      constexpr uint32_t idesc = idesc_f16(kFmtBF16, kFmtBF16, false, false, 2 * kTok, 2 * kTok);
       bool ok = true;
       for (int k = 0; k < nk; ++k) {
         const int s = k % kRing;
         if (!mbar_wait(&bar->full[s], (k / kRing) & 1, dev_status, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t ya = smem_u32(ring + s * kStageBytes), xa = ya + kSlab;
+        const uint32_t ya = smem_u32(ring + s * kStageBytes);  // 64 rows of y, 64 of x
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {  // 16 channels per MMA
-          const uint64_t yd = smem_desc_sw128(ya + kk * 32, 16, 1024), xd = smem_desc_sw128(xa + kk * 32, 16, 1024);
+          const uint64_t yd = smem_desc_sw128(ya + kk * 32, 16, 1024);
           mma_ss(tmem, yd, yd, idesc, k > 0 || kk > 0);
-          mma_ss(tmem + kTok, xd, xd, idesc, k > 0 || kk > 0);
         }
         mma_commit(&bar->empty[s]);
       }
       if (ok) mma_commit(&bar->done);
     }
-  } else {
-    const int r = threadIdx.x;  // token = tensor-memory lane (warp 0: lanes 0..31, warp 1: 32..63)
-    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
-    // one answer per warp: the tensor-memory loads below are warp-wide operations
-    if (__all_sync(0xffffffffu, mbar_wait(&bar->done, 0, dev_status, abort_flag))) {
-      tc_fence_after();
+  }
+  __syncwarp();
+  const int r = threadIdx.x & (kTok - 1);  // token; threadIdx.x = its tensor-memory lane
+  if (mbar_wait_warp(&bar->done, 0, dev_status, abort_flag)) {
+    tc_fence_after();
+    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (warp < 2 ? 0 : kTok);
 #pragma unroll
-      for (int c0 = 0; c0 < kTok; c0 += 32) {  // S_q[r][c] = rint(<y_r, y_c> * 4096), the diagonal by definition
-        uint32_t v[32];
-        tmem_ld32(taddr + c0, v);
-        tmem_wait_ld();
+    for (int c0 = 0; c0 < kTok; c0 += 32) {
+      uint32_t v[32];
+      tmem_ld32(taddr + c0, v);
+      tmem_wait_ld();
+      if (warp < 2) {  // S_q[r][c] = rint(<y_r, y_c> * 4096), the diagonal by definition
 #pragma unroll
         for (int e = 0; e < 32; ++e)
           S[(c0 + e) * kTok + r] = (uint16_t)((c0 + e == r ? kDiagQ : __float2int_rn(__uint_as_float(v[e]) * 4096.f)) + kSqBias);
-      }
-#pragma unroll
-      for (int c0 = 0; c0 < kTok; c0 += 32) {
-        uint32_t v[32];
-        tmem_ld32(taddr + kTok + c0, v);
-        tmem_wait_ld();
+      } else {
 #pragma unroll
         for (int e = 0; e < 32; ++e) G[r * kPitch + c0 + e] = __uint_as_float(v[e]);
       }
     }
-    rows_sync();  // S_q and G are complete in shared memory - or somebody's wait ran out
-    if (r == 0) bar->go = *abort_flag ? 0 : 1;  // one decision for both warps: the barriers below need all 64 threads
+  }
+  __syncthreads();  // S_q and G are complete in shared memory - or somebody's wait ran out, the last of them
+  const bool go = *abort_flag == 0;
+  const int Dl = p.Dloc;
+  if (go && warp < 2) {
+    // ---- Algorithm 2
+    if (warp == 0) greedy_one_warp(reinterpret_cast<const uint32_t*>(S), Dl, lane, *lists, sel, p.idx + (size_t)tile_b * Dl);
     rows_sync();
-    if (bar->go) {
-      // ---- Algorithm 2
-      if (warp == 0) greedy_one_warp(reinterpret_cast<const uint32_t*>(S), p.Dloc, lane, *lists, sel, p.idx + (size_t)tile_b * p.Dloc);
-      rows_sync();
-      // ---- Sec. 4.2.1: thread = source token k; logit of destination i is G[idx_i][k] / (tau sqrt(d))
-      const int Dl = p.Dloc;
-      float mx = -INFINITY;
-      for (int i = 0; i < Dl; ++i) mx = fmaxf(mx, G[sel[i] * kPitch + r]);
-      const float neg_m = -mx * p.scale_log2;
-      float sum = 0.f;
-      for (int i = 0; i < Dl; ++i) sum += ex2(fmaf(G[sel[i] * kPitch + r], p.scale_log2, neg_m));
-      const float inv = 1.f / sum;
-      for (int i = 0; i < Dl; ++i) A[i * kPitch + r] = ex2(fmaf(G[sel[i] * kPitch + r], p.scale_log2, neg_m)) * inv;
-      rows_sync();
-      if (r < Dl) {  // row sum of destination r over the tile's sources, in source order
-        float z = 0.f;
-        for (int k = 0; k < kTok; ++k) z += A[r * kPitch + k];
-        zinv[r] = z > 0.f ? 1.f / z : 0.f;  // a row sum that underflowed to 0 gives a zero row
-      }
-      rows_sync();
-      // A~^T[k][i] = A[i][k] / Z_i as hi + lo bf16 planes; a source's D_loc weights are contiguous (D_loc % 8 == 0)
-      __nv_bfloat16* hi_row = p.w + ((size_t)tile_b * 2 * kTok + r) * Dl;
-      __nv_bfloat16* lo_row = hi_row + (size_t)kTok * Dl;
-      for (int i0 = 0; i0 < Dl; i0 += 8) {
-        __align__(16) __nv_bfloat16 hi[8], lo[8];
+    // ---- Sec. 4.2.1: thread = source token k; logit of destination i is G[idx_i][k] / (tau sqrt(d)).  Eight at a time, so that
+    // their reads are in flight together (one behind the other: 2.5 us).
+    float mx = -INFINITY;
+    for (int i0 = 0; i0 < Dl; i0 += 8) {
+      float g[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float v = A[(i0 + e) * kPitch + r] * zinv[i0 + e];
-          hi[e] = __float2bfloat16_rn(v);
-          lo[e] = __float2bfloat16_rn(v - __bfloat162float(hi[e]));
-        }
-        *reinterpret_cast<uint4*>(hi_row + i0) = *reinterpret_cast<const uint4*>(hi);
-        *reinterpret_cast<uint4*>(lo_row + i0) = *reinterpret_cast<const uint4*>(lo);
+      for (int e = 0; e < 8; ++e) g[e] = G[sel[i0 + e] * kPitch + r];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) mx = fmaxf(mx, g[e]);
+    }
+    const float neg_m = -mx * p.scale_log2;
+    float sum = 0.f;
+    for (int i0 = 0; i0 < Dl; i0 += 8) {
+      float g[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) g[e] = G[sel[i0 + e] * kPitch + r];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) g[e] = ex2(fmaf(g[e], p.scale_log2, neg_m));
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        A[(i0 + e) * kPitch + r] = g[e];
+        sum += g[e];
       }
+    }
+    const float inv = 1.f / sum;
+    for (int i0 = 0; i0 < Dl; i0 += 8) {
+      float g[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) g[e] = A[(i0 + e) * kPitch + r];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) A[(i0 + e) * kPitch + r] = g[e] * inv;
+    }
+    rows_sync();
+    if (r < Dl) {  // row sum of destination r over the tile's sources, in source order
+      float z = 0.f;
+      for (int k = 0; k < kTok; ++k) z += A[r * kPitch + k];
+      zinv[r] = z > 0.f ? 1.f / z : 0.f;  // a row sum that underflowed to 0 gives a zero row
+    }
+  }
+  __syncthreads();
+  if (go) {
+    // A~^T[k][i] = A[i][k] / Z_i as hi + lo bf16 planes; a source's D_loc weights are contiguous (D_loc % 8 == 0), and two
+    // threads take every second eight of them
+    __nv_bfloat16* hi_row = p.w + ((size_t)tile_b * 2 * kTok + r) * Dl;
+    __nv_bfloat16* lo_row = hi_row + (size_t)kTok * Dl;
+    for (int i0 = (warp >> 1) * 8; i0 < Dl; i0 += 16) {
+      __align__(16) __nv_bfloat16 hi[8], lo[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const float v = A[(i0 + e) * kPitch + r] * zinv[i0 + e];
+        hi[e] = __float2bfloat16_rn(v);
+        lo[e] = __float2bfloat16_rn(v - __bfloat162float(hi[e]));
+      }
+      *reinterpret_cast<uint4*>(hi_row + i0) = *reinterpret_cast<const uint4*>(hi);
+      *reinterpret_cast<uint4*>(lo_row + i0) = *reinterpret_cast<const uint4*>(lo);
     }
   }
   tc_fence_before();
@@ -229,7 +248,7 @@ refresh_small_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_cons
   }
 }
 
-constexpr int kRefreshSmem = 1024 + kRing * kStageBytes + kSlab + kTok * kTok * 2 + 2 * kTok * kPitch * 4 + 2 * kTok * 4 + (int)sizeof(greedy::Shared<kTok>) + 256;
+constexpr int kRefreshSmem = 1024 + kRing * kStageBytes + kTok * kTok * 2 + 2 * kTok * kPitch * 4 + 2 * kTok * 4 + (int)sizeof(greedy::Shared<kTok>) + 256;
 static_assert(sizeof(RBars) <= 256, "barrier block outgrew its reservation");
 
 }  // namespace
