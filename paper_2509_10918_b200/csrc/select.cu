@@ -12,14 +12,13 @@ namespace toma {
 // written tile-major: row (b*P + p)*N_loc + l.  Defined in fp64 (the squares added up per lane in channel order, then by
 // the tree below; scale, product and rounding), so that the CPU definition can be matched bit for bit.
 // The fp64 pipe and its conversions bounded this kernel (4 x 16384 tokens of 640 channels: 65 us, where reading and writing
-// them takes 26; now 50).  bf16 tokens therefore get their squares' sum from the same fp64 additions, but of doubles put together
+// them takes 26; now 49).  bf16 tokens therefore get their squares' sum from the same fp64 additions, but of doubles put together
 // from the bits, and the products as pairs of floats: x * scale = hi + lo to about 2^-45 of it, and what is not within 2^-20
 // of the middle between two integers rounds as the fp64 product does.  A token with a channel that is (one in some
 // thousands), or with a norm far from 1, is done again in fp64.
 // ---------------------------------------------------------------------------
 // Eight consecutive elements as floats (16-byte aligned source).
-__device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&v)[8]) {
-  const uint4 raw = *reinterpret_cast<const uint4*>(p);
+__device__ __forceinline__ void widen8(const uint4& raw, float (&v)[8]) {
   const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
@@ -27,6 +26,7 @@ __device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&v)[8]) {
     v[2 * e + 1] = __uint_as_float(w[e] & 0xFFFF0000u);
   }
 }
+__device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&v)[8]) { widen8(*reinterpret_cast<const uint4*>(p), v); }
 __device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
   const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
   v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
@@ -67,27 +67,32 @@ __device__ __forceinline__ double widen(float v) {
   const uint32_t b = __float_as_uint(v);
   return __hiloint2double((int)(((b & 0x7FFFFFFFu) >> 3) + 0x38000000u), 0);  // without the sign: it is squared
 }
-// False: not this way.
+// kTrips > 0: the warp's trips over the token's channels, all on their way before the first is used and kept in registers for
+// the products.  0: one at a time, read twice.  False: not this way.
+template <int kTrips>
 __device__ __forceinline__ bool quantise_fast(const __nv_bfloat16* row, __nv_bfloat16* out, int d, int lane) {
   double ss = 0.0;
-  for (int c = lane * 8; c < d; c += 256) {
+  auto add_squares = [&](const uint4& raw) {
     float v[8];
-    load8(row + c, v);
+    widen8(raw, v);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const double x = widen(v[e]);
       ss = fma(x, x, ss);  // the square is exact
     }
-  }
-  ss = warp_sum(ss);
-  // no infinities, no sum that 2^-254 for a zero could change, no scale whose parts leave the range of floats
-  if (!(ss > 1e-40 && ss < 1e40)) return false;
-  const double scale = kCosScaleTimesOne / sqrt(ss);
-  const float s_hi = (float)scale, s_lo = (float)(scale - (double)s_hi);
-  float off = 0.f;  // largest distance from an integer
-  for (int c = lane * 8; c < d; c += 256) {
+  };
+  float s_hi, s_lo, off = 0.f;  // the scale; largest distance from an integer
+  auto set_scale = [&] {
+    ss = warp_sum(ss);
+    // no infinities, no sum that 2^-254 for a zero could change, no scale whose parts leave the range of floats
+    if (!(ss > 1e-40 && ss < 1e40)) return false;
+    const double scale = kCosScaleTimesOne / sqrt(ss);
+    s_hi = (float)scale, s_lo = (float)(scale - (double)s_hi);
+    return true;
+  };
+  auto write = [&](const uint4& raw, int c) {
     float v[8];
-    load8(row + c, v);
+    widen8(raw, v);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const float p = v[e] * s_hi;
@@ -97,11 +102,29 @@ __device__ __forceinline__ bool quantise_fast(const __nv_bfloat16* row, __nv_bfl
       v[e] = k;
     }
     store8(out + c, v);
+  };
+  auto at = [&](int c) { return *reinterpret_cast<const uint4*>(row + c); };
+  if constexpr (kTrips > 0) {
+    uint4 raw[kTrips];
+#pragma unroll
+    for (int t = 0; t < kTrips; ++t)
+      if (t * 256 + lane * 8 < d) raw[t] = at(t * 256 + lane * 8);
+#pragma unroll
+    for (int t = 0; t < kTrips; ++t)
+      if (t * 256 + lane * 8 < d) add_squares(raw[t]);
+    if (!set_scale()) return false;
+#pragma unroll
+    for (int t = 0; t < kTrips; ++t)
+      if (t * 256 + lane * 8 < d) write(raw[t], t * 256 + lane * 8);
+  } else {
+    for (int c = lane * 8; c < d; c += 256) add_squares(at(c));
+    if (!set_scale()) return false;
+    for (int c = lane * 8; c < d; c += 256) write(at(c), c);  // second read of the row: an L1/L2 hit
   }
   return !__any_sync(0xffffffffu, off > 0.5f - 0x1p-20f);
 }
 
-template <typename T>
+template <typename T, int kTrips>
 __global__ void __launch_bounds__(256) quantise_kernel(const T* __restrict__ x, __nv_bfloat16* __restrict__ y, int B,
                                                        int N, int n_all, int d, int W, int th, int tw, int tiles_x,
                                                        int P, int Nloc) {
@@ -117,7 +140,7 @@ __global__ void __launch_bounds__(256) quantise_kernel(const T* __restrict__ x, 
   const T* row = x + ((size_t)b * n_all + n) * d;
   __nv_bfloat16* out = y + ((size_t)(b * P + p) * Nloc + l) * d;
   if constexpr (sizeof(T) == 2) {
-    if (quantise_fast(row, out, d, lane)) return;
+    if (quantise_fast<kTrips>(row, out, d, lane)) return;
   }
   quantise_f64(row, out, d, lane);
 }
@@ -125,13 +148,17 @@ __global__ void __launch_bounds__(256) quantise_kernel(const T* __restrict__ x, 
 cudaError_t launch_quantise(const Geom& g, const void* x, __nv_bfloat16* y, cudaStream_t s) {
   const long long warps = (long long)g.B * g.N;
   const int blocks = (int)((warps * 32 + 255) / 256);
-  cudaError_t e;
-  if (g.f32)
-    e = launch_dependent(quantise_kernel<float>, dim3(blocks), dim3(256), 0, s, (const float*)x, y, g.B, g.N, (int)g.tokens_all(), g.d, g.W, g.th,
-                                                  g.tw, g.tiles_x, g.P, g.Nloc);
-  else
-    e = launch_dependent(quantise_kernel<__nv_bfloat16>, dim3(blocks), dim3(256), 0, s, (const __nv_bfloat16*)x, y, g.B, g.N, (int)g.tokens_all(),
-                                                          g.d, g.W, g.th, g.tw, g.tiles_x, g.P, g.Nloc);
+  auto launch = [&](auto kernel, auto* tokens) {
+    return launch_dependent(kernel, dim3(blocks), dim3(256), 0, s, tokens, y, g.B, g.N, (int)g.tokens_all(), g.d, g.W, g.th, g.tw, g.tiles_x, g.P, g.Nloc);
+  };
+  // Channels kept in registers: 4096 tokens of 3072 channels 6 us less, 2 x 4096 of 640 1.5 less.  Where a warp runs once, the long
+  // straight code of more than four trips costs more than that gains (2048 tokens of 1280 channels: 1 us).
+  const __nv_bfloat16* h = (const __nv_bfloat16*)x;
+  const bool once = warps <= 16LL * sm_count();
+  const cudaError_t e = g.f32 ? launch(quantise_kernel<float, 0>, (const float*)x)
+                        : g.d <= 1024 ? launch(quantise_kernel<__nv_bfloat16, 4>, h)
+                        : once || g.d > 4096 ? launch(quantise_kernel<__nv_bfloat16, 0>, h)
+                        : g.d <= 2048 ? launch(quantise_kernel<__nv_bfloat16, 8>, h) : launch(quantise_kernel<__nv_bfloat16, 16>, h);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }

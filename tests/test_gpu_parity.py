@@ -1503,3 +1503,16 @@ def test_f32_weights_of_every_tile_form(toma, batch, gy, gx, th, tw, dim, ratio)
     shares = torch.softmax(dest @ xt.transpose(2, 3) / (cfg.tau * dim ** 0.5), dim=2)
     # a logit l is rounded to 2^-24 l once more, which moves a share by as much: 6e-5 at the largest ones here (about 1000)
     assert float((dense - shares / shares.sum(3, keepdim=True)).abs().max()) <= 1e-4
+
+
+@pytest.mark.parametrize("d", [1024, 1032, 2048, 2056, 4096])
+@pytest.mark.parametrize("tokens_per_side", [16, 64])
+def test_selection_with_channels_kept_in_registers(toma, d, tokens_per_side):
+    """The quantisation's forms by channels (up to 4, 8 and 16 trips of a warp) and tokens (one trip at a time for few)."""
+    side = tokens_per_side
+    cfg = gen.config("cfg2", batch=1, grid_h=side, grid_w=side, tile_h=8, tile_w=4, dim=d, n_heads=d // 8, head_dim=8)
+    x = gen.features(cfg)
+    idx = Run(toma, cfg, x).select()
+    for b, p in sample_tiles(cfg, 12):
+        want, _ = O.select_tile(tile_tokens(cfg, x, b, p).astype(np.float64), od(cfg))
+        assert np.array_equal(idx[b, p], want)
