@@ -35,6 +35,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tile = blockIdx.x, m0 = blockIdx.y * 128, n0 = blockIdx.z * n_cols;
   const int nk = (d + kKC - 1) / kKC;
+  const bool same = m0 == n0 && n_cols == 128;  // a block on the diagonal: one operand
   const uint32_t ncols = n_cols > 128 ? 256u : n_cols > 64 ? 128u : n_cols > 32 ? 64u : 32u;
 
   if (threadIdx.x == 0) {
@@ -63,9 +64,9 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       for (int k = 0, s = 0, round = 0; k < nk; ++k, round += s + 1 == stages, s = s + 1 == stages ? 0 : s + 1) {
         if (round > 0 && !mbar_wait(&bar->empty[s], (round - 1) & 1, dev_status, abort_flag)) break;
         uint8_t* sa = smem + s * stage_bytes;
-        mbar_expect_tx(&bar->full[s], stage_bytes);
+        mbar_expect_tx(&bar->full[s], same ? a_bytes : stage_bytes);
         tma_load_3d(sa, &tm_a, &bar->full[s], k * kKC, m0, tile);
-        tma_load_3d(sa + a_bytes, &tm_b, &bar->full[s], k * kKC, n0, tile);
+        if (!same) tma_load_3d(sa + a_bytes, &tm_b, &bar->full[s], k * kKC, n0, tile);
       }
     }
   } else if (warp == 1) {
@@ -75,7 +76,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       for (int k = 0, s = 0, round = 0; k < nk; ++k, round += s + 1 == stages, s = s + 1 == stages ? 0 : s + 1) {
         if (!mbar_wait(&bar->full[s], round & 1, dev_status, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t aa = smem_u32(smem + s * stage_bytes), ba = aa + a_bytes;
+        const uint32_t aa = smem_u32(smem + s * stage_bytes), ba = same ? aa : aa + a_bytes;
 #pragma unroll
         for (int kk = 0; kk < kKC / 16; ++kk)
           mma_ss(tmem, smem_desc_sw128(aa + kk * 32, 16, 1024), smem_desc_sw128(ba + kk * 32, 16, 1024), idesc,
@@ -136,7 +137,11 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 }  // namespace
 
 cudaError_t launch_gram_tc(const Geom& g, const __nv_bfloat16* y, uint16_t* sq, uint32_t* dev_status, cudaStream_t s) {
-  const int n_cols = g.Nloc > 256 ? 256 : (g.Nloc + 15) & ~15;  // MMA N: a multiple of 16
+  // MMA N: a multiple of 16, 256 columns at most.  128 where that still leaves every block an SM of its own: a block then takes in
+  // two thirds of the bytes per step, one on the diagonal a third (16 tiles of 256 tokens, 3072 channels: 5.3 us less for the
+  // refresh step of 208; 32 tiles of 252, 640 channels: 1.5 of 436).
+  int n_cols = g.Nloc > 256 ? 256 : (g.Nloc + 15) & ~15;
+  if (n_cols > 128 && 2LL * g.B * g.P * ((g.Nloc + 127) / 128) * ((g.Nloc + n_cols - 1) / n_cols) <= sm_count()) n_cols = 128;
   CUtensorMap ta, tb;
   const uint64_t dims[3] = {(uint64_t)g.d, (uint64_t)g.Nloc, (uint64_t)g.B * g.P};
   const uint64_t strides[2] = {(uint64_t)g.d * 2, (uint64_t)g.Nloc * g.d * 2};

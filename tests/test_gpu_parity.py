@@ -1516,3 +1516,14 @@ def test_selection_with_channels_kept_in_registers(toma, d, tokens_per_side):
     for b, p in sample_tiles(cfg, 12):
         want, _ = O.select_tile(tile_tokens(cfg, x, b, p).astype(np.float64), od(cfg))
         assert np.array_equal(idx[b, p], want)
+
+
+@pytest.mark.parametrize("tiles", [1, 100])  # column blocks of 128, diagonal ones among them, and of up to 256
+@pytest.mark.parametrize("th,tw", [(3, 43), (16, 15), (15, 17), (16, 16), (19, 20)])
+def test_selection_by_column_blocks_of_the_gram_matrix(toma, tiles, th, tw):
+    cfg = gen.config("cfg2", batch=1, grid_h=tiles * th, grid_w=tw, tile_h=th, tile_w=tw, dim=200, n_heads=25, head_dim=8)
+    x = gen.features(cfg)
+    idx = Run(toma, cfg, x).select()
+    for b, p in sample_tiles(cfg, 4):
+        want, _ = O.select_tile(tile_tokens(cfg, x, b, p).astype(np.float64), od(cfg))
+        assert np.array_equal(idx[b, p], want)
