@@ -227,7 +227,7 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
 }
 
 // ------------------------------------------------------------------------------------------------
-// merge with destinations on M: X_m [D_loc x ch] = A~ [D_loc x N_loc] * X [N_loc x ch], for launches that the SMs hold at once.
+// merge with destinations on M: X_m [D_loc x ch] = A~ [D_loc x N_loc] * X [N_loc x ch], for up to four CTAs per SM.
 // One CTA = (128 destinations, 128 channels); both operands MN-major as they lie in memory.  The same bytes and products per
 // CTA as with channels on M, but a thread then owns an output row and stages 16 bytes at a time where the other form stages 2:
 // the epilogue was 2.3 us of a launch of 8 (32 tiles of 256 tokens, 128 destinations, 640 channels).
@@ -930,6 +930,21 @@ cudaError_t launch_merge_tc(const Geom& g, const void* w, const void* x, void* x
   const int smem = 1024 + p.stages * stage_bytes + 256;
   dim3 grid(g.B * g.P, (g.d + 127) / 128, (g.Dloc + p.dest_block - 1) / p.dest_block);
   cudaError_t e;
+  // Destinations on M as long as an SM has up to four of its CTAs, two at a time: 16 tiles of 256 tokens, 128 destinations, 3072
+  // channels (2.6) 13.5 us one CTA per SM walking over the items, 12.2 so; at 3.9 16.3 and 14.4, at 4.3 18.6 and 18.4, at 8.7
+  // 31.6 and 36.2; 192 destinations, two blocks of which read the tokens twice, at 5.2 15.7 and 17.3.
+  const dim3 rgrid(g.B * g.P, (g.d + 127) / 128, (g.Dloc + 127) / 128);
+  if (g.Dloc <= kMaxCols && (long long)rgrid.x * rgrid.y * rgrid.z <= 4LL * sm_count()) {
+    const uint32_t rbox[4] = {64, 32, 1, 1};  // a warp's 32 destinations
+    if (!encode_tmap_16bit(&to, xm, 4, odims, ostrides, rbox)) return cudaErrorInvalidValue;
+    constexpr int kStage = 6 * kSlab;
+    p.stages = g.Nloc / kKC < 2 ? g.Nloc / kKC : 2;  // two CTAs per SM hide each other's latencies
+    if (copied_beside(rows, rgrid.x * rgrid.y * rgrid.z * kRowsCopyThreads)) p.extra = rows;
+    static std::atomic<unsigned long long> raised_m{0};
+    if (e = raise_dynamic_smem(merge_rows_kernel, 1024 + 2 * kStage + 256, raised_m); e != cudaSuccess) return e;
+    e = launch_dependent(merge_rows_kernel, rgrid, dim3(kRowsThreads), (size_t)(1024 + p.stages * kStage + 256), s, tx, tw, to, p, dev_status);
+    return finish_launch(e, rows, p.extra, s);
+  }
   const int n_chunks = (g.d + 127) / 128, n_blocks = (g.Dloc + p.dest_block - 1) / p.dest_block, n_items = g.B * g.P * n_blocks * n_chunks;
   if (n_items > 2 * sm_count()) {
     // more items than the SMs hold at once: one CTA per SM walks them with the ring and two accumulators kept busy
@@ -951,18 +966,6 @@ cudaError_t launch_merge_tc(const Geom& g, const void* w, const void* x, void* x
       return finish_launch(e, rows, p.extra, s);
     }
     p.stages = 2;
-  }
-  if (g.Dloc <= kMaxCols) {
-    const uint32_t rbox[4] = {64, 32, 1, 1};  // a warp's 32 destinations
-    if (!encode_tmap_16bit(&to, xm, 4, odims, ostrides, rbox)) return cudaErrorInvalidValue;
-    constexpr int kStage = 6 * kSlab;
-    p.stages = g.Nloc / kKC < 2 ? g.Nloc / kKC : 2;  // two CTAs per SM hide each other's latencies
-    const dim3 rgrid(g.B * g.P, (g.d + 127) / 128, (g.Dloc + 127) / 128);
-    if (copied_beside(rows, rgrid.x * rgrid.y * rgrid.z * kRowsCopyThreads)) p.extra = rows;
-    static std::atomic<unsigned long long> raised_m{0};
-    if (e = raise_dynamic_smem(merge_rows_kernel, 1024 + 2 * kStage + 256, raised_m); e != cudaSuccess) return e;
-    e = launch_dependent(merge_rows_kernel, rgrid, dim3(kRowsThreads), (size_t)(1024 + p.stages * kStage + 256), s, tx, tw, to, p, dev_status);
-    return finish_launch(e, rows, p.extra, s);
   }
   if (copied_beside(rows, grid.x * grid.y * grid.z * kCopyThreads)) p.extra = rows;
   static std::atomic<unsigned long long> raised{0};
