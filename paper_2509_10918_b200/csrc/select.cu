@@ -14,8 +14,8 @@ namespace toma {
 // The fp64 pipe and its conversions bounded this kernel (4 x 16384 tokens of 640 channels: 65 us, where reading and writing
 // them takes 26; now 49).  bf16 tokens therefore get their squares' sum from the same fp64 additions, but of doubles put together
 // from the bits, and the products as pairs of floats: x * scale = hi + lo to about 2^-45 of it, and what is not within 2^-20
-// of the middle between two integers rounds as the fp64 product does.  A token with a channel that is (one in some
-// thousands), or with a norm far from 1, is done again in fp64.
+// of the middle between two integers rounds as the fp64 product does.  A token with a channel that is (one in four
+// hundred of 640 to 3072 normally distributed channels), or with a norm far from 1, is done again in fp64.
 // ---------------------------------------------------------------------------
 // Eight consecutive elements as floats (16-byte aligned source).
 __device__ __forceinline__ void widen8(const uint4& raw, float (&v)[8]) {
@@ -95,10 +95,12 @@ __device__ __forceinline__ bool quantise_fast(const __nv_bfloat16* row, __nv_bfl
     widen8(raw, v);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const float p = v[e] * s_hi;
+      // rounded one by one whatever the compiler would fuse: lo is what the product p has lost (p - k of the unrounded product
+      // would count it twice, 2^-13 at most, and let wrong roundings pass)
+      const float p = __fmul_rn(v[e], s_hi);
       const float lo = fmaf(v[e], s_lo, fmaf(v[e], s_hi, -p));
-      const float k = (p + 12582912.f) - 12582912.f;  // |p| <= 4056: the nearest integer
-      off = fmaxf(off, fabsf((p - k) + lo));
+      const float k = __fsub_rn(__fadd_rn(p, 12582912.f), 12582912.f);  // |p| <= 4056: the nearest integer
+      off = fmaxf(off, fabsf(__fadd_rn(__fsub_rn(p, k), lo)));
       v[e] = k;
     }
     store8(out + c, v);

@@ -1527,3 +1527,35 @@ def test_selection_by_column_blocks_of_the_gram_matrix(toma, tiles, th, tw):
     for b, p in sample_tiles(cfg, 4):
         want, _ = O.select_tile(tile_tokens(cfg, x, b, p).astype(np.float64), od(cfg))
         assert np.array_equal(idx[b, p], want)
+
+
+@pytest.mark.parametrize("batch,side,d", [
+    (1, 32, 72), (4, 128, 640),  # channels kept in registers, four trips of a warp
+    (2, 32, 1288),   # ... one trip at a time (few tokens, many channels)
+    (2, 64, 1032), (1, 64, 2056),  # ... eight and sixteen trips
+    (2, 64, 8),
+])
+def test_quantised_tokens_are_the_definition(toma, batch, side, d):
+    """Every channel of every quantised token (they lie at the workspace's start, a tile's behind one another) against
+    rint(x 0.99 * 4096 / |x|) in doubles, rounded to bf16.  What floats cannot tell apart - products within 2^-20 of the middle
+    between two integers - is among the tokens; what doubles cannot (2^-30, a norm summed in another order) is left out."""
+    cfg = gen.config("cfg2", batch=batch, grid_h=side, grid_w=side, tile_h=8, tile_w=8, dim=d, n_heads=d // 8, head_dim=8)
+    desc = toma.desc_from_config(cfg)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    x = torch.randn(batch, side * side, d, generator=g, device="cuda")
+    x[:, 0] = 0.0
+    x[:, 1, 1:] = 0.0
+    x[:, 2, ::3] = 2.0 ** -133  # the smallest bf16 number
+    x[:, 3:64] *= torch.exp2(torch.linspace(-110, 110, 61, device="cuda").floor())[:, None]
+    x = x.to(torch.bfloat16)
+    ws = toma.alloc_workspace(desc).fill_(255)
+    toma.toma_select(desc, x, toma.alloc_idx(desc), ws)
+    y = _regions(cfg, torch.zeros_like(x))  # shape [batch, tiles, 64, d]
+    y = ws[: x.numel() * 2].view(torch.bfloat16).double().reshape(y.shape) * 4096
+    xt = _regions(cfg, x)
+    p = xt * (0.99 * 4096 / xt.square().sum(3, keepdim=True).sqrt().clamp(min=1e-30))
+    off = ((p - p.floor()) - 0.5).abs()
+    wrong = (y != p.round().float().to(torch.bfloat16).double()) & (off > 2.0 ** -30)
+    assert not bool(wrong.any())
+    assert x.numel() < 1e7 or int((off < 2.0 ** -20).any(3).sum()) > 20
