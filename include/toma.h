@@ -118,6 +118,10 @@ TOMA_API uint64_t toma_launch_counter(void);
  *                    the library chooses */
 TOMA_API void toma_test_set_tuning(int32_t attention_split, int32_t attention_ctas, int32_t linear_tile,
                                    int32_t block_unfused);
+/* TEST-ONLY (no counterpart in the paper; host only, no device needed): the tile form, in linear_tile's numbers, that a bf16
+ * projection c_i[m][n] = a[m][k] w_i[k][n], i < n_mats, takes on a device of `sms` SMs that holds `pairs` clusters of two
+ * CTAs of its 256 x 256 form at once (0: none, that form is then never taken); 0 for arguments out of range. */
+TOMA_API int32_t toma_test_linear_form(int32_t m, int32_t n, int32_t k, int32_t n_mats, int32_t sms, int32_t pairs);
 /* TEST-ONLY (no counterpart in the paper): launches one CTA that waits, with the library's bounded wait and
  * a limit of `polls` polls (1..100000), on a barrier that nobody signals.  The wait gives up, ORs
  * TOMA_ERR_TIMEOUT's bit (bit 0) into *dev_status (device, may be NULL), writes 2 to *outcome (device, may be

@@ -19,7 +19,7 @@ TOMA_BF16, TOMA_F32 = 0, 1
 STATUS_NAMES = ["OK", "ERR_NULL", "ERR_SHAPE", "ERR_DTYPE", "ERR_RATIO", "ERR_TAU", "ERR_WORKSPACE",
                 "ERR_UNSUPPORTED", "ERR_CUDA", "ERR_TIMEOUT", "ERR_SCRATCH_LIMIT"]
 
-EXPORTS = ["toma_select_static", "toma_launch_counter", "toma_test_set_tuning", "toma_test_wait_timeout", "toma_workspace_bytes", "toma_weights_bytes", "toma_dest_per_tile", "toma_validate", "toma_status_str",
+EXPORTS = ["toma_select_static", "toma_launch_counter", "toma_test_set_tuning", "toma_test_linear_form", "toma_test_wait_timeout", "toma_workspace_bytes", "toma_weights_bytes", "toma_dest_per_tile", "toma_validate", "toma_status_str",
            "toma_select", "toma_merge_weights", "toma_merge", "toma_attention_workspace_bytes", "toma_attention_plan", "toma_attention",
            "toma_unmerge", "toma_block", "toma_block_host", "toma_linear", "toma_block_proj", "toma_attention_proj_workspace_bytes",
            "toma_attention_proj", "toma_block_mlp", "toma_mlp_workspace_bytes", "toma_mlp",
@@ -63,6 +63,8 @@ def _load() -> ctypes.CDLL:
     lib.toma_launch_counter.argtypes = []
     lib.toma_test_set_tuning.restype = None
     lib.toma_test_set_tuning.argtypes = [c_int32, c_int32, c_int32, c_int32]
+    lib.toma_test_linear_form.restype = c_int32
+    lib.toma_test_linear_form.argtypes = [c_int32] * 6
     lib.toma_test_wait_timeout.restype = c_int32
     lib.toma_test_wait_timeout.argtypes = [ctypes.c_uint32, c_void_p, c_void_p, c_void_p]
     lib.toma_validate.restype = c_int32
@@ -182,6 +184,11 @@ def toma_test_set_tuning(attention_split: int = -1, attention_ctas: int = 0, lin
     """Test-only: force the attention work plan / the projection tile form / the three-kernel block path
     (defaults restore the library's own choices)."""
     lib.toma_test_set_tuning(attention_split, attention_ctas, linear_tile, block_unfused)
+
+
+def toma_test_linear_form(m, n, k, n_mats=1, sms=148, pairs=74) -> int:
+    """Test-only: the tile form of a bf16 projection on a device of that many SMs and clusters of two (see include/toma.h)."""
+    return lib.toma_test_linear_form(m, n, k, n_mats, sms, pairs)
 
 
 def toma_test_wait_timeout(polls, dev_status, outcome) -> None:

@@ -132,6 +132,8 @@ cudaError_t launch_global_idx(const Geom& g, const int32_t* idx, int32_t* gidx, 
 // `act`: kActNone, or kActGelu to apply the exact (erf) GELU to the fp32 result before it is stored.
 constexpr int kActNone = 0, kActGelu = 1;
 bool linear_tc_shape_ok(int M, int N, int K);
+// The tile form launch_linear_tc takes on a device of `sms` SMs that holds `pairs` clusters of two at once.
+int linear_tc_form(int M, int N, int K, int n_mats, int sms, int pairs);
 cudaError_t launch_linear_tc(int M, int N, int K, const void* a, const void* const* w, void* const* c, int n_mats, int act,
                              uint32_t* dev_status, cudaStream_t s);
 cudaError_t launch_linear_simt(int M, int N, int K, bool f32, const void* a, const void* w, void* c, int act, cudaStream_t s);

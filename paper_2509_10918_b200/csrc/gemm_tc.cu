@@ -381,7 +381,53 @@ cudaError_t run_persistent(int M, int N, int K, int n_mats, const CUtensorMap& t
                           tc[0], tc[1], tc[2], M, N, K, (int)items, act, dev_status);
 }
 
+// How many pairs the device holds at once: 0 where it places no cluster of this size (asked once per device; the other forms
+// need none).
+int pairs_at_once() {
+  static std::atomic<unsigned long long> raised{0};
+  static std::atomic<int> known[64];  // per device: 0 unknown, else the answer + 1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (const int k = known[dev].load(std::memory_order_relaxed)) return k - 1;
+  int clusters = 0;
+  bool ok = raise_dynamic_smem(linear_pair_kernel, kPairSmem, raised) == cudaSuccess;
+  if (ok) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2);
+    cfg.blockDim = dim3((2 + kEpiWarps) * 32);
+    cfg.dynamicSmemBytes = kPairSmem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    ok = cudaOccupancyMaxActiveClusters(&clusters, linear_pair_kernel, &cfg) == cudaSuccess;
+  }
+  if (!ok) (void)cudaGetLastError();  // a failed query is an answer, not an error of the caller's stream
+  if (!ok || clusters < 0) clusters = 0;
+  known[dev].store(clusters + 1, std::memory_order_relaxed);
+  return clusters;
+}
+
 }  // namespace
+
+// Tile form: the one with the least serial work per SM, i.e. tiles per SM (rounded up) times the time of one, which was
+// timed on seventeen shapes between 200 x 640 x 640 and 16384 x 8192 x 4096: a tile of 128 x 192 takes 1.2 times, one of
+// 128 x 256 1.35 times as long as one of 128 x 128 (they read fewer operand bytes per multiply-add), a pair's of 256 x 256
+// 1.25 times - 1.1 from about 2048 contraction elements on - and a fifth more per launch for the cluster's start and end.
+// Returns 128 x 256 (1), 128 x 192 (2), 256 x 256 by pairs (3) or 128 x 128 (4).
+int linear_tc_form(int M, int N, int K, int n_mats, int sms, int pairs) {
+  auto cost = [&](int rows, int cols, int tile, int at_once) {
+    const long long tiles = (long long)((M + rows - 1) / rows) * ((N + cols - 1) / cols) * n_mats;
+    return (tiles + at_once - 1) / at_once * tile;
+  };
+  const long long cost128 = cost(128, 128, 20, sms), cost192 = cost(128, 192, 24, sms), cost256 = cost(128, 256, 27, sms);
+  const long long cost_pair = M > 128 && pairs > 0 ? cost(kPairRows, kPairCols, K >= 2048 ? 22 : 25, pairs) + 4 : LLONG_MAX;
+  if (cost_pair < cost128 && cost_pair < cost192 && cost_pair < cost256) return 3;
+  return cost128 <= cost192 && cost128 <= cost256 ? 4 : cost192 <= cost256 ? 2 : 1;
+}
 
 bool linear_tc_shape_ok(int M, int N, int K) { return M >= 1 && N >= 8 && K >= 8 && N % 8 == 0 && K % 8 == 0; }
 
@@ -403,28 +449,15 @@ cudaError_t launch_linear_tc(int M, int N, int K, const void* a, const void* con
     if (!encode_tmap_16bit(&tw[i], w[j], 2, wdims, wstr, wbox) || !encode_tmap_16bit(&tc_[i], c[j], 2, cdims, wstr, cbox))
       return cudaErrorInvalidValue;
   }
-  // Tile form: the one with the least serial work per SM, i.e. tiles per SM (rounded up) times the time of one, which was
-  // timed on seventeen shapes between 200 x 640 x 640 and 16384 x 8192 x 4096: a tile of 128 x 192 takes 1.2 times, one of
-  // 128 x 256 1.35 times as long as one of 128 x 128 (they read fewer operand bytes per multiply-add), a pair's of 256 x 256
-  // 1.25 times - 1.1 from about 2048 contraction elements on - and a fifth more per launch for the cluster's start and end.
-  const int sms = sm_count();
-  auto cost = [&](int rows, int cols, int tile, int at_once) {
-    const long long tiles = (long long)((M + rows - 1) / rows) * ((N + cols - 1) / cols) * n_mats;
-    return (tiles + at_once - 1) / at_once * tile;
-  };
-  const long long cost128 = cost(128, 128, 20, sms), cost192 = cost(128, 192, 24, sms), cost256 = cost(128, 256, 27, sms);
-  const long long cost_pair = M > 128 && sms >= 2 ? cost(kPairRows, kPairCols, K >= 2048 ? 22 : 25, sms / 2) + 4 : LLONG_MAX;
-  int form = cost128 <= cost192 && cost128 <= cost256 ? 4 : cost192 <= cost256 ? 2 : 1;
-  if (cost_pair < cost128 && cost_pair < cost192 && cost_pair < cost256) form = 3;
-  // test-only override: 128 x 256 (1), 128 x 192 (2), 256 x 256 (3) or 128 x 128 (4) tiles
-  if (const int v = g_tune_linear_tile.load(std::memory_order_relaxed); v && (v != 3 || M > 128)) form = v;
+  const int at_once = pairs_at_once();
+  int form = linear_tc_form(M, N, K, n_mats, sm_count(), at_once);
+  // test-only override
+  if (const int v = g_tune_linear_tile.load(std::memory_order_relaxed); v && (v != 3 || (M > 128 && at_once > 0))) form = v;
   cudaError_t e;
   if (form == 3) {
-    static std::atomic<unsigned long long> raised{0};
-    if (e = raise_dynamic_smem(linear_pair_kernel, kPairSmem, raised); e != cudaSuccess) return e;
     const long long items = (long long)((M + kPairRows - 1) / kPairRows) * ((N + kPairCols - 1) / kPairCols) * n_mats;
     if (items > INT32_MAX / 2) return cudaErrorInvalidValue;
-    const int pairs = items < sms / 2 ? (int)items : sms / 2;
+    const int pairs = items < at_once ? (int)items : at_once;
     e = launch_dependent_cluster(linear_pair_kernel, dim3(2 * pairs), dim3((2 + kEpiWarps) * 32), (size_t)kPairSmem, 2, s, ta, tw[0], tw[1], tw[2],
                                  tc_[0], tc_[1], tc_[2], M, N, K, (int)items, act, dev_status);
   } else {

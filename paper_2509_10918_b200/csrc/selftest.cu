@@ -1,4 +1,5 @@
-// Test-only entry point: makes a bounded device-side wait run out, the way every wait in the
+// Test-only entry points.  toma_test_linear_form: the projections' rule of tile forms for any device, without one.
+// toma_test_wait_timeout: makes a bounded device-side wait run out, the way every wait in the
 // tensor-core kernels would if its producer never came, and shows that the kernel then reports
 // through the status word and returns instead of hanging.
 #include "common.cuh"
@@ -25,6 +26,11 @@ __global__ void wait_that_runs_out_kernel(uint32_t polls, uint32_t* dev_status, 
 
 }  // namespace
 }  // namespace toma
+
+extern "C" int32_t toma_test_linear_form(int32_t m, int32_t n, int32_t k, int32_t n_mats, int32_t sms, int32_t pairs) {
+  if (m < 1 || n < 1 || k < 1 || n_mats < 1 || n_mats > 3 || sms < 1 || pairs < 0) return 0;
+  return toma::linear_tc_form(m, n, k, n_mats, sms, pairs);
+}
 
 extern "C" toma_status toma_test_wait_timeout(uint32_t polls, uint32_t* dev_status, uint32_t* outcome, void* stream) {
   if (polls < 1 || polls > 100000) return TOMA_ERR_SHAPE;

@@ -182,3 +182,15 @@ def test_attention_work_plan_covers_every_key_tile_once(toma, shape, split):
     else:
         assert all(x % nblk == 0 for x in b) and max(sizes) - min(sizes) <= nblk
     assert toma.toma_attention_plan(B, L, h, dh, "f32") is None
+
+
+def test_projections_take_no_pairs_where_no_cluster_can_be_placed(toma):
+    shapes = [(m, n, k, mats) for m in (1, 128, 129, 300, 4096, 16384) for n in (8, 640, 2560, 8192) for k in (8, 640, 2048, 12288) for mats in (1, 3)]
+    whole = [toma.toma_test_linear_form(*s, sms=148, pairs=74) for s in shapes]
+    assert 3 in whole and not any(f == 3 and s[0] <= 128 for f, s in zip(whole, shapes))
+    assert all(toma.toma_test_linear_form(*s, sms=148, pairs=0) in (1, 2, 4) for s in shapes)
+    # fewer at once make the form dearer, never cheaper; a part of a device has fewer SMs too
+    fewer = [toma.toma_test_linear_form(*s, sms=148, pairs=40) for s in shapes]
+    assert all(f == w for f, w in zip(fewer, whole) if w != 3 or f == 3)
+    assert all(toma.toma_test_linear_form(*s, sms=1, pairs=0) in (1, 2, 4) for s in shapes)
+    assert toma.toma_test_linear_form(0, 8, 8) == 0 and toma.toma_test_linear_form(8, 8, 8, pairs=-1) == 0
