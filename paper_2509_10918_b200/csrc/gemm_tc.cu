@@ -244,6 +244,10 @@ linear_persistent_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_
 // Both CTAs' loads count on the first one's barrier; MMA completion is committed to both.
 // ------------------------------------------------------------------------------------------------
 constexpr int kPairRows = 256, kPairCols = 256, kPairStages = 6;
+// Row blocks that are walked over together.  The 74 tiles under way then need about 8 row blocks of A and 9 column blocks of W at a
+// time, which they read in step; with all rows of A first (61 blocks and one) every k-step came out of DRAM where A is larger
+// than L2.
+constexpr int kPanel = 8;
 constexpr int kPairStageBytes = kABytes + 2 * kSlab;     // a CTA's half
 constexpr int kPairStaging = kEpiWarps * 32 * 128;
 constexpr int kPairSmem = 1024 + kPairStages * kPairStageBytes + kPairStaging + 256;
@@ -270,10 +274,13 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
   const int nk = (K + kKC - 1) / kKC;
   const int mb = (M + kPairRows - 1) / kPairRows, nb = (N + kPairCols - 1) / kPairCols;
   const int pair = blockIdx.x / 2, pairs = gridDim.x / 2;
-  // item -> row block (fastest), column block, matrix; this CTA's rows and columns of it
-  auto m_of = [&](int item) { return item % mb * kPairRows; };
-  auto n_of = [&](int item) { return item / mb % nb * kPairCols; };
-  auto z_of = [&](int item) { return item / mb / nb; };
+  // item -> matrix, panel of kPanel row blocks, column block, row block (fastest)
+  auto place = [&](int item, int& m0, int& n0, int& z) {
+    z = item / (mb * nb);
+    const int in_z = item - z * mb * nb, first = in_z / (kPanel * nb) * kPanel, in_panel = in_z - first * nb, rows = min(kPanel, mb - first);
+    n0 = in_panel / rows * kPairCols;
+    m0 = (first + in_panel % rows) * kPairRows;
+  };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kPairStages; ++s) {
@@ -305,7 +312,9 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
       int kc = 0;  // k-steps so far, over all items: ring slot and phase follow it
       bool ok = true;
       for (int item = pair; ok && item < n_items; item += pairs) {
-        const int m0 = m_of(item) + rank * 128, n0 = n_of(item) + rank * 128, z = z_of(item);
+        int m0, n0, z;
+        place(item, m0, n0, z);
+        m0 += rank * 128, n0 += rank * 128;  // this CTA's rows and columns
         const CUtensorMap* tm_w = z == 0 ? &tm_w0 : z == 1 ? &tm_w1 : &tm_w2;
         for (int k = 0; k < nk; ++k, ++kc) {
           const int s = kc % kPairStages;
@@ -347,7 +356,10 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
     uint8_t* mine = staging + (warp - 2) * 4096;
     int n = 0;
     for (int item = pair; item < n_items; item += pairs, ++n) {
-      const int a = n & 1, m0 = m_of(item) + rank * 128 + quarter * 32, n0 = n_of(item), z = z_of(item), slabs = (min(kPairCols, N - n0) + 63) / 64;
+      int m0, n0, z;
+      place(item, m0, n0, z);
+      m0 += rank * 128 + quarter * 32;
+      const int a = n & 1, slabs = (min(kPairCols, N - n0) + 63) / 64;
       const CUtensorMap* tm_c = z == 0 ? &tm_c0 : z == 1 ? &tm_c1 : &tm_c2;
       // one answer per warp: the tensor-memory loads below are warp-wide operations
       if (!__all_sync(0xffffffffu, mbar_wait(&bar->acc_full[a], (n >> 1) & 1, dev_status, abort_flag))) break;
