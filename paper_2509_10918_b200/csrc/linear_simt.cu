@@ -6,6 +6,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "spread.cuh"
 #include "tc.cuh"
 
 namespace toma {
@@ -288,8 +289,9 @@ struct UnmergeOp {
 template <class Op, int BM, int BN, int TM, int TN>
 static void run_tile(const Op& op, int batches, cudaStream_t s) {
   const dim3 grid((op.N + BN - 1) / BN, (op.M + BM - 1) / BM, batches);
-  launch_dependent(simt_gemm_kernel<Op, BM, BN, TM, TN>, grid, dim3((BM / TM) * (BN / TN)), 0, s, op);  // errors: cudaGetLastError
+  static SpreadState state;
   count_launch();
+  launch_spread(simt_gemm_kernel<Op, BM, BN, TM, TN>, state, true, grid, dim3((BM / TM) * (BN / TN)), 2 * kBK * (BM + BN) * 4, 0, s, op);  // errors: cudaGetLastError
 }
 
 // Tile form: the least work on the fullest SM, padding included.  A larger tile reads its operands less often per
@@ -361,11 +363,11 @@ __global__ void __launch_bounds__(kSoftThreads) softmax_dest_kernel(float* __res
     for (int i = warp; i < Dloc; i += kWarps) L[(size_t)i * Nloc] = e_smem[i * kSoftTok + lane] * inv;
   }
 }
-// The same without shared memory for more destinations than it holds (global merge): one thread per source token.
+// The same without shared memory for more destinations than it holds (global merge): one thread per source token.  Neither placed
+// beside its predecessor's last CTAs nor beside its successor's first: its few CTAs, which wait for memory most of the
+// time, then crowd on the SMs that come free first (2 x 4416 tokens of 256 channels, the weights as a whole 1357 -> 1610 us).
 __global__ void __launch_bounds__(128) softmax_dest_long_kernel(float* __restrict__ logits, int Nloc, int Dloc) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  tc::dependency_wait();
-  if (threadIdx.x == 0) tc::release_dependents();
   if (k >= Nloc) return;
   float* L = logits + (size_t)blockIdx.y * Dloc * Nloc + k;
   float mx = -INFINITY;
@@ -534,11 +536,10 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) logits_kernel(const Log
 
 template <int BM, int BN, int TM, int TN>
 static cudaError_t run_logits(const LogitsOp<__nv_bfloat16>& op, int batches, cudaStream_t s) {
-  static std::atomic<unsigned long long> raised{0};
-  if (cudaError_t e = raise_dynamic_smem(logits_kernel<BM, BN, TM, TN>, logit_smem<BM, BN>(), raised); e != cudaSuccess) return e;
+  static SpreadState state;
   const dim3 grid((op.N + BN - 1) / BN, (op.M + BM - 1) / BM, batches);
   count_launch();
-  return launch_dependent(logits_kernel<BM, BN, TM, TN>, grid, dim3((BM / TM) * (BN / TN)), logit_smem<BM, BN>(), s, op);
+  return launch_spread(logits_kernel<BM, BN, TM, TN>, state, false, grid, dim3((BM / TM) * (BN / TN)), 0, logit_smem<BM, BN>(), s, op);
 }
 // The same of fp32 tokens, summed in double (the order of addition does not show in the fp32 result).  Their way into double
 // is the bound where there is enough to do (eight conversions, at a quarter of the rate, for sixteen multiply-adds); few and
@@ -643,11 +644,10 @@ __global__ void __launch_bounds__(BM / 4 * (BN / 4) * KG) logits64_kernel(const 
 
 template <int BM, int BN, int KG>
 static cudaError_t run_logits64(const LogitsOp<float>& op, int batches, cudaStream_t s) {
-  static std::atomic<unsigned long long> raised{0};
-  if (cudaError_t e = raise_dynamic_smem(logits64_kernel<BM, BN, KG>, logit64_smem<BM, BN, KG>(), raised); e != cudaSuccess) return e;
+  static SpreadState state;
   const dim3 grid((op.N + BN - 1) / BN, (op.M + BM - 1) / BM, batches);
   count_launch();
-  return launch_dependent(logits64_kernel<BM, BN, KG>, grid, dim3(BM / 4 * (BN / 4) * KG), logit64_smem<BM, BN, KG>(), s, op);
+  return launch_spread(logits64_kernel<BM, BN, KG>, state, false, grid, dim3(BM / 4 * (BN / 4) * KG), 0, logit64_smem<BM, BN, KG>(), s, op);
 }
 // Timed on thirteen shapes (microseconds per tile and 640 channels on the fullest SM): 16 x 16 takes 3.2 among many; 64 x 64
 // takes 44, one or two of them 90, and wins where every SM has several.  The weights as a whole (with logits in stages of 16
@@ -686,11 +686,12 @@ cudaError_t launch_weights_simt(const Geom& g, const void* x, const int32_t* idx
   }
   const size_t smem = (size_t)g.Dloc * kSoftTok * 4;
   if (smem <= 200 * 1024) {
-    static std::atomic<unsigned long long> raised{0};
-    if ((e = raise_dynamic_smem(softmax_dest_kernel, 200 * 1024, raised)) != cudaSuccess) return e;
-    e = launch_dependent(softmax_dest_kernel, dim3((g.Nloc + kSoftTok - 1) / kSoftTok, batches), dim3(kSoftThreads), smem, s, logits, g.Nloc, g.Dloc);
+    static SpreadState state;
+    e = launch_spread(softmax_dest_kernel, state, false, dim3((g.Nloc + kSoftTok - 1) / kSoftTok, batches), dim3(kSoftThreads), kSoftThreads * 4, (int)smem, s, logits,
+                      g.Nloc, g.Dloc);
   } else {
-    e = launch_dependent(softmax_dest_long_kernel, dim3((g.Nloc + 127) / 128, batches), dim3(128), 0, s, logits, g.Nloc, g.Dloc);
+    softmax_dest_long_kernel<<<dim3((g.Nloc + 127) / 128, batches), 128, 0, s>>>(logits, g.Nloc, g.Dloc);
+    e = cudaGetLastError();
   }
   if (e != cudaSuccess) return e;
   count_launch();
@@ -699,8 +700,10 @@ cudaError_t launch_weights_simt(const Geom& g, const void* x, const int32_t* idx
   int row_parts = 1;
   while (row_parts < 8 && (long long)blocks * batches * row_parts < sm_count() && row_parts * 256 < g.Nloc) row_parts *= 2;
   const dim3 grid(blocks, batches, row_parts);
-  e = g.f32 ? launch_dependent(rownorm_kernel<float>, grid, dim3(256), 0, s, logits, (float*)w, (float*)wu, g.Nloc, g.Dloc)
-            : launch_dependent(rownorm_kernel<__nv_bfloat16>, grid, dim3(256), 0, s, logits, (__nv_bfloat16*)w, (__nv_bfloat16*)wu, g.Nloc, g.Dloc);
+  static SpreadState state_f, state_h;
+  constexpr int kRowSmem = (32 + 8 * 32 * 33) * 4;
+  e = g.f32 ? launch_spread(rownorm_kernel<float>, state_f, false, grid, dim3(256), kRowSmem, 0, s, logits, (float*)w, (float*)wu, g.Nloc, g.Dloc)
+            : launch_spread(rownorm_kernel<__nv_bfloat16>, state_h, false, grid, dim3(256), kRowSmem, 0, s, logits, (__nv_bfloat16*)w, (__nv_bfloat16*)wu, g.Nloc, g.Dloc);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -1559,3 +1559,16 @@ def test_quantised_tokens_are_the_definition(toma, batch, side, d):
     wrong = (y != p.round().float().to(torch.bfloat16).double()) & (off > 2.0 ** -30)
     assert not bool(wrong.any())
     assert x.numel() < 1e7 or int((off < 2.0 ** -20).any(3).sum()) > 20
+
+
+@pytest.mark.parametrize("m,n,k", [(373, 4608, 64), (1750, 704, 40), (105, 2304, 72), (64, 64, 8), (1300, 1100, 20)])
+def test_ffma_projection_on_an_evenly_filled_chip(toma, m, n, k):
+    """Three CTAs per SM where four fit (the launch asks for shared memory that it does not use), one, one in all."""
+    rng = np.random.default_rng(m)
+    a = torch.from_numpy(rng.standard_normal((m, k)).astype(np.float32)).cuda()
+    w = torch.from_numpy((rng.standard_normal((k, n)) / np.sqrt(k)).astype(np.float32)).cuda()
+    c = torch.full((m, n), float("nan"), device="cuda")
+    for _ in range(3):
+        toma.toma_linear(a, w, c)
+    # a chain of k products of about 1 / sqrt(k): k 2^-24 of their sum of magnitudes, sqrt(k)
+    assert float((c.double() - a.double() @ w.double()).abs().max()) <= 2 * k ** 1.5 * 2.0 ** -24
