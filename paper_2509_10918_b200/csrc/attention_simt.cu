@@ -9,12 +9,15 @@
 // registers (row maxima and sums by shuffles within the sixteen lanes) and pass through shared memory once, between
 // lanes of one half warp.  Bound by the FMA pipe where there are queries enough to fill it (16 warps per SM).  Where there are
 // not, the four warps of 32 queries wait for their own latencies - 10 heads x 512 tokens x 64 channels, fp32: 46 us, 9 of
-// them multiply-adds -, and so three or four groups of warps share the queries, each with every third or fourth key tile, a
+// them multiply-adds -, and so two to four groups of warps share the queries, each with every second to fourth key tile, a
 // reference and sums of its own, added up at the end (KG): 28 us.  512 tokens of 20 heads of 128 223 -> 206, bound by reads of
 // shared memory, as are all (2.8 cycles for each of them, eight for 32 packed multiply-adds).
 #include <float.h>
 
+#include <type_traits>
+
 #include "common.cuh"
+#include "spread.cuh"
 #include "tc.cuh"
 
 namespace toma {
@@ -73,9 +76,15 @@ __global__ void __launch_bounds__(BQ * 4 * KG) attention_simt_kernel(const T* __
     }
   };
   auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
-  auto load_tile = [&](int k0, int st) {
-    load_one(Ks + st * C::kTile, k, k0);
-    load_one(Vs + st * C::kTile, v, k0);
+  auto load_tile = [&](int k0, int st) {  // (in one loop: bf16 packets pass through registers, and so twice as many are on their way)
+#pragma unroll 4
+    for (int e = tid; e < kKeys * (DH / 4); e += kThreads) {
+      const int r = e / (DH / 4), c = (e % (DH / 4)) * 4, dst = st * C::kTile + r * C::kPitch + c;
+      const bool in = k0 + r < L;
+      const size_t off = base + (size_t)(in ? k0 + r : 0) * row_stride + c;
+      copy16(Ks + dst, k + off, in);
+      copy16(Vs + dst, v + off, in);
+    }
     commit();
   };
   auto group_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(kThreads) : "memory"); };
@@ -83,6 +92,9 @@ __global__ void __launch_bounds__(BQ * 4 * KG) attention_simt_kernel(const T* __
   if (threadIdx.x == 0) tc::release_dependents();
   if constexpr (KG == 1) {
     load_tile(0, 0);
+  } else if constexpr (sizeof(T) == 2) {
+    load_tile(group * kKeys, 0);
+    commit();
   } else {
     load_one(Ks, k, group * kKeys);
     commit();
@@ -93,9 +105,10 @@ __global__ void __launch_bounds__(BQ * 4 * KG) attention_simt_kernel(const T* __
     const int r = e / DH, c = e % DH;
     Qs[r * C::kPitch + c] = q0 + r < L ? to_f32(q[base + (size_t)(q0 + r) * row_stride + c]) * scale : 0.f;
   }
-  // outputs of two channels in a register pair (one for DV = 1: the second of the pair is not used)
+  // outputs of two channels in a register pair; a single one (DV = 1) in a register
   constexpr int kPairs = (DV + 1) / 2;
-  uint64_t acc[4][kPairs] = {};
+  using Acc = std::conditional_t<DV == 1, float, uint64_t>;
+  Acc acc[4][kPairs] = {};
   float m[4], l[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) m[i] = KG > 1 ? -FLT_MAX : -INFINITY, l[i] = 0.f;  // one group's keys may all be at -infinity
@@ -167,7 +180,10 @@ __global__ void __launch_bounds__(BQ * 4 * KG) attention_simt_kernel(const T* __
       }
       l[i] = l[i] * corr + sum;  // this lane's keys; the sixteen lanes' sums meet at the end
 #pragma unroll
-      for (int c = 0; c < kPairs; ++c) acc[i][c] = tc::mul2(acc[i][c], tc::pack2(corr, corr));
+      for (int c = 0; c < kPairs; ++c) {
+        if constexpr (DV == 1) acc[i][c] *= corr;
+        else acc[i][c] = tc::mul2(acc[i][c], tc::pack2(corr, corr));
+      }
     }
     if constexpr (KG > 1) {
       group_sync();  // K has been read
@@ -187,7 +203,7 @@ __global__ void __launch_bounds__(BQ * 4 * KG) attention_simt_kernel(const T* __
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const float* vr = Vt + (kk + u) * C::kPitch;
-        uint64_t vv[kPairs];  // channels tx DV .. (DV <= 4), or tx 4 .. and 64 + tx 4 ..
+        Acc vv[kPairs];  // channels tx DV .. (DV <= 4), or tx 4 .. and 64 + tx 4 ..
         if constexpr (DV >= 4) {
 #pragma unroll
           for (int g = 0; g < DV / 4; ++g) {
@@ -197,14 +213,16 @@ __global__ void __launch_bounds__(BQ * 4 * KG) attention_simt_kernel(const T* __
         } else if constexpr (DV == 2) {
           vv[0] = *reinterpret_cast<const uint64_t*>(vr + tx * 2);
         } else {
-          vv[0] = tc::pack2(vr[tx], 0.f);
+          vv[0] = vr[tx];
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float pu = u == 0 ? p[i].x : u == 1 ? p[i].y : u == 2 ? p[i].z : p[i].w;
-          const uint64_t p2 = tc::pack2(pu, pu);
 #pragma unroll
-          for (int c = 0; c < kPairs; ++c) acc[i][c] = tc::fma2(p2, vv[c], acc[i][c]);
+          for (int c = 0; c < kPairs; ++c) {
+            if constexpr (DV == 1) acc[i][c] = fmaf(pu, vv[c], acc[i][c]);
+            else acc[i][c] = tc::fma2(tc::pack2(pu, pu), vv[c], acc[i][c]);
+          }
         }
       }
     }
@@ -220,7 +238,10 @@ __global__ void __launch_bounds__(BQ * 4 * KG) attention_simt_kernel(const T* __
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int c = 0; c < kPairs; ++c) tc::unpack2(acc[i][c], out[i][2 * c], out[i][2 * c + 1]);
+    for (int c = 0; c < kPairs; ++c) {
+      if constexpr (DV == 1) out[i][c] = acc[i][c];
+      else tc::unpack2(acc[i][c], out[i][2 * c], out[i][2 * c + 1]);
+    }
   if constexpr (KG > 1) {
     // the groups' outputs and sums, to where their tiles were, and from there into one
     asm volatile("cp.async.wait_group 0;" ::: "memory");  // a group without a tile has fetched zeros
@@ -277,28 +298,35 @@ __global__ void __launch_bounds__(BQ * 4 * KG) attention_simt_kernel(const T* __
 template <typename T, int DH, int BQ, int KG>
 cudaError_t run_one(int B, int L, int heads, const void* q, const void* k, const void* v, void* o, cudaStream_t s) {
   using C = SimtCfg<DH, BQ, KG>;
-  static std::atomic<unsigned long long> raised{0};
-  if (cudaError_t e = raise_dynamic_smem(attention_simt_kernel<T, DH, BQ, KG>, (int)C::kSmem, raised); e != cudaSuccess) return e;
+  static SpreadState state;
   const dim3 grid((L + BQ - 1) / BQ, heads, B);
   count_launch();
-  return launch_dependent(attention_simt_kernel<T, DH, BQ, KG>, grid, dim3(BQ * 4 * KG), C::kSmem, s, (const T*)q, (const T*)k, (const T*)v, (T*)o, L,
-                          heads, 1.0f / sqrtf((float)DH));
+  return launch_spread(attention_simt_kernel<T, DH, BQ, KG>, state, false, grid, dim3(BQ * 4 * KG), 0, (int)C::kSmem, s, (const T*)q, (const T*)k, (const T*)v,
+                       (T*)o, L, heads, 1.0f / sqrtf((float)DH));
 }
 
 template <typename T, int DH>
 cudaError_t run(int B, int L, int heads, const void* q, const void* k, const void* v, void* o, cudaStream_t s) {
-  // 64 queries per CTA read K and V half as often and two CTAs fill an SM.  Where that would not give every SM two CTAs, 32 or
-  // 40, one CTA per SM, their keys dealt out to as many groups of warps as shared memory and registers hold: whichever leaves
-  // the fullest SM fewer queries (512 tokens of 10 heads are 160 CTAs of 32 on 148 SMs, and 130 of 40).
-  const long long ctas64 = (long long)((L + 63) / 64) * heads * B;
-  if (ctas64 >= 2LL * sm_count()) return run_one<T, DH, 64, 1>(B, L, heads, q, k, v, o, s);
-  auto fullest = [&](int bq) { return ((long long)((L + bq - 1) / bq) * heads * B + sm_count() - 1) / sm_count() * bq; };
+  // Queries per CTA and groups of warps that share them, timed in all forms on 270 shapes, 32 to 1200 tokens, 0.05 to 24 CTAs of 32
+  // queries per SM (us; fp32 unless said otherwise).
+  auto per_sm = [&](int bq) { return (double)((long long)((L + bq - 1) / bq) * heads * B) / sm_count(); };
   if constexpr (DH == 128) {
-    // bound by shared-memory reads, and two groups would not have a second K and V: one group, 64 queries where the fullest SM
-    // has no more of them so (3 x 300 tokens, 7 heads: 60 us with 32, 46 with 64)
-    return fullest(64) <= fullest(32) ? run_one<T, DH, 64, 1>(B, L, heads, q, k, v, o, s) : run_one<T, DH, 32, 1>(B, L, heads, q, k, v, o, s);
+    // Bound by shared-memory reads, and two groups would not have a second K and V: one group.  64 queries read K and V half as
+    // often: two CTAs of them per SM, or where the fullest SM has no more queries with them (3 x 300 tokens, 7 heads: 60
+    // with 32, 46 with 64).
+    const bool wide = per_sm(64) >= 2 || ceil(per_sm(64)) * 64 <= ceil(per_sm(32)) * 32;
+    return wide ? run_one<T, DH, 64, 1>(B, L, heads, q, k, v, o, s) : run_one<T, DH, 32, 1>(B, L, heads, q, k, v, o, s);
   } else {
-    return fullest(40) < fullest(32) ? run_one<T, DH, 40, 3>(B, L, heads, q, k, v, o, s) : run_one<T, DH, 32, 4>(B, L, heads, q, k, v, o, s);
+    // Groups hide latencies while an SM has one CTA: four (head_dim 64, 260 tokens: 18.8 with one group, 15.6 with four), or
+    // three with 40 queries where 32 would leave a second CTA to some SMs (705 tokens, 0.85 per SM: 59 and 37).  With
+    // more CTAs two groups (606 tokens of head_dim 64, 2.3 CTAs of 64 queries per SM: 64 queries 133, 32 in one group 131,
+    // in two 115, in four 129).  Below head_dim 64 there is too little to a key tile for that to pay in the long run: two groups
+    // for four tiles and two CTAs per SM at most, else one (head_dim 16, 450 tokens, 3.65 per SM: one 30.9, two 31.4, three 37.4).
+    if (per_sm(32) <= 1) return run_one<T, DH, 32, 4>(B, L, heads, q, k, v, o, s);
+    if (per_sm(40) <= 1) return run_one<T, DH, 40, 3>(B, L, heads, q, k, v, o, s);
+    if constexpr (DH < 64)
+      if (L > 4 * kKeys || per_sm(32) > 2) return run_one<T, DH, 32, 1>(B, L, heads, q, k, v, o, s);
+    return run_one<T, DH, 32, 2>(B, L, heads, q, k, v, o, s);
   }
 }
 
