@@ -227,20 +227,21 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
 }
 
 // ------------------------------------------------------------------------------------------------
-// merge with destinations on M: X_m [D_loc x ch] = A~ [D_loc x N_loc] * X [N_loc x ch], for up to four CTAs per SM.
+// merge with destinations on M: X_m [D_loc x ch] = A~ [D_loc x N_loc] * X [N_loc x ch], for launches that the SMs hold at once
+// and a little beyond (see launch_merge_tc).
 // One CTA = (128 destinations, 128 channels); both operands MN-major as they lie in memory.  The same bytes and products per
 // CTA as with channels on M, but a thread then owns an output row and stages 16 bytes at a time where the other form stages 2:
 // the epilogue was 2.3 us of a launch of 8 (32 tiles of 256 tokens, 128 destinations, 640 channels).
-// A block of 64 destinations or fewer loads one slab of a weight plane: the rows of the product that the other one would have
-// made are made of whatever lies there, and not stored.
+// A block of 64 destinations or fewer loads one slab of a weight plane (and with no more destinations in the region a stage has
+// room for no more): the rows of the product that the other one would have made are made of whatever lies there, and not stored.
 // ------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kRowsThreads, 2)
 merge_rows_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                   const __grid_constant__ CUtensorMap tm_o, const LinParams p, uint32_t* dev_status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  constexpr int kStage = 6 * kSlab;  // two planes of two slabs of weights, two slabs of tokens
-  PipeBars* bar = reinterpret_cast<PipeBars*>(smem + p.stages * kStage);
+  const int w_bytes = p.Dloc > 64 ? 2 * kSlab : kSlab, stage_bytes = 2 * w_bytes + 2 * kSlab;  // two planes of weights, two slabs of tokens
+  PipeBars* bar = reinterpret_cast<PipeBars*>(smem + p.stages * stage_bytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int batch = blockIdx.x, c0 = blockIdx.y * 128, i_base = blockIdx.z * 128;
   const int w_slabs = p.Dloc - i_base > 64 ? 2 : 1, x_slabs = p.d - c0 > 64 ? 2 : 1;
@@ -258,12 +259,12 @@ merge_rows_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   // k-step k of the operands into its stage
   auto load = [&](int k) {
     const int s = k % p.stages;
-    uint8_t* sw = smem + s * kStage;
-    uint8_t* sx = sw + 4 * kSlab;
+    uint8_t* sw = smem + s * stage_bytes;
+    uint8_t* sx = sw + 2 * w_bytes;
     mbar_expect_tx(&bar->full[s], (2 * w_slabs + x_slabs) * kSlab);
     for (int pl = 0; pl < 2; ++pl)
       for (int c = 0; c < w_slabs; ++c)
-        tma_load_3d(sw + (2 * pl + c) * kSlab, &tm_w, &bar->full[s], i_base + c * 64, k * kKC, 2 * batch + pl);
+        tma_load_3d(sw + pl * w_bytes + c * kSlab, &tm_w, &bar->full[s], i_base + c * 64, k * kKC, 2 * batch + pl);
     for (int c = 0; c < x_slabs; ++c)
       tma_load_4d(sx + c * kSlab, &tm_x, &bar->full[s], c0 + c * 64, tx * p.tw, ty * p.th + k * rows_per_chunk, b);
   };
@@ -303,12 +304,12 @@ merge_rows_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         const int s = k % p.stages;
         if (!mbar_wait(&bar->full[s], (k / p.stages) & 1, dev_status, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t wa = smem_u32(smem + s * kStage), xa = wa + 4 * kSlab;
+        const uint32_t wa = smem_u32(smem + s * stage_bytes), xa = wa + 2 * w_bytes;
 #pragma unroll
         for (int kk = 0; kk < kKC / 16; ++kk) {  // 16 tokens per MMA: 16 rows of 128 B in every slab
           const uint64_t xd = smem_desc_sw128(xa + kk * 2048, kSlab, 1024);
           mma_ss(tmem, smem_desc_sw128(wa + kk * 2048, kSlab, 1024), xd, idesc, k > 0 || kk > 0);
-          mma_ss(tmem, smem_desc_sw128(wa + 2 * kSlab + kk * 2048, kSlab, 1024), xd, idesc, true);
+          mma_ss(tmem, smem_desc_sw128(wa + w_bytes + kk * 2048, kSlab, 1024), xd, idesc, true);
         }
         mma_commit(&bar->empty[s]);
       }
@@ -930,19 +931,27 @@ cudaError_t launch_merge_tc(const Geom& g, const void* w, const void* x, void* x
   const int smem = 1024 + p.stages * stage_bytes + 256;
   dim3 grid(g.B * g.P, (g.d + 127) / 128, (g.Dloc + p.dest_block - 1) / p.dest_block);
   cudaError_t e;
-  // Destinations on M as long as an SM has up to four of its CTAs, two at a time: 16 tiles of 256 tokens, 128 destinations, 3072
-  // channels (2.6) 13.5 us one CTA per SM walking over the items, 12.2 so; at 3.9 16.3 and 14.4, at 4.3 18.6 and 18.4, at 8.7
-  // 31.6 and 36.2; 192 destinations, two blocks of which read the tokens twice, at 5.2 15.7 and 17.3.
+  // Destinations on M while the SMs hold all CTAs at once, two each.  With more, one CTA per SM that walks over the items keeps its
+  // ring filled where these start anew, and wins the more the longer they are.  Timed over 64 to 1024 tokens, 16 to 256
+  // destinations and 0.3 to 4.5 CTAs per SM, this form's time over the other's: up to 2 per SM 0.55 to 1.07 (4 us and 16
+  // destinations).  2.3 to 3.9 per SM, up to 128 destinations: 64 tokens 0.88 to 1.02, 128 tokens 0.76 to 1.0 (1.07 with 16 or 32
+  // destinations from 3.3 on), 256 tokens 0.92 to 1.2, 512 and 1024 tokens 0.97 to 1.3; more than 128, two blocks of
+  // them, 0.68 to 0.98 (1.13 in one place).  4.5 per SM: 0.94 to 1.3.
   const dim3 rgrid(g.B * g.P, (g.d + 127) / 128, (g.Dloc + 127) / 128);
-  if (g.Dloc <= kMaxCols && (long long)rgrid.x * rgrid.y * rgrid.z <= 4LL * sm_count()) {
+  const long long rctas = (long long)rgrid.x * rgrid.y * rgrid.z, sms = sm_count();
+  const bool at_once = rctas <= 2 * sms, few = rctas <= 4 * sms, brief = g.Nloc <= 2 * kKC && (g.Dloc >= 64 || rctas <= 3 * sms);
+  if (g.Dloc <= kMaxCols && (at_once || (few && (brief || g.Dloc > 128)))) {
     const uint32_t rbox[4] = {64, 32, 1, 1};  // a warp's 32 destinations
     if (!encode_tmap_16bit(&to, xm, 4, odims, ostrides, rbox)) return cudaErrorInvalidValue;
-    constexpr int kStage = 6 * kSlab;
-    p.stages = g.Nloc / kKC < 2 ? g.Nloc / kKC : 2;  // two CTAs per SM hide each other's latencies
+    const int rstage = (g.Dloc > 64 ? 6 : 4) * kSlab;
+    // two CTAs per SM hide each other's latencies, one alone has a deeper ring
+    p.stages = (rctas <= sms ? 200 * 1024 : 100 * 1024) / rstage;
+    p.stages = p.stages > 4 ? 4 : p.stages;
+    if (p.stages > g.Nloc / kKC) p.stages = g.Nloc / kKC;
     if (copied_beside(rows, rgrid.x * rgrid.y * rgrid.z * kRowsCopyThreads)) p.extra = rows;
     static std::atomic<unsigned long long> raised_m{0};
-    if (e = raise_dynamic_smem(merge_rows_kernel, 1024 + 2 * kStage + 256, raised_m); e != cudaSuccess) return e;
-    e = launch_dependent(merge_rows_kernel, rgrid, dim3(kRowsThreads), (size_t)(1024 + p.stages * kStage + 256), s, tx, tw, to, p, dev_status);
+    if (e = raise_dynamic_smem(merge_rows_kernel, 202 * 1024, raised_m); e != cudaSuccess) return e;
+    e = launch_dependent(merge_rows_kernel, rgrid, dim3(kRowsThreads), (size_t)(1024 + p.stages * rstage + 256), s, tx, tw, to, p, dev_status);
     return finish_launch(e, rows, p.extra, s);
   }
   const int n_chunks = (g.d + 127) / 128, n_blocks = (g.Dloc + p.dest_block - 1) / p.dest_block, n_items = g.B * g.P * n_blocks * n_chunks;
