@@ -68,7 +68,7 @@ __device__ __forceinline__ double widen(float v) {
   return __hiloint2double((int)(((b & 0x7FFFFFFFu) >> 3) + 0x38000000u), 0);  // without the sign: it is squared
 }
 // kTrips > 0: the warp's trips over the token's channels, all on their way before the first is used and kept in registers for
-// the products.  0: one at a time, read twice.  False: not this way.
+// the products.  0: one at a time, read twice.  False: not this way.  (quantise_kernel, kTrips < 0: never this way.)
 template <int kTrips>
 __device__ __forceinline__ bool quantise_fast(const __nv_bfloat16* row, __nv_bfloat16* out, int d, int lane) {
   double ss = 0.0;
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(256) quantise_kernel(const T* __restrict__ x, 
   const int l = (yy % th) * tw + xx % tw;
   const T* row = x + ((size_t)b * n_all + n) * d;
   __nv_bfloat16* out = y + ((size_t)(b * P + p) * Nloc + l) * d;
-  if constexpr (sizeof(T) == 2) {
+  if constexpr (sizeof(T) == 2 && kTrips >= 0) {
     if (quantise_fast<kTrips>(row, out, d, lane)) return;
   }
   quantise_f64(row, out, d, lane);
@@ -154,12 +154,16 @@ cudaError_t launch_quantise(const Geom& g, const void* x, __nv_bfloat16* y, cuda
     return launch_dependent(kernel, dim3(blocks), dim3(256), 0, s, tokens, y, g.B, g.N, (int)g.tokens_all(), g.d, g.W, g.th, g.tw, g.tiles_x, g.P, g.Nloc);
   };
   // Channels kept in registers: 4096 tokens of 3072 channels 6 us less, 2 x 4096 of 640 1.5 less.  Where a warp runs once, the long
-  // straight code of more than four trips costs more than that gains (2048 tokens of 1280 channels: 1 us).
+  // straight code of more than four trips costs more than that gains (2048 tokens of 1280 channels: 1 us), and where an SM has
+  // one CTA the fp64 pipe is not the bound and the definition's short code is through first (selection of 1024 tokens of 1088
+  // channels 21.5 us, 22.3 by floats; of 672 of 1280 17.1 and 17.7; of 2048 of 1280 24.4 and 24.1).
   const __nv_bfloat16* h = (const __nv_bfloat16*)x;
-  const bool once = warps <= 16LL * sm_count();
-  const cudaError_t e = g.f32 ? launch(quantise_kernel<float, 0>, (const float*)x)
+  const bool few = warps <= 8LL * sm_count(), once = warps <= 16LL * sm_count();
+  static_assert(kMaxDim <= 16 * 256, "sixteen trips hold a token's channels");
+  const cudaError_t e = g.f32 ? launch(quantise_kernel<float, -1>, (const float*)x)
+                        : few ? launch(quantise_kernel<__nv_bfloat16, -1>, h)
                         : g.d <= 1024 ? launch(quantise_kernel<__nv_bfloat16, 4>, h)
-                        : once || g.d > 4096 ? launch(quantise_kernel<__nv_bfloat16, 0>, h)
+                        : once ? launch(quantise_kernel<__nv_bfloat16, 0>, h)
                         : g.d <= 2048 ? launch(quantise_kernel<__nv_bfloat16, 8>, h) : launch(quantise_kernel<__nv_bfloat16, 16>, h);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();

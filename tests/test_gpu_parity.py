@@ -2231,7 +2231,8 @@ def test_selection_by_column_blocks_of_the_gram_matrix(toma, tiles, th, tw):
 
 
 @pytest.mark.parametrize("batch,side,d", [
-    (1, 32, 72), (4, 128, 640),  # channels kept in registers, four trips of a warp
+    (1, 32, 72),     # few tokens: by the definition in doubles
+    (4, 128, 640),   # by pairs of floats: channels kept in registers, four trips of a warp
     (2, 32, 1288),   # ... one trip at a time (few tokens, many channels)
     (2, 64, 1032), (1, 64, 2056),  # ... eight and sixteen trips
     (2, 64, 8),
