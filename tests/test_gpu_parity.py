@@ -1498,7 +1498,7 @@ def test_ffma_attention_of_keys_at_minus_infinity(toma):
 
 @pytest.mark.parametrize("batch,gy,gx,th,tw,dim,ratio", [
     (8, 4, 4, 16, 16, 40, 0.5),   # logits in tiles of 64 x 64, many per SM; a last stage of 8 channels
-    (4, 6, 6, 19, 15, 32, 0.5),   # ... partial in both directions; one stage
+    (8, 4, 4, 15, 16, 32, 0.5),   # ... partial in both directions (120 destinations, 240 tokens); one stage
     (1, 1, 1, 1, 1, 8, 0.0),      # 16 x 16: one token
     (2, 2, 3, 7, 5, 264, 0.5),    # ... 35 tokens, 17 destinations
     (1, 1, 2, 16, 3, 320, 0.65),  # ... more stages than the ring holds; one tile of destinations, three of tokens
