@@ -47,10 +47,17 @@ struct SimtCfg {
   static constexpr int kTile = kKeys * kPitch;
   static constexpr int kPPitch = kKeys + 4;
   static constexpr int kBufs = KG == 1 ? 2 : 1;
+  static constexpr bool kByTile = KG <= 2 && BQ == 32;
   static constexpr int kGroup = 2 * kBufs * kTile + BQ * kPPitch;
   static constexpr size_t kSmem = ((size_t)BQ * kPitch + (size_t)KG * kGroup) * 4;
   static_assert(BQ * DH <= kTile && 2 * BQ <= kPPitch * BQ, "a group's outputs and sums fit where its tiles were");
 };
+
+template <bool kSecond, typename A>
+__device__ __forceinline__ A& select_sum(A& first, A& second) {
+  if constexpr (kSecond) return second;
+  else return first;
+}
 
 template <typename T, int DH, int BQ, int KG>
 __global__ void __launch_bounds__(BQ * 4 * KG) attention_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
@@ -76,14 +83,19 @@ __global__ void __launch_bounds__(BQ * 4 * KG) attention_simt_kernel(const T* __
     }
   };
   auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
-  auto load_tile = [&](int k0, int st) {  // (in one loop: bf16 packets pass through registers, and so twice as many are on their way)
+  auto load_tile = [&](int k0, int st) {
+    if constexpr (sizeof(T) == 4) {
+      load_one(Ks + st * C::kTile, k, k0);
+      load_one(Vs + st * C::kTile, v, k0);
+    } else {  // bf16 packets pass through registers: in one loop twice as many are on their way
 #pragma unroll 4
-    for (int e = tid; e < kKeys * (DH / 4); e += kThreads) {
-      const int r = e / (DH / 4), c = (e % (DH / 4)) * 4, dst = st * C::kTile + r * C::kPitch + c;
-      const bool in = k0 + r < L;
-      const size_t off = base + (size_t)(in ? k0 + r : 0) * row_stride + c;
-      copy16(Ks + dst, k + off, in);
-      copy16(Vs + dst, v + off, in);
+      for (int e = tid; e < kKeys * (DH / 4); e += kThreads) {
+        const int r = e / (DH / 4), c = (e % (DH / 4)) * 4, dst = st * C::kTile + r * C::kPitch + c;
+        const bool in = k0 + r < L;
+        const size_t off = base + (size_t)(in ? k0 + r : 0) * row_stride + c;
+        copy16(Ks + dst, k + off, in);
+        copy16(Vs + dst, v + off, in);
+      }
     }
     commit();
   };
@@ -194,6 +206,11 @@ __global__ void __launch_bounds__(BQ * 4 * KG) attention_simt_kernel(const T* __
     } else {
       __syncwarp();  // a row's probabilities are written and read by the same half warp
     }
+    // One or two groups with 32 queries: a tile's outputs are summed by themselves and added to the others'.  Chains of 64 keys and one
+    // of tiles, instead of one of a group's keys, take a third off the error of an output, so that fewer groups (longer
+    // chains) lose nothing against four; a query's registers have no room for it with more threads to an SM.
+    [[maybe_unused]] Acc part[4][kPairs] = {};
+    Acc(&sum)[4][kPairs] = select_sum<C::kByTile>(acc, part);
     const float* Vt = Vs + st * C::kTile;
 #pragma unroll 4
     for (int kk = 0; kk < kKeys; kk += 4) {
@@ -220,11 +237,20 @@ __global__ void __launch_bounds__(BQ * 4 * KG) attention_simt_kernel(const T* __
           const float pu = u == 0 ? p[i].x : u == 1 ? p[i].y : u == 2 ? p[i].z : p[i].w;
 #pragma unroll
           for (int c = 0; c < kPairs; ++c) {
-            if constexpr (DV == 1) acc[i][c] = fmaf(pu, vv[c], acc[i][c]);
-            else acc[i][c] = tc::fma2(tc::pack2(pu, pu), vv[c], acc[i][c]);
+            if constexpr (DV == 1) sum[i][c] = fmaf(pu, vv[c], sum[i][c]);
+            else sum[i][c] = tc::fma2(tc::pack2(pu, pu), vv[c], sum[i][c]);
           }
         }
       }
+    }
+    if constexpr (C::kByTile) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int c = 0; c < kPairs; ++c) {
+          if constexpr (DV == 1) acc[i][c] += part[i][c];
+          else acc[i][c] = tc::add2(acc[i][c], part[i][c]);
+        }
     }
     if constexpr (KG > 1) {
       group_sync();  // V and the probabilities have been read
@@ -307,23 +333,24 @@ cudaError_t run_one(int B, int L, int heads, const void* q, const void* k, const
 
 template <typename T, int DH>
 cudaError_t run(int B, int L, int heads, const void* q, const void* k, const void* v, void* o, cudaStream_t s) {
-  // Queries per CTA and groups of warps that share them, timed in all forms on 270 shapes, 32 to 1200 tokens, 0.05 to 24 CTAs of 32
-  // queries per SM (us; fp32 unless said otherwise).
+  // Queries per CTA and groups of warps that share them, timed in all forms on 300 shapes, 32 to 2300 tokens, 0.05 to 27 CTAs of 32
+  // queries per SM (us; fp32).  64 queries read K and V half as often: from two CTAs of them per SM on, which fill it.
   auto per_sm = [&](int bq) { return (double)((long long)((L + bq - 1) / bq) * heads * B) / sm_count(); };
+  if (per_sm(64) >= 2) return run_one<T, DH, 64, 1>(B, L, heads, q, k, v, o, s);
   if constexpr (DH == 128) {
-    // Bound by shared-memory reads, and two groups would not have a second K and V: one group.  64 queries read K and V half as
-    // often: two CTAs of them per SM, or where the fullest SM has no more queries with them (3 x 300 tokens, 7 heads: 60
-    // with 32, 46 with 64).
-    const bool wide = per_sm(64) >= 2 || ceil(per_sm(64)) * 64 <= ceil(per_sm(32)) * 32;
+    // bound by shared-memory reads, and two groups would not have a second K and V: one group, 64 queries where the fullest SM
+    // has no more of them so (3 x 300 tokens, 7 heads: 60 with 32, 46 with 64)
+    const bool wide = ceil(per_sm(64)) * 64 <= ceil(per_sm(32)) * 32;
     return wide ? run_one<T, DH, 64, 1>(B, L, heads, q, k, v, o, s) : run_one<T, DH, 32, 1>(B, L, heads, q, k, v, o, s);
   } else {
     // Groups hide latencies while an SM has one CTA: four (head_dim 64, 260 tokens: 18.8 with one group, 15.6 with four), or
-    // three with 40 queries where 32 would leave a second CTA to some SMs (705 tokens, 0.85 per SM: 59 and 37).  With
-    // more CTAs two groups (606 tokens of head_dim 64, 2.3 CTAs of 64 queries per SM: 64 queries 133, 32 in one group 131,
-    // in two 115, in four 129).  Below head_dim 64 there is too little to a key tile for that to pay in the long run: two groups
-    // for four tiles and two CTAs per SM at most, else one (head_dim 16, 450 tokens, 3.65 per SM: one 30.9, two 31.4, three 37.4).
+    // three with 40 queries where 32 would leave one more CTA to some SMs (705 tokens, 0.85 per SM: 59 and 37; 2271 tokens, 1.95
+    // per SM: 198, two groups of 32 235; not at head_dim 16, 386 tokens, 1.55 per SM: 23.6, one group of 32 22.2).  With more
+    // CTAs two groups (652 tokens, 2.7 of 32 queries per SM: one 92, two 79, four 85).  Below head_dim 64 there is too little to a key tile
+    // for that to pay in the long run: two groups for four tiles and two CTAs per SM at most, else one (head_dim 16,
+    // 450 tokens, 3.65 per SM: one 30.9, two 31.4, three 37.4).
     if (per_sm(32) <= 1) return run_one<T, DH, 32, 4>(B, L, heads, q, k, v, o, s);
-    if (per_sm(40) <= 1) return run_one<T, DH, 40, 3>(B, L, heads, q, k, v, o, s);
+    if (per_sm(40) <= 1 || (DH > 16 && per_sm(32) > 2 && per_sm(40) <= 2)) return run_one<T, DH, 40, 3>(B, L, heads, q, k, v, o, s);
     if constexpr (DH < 64)
       if (L > 4 * kKeys || per_sm(32) > 2) return run_one<T, DH, 32, 1>(B, L, heads, q, k, v, o, s);
     return run_one<T, DH, 32, 2>(B, L, heads, q, k, v, o, s);

@@ -1591,7 +1591,8 @@ def test_ffma_projection_on_an_evenly_filled_chip(toma, m, n, k):
     ("f32", 4, 200, 10, 32), ("bf16", 4, 200, 10, 16),  # two groups of warps: four key tiles, up to two CTAs per SM
     ("f32", 3, 300, 12, 16), ("bf16", 2, 700, 12, 32),  # one group: more of either
     ("bf16", 1, 600, 9, 16), ("f32", 1, 600, 9, 32),    # three groups of 40 queries
-    ("f32", 4, 65, 24, 64), ("f32", 4, 1, 24, 64),      # two groups at head_dim 64, one of them without a key tile
+    ("f32", 4, 65, 24, 64), ("f32", 8, 1, 24, 64),      # two groups at head_dim 64, one of them without a key tile
+    ("f32", 1, 1000, 10, 64),                           # three groups of 40 queries, two CTAs after another
 ])
 def test_ffma_attention_of_every_form(toma, dtype, B, L, h, dh):
     test_ffma_attention_with_its_keys_dealt_out(toma, dtype, B, L, h, dh)
