@@ -268,7 +268,7 @@ merge_rows_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     for (int c = 0; c < x_slabs; ++c)
       tma_load_4d(sx + c * kSlab, &tm_x, &bar->full[s], c0 + c * 64, tx * p.tw, ty * p.th + k * rows_per_chunk, b);
   };
-  const int early = min(nk, p.stages);
+  const int early = min(min(nk, p.stages), 2);  // (more than that delays the others: 0.3 us of 4.1 for 8 regions of 256 tokens, 256 channels)
   dependency_wait();
   if (threadIdx.x == 0) release_dependents();
   if (warp == 0) {
@@ -292,7 +292,7 @@ merge_rows_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   if (warp == 0) {
     if (elect_one()) {
       for (int k = early; k < nk; ++k) {
-        if (!mbar_wait(&bar->empty[k % p.stages], ((k / p.stages) - 1) & 1, dev_status, abort_flag)) break;
+        if (k >= p.stages && !mbar_wait(&bar->empty[k % p.stages], ((k / p.stages) - 1) & 1, dev_status, abort_flag)) break;
         load(k);
       }
     }
