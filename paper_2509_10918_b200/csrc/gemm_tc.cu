@@ -244,10 +244,11 @@ linear_persistent_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_
 // Both CTAs' loads count on the first one's barrier; MMA completion is committed to both.
 // ------------------------------------------------------------------------------------------------
 constexpr int kPairRows = 256, kPairCols = 256, kPairStages = 6;
-// Row blocks that are walked over together.  The 74 tiles under way then need about 8 row blocks of A and 9 column blocks of W at a
-// time, which they read in step; with all rows of A first (61 blocks and one) every k-step came out of DRAM where A is larger
-// than L2.
-constexpr int kPanel = 8;
+// Row blocks that are walked over together.  The 74 tiles under way then need 12 row blocks of A and six or seven column blocks
+// of W at a time, which they read in step; with all rows of A first (61 blocks and one) every k-step came out of DRAM where A is
+// larger than L2.  Panels of 4 to 16 timed on 23 shapes: 12 takes 0.95 to 1.0 of the time of all rows first (1.01 once), 8 and 16 up
+// to 1 and 2 % more than 12.
+constexpr int kPanel = 12;
 constexpr int kPairStageBytes = kABytes + 2 * kSlab;     // a CTA's half
 constexpr int kPairStaging = kEpiWarps * 32 * 128;
 constexpr int kPairSmem = 1024 + kPairStages * kPairStageBytes + kPairStaging + 256;
