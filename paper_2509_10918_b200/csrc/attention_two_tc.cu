@@ -132,10 +132,12 @@ __device__ __forceinline__ void flush_slab(const OutStage& os, int lane, int ch0
   if (lane == 0 && row0 < L) {
     tma_store_3d(os.tm_o, os.stage, ch0, row0, b);
     tma_store_commit();
-    // The slab may be staged again, and the block may end.  (Waited for here: at the slab's next use and at the block's end 0.1 to
-    // 0.5 us of 20 more - 636 tokens of 11 heads of 64 channels 21.1 -> 21.4, 428 of 8 of 128 33.7 -> 33.9 -, a span having few pieces.)
-    tma_store_wait_read();
   }
+}
+// Before the slab is staged again, and before the block ends.  (Units kept whole: 170 tokens of 15 heads of 64 channels 7.6 us waiting
+// right behind the store, 7.3 so.  Pieces are stored at a span's end, and wait there: 636 tokens of 11 heads 21.1 and 21.4.)
+__device__ __forceinline__ void staging_free(int lane) {
+  if (lane == 0) tma_store_wait_read();
   __syncwarp();
 }
 // End of a piece that covers all keys of its unit (the only kind when units are kept whole), run by
@@ -162,6 +164,7 @@ __device__ __forceinline__ void finish_whole(const Row& t, Barriers* bar, int un
     uint32_t r[32];
     tmem_ld32(t.ob + c * 32, r);
     tmem_wait_ld();
+    if (!(c & 1)) staging_free(t.lane);
     stage_half(os, t.lane, c & 1, r, inv);
     if (c & 1) flush_slab(os, t.lane, ch0 + (c >> 1) * 64, row0, b, L);
   }
@@ -272,8 +275,12 @@ __device__ __noinline__ void finish_partial(Row t, Barriers* bar, Piece p, int p
             r[4 * q + e] = __float_as_uint(own_first ? fmaf(w_o, vv[e], w_own * own) : fmaf(w_own, own, w_o * vv[e]));
           }
         }
+        if (c == 0) staging_free(lane);
         stage_quarter(os, t.lane, c & 3, r, inv);
-        if ((c & 3) == 3) flush_slab(os, t.lane, ch0 + (c >> 2) * 64, row0, b_item, L);
+        if ((c & 3) == 3) {
+          flush_slab(os, t.lane, ch0 + (c >> 2) * 64, row0, b_item, L);
+          staging_free(lane);
+        }
       }
     } else {
 #pragma unroll
@@ -305,8 +312,12 @@ __device__ __noinline__ void finish_partial(Row t, Barriers* bar, Piece p, int p
             r[4 * q + e] = __float_as_uint(own_first ? fmaf(w_o, vv[e], w_own * own) : fmaf(w_own, own, w_o * vv[e]));
           }
         }
+        if (c == 0) staging_free(lane);
         stage_half(os, t.lane, c & 1, r, inv);
-        if (c & 1) flush_slab(os, t.lane, ch0 + (c >> 1) * 64, row0, b_item, L);
+        if (c & 1) {
+          flush_slab(os, t.lane, ch0 + (c >> 1) * 64, row0, b_item, L);
+          staging_free(lane);
+        }
       } else {
         to_scratch(c, r);
       }
@@ -598,6 +609,7 @@ attention_two_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
       else finish_partial<DH>(t, bar, p, pc, it >= it_end, m_used, l, o, &tm_o, L, heads, sp, tickets, pieces, dev_status);
     }
     settle_first_piece<DH>(bar, it_begin, it_end, t, o, L, heads, sp, pieces, dev_status);
+    staging_free(lane);  // shared memory must outlive the engine's reads
   }
   tc_fence_before();
   __syncthreads();
