@@ -46,29 +46,21 @@ struct Spans {
 };
 
 // What the ends of a CTA's span need of the plan, in shared memory: at the end of a piece the parameter memory is cold, and
-// its reads, one behind the other, cost a microsecond.  Where units are cut, lanes 0 and 1 of a warp with nothing else to do fill
-// this in while the first tiles are on their way (in front of the setup's barrier the same microsecond was the launch's: 636 tokens
-// of 11 heads of 64 channels 21.5 -> 22.5 us).
+// its reads, one behind the other, cost a microsecond.  Filled in by lanes 0 and 1 of a warp at the start.
 struct Edges {
-  uint64_t ready;    // filled in (one arrival)
   int lo[2], hi[2];  // lowest and highest CTA with key tiles of the unit the span starts in, and of the one it ends in
   int first_unit;    // the unit the span starts in
   int other_slot;    // scratch slot of the last unit's other contributor, where it has one
-  // Whole warp.
   __device__ __forceinline__ void fill(const Spans& sp, int it_begin, int it_end, int lane) {
-    if (lane < 2) {
-      const int u = (lane ? it_end - 1 : it_begin) / sp.nblk;
-      lo[lane] = sp.unit_lo[lane][blockIdx.x];
-      hi[lane] = sp.unit_hi[lane][blockIdx.x];
-      if (lane == 0) {
-        first_unit = u;
-      } else {  // a CTA's first piece sits in slot 0 of its two, a later partial piece in slot 1
-        const int g = lo[1] == (int)blockIdx.x ? hi[1] : lo[1];
-        other_slot = 2 * g + (u > sp.bound(g) / sp.nblk ? 1 : 0);
-      }
+    const int u = (lane ? it_end - 1 : it_begin) / sp.nblk;
+    lo[lane] = sp.unit_lo[lane][blockIdx.x];
+    hi[lane] = sp.unit_hi[lane][blockIdx.x];
+    if (lane == 0) {
+      first_unit = u;
+    } else {  // a CTA's first piece sits in slot 0 of its two, a later partial piece in slot 1
+      const int g = lo[1] == (int)blockIdx.x ? hi[1] : lo[1];
+      other_slot = 2 * g + (u > sp.bound(g) / sp.nblk ? 1 : 0);
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&ready);
   }
 };
 

@@ -219,7 +219,6 @@ __device__ __noinline__ bool finish_partial(Row t, Barriers* bar, Piece p, int p
   const int row = t.row, lane = t.lane, c0 = t.half * (DH / 2);
   uint32_t* ticket = tickets + (size_t)p.u * kTicketCols + t.warp;
   // a partial piece lies in the unit the span starts in or in the one it ends in
-  if (!mbar_wait_warp(&bar->edge.ready, 0, dev_status, &bar->abort_flag)) return false;  // (it has been for long)
   const int which = p.u == bar->edge.first_unit ? 0 : 1;
   const int g_first = bar->edge.lo[which], g_last = bar->edge.hi[which];
   bool own_first = false;  // this CTA is the lower of the two contributors
@@ -408,11 +407,11 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     }
     mbar_init(&bar->pub_ready, kSoftWarps);
     mbar_init(&bar->pub_done, 1);
-    mbar_init(&bar->edge.ready, 1);
     bar->others_done = 0;
     bar->abort_flag = 0;
     mbar_fence_init();
   }
+  if (warp == kSoftWarps + 3 && lane < 2) bar->edge.fill(sp, it_begin, it_end, lane);
   if (threadIdx.x == kSoftWarps * 32) {  // descriptor fetches overlap the previous kernel's tail
     prefetch_tmap(&tm_q);
     prefetch_tmap(&tm_k);
@@ -560,8 +559,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         }
       }
     }
-  } else if (warp == kSoftWarps + 3) {
-    if (sp.split) bar->edge.fill(sp, it_begin, it_end, lane);
   } else if (warp < kSoftWarps) {
     // ------------------------------------------------------------------ softmax / epilogue
     Row t;

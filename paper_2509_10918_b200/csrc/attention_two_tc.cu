@@ -134,8 +134,7 @@ __device__ __forceinline__ void flush_slab(const OutStage& os, int lane, int ch0
     tma_store_commit();
   }
 }
-// Before the slab is staged again, and before the block ends.  (Units kept whole: 170 tokens of 15 heads of 64 channels 7.6 us waiting
-// right behind the store, 7.3 so.  Pieces are stored at a span's end, and wait there: 636 tokens of 11 heads 21.1 and 21.4.)
+// Before the slab is staged again, and before the block ends.
 __device__ __forceinline__ void staging_free(int lane) {
   if (lane == 0) tma_store_wait_read();
   __syncwarp();
@@ -194,7 +193,6 @@ __device__ __noinline__ void finish_partial(Row t, Barriers* bar, Piece p, int p
   const int row = t.row, lane = t.lane;
   uint32_t* ticket = tickets + (size_t)p.u * kTicketCols + t.warp;
   // a partial piece lies in the unit the span starts in or in the one it ends in
-  if (!mbar_wait_warp(&bar->edge.ready, 0, dev_status, &bar->abort_flag)) return;  // (it has been for long)
   const int which = p.u == bar->edge.first_unit ? 0 : 1;
   const int g_first = bar->edge.lo[which], g_last = bar->edge.hi[which];
   bool own_first = false;  // this CTA is the lower of the two contributors
@@ -275,12 +273,9 @@ __device__ __noinline__ void finish_partial(Row t, Barriers* bar, Piece p, int p
             r[4 * q + e] = __float_as_uint(own_first ? fmaf(w_o, vv[e], w_own * own) : fmaf(w_own, own, w_o * vv[e]));
           }
         }
-        if (c == 0) staging_free(lane);
+        if ((c & 3) == 0) staging_free(lane);
         stage_quarter(os, t.lane, c & 3, r, inv);
-        if ((c & 3) == 3) {
-          flush_slab(os, t.lane, ch0 + (c >> 2) * 64, row0, b_item, L);
-          staging_free(lane);
-        }
+        if ((c & 3) == 3) flush_slab(os, t.lane, ch0 + (c >> 2) * 64, row0, b_item, L);
       }
     } else {
 #pragma unroll
@@ -312,12 +307,9 @@ __device__ __noinline__ void finish_partial(Row t, Barriers* bar, Piece p, int p
             r[4 * q + e] = __float_as_uint(own_first ? fmaf(w_o, vv[e], w_own * own) : fmaf(w_own, own, w_o * vv[e]));
           }
         }
-        if (c == 0) staging_free(lane);
+        if (!(c & 1)) staging_free(lane);
         stage_half(os, t.lane, c & 1, r, inv);
-        if (c & 1) {
-          flush_slab(os, t.lane, ch0 + (c >> 1) * 64, row0, b_item, L);
-          staging_free(lane);
-        }
+        if (c & 1) flush_slab(os, t.lane, ch0 + (c >> 1) * 64, row0, b_item, L);
       } else {
         to_scratch(c, r);
       }
@@ -403,7 +395,6 @@ attention_two_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     }
     mbar_init(&bar->pub_ready, 8);
     mbar_init(&bar->pub_done, 1);
-    mbar_init(&bar->edge.ready, 1);
     bar->others_done = 0;
     bar->abort_flag = 0;
     mbar_fence_init();
@@ -418,6 +409,7 @@ attention_two_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     prefetch_tmap(&tm_v);
     prefetch_tmap(&tm_o);
   }
+  if (warp == 10 && lane < 2) bar->edge.fill(sp, it_begin, it_end, lane);
   dependency_wait();
   if (threadIdx.x == 0) release_dependents();
   if (warp == 9) tmem_alloc(&bar->tmem_base, C::kTmemCols);
@@ -544,7 +536,6 @@ attention_two_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     }
   } else if (warp == 10) {
     // ------------------------------------------------------------------ publisher
-    if (sp.split) bar->edge.fill(sp, it_begin, it_end, lane);
     if (lane == 0) {
       // When the span's first piece is partial and more pieces follow, make that piece
       // visible to the other CTAs and draw its eight tickets here, off the softmax warps' path.

@@ -937,12 +937,15 @@ cudaError_t launch_merge_tc(const Geom& g, const void* w, const void* x, void* x
   // destinations).  2.3 to 3.9 per SM, up to 128 destinations: 64 tokens 0.88 to 1.02, 128 tokens 0.76 to 1.0 (1.07 with 16 or 32
   // destinations from 3.3 on), 256 tokens 0.92 to 1.2, 512 and 1024 tokens 0.97 to 1.3; more than 128, two blocks of
   // them, 0.68 to 0.98 (1.13 in one place).  4.5 per SM: 0.94 to 1.3.  256 tokens and 128 destinations come out in front from 3.2 on
-  // (0.92 to 0.95), where the other form has a fourth item on some SMs.
+  // (0.92 to 0.95), where the other form has a fourth item on some SMs, and so does any region with many text tokens: the four
+  // warps that store the items copy them first (16 regions of 256 tokens, 128 destinations, 3072 channels, 512 text tokens: a step of
+  // 120.4 us walked, 117.2 so; without text tokens 14.0 and 14.1 for the merge).
   const dim3 rgrid(g.B * g.P, (g.d + 127) / 128, (g.Dloc + 127) / 128);
   const long long rctas = (long long)rgrid.x * rgrid.y * rgrid.z, sms = sm_count();
   const bool at_once = rctas <= 2 * sms, few = rctas <= 4 * sms, brief = g.Nloc <= kKC || (g.Nloc <= 2 * kKC && (g.Dloc >= 64 || rctas <= 3 * sms));
   const bool even = g.Dloc > 64 && g.Nloc <= 4 * kKC && rctas > 3 * sms;  // two full waves of two against four items per SM
-  if (g.Dloc <= kMaxCols && (at_once || (few && (brief || even || g.Dloc > 128)))) {
+  const bool copies = (long long)rows.per * rows.batches > 4 * sms * kCopyThreads;
+  if (g.Dloc <= kMaxCols && (at_once || (few && (brief || even || copies || g.Dloc > 128)))) {
     const uint32_t rbox[4] = {64, 32, 1, 1};  // a warp's 32 destinations
     if (!encode_tmap_16bit(&to, xm, 4, odims, ostrides, rbox)) return cudaErrorInvalidValue;
     const int rstage = (g.Dloc > 64 ? 6 : 4) * kSlab;
