@@ -542,7 +542,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         mbar_arrive(&bar->pub_done);
       }
       // When the span ends inside a unit that one other CTA shares, that CTA ran its part at the
-      // start of its span and has normally published it long since.  Watch its tickets (acquire)
+      // start of its span and has normally published it long since.  Watch its tickets (plain loads, one fence behind them)
       // and leave the answer in shared memory for the softmax warps: they add the two pieces up
       // straight from tensor memory if the answer is there when their last piece ends, and go
       // through scratch and tickets otherwise.  Polling keeps the ticket out of their registers.

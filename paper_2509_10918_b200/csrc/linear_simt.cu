@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kSoftThreads) softmax_dest_kernel(float* __res
 }
 // The same without shared memory for more destinations than it holds (global merge): one thread per source token.  Neither placed
 // beside its predecessor's last CTAs nor beside its successor's first: its few CTAs, which wait for memory most of the
-// time, then crowd on the SMs that come free first (2 x 4416 tokens of 256 channels, the weights as a whole 1357 -> 1610 us).
+// time, then crowd on the SMs that come free first (2 x 4416 tokens of 256 channels, the weights as a whole 1399 -> 1505 us, now 1373).
 __global__ void __launch_bounds__(128) softmax_dest_long_kernel(float* __restrict__ logits, int Nloc, int Dloc) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= Nloc) return;
@@ -435,9 +435,9 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const float* __restrict__ 
   }
 }
 
-// Logits of bf16 tokens, <X[idx_i], X_k> * scale, every sum one chain of fused multiply-adds in ascending channels: the same
-// bits as the general kernel above gives.  What bounds it is the FMA pipe (a product is 2 N_loc D_loc d operations of the
-// 75 TFLOP/s it has) as long as operands keep coming, and the general kernel's did not: its stages of 16 channels, one
+// Logits of bf16 tokens, <X[idx_i], X_k> * scale, every sum one chain of fused multiply-adds in ascending channels, whatever the
+// tile form.  What bounds it is the FMA pipe (a product is 2 N_loc D_loc d operations of the
+// 75 TFLOP/s it has) as long as operands keep coming, and those of the general kernel above, which made them once, did not: its stages of 16 channels, one
 // ahead, cover a third of a load's latency, and it converts and transposes them on the way.  Here the rows travel as they
 // are, by cp.async, kStages - 1 stages of 64 channels ahead, and are widened in registers as they are read (a shift or a mask,
 // on the ALU pipe beside the FMAs).  Rows lie 144 bytes apart, so that eight threads read eight rows' 16 bytes at once.
@@ -541,7 +541,8 @@ static cudaError_t run_logits(const LogitsOp<__nv_bfloat16>& op, int batches, cu
   count_launch();
   return launch_spread(logits_kernel<BM, BN, TM, TN>, state, false, grid, dim3((BM / TM) * (BN / TN)), 0, logit_smem<BM, BN>(), s, op);
 }
-// The same of fp32 tokens, summed in double (the order of addition does not show in the fp32 result).  Their way into double
+// The same of fp32 tokens, summed in double: one chain with 64 x 64 tiles, eight with 16 x 16, so that a logit within some
+// 2^-50 of the middle between two fp32 numbers may round either way with the form, which depends on the number of regions.  Their way into double
 // is the bound where there is enough to do (eight conversions, at a quarter of the rate, for sixteen multiply-adds); few and
 // small regions wait for loads instead, and so KG groups of threads share a tile, each with every KG-th four channels of a
 // stage of 32, and add up through shared memory at the end.  Thread = 4 x 4 outputs.

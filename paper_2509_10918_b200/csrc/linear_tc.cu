@@ -22,7 +22,7 @@ constexpr int kKC = 64;           // contraction elements per pipeline stage
 constexpr int kSlab = kKC * 128;  // bytes of a 64-row x 128-byte slab
 constexpr int kMaxCols = 256;     // output columns (MMA N) per merge CTA
 constexpr int kUnmergeTok = 128;  // tokens per unmerge CTA: small enough that two CTAs share an SM
-constexpr int kRowsEpiWarps = 8, kRowsThreads = (2 + kRowsEpiWarps) * 32;  // of the kernels with tokens on M
+constexpr int kRowsEpiWarps = 8, kRowsThreads = (2 + kRowsEpiWarps) * 32;  // of the kernels with tokens or destinations on M
 
 struct PipeBars {
   uint64_t full[4], empty[4], done;
@@ -601,7 +601,7 @@ unmerge_tc_kernel(const __grid_constant__ CUtensorMap tm_y, const __grid_constan
 // 4.2 MFLOP, the weights are read twice instead of five times, and the 128 CTAs of the 64x64-token
 // case fit the SMs in one wave with a three-stage pipeline; each thread then owns a token row, which it
 // stages in shared memory (the pipeline's stages, free by then) as 64-channel slabs in the layout of the
-// output tensor map's box: the CTA's 128 tokens are whole tile rows, one TMA store per slab.
+// output tensor map's box: a warp's 32 tokens are whole tile rows (or half of one of 64), one TMA store per warp and slab.
 // ------------------------------------------------------------------------------------------------
 constexpr int kRowsChBlock = 320;  // channels per CTA (five 64-channel slabs)
 

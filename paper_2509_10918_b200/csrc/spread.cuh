@@ -2,7 +2,7 @@
 //
 // CTAs of a dependent launch (launch_dependent()) are placed while the predecessor's retire, all that fit on the first SM that
 // comes free.  432 CTAs of a kernel four of which fit an SM came to lie four on some SMs and two on others instead of three on
-// each (fp32 projection of 373 x 4608 x 1152: 126 us so, 100 us evenly; of 1750 x 704 x 704 79 and 62), 18 of a softmax on five
+// each (fp32 projection of 373 x 4608 x 1152: 126 us so, 100 us evenly; of 1750 x 704 x 704 79 and 62), 18 of a softmax on a few
 // SMs (fp32 weights of a region of 572 tokens, 384 channels: 43 and 34).  So a launch asks for as much shared memory as
 // makes an SM hold no more of its CTAs than an even distribution gives it.  Not where it follows its like and fits beside it: nothing
 // is uneven then, and an SM of its own for every CTA costs (projection of 103 x 2304 x 2304, 144 CTAs: 93 us, 101 so).

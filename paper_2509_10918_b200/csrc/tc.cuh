@@ -1,7 +1,8 @@
 // sm_100a building blocks used by the tensor-core kernels: mbarriers with bounded
 // waits, TMA (cp.async.bulk.tensor) loads and stores, tensor-memory allocation and
 // tcgen05 MMA / load / store wrappers, and the shared-memory / instruction descriptors.
-// Every TMA load in this library is issued by the CTA that consumes it.
+// Every TMA load in this library is issued by the CTA into whose shared memory it goes (a pair of CTAs multiplies what both
+// have loaded, and the bytes of both count on the first one's barrier: tma_load_2d_pair).
 #pragma once
 
 #include <cuda.h>
