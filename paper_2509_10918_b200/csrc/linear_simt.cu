@@ -363,26 +363,49 @@ __global__ void __launch_bounds__(kSoftThreads) softmax_dest_kernel(float* __res
     for (int i = warp; i < Dloc; i += kWarps) L[(size_t)i * Nloc] = e_smem[i * kSoftTok + lane] * inv;
   }
 }
-// The same without shared memory for more destinations than it holds (global merge): one thread per source token.  Neither placed
-// beside its predecessor's last CTAs nor beside its successor's first: its few CTAs, which wait for memory most of the
-// time, then crowd on the SMs that come free first (2 x 4416 tokens of 256 channels, the weights as a whole 1399 -> 1505 us, now 1373).
-__global__ void __launch_bounds__(128) softmax_dest_long_kernel(float* __restrict__ logits, int Nloc, int Dloc) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= Nloc) return;
-  float* L = logits + (size_t)blockIdx.y * Dloc * Nloc + k;
+// The same for more destinations than shared memory holds (global merge): the exponentials stay where the logits were.  The same
+// sums in the same order.  (One thread per source token took three passes of its own over them: a millisecond of latencies in
+// 30 to 90 CTAs, whose time depended on where a dependent launch had placed them - 2 x 4416 tokens of 256 channels, the weights
+// as a whole 1407 us launched by itself, 1615 behind its predecessor; 3528 tokens of 640 channels 1461 and 1200.)
+__global__ void __launch_bounds__(kSoftThreads) softmax_dest_long_kernel(float* __restrict__ logits, int Nloc, int Dloc) {
+  __shared__ float red[kSoftThreads / 32][kSoftTok];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = blockIdx.x * kSoftTok + lane;
+  constexpr int kWarps = kSoftThreads / 32;
+  const bool live = k < Nloc;
+  tc::dependency_wait();
+  if (threadIdx.x == 0) tc::release_dependents();
+  float* L = logits + (size_t)blockIdx.y * Dloc * Nloc + (live ? k : 0);
   float mx = -INFINITY;
 #pragma unroll 8
-  for (int i = 0; i < Dloc; ++i) mx = fmaxf(mx, L[(size_t)i * Nloc]);
-  float sum = 0.f;
+  for (int i = warp; i < Dloc; i += kWarps) mx = fmaxf(mx, L[(size_t)i * Nloc]);
+  red[warp][lane] = mx;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) mx = fmaxf(mx, red[w][lane]);
+  if (live) {
 #pragma unroll 8
-  for (int i = 0; i < Dloc; ++i) {
-    const float e = expf(L[(size_t)i * Nloc] - mx);
-    L[(size_t)i * Nloc] = e;
-    sum += e;
+    for (int i = warp; i < Dloc; i += kWarps) L[(size_t)i * Nloc] = expf(L[(size_t)i * Nloc] - mx);
   }
-  const float inv = 1.f / sum;
+  __syncthreads();  // the block's exponentials are in memory, and red has been read
+  if (warp == 0 && live) {
+    float sum = 0.f;
+    int i = 0;
+    for (; i + 32 <= Dloc; i += 32) {  // 32 loads on their way, added up in destination order
+      float e[32];
+#pragma unroll
+      for (int u = 0; u < 32; ++u) e[u] = L[(size_t)(i + u) * Nloc];
+#pragma unroll
+      for (int u = 0; u < 32; ++u) sum += e[u];
+    }
+    for (; i < Dloc; ++i) sum += L[(size_t)i * Nloc];
+    red[0][lane] = 1.f / sum;
+  }
+  __syncthreads();
+  const float inv = red[0][lane];
+  if (live) {
 #pragma unroll 8
-  for (int i = 0; i < Dloc; ++i) L[(size_t)i * Nloc] *= inv;
+    for (int i = warp; i < Dloc; i += kWarps) L[(size_t)i * Nloc] *= inv;
+  }
 }
 
 // Row normalisation of 32 destinations of a region: A~^T[k][i] = A_ik / sum_k' A_ik' and, when wu is given, the shares
@@ -691,8 +714,9 @@ cudaError_t launch_weights_simt(const Geom& g, const void* x, const int32_t* idx
     e = launch_spread(softmax_dest_kernel, state, false, dim3((g.Nloc + kSoftTok - 1) / kSoftTok, batches), dim3(kSoftThreads), kSoftThreads * 4, (int)smem, s, logits,
                       g.Nloc, g.Dloc);
   } else {
-    softmax_dest_long_kernel<<<dim3((g.Nloc + 127) / 128, batches), 128, 0, s>>>(logits, g.Nloc, g.Dloc);
-    e = cudaGetLastError();
+    static SpreadState state;
+    e = launch_spread(softmax_dest_long_kernel, state, false, dim3((g.Nloc + kSoftTok - 1) / kSoftTok, batches), dim3(kSoftThreads), kSoftThreads * 4, 0, s,
+                      logits, g.Nloc, g.Dloc);
   }
   if (e != cudaSuccess) return e;
   count_launch();
@@ -701,10 +725,10 @@ cudaError_t launch_weights_simt(const Geom& g, const void* x, const int32_t* idx
   int row_parts = 1;
   while (row_parts < 8 && (long long)blocks * batches * row_parts < sm_count() && row_parts * 256 < g.Nloc) row_parts *= 2;
   const dim3 grid(blocks, batches, row_parts);
-  static SpreadState state_f, state_h;
-  constexpr int kRowSmem = (32 + 8 * 32 * 33) * 4;
-  e = g.f32 ? launch_spread(rownorm_kernel<float>, state_f, false, grid, dim3(256), kRowSmem, 0, s, logits, (float*)w, (float*)wu, g.Nloc, g.Dloc)
-            : launch_spread(rownorm_kernel<__nv_bfloat16>, state_h, false, grid, dim3(256), kRowSmem, 0, s, logits, (__nv_bfloat16*)w, (__nv_bfloat16*)wu, g.Nloc, g.Dloc);
+  // (Not spread: what counts is that its CTAs are there when the softmax ends.  21 regions of 264 tokens, 1536 channels: 100 us for the
+  // weights as a whole, 137 spread.)
+  e = g.f32 ? launch_dependent(rownorm_kernel<float>, grid, dim3(256), 0, s, logits, (float*)w, (float*)wu, g.Nloc, g.Dloc)
+            : launch_dependent(rownorm_kernel<__nv_bfloat16>, grid, dim3(256), 0, s, logits, (__nv_bfloat16*)w, (__nv_bfloat16*)wu, g.Nloc, g.Dloc);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -1609,3 +1609,23 @@ def test_ffma_attention_of_every_form(toma, dtype, B, L, h, dh):
 ])
 def test_merge_by_ctas_per_sm(toma, th, tw, ratio, dim, batch):
     test_merge_and_unmerge_of_box_regions(toma, th, tw, ratio, dim, batch)
+
+
+@pytest.mark.parametrize("dtype,gh,gw,th,tw,ratio", [("bf16", 50, 66, 25, 22, 0.5), ("f32", 50, 66, 25, 22, 0.5), ("f32", 45, 45, 15, 9, 0.1)])
+def test_global_weights_of_more_destinations_than_shared_memory_holds(toma, dtype, gh, gw, th, tw, ratio):
+    """1650 and 1830 destinations, the last warps of tokens and destinations partly filled: every weight against 64-bit arithmetic."""
+    cfg = gen.config("cfg2", batch=2, grid_h=gh, grid_w=gw, tile_h=th, tile_w=tw, dim=64, n_heads=1, merge_ratio=ratio, dtype=dtype)
+    run = Run(toma, cfg, gen.features(cfg), global_merge=True)
+    idx = run.select()
+    d = cfg.n_tiles * run.d_loc
+    run.t.toma_merge_weights(run.desc, run.x, run.idx, run.w, run.ws, run.status)
+    dense = torch.empty((cfg.batch, 1, d, cfg.n_tokens), dtype=torch.float32, device="cuda")
+    run.t.toma_weights_export(run.desc, run.w, dense)
+    run.ok()
+    ids = O.tile_token_ids(gh, gw, th, tw)
+    x = run.x.double()
+    for b in range(cfg.batch):
+        dest = torch.from_numpy(np.asarray(O.global_destinations(idx[b], ids)).reshape(-1)).cuda()
+        shares = torch.softmax(x[b, dest] @ x[b].T / (cfg.tau * 8.0), dim=0)
+        want = shares / shares.sum(1, keepdim=True)
+        assert float((dense[b, 0].double() - want).abs().max()) <= (1e-4 if dtype == "f32" else 6e-4)  # as in the tests of local weights
