@@ -345,12 +345,14 @@ cudaError_t run(int B, int L, int heads, const void* q, const void* k, const voi
   } else {
     // Groups hide latencies while an SM has one CTA: four (head_dim 64, 260 tokens: 18.8 with one group, 15.6 with four), or
     // three with 40 queries where 32 would leave one more CTA to some SMs (705 tokens, 0.85 per SM: 59 and 37; 2271 tokens, 1.95
-    // per SM: 198, two groups of 32 235; not at head_dim 16, 386 tokens, 1.55 per SM: 23.6, one group of 32 22.2).  With more
+    // per SM: 198, two groups of 32 235; 1986 tokens, 2.7 per SM: 265 and 273, but 343 tokens, 2.8 per SM: 63 and 59; not at head_dim
+    // 16, 386 tokens, 1.55 per SM: 23.6, one group of 32 22.2).  With more
     // CTAs two groups (652 tokens, 2.7 of 32 queries per SM: one 92, two 79, four 85).  Below head_dim 64 there is too little to a key tile
     // for that to pay in the long run: two groups for four tiles and two CTAs per SM at most, else one (head_dim 16,
     // 450 tokens, 3.65 per SM: one 30.9, two 31.4, three 37.4).
     if (per_sm(32) <= 1) return run_one<T, DH, 32, 4>(B, L, heads, q, k, v, o, s);
-    if (per_sm(40) <= 1 || (DH > 16 && per_sm(32) > 2 && per_sm(40) <= 2)) return run_one<T, DH, 40, 3>(B, L, heads, q, k, v, o, s);
+    const bool rounds = (per_sm(32) > 2 && per_sm(40) <= 2) || (L > 1024 && per_sm(32) > 3 && per_sm(40) <= 3);
+    if (per_sm(40) <= 1 || (DH > 16 && rounds)) return run_one<T, DH, 40, 3>(B, L, heads, q, k, v, o, s);
     if constexpr (DH < 64)
       if (L > 4 * kKeys || per_sm(32) > 2) return run_one<T, DH, 32, 1>(B, L, heads, q, k, v, o, s);
     return run_one<T, DH, 32, 2>(B, L, heads, q, k, v, o, s);
