@@ -247,7 +247,8 @@ constexpr int kPairRows = 256, kPairCols = 256, kPairStages = 6;
 // Row blocks that are walked over together.  The 74 tiles under way then need 12 row blocks of A and six or seven column blocks
 // of W at a time, which they read in step; with all rows of A first (61 blocks and one) every k-step came out of DRAM where A is
 // larger than L2.  Panels of 4 to 16 timed on 23 shapes: 12 takes 0.95 to 1.0 of the time of all rows first (1.01 once), 8 and 16 up
-// to 1 and 2 % more than 12.
+// to 1 and 2 % more than 12.  Twelve at most, all panels of a matrix alike: a last one of a few rows shares nothing (6585 x 8448 x 2112 and
+// others of 13 to 37 row blocks 3 % slower with panels of twelve and a rest).
 constexpr int kPanel = 12;
 constexpr int kPairStageBytes = kABytes + 2 * kSlab;     // a CTA's half
 constexpr int kPairStaging = kEpiWarps * 32 * 128;
@@ -275,10 +276,11 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
   const int nk = (K + kKC - 1) / kKC;
   const int mb = (M + kPairRows - 1) / kPairRows, nb = (N + kPairCols - 1) / kPairCols;
   const int pair = blockIdx.x / 2, pairs = gridDim.x / 2;
-  // item -> matrix, panel of kPanel row blocks, column block, row block (fastest)
+  const int panels = (mb + kPanel - 1) / kPanel, panel = (mb + panels - 1) / panels;  // row blocks of a panel, alike but for the last
+  // item -> matrix, panel, column block, row block (fastest)
   auto place = [&](int item, int& m0, int& n0, int& z) {
     z = item / (mb * nb);
-    const int in_z = item - z * mb * nb, first = in_z / (kPanel * nb) * kPanel, in_panel = in_z - first * nb, rows = min(kPanel, mb - first);
+    const int in_z = item - z * mb * nb, first = in_z / (panel * nb) * panel, in_panel = in_z - first * nb, rows = min(panel, mb - first);
     n0 = in_panel / rows * kPairCols;
     m0 = (first + in_panel % rows) * kPairRows;
   };
